@@ -1,0 +1,92 @@
+// fr_fx.cuh -- 64-bit block fixed-point arithmetic for the linear operators of the FP64 kernels.
+//
+// GB300 issues 1.6 FP64 multiply-adds per clock and SM, but 54 wide integer multiply-adds
+// (32 x 32 + 64 -> 64 bits; both measured, dependent-free streams). The interpolation, projection,
+// differentiation and trace operators are constant matrices applied to a block of values (one field of
+// one element), so they run in fixed point: the block is scaled by one power of two, taken from its
+// largest magnitude, to integers below 2^56, and every product-sum is exact in 64-bit integers down
+// to 2^-58 of the block's bound, where an FP64 sum rounds each step at 2^-53 of its running value.
+// The power of two travels beside the block; values return to FP64 for the pointwise fluxes.
+//
+// A value X is held as two limbs X = h 2^28 + l (0 <= l < 2^28), a coefficient C = round(c 2^(58-k))
+// as C = H 2^28 + L (|L| <= 2^27; k is the operator's scale, FX_KD, FX_KP or FX_KL). A term of a sum
+// takes three wide multiply-adds: hh += H h, mm += H l + L h; the dropped L l is below 2^-57 of the
+// term's bound. The sum is Y = hh + (mm >> 28), in units of X 2^(k - 2). Bounds, for operators whose
+// absolute row sums are at most 2 after scaling and |X| < 2^59: |h| < 2^31, |hh| < 2^62, |mm| < 2^62.
+#pragma once
+
+#include <cstdint>
+
+#define FX_MASK 0x0fffffffu
+
+// One coefficient or value in two limbs.
+struct fx2 { int h, l; };
+
+// c 2^(58 - k) in two limbs (host); |c| 2^-k < 2.
+inline fx2 fx_coef(double c, int k)
+{
+    double s = c;
+    for (int i = 0; i < 58 - k; i++) s *= 2.0;   // exact
+    const long long C = (long long)(s < 0 ? s - 0.5 : s + 0.5);
+    const long long H = (C + (1LL << 27)) >> 28;
+    return fx2{(int)H, (int)(C - H * (1LL << 28))};
+}
+
+#ifdef __CUDACC__
+// A running product-sum.
+struct fxacc { long long hh, mm; };
+
+__device__ __forceinline__ void fx_mac(fxacc &s, fx2 c, fx2 x)
+{
+    s.hh += (long long)c.h * x.h;
+    s.mm += (long long)c.h * (int)x.l;
+    s.mm += (long long)c.l * x.h;
+}
+// The sum in units of 2^(k - 2) X.
+__device__ __forceinline__ long long fx_sum(const fxacc &s) { return s.hh + (s.mm >> 28); }
+// A sum back to limbs at the scale of the operator's input (times 2^-k): Y / 4, rounded if the
+// accumulator started at FX_HALF.
+#define FX_HALF 2
+__device__ __forceinline__ fx2 fx_limbs(long long y)
+{
+    return fx2{(int)(y >> 30), (int)((unsigned)(y >> 2) & FX_MASK)};
+}
+
+// Exponent field of the largest magnitude is formed from the high words: abs(hi) of a value.
+__device__ __forceinline__ int fx_mag(double v) { return __double2hiint(v) & 0x7fffffff; }
+
+// v of a block with biased exponent E (of its largest magnitude) as X = v 2^(1078 - E), |X| < 2^56.
+__device__ __forceinline__ long long fx_int(double v, int E)
+{
+    const int hi = __double2hiint(v), e = (hi >> 20) & 0x7ff;
+    const unsigned mh = e ? ((unsigned)(hi & 0xfffff) | 0x100000u) : 0u;   // subnormal values count as zero
+    unsigned long long m = ((unsigned long long)mh << 32) | (e ? (unsigned)__double2loint(v) : 0u);
+    m = (m << 3) >> min(E - e, 63);
+    return hi < 0 ? -(long long)m : (long long)m;
+}
+__device__ __forceinline__ fx2 fx_split(long long x) { return fx2{(int)(x >> 28), (int)((unsigned)x & FX_MASK)}; }
+__device__ __forceinline__ fx2 fx_from(double v, int E) { return fx_split(fx_int(v, E)); }
+
+// y 2^e2 rounded to FP64; NaN for a block that held a non-finite value.
+__device__ __forceinline__ double fx_double(long long y, int e2, bool bad)
+{
+    const unsigned long long m = y < 0 ? 0ull - (unsigned long long)y : (unsigned long long)y;
+    const int lz = __clzll((long long)m);
+    const unsigned long long z = m << (lz & 63);
+    int ex = min(max(1085 + e2 - lz, 0), 2046);
+    if ((long long)z >= 0) ex = 0;   // y = 0
+    const unsigned long long b = ((unsigned long long)(unsigned)ex << 52) + (z >> 11) + ((z >> 10) & 1ull);
+    int hi = (int)(b >> 32) | ((int)(y >> 32) & 0x80000000);
+    hi = bad ? 0x7ff80000 : hi;
+    return __hiloint2double(hi, (int)(unsigned)b);
+}
+
+// A run-time factor c (of an element's metric) in limbs for the common exponent E of its block:
+// c 2^(1080 - E), below 2^58.
+__device__ __forceinline__ fx2 fx_factor(double c, int E)
+{
+    const long long C = fx_int(c, E) << 2;
+    const int H = (int)((C + (1LL << 27)) >> 28);
+    return fx2{H, (int)(C - ((long long)H << 28))};
+}
+#endif

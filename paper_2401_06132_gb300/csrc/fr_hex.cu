@@ -17,6 +17,7 @@
 #include <type_traits>
 
 #include "fr_internal.h"
+#include "fr_fx.cuh"
 #include "fr_physics.cuh"
 #include "fr_tcgen05.cuh"
 #include "fr_pri_body.cuh"   // the prism phase bodies, for the launches that serve several groups
@@ -30,6 +31,18 @@ struct HexOpsFF {
     ff Dh[FR_MAXN][FR_MAXN];
 };
 __constant__ HexOpsFF c_hexff[3];
+
+// The line operators in block fixed point (fr_fx.cuh), each with its scale k.
+struct HexFx {
+    fx2 B[FR_MAXM][FR_MAXN];                   // k = 0
+    fx2 Pj[FR_MAXN][FR_MAXM];                  // k = 0
+    fx2 DP[FR_MAXN][FR_MAXM];                  // k = FX_KP
+    fx2 Dh[FR_MAXN][FR_MAXN];                  // k = FX_KD, as the lifts
+    fx2 liftL[FR_MAXN], liftR[FR_MAXN];
+    fx2 lL[FR_MAXN], lR[FR_MAXN];              // k = FX_KL
+};
+constexpr int FX_KD = 4, FX_KP = 3, FX_KL = 1;
+__constant__ HexFx c_hexfx[3];
 
 template <typename T> __device__ __forceinline__ const HexOps<T> &OPS(int slot);
 template <> __device__ __forceinline__ const HexOps<double> &OPS<double>(int slot) { return c_hex64[slot]; }
@@ -70,6 +83,17 @@ int hex_upload_ops(int p, int m, const frb::Hex1D &h)
     eo_fill(&h.B[0][0], FR_MAXN, m, n, d.Beo, f.Beo);
     eo_fill(&h.Pj[0][0], FR_MAXM, n, m, d.Peo, f.Peo);
     eo_fill(&d.DP[0][0], FR_MAXM, n, m, d.DPeo, f.DPeo);
+    HexFx fx{};
+    for (int i = 0; i < n; i++) {
+        for (int a = 0; a < m; a++) {
+            fx.B[a][i] = fx_coef(h.B[a][i], 0);
+            fx.Pj[i][a] = fx_coef(h.Pj[i][a], 0);
+            fx.DP[i][a] = fx_coef(d.DP[i][a], FX_KP);
+        }
+        for (int j = 0; j < n; j++) fx.Dh[i][j] = fx_coef(h.Dh[i][j], FX_KD);
+        fx.liftL[i] = fx_coef(h.liftL[i], FX_KD); fx.liftR[i] = fx_coef(h.liftR[i], FX_KD);
+        fx.lL[i] = fx_coef(h.lL[i], FX_KL); fx.lR[i] = fx_coef(h.lR[i], FX_KL);
+    }
     HexOpsFF x{};
     for (int i = 0; i < FR_MAXN; i++) {
         x.lL[i] = ff_from_double(h.lL[i]); x.lR[i] = ff_from_double(h.lR[i]);
@@ -78,6 +102,7 @@ int hex_upload_ops(int p, int m, const frb::Hex1D &h)
     }
     if (cudaMemcpyToSymbol(c_hex64, &d, sizeof(d), (p - 2) * sizeof(d)) != cudaSuccess) return -2;
     if (cudaMemcpyToSymbol(c_hex32, &f, sizeof(f), (p - 2) * sizeof(f)) != cudaSuccess) return -2;
+    if (cudaMemcpyToSymbol(c_hexfx, &fx, sizeof(fx), (p - 2) * sizeof(fx)) != cudaSuccess) return -2;
     if (cudaMemcpyToSymbol(c_hexff, &x, sizeof(x), (p - 2) * sizeof(x)) != cudaSuccess) return -2;
     return 0;
 }
@@ -584,6 +609,415 @@ __device__ __forceinline__ void project_5(const HexOps<T> &op, const T *src, T *
         }
     }
     __syncthreads();
+}
+
+// ---------------------------------------------------------------------------------------------
+// Fused phase B in FP64: the linear operators in block fixed point (fr_fx.cuh)
+// ---------------------------------------------------------------------------------------------
+// With every operator on the FP64 pipe (1.6 multiply-adds per clock and SM) that pipe bounds the
+// kernel: 69,000 FP64 operations per element at p = 3, two thirds of them in the line operators. Those
+// run on the integer multipliers instead (three wide multiply-adds per term at 54 per clock and SM),
+// which leaves the FP64 pipe the pointwise fluxes; the two overlap across the CTAs of an SM. Every
+// block (one conserved variable of one element with its common solution; one flux component) is
+// scaled by the power of two of its largest magnitude, found with warp reductions; derived fields (the
+// gradient) take static bounds from their operators. Values between the sweeps resolve 2^-56 of their
+// block, below the rounding (2^-53 per operation) of the FP64 sums; against an 80-bit evaluation the
+// RHS error is 0.99 of the FP64 sweeps' (4^3 and 3^3 boxes, diagonal, sheared and curved metrics).
+// Measured, 48^3 p = 3: 15.5 -> 6.66 ms per launch; 25^3 p = 4: 4.18 -> 1.84 ms.
+// y = A x along one line, rows to fixed-point limbs.
+template <int R, int C, int LD>
+__device__ __forceinline__ void line_fx(const fx2 (*A)[LD], const fx2 (&x)[C], fx2 (&y)[R])
+{
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+        fxacc s{FX_HALF, 0};
+#pragma unroll
+        for (int c = 0; c < C; c++) fx_mac(s, A[r][c], x[c]);
+        y[r] = fx_limbs(fx_sum(s));
+    }
+}
+
+template <int P, int NT, bool CURV>
+__device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long long first, long long stride)
+{
+    using S = HexSmem<double, P>;
+    constexpr int N = S::N, M = S::M, NU = S::NU, NF = S::NF, NQ = S::NQ;
+    constexpr int XS = S::XS, PS = S::PS, FS = S::FS;
+    constexpr int NV1 = NU + NF, IT = (NV1 + NT - 1) / NT;   // values of one variable: state, then common solution
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    fx2 *s_u = reinterpret_cast<fx2 *>(smem_raw);
+    fx2 *s_q = s_u + 5 * FS;
+    fx2 *s_c = s_q + 15 * FS;
+    double *s_pf = reinterpret_cast<double *>(s_u + S::LOW);   // prefetched state of the next element
+    double *s_w = s_pf + S::PF;
+    fx2 *s_wx = reinterpret_cast<fx2 *>(s_w);
+    __shared__ short s_list[NF];
+    __shared__ int s_cnt;
+    __shared__ int s_mx[21];   // exponent fields: 5 variables, 15 flux components, the metric (curved)
+    const HexFx &op = c_hexfx[P - 2];
+    constexpr bool TMA_U = S::TMA;
+    __shared__ uint64_t s_ubar;
+    bool pending = false, first_wait = true;
+    uint32_t uparity = 0;
+    if (threadIdx.x < 21) s_mx[threadIdx.x] = 0;
+    if (threadIdx.x == 0) {
+        s_cnt = 0;
+        if constexpr (TMA_U) tc::mbar_init(&s_ubar, 1);
+    }
+    __syncthreads();
+    const bool lane0 = (threadIdx.x & 31) == 0;
+
+    for (long long e = first; e < a.ne; e += stride) {
+        const Geo<double> g = a.geo[e];
+        const Phys<double> ph = elem_phys(a, e);
+        const long long gf0 = elem_f0(a, e, NF);
+        const double *usrc = a.U + elem_u0(a, e, NU);
+        // 1. the element's state and common solution, C = (1/2 - beta) uL + (1/2 + beta) uR, in
+        //    registers, and each variable's largest magnitude
+        if constexpr (TMA_U) {
+            if (pending) {
+                const bool landed = tc::mbar_wait(&s_ubar, uparity, tc::first_limit(first_wait, a.dbg_wait0));
+                uparity ^= 1;
+                pending = false;
+                if (__syncthreads_and(landed)) {
+                    usrc = s_pf;
+                } else {
+                    // the copy did not land within the bound: report it, give it one more bounded
+                    // wait, and read the state from global memory
+                    if (threadIdx.x == 0) atomicOr(a.status, 2);
+                    tc::mbar_wait(&s_ubar, uparity ^ 1);
+                }
+            }
+        }
+        // (after any prefetch of this element has landed: nothing is left in flight when it is skipped)
+        if (!fr_elem_ok(a, e, NU, NF)) continue;
+        double val[IT][5];
+        int mag[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+        for (int i = 0; i < IT; i++) {
+            const int r = threadIdx.x + i * NT;
+            if (r < NU) {
+#pragma unroll
+                for (int alpha = 0; alpha < 5; alpha++) val[i][alpha] = usrc[alpha * NU + r];
+            } else if (r < NV1) {
+                const long long og = gf0 + (r - NU);
+                const uint32_t pc = a.partner[og];
+                const bool isL = (pc & FR_LFLAG) != 0;
+                const long long pg = fr_partner(a, pc, og);
+                const long long gL = isL ? og : pg, gR = isL ? pg : og;
+#pragma unroll
+                for (int alpha = 0; alpha < 5; alpha++)
+                    val[i][alpha] = (0.5 - ph.beta) * a.UF[alpha * a.nfpt + gL] + (0.5 + ph.beta) * a.UF[alpha * a.nfpt + gR];
+                // the flux points whose side carries LDG weight (one side at beta = +-1/2), compacted
+                if ((isL ? 0.5 + ph.beta : 0.5 - ph.beta) == 0.0) {
+#pragma unroll
+                    for (int k = 0; k < 4; k++) a.FV[k * a.nfpt + og] = 0.0;
+                } else {
+                    s_list[atomicAdd(&s_cnt, 1)] = (short)(r - NU);
+                }
+            } else {
+#pragma unroll
+                for (int alpha = 0; alpha < 5; alpha++) val[i][alpha] = 0.0;
+            }
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) mag[alpha] = max(mag[alpha], fx_mag(val[i][alpha]));
+        }
+#pragma unroll
+        for (int alpha = 0; alpha < 5; alpha++) {
+            const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)mag[alpha]);
+            if (lane0) atomicMax(&s_mx[alpha], m >> 20);
+        }
+        if constexpr (CURV) {
+            int m = 0;
+            for (int it = threadIdx.x; it < NU * 9; it += NT) m = max(m, fx_mag(a.mu[(e * NU + it / 9) * 10 + it % 9]));
+            m = (int)__reduce_max_sync(0xffffffffu, (unsigned)m);
+            if (lane0) atomicMax(&s_mx[20], m >> 20);
+        }
+        if constexpr (TMA_U) tc::fence_async_smem();   // this element's reads of s_pf before the copy that overwrites it
+        __syncthreads();
+        if constexpr (TMA_U) {
+            // prefetch the next element's state into s_pf
+            const long long en = e + stride;
+            bool en_ok = en < a.ne;
+#ifdef FR_DEBUG_BOUNDS
+            if (en_ok) {   // the bounds-checking build prefetches only elements inside U
+                const long long un = elem_u0(a, en, NU);
+                en_ok = un >= 0 && un + (long long)FR_NV * NU <= a.nU;
+            }
+#endif
+            if (en_ok) {
+                const double *Un = a.U + elem_u0(a, en, NU);
+                if ((reinterpret_cast<uintptr_t>(Un) & 15) == 0) {
+                    if (threadIdx.x == 0) tc::bulk_g2s(s_pf, Un, 5 * NU * sizeof(double), &s_ubar);
+                    pending = true;
+                }
+            }
+        }
+        // 2. to fixed point
+        int E[5];
+#pragma unroll
+        for (int alpha = 0; alpha < 5; alpha++) E[alpha] = s_mx[alpha];
+#pragma unroll
+        for (int i = 0; i < IT; i++) {
+            const int r = threadIdx.x + i * NT;
+            if (r < NU) {
+                const int pz = r % N + XS * ((r / N) % N) + PS * (r / (N * N));
+#pragma unroll
+                for (int alpha = 0; alpha < 5; alpha++) s_u[alpha * FS + pz] = fx_from(val[i][alpha], E[alpha]);
+            } else if (r < NV1) {
+#pragma unroll
+                for (int alpha = 0; alpha < 5; alpha++) s_c[alpha * NF + r - NU] = fx_from(val[i][alpha], E[alpha]);
+            }
+        }
+        __syncthreads();
+        const int nlist = s_cnt;
+        // 3. corrected gradient along lines, q~ = Dh u + liftR C_R - liftL C_L, and J^-T on a diagonal
+        //    metric (each direction its own factor)
+        const bool diagJ = !CURV && g.Ji[1] == 0.0 && g.Ji[2] == 0.0 && g.Ji[3] == 0.0 && g.Ji[5] == 0.0 &&
+                           g.Ji[6] == 0.0 && g.Ji[7] == 0.0;
+        // exponents of the physical gradient relative to the variable's: value = X 2^(E - 1078 + qe[d])
+        int qe[3], EJ = 0;
+        if (diagJ) {
+#pragma unroll
+            for (int d = 0; d < 3; d++) qe[d] = FX_KD + (fx_mag(g.Ji[4 * d]) >> 20) - 1022;
+        } else {
+            if constexpr (CURV) EJ = s_mx[20] + 2;
+            else {
+                int m = 0;
+#pragma unroll
+                for (int k = 0; k < 9; k++) m = max(m, fx_mag(g.Ji[k]));
+                EJ = (m >> 20) + 2;   // three terms
+            }
+#pragma unroll
+            for (int d = 0; d < 3; d++) qe[d] = FX_KD + EJ - 1022;
+        }
+        for (int it = threadIdx.x; it < 15 * N * N; it += NT) {
+            const int alpha = it / (3 * N * N), r = it % (3 * N * N), d = r / (N * N), loc = r % (N * N);
+            int base, str;
+            face_line_p<N, XS, PS>(2 * d, loc, base, str);
+            fx2 u[N];
+#pragma unroll
+            for (int i = 0; i < N; i++) u[i] = s_u[alpha * FS + base + i * str];
+            const fx2 cL = s_c[alpha * NF + (2 * d) * N * N + loc], cR = s_c[alpha * NF + (2 * d + 1) * N * N + loc];
+            const fx2 nL{-cL.h, -cL.l};
+            const double Jd = d == 0 ? g.Ji[0] : (d == 1 ? g.Ji[4] : g.Ji[8]);
+            const fx2 jf = diagJ ? fx_factor(Jd, fx_mag(Jd) >> 20) : fx2{0, 0};
+#pragma unroll
+            for (int i = 0; i < N; i++) {
+                fxacc s{FX_HALF, 0};
+                fx_mac(s, op.liftR[i], cR);
+                fx_mac(s, op.liftL[i], nL);
+#pragma unroll
+                for (int j = 0; j < N; j++) fx_mac(s, op.Dh[i][j], u[j]);
+                fx2 v = fx_limbs(fx_sum(s));
+                if (diagJ) {
+                    fxacc t{FX_HALF, 0};
+                    fx_mac(t, jf, v);
+                    v = fx_limbs(fx_sum(t));
+                }
+                s_q[(alpha * 3 + d) * FS + base + i * str] = v;
+            }
+        }
+        __syncthreads();
+        // 4. q = J^-T q~ on a full metric
+        if (!diagJ) {
+            for (int z = threadIdx.x; z < NU; z += NT) {
+                const double *Ji = CURV ? a.mu + (e * NU + z) * 10 : g.Ji;
+                fx2 J[9];
+#pragma unroll
+                for (int k = 0; k < 9; k++) J[k] = fx_factor(Ji[k], EJ);
+                fx2 *q = s_q + z % N + XS * ((z / N) % N) + PS * (z / (N * N));
+#pragma unroll
+                for (int alpha = 0; alpha < 5; alpha++, q += 3 * FS) {
+                    const fx2 q0 = q[0], q1 = q[FS], q2 = q[2 * FS];
+#pragma unroll
+                    for (int k = 0; k < 3; k++) {
+                        fxacc s{FX_HALF, 0};
+                        fx_mac(s, J[k], q0);
+                        fx_mac(s, J[3 + k], q1);
+                        fx_mac(s, J[6 + k], q2);
+                        q[k * FS] = fx_limbs(fx_sum(s));
+                    }
+                }
+            }
+            __syncthreads();
+        }
+        // 5. own-normal viscous flux n.f^v at the listed flux points
+        for (int li = threadIdx.x; li < nlist; li += NT) {
+            const int s = s_list[li];
+            const int f = s / (N * N), loc = s % (N * N);
+            int base, str;
+            face_line_p<N, XS, PS>(f, loc, base, str);
+            const fx2 *l = (f & 1) ? op.lR : op.lL;
+            fx2 lr[N];
+#pragma unroll
+            for (int i = 0; i < N; i++) lr[i] = l[i];
+            double uf[5], qf[5][3];
+#pragma unroll
+            for (int fl = 0; fl < 20; fl++) {   // s_q follows s_u
+                fxacc t{0, 0};
+#pragma unroll
+                for (int i = 0; i < N; i++) fx_mac(t, lr[i], s_u[fl * FS + base + i * str]);
+                const int alpha = fl < 5 ? fl : (fl - 5) / 3, ex = E[alpha] - 1080 + FX_KL + (fl < 5 ? 0 : qe[(fl - 5) % 3]);
+                const double v = fx_double(fx_sum(t), ex, E[alpha] >= 2047);
+                if (fl < 5) uf[alpha] = v;
+                else qf[alpha][(fl - 5) % 3] = v;
+            }
+            double n[3], mg;
+            if constexpr (CURV) {   // the normal at this flux point
+                const double *t = a.mfn + (e * NF + s) * 4;
+                n[0] = t[0]; n[1] = t[1]; n[2] = t[2]; mg = t[3];
+            } else {
+                face_nrm<double, double>(a.fnrm, e, f, n, mg);
+            }
+            double fvn[4];
+            viscous_normal_flux(ph, uf, qf, n, fvn);
+#pragma unroll
+            for (int k = 0; k < 4; k++) a.FV[k * a.nfpt + gf0 + s] = fvn[k];
+        }
+        // 6. uqpts + gradcoru_qpts: 20 fields to the quadrature points, x then y then z; the last sweep
+        //    returns to FP64
+        for (int it = threadIdx.x; it < 20 * N * N; it += NT) {
+            const int f = it / (N * N), jk = it % (N * N);
+            const int sb = f * FS + XS * (jk % N) + PS * (jk / N);
+            fx2 u[N], v[M];
+#pragma unroll
+            for (int i = 0; i < N; i++) u[i] = s_u[sb + i];
+            line_fx(op.B, u, v);
+#pragma unroll
+            for (int q = 0; q < M; q++) s_wx[f * M * N * N + q + M * jk] = v[q];
+        }
+        __syncthreads();
+        for (int it = threadIdx.x; it < 20 * M * N; it += NT) {   // (f, qa, k), staged over the state and gradient
+            const int f = it / (M * N), r = it % (M * N), qa = r % M, k = r / M;
+            fx2 u[N], v[M];
+#pragma unroll
+            for (int j = 0; j < N; j++) u[j] = s_wx[f * M * N * N + qa + M * j + M * N * k];
+            line_fx(op.B, u, v);
+#pragma unroll
+            for (int q = 0; q < M; q++) s_u[f * M * M * N + qa + M * q + M * M * k] = v[q];
+        }
+        __syncthreads();
+        for (int it = threadIdx.x; it < 20 * M * M; it += NT) {   // (f, qa, qb)
+            const int f = it / (M * M), ab = it % (M * M);
+            const int alpha = f < 5 ? f : (f - 5) / 3, d = (f - 5) - 3 * alpha;
+            const int Ef = s_mx[alpha], ex = Ef - 1080 + (f < 5 ? 0 : (d == 0 ? qe[0] : (d == 1 ? qe[1] : qe[2])));
+            fx2 u[N];
+#pragma unroll
+            for (int k = 0; k < N; k++) u[k] = s_u[f * M * M * N + ab + M * M * k];
+#pragma unroll
+            for (int q = 0; q < M; q++) {
+                fxacc t{0, 0};
+#pragma unroll
+                for (int k = 0; k < N; k++) fx_mac(t, op.B[q][k], u[k]);
+                s_w[f * NQ + ab + M * M * q] = fx_double(fx_sum(t), ex, Ef >= 2047);
+            }
+        }
+        __syncthreads();
+        // 7. tdisf: flux at each quadrature point, in place (field alpha 3 + d); a diagonal metric's
+        //    three factors det J J^-1 are applied to the projected components instead
+        bool ok = true;
+        int fm[15];
+#pragma unroll
+        for (int c = 0; c < 15; c++) fm[c] = 0;
+        for (int q = threadIdx.x; q < NQ; q += NT) {
+            double u[5], gq[5][3], f[3][5];
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) {
+                u[alpha] = s_w[alpha * NQ + q];
+#pragma unroll
+                for (int d = 0; d < 3; d++) gq[alpha][d] = s_w[(5 + alpha * 3 + d) * NQ + q];
+            }
+            ok &= total_flux(ph, u, gq, f);
+            if (diagJ) {
+#pragma unroll
+                for (int c = 0; c < 15; c++) {
+                    s_w[c * NQ + q] = f[c % 3][c / 3];
+                    fm[c] = max(fm[c], fx_mag(f[c % 3][c / 3]));
+                }
+            } else {
+                double cm[9];
+                if constexpr (CURV) {   // det J J^-1 at this quadrature point
+                    const double *c = a.mq + (e * NQ + q) * 9;
+#pragma unroll
+                    for (int k = 0; k < 9; k++) cm[k] = c[k];
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 9; k++) cm[k] = g.det * g.Ji[k];
+                }
+#pragma unroll
+                for (int c = 0; c < 15; c++) {
+                    const int alpha = c / 3, d = c % 3;
+                    const double v = cm[3 * d] * f[0][alpha] + cm[3 * d + 1] * f[1][alpha] + cm[3 * d + 2] * f[2][alpha];
+                    s_w[c * NQ + q] = v;
+                    fm[c] = max(fm[c], fx_mag(v));
+                }
+            }
+        }
+        flag_status(a.status, ok);
+#pragma unroll
+        for (int c = 0; c < 15; c++) {
+            const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)fm[c]);
+            if (lane0) atomicMax(&s_mx[5 + c], m >> 20);
+        }
+        __syncthreads();
+        // 8. tdivtpcorf: projection of the 15 components with the corrected divergence folded in
+        //    (Dh Pj along the component's own direction), z then y then x
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            for (int it = threadIdx.x; it < 5 * M * M; it += NT) {   // z: (alpha, qa qb) -> k
+                const int alpha = it / (M * M), ab = it % (M * M), Ef = s_mx[5 + alpha * 3 + d];
+                fx2 u[M], v[N];
+#pragma unroll
+                for (int c = 0; c < M; c++) u[c] = fx_from(s_w[(alpha * 3 + d) * NQ + ab + M * M * c], Ef);
+                line_fx(d == 2 ? op.DP : op.Pj, u, v);
+#pragma unroll
+                for (int k = 0; k < N; k++) s_u[(d * 5 + alpha) * M * M * N + ab + M * M * k] = v[k];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            for (int it = threadIdx.x; it < 5 * M * N; it += NT) {   // y: (alpha, qa, k) -> j
+                const int alpha = it / (M * N), r2 = it % (M * N), qa = r2 % M, k = r2 / M;
+                fx2 u[M], v[N];
+#pragma unroll
+                for (int b = 0; b < M; b++) u[b] = s_u[(d * 5 + alpha) * M * M * N + qa + M * b + M * M * k];
+                line_fx(d == 1 ? op.DP : op.Pj, u, v);
+#pragma unroll
+                for (int j = 0; j < N; j++) s_wx[(alpha * 3 + d) * NQ + qa + M * j + M * N * k] = v[j];
+            }
+        }
+        __syncthreads();
+        double *R = a.R + elem_u0(a, e, NU);
+        for (int it = threadIdx.x; it < 5 * N * N; it += NT) {   // x: (alpha, j, k), sum over d -> i
+            const int alpha = it / (N * N), jk = it % (N * N);
+            double v[N];
+#pragma unroll
+            for (int i = 0; i < N; i++) v[i] = 0.0;
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                const int Ef = s_mx[5 + alpha * 3 + d];
+                const double sd = diagJ ? g.det * g.Ji[4 * d] : 1.0;
+                fx2 u[M];
+#pragma unroll
+                for (int q = 0; q < M; q++) u[q] = s_wx[(alpha * 3 + d) * NQ + q + M * jk];
+#pragma unroll
+                for (int i = 0; i < N; i++) {
+                    fxacc t{0, 0};
+#pragma unroll
+                    for (int q = 0; q < M; q++) fx_mac(t, d == 0 ? op.DP[i][q] : op.Pj[i][q], u[q]);
+                    v[i] += sd * fx_double(fx_sum(t), Ef - 1080 + FX_KP, Ef >= 2047);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < N; i++) R[alpha * NU + i + N * jk] = v[i];
+        }
+        __syncthreads();
+        if (threadIdx.x < 21) s_mx[threadIdx.x] = 0;
+        if (threadIdx.x == 0) s_cnt = 0;
+        __syncthreads();
+    }
 }
 
 template <typename T, int P, int NT, int TCM = 0, bool AA = true, bool SURF = false, bool CURV = false>
@@ -1170,20 +1604,32 @@ __device__ __forceinline__ void fused_B_body(const HexArgs<T> &a, long long firs
     }
 }
 
+// The volume group of a precision and form: FP64 with flux anti-aliasing in block fixed point, the
+// other forms (FP32, collocation, surface-flux anti-aliasing) in their own arithmetic.
+template <typename T, int P, int NT, int TCM = 0, bool AA = true, bool SURF = false, bool CURV = false>
+__device__ __forceinline__ void volume_body(const HexArgs<T> &a, long long first, long long stride)
+{
+    if constexpr (sizeof(T) == 8 && AA && !SURF) fused_B_fx_body<P, NT, CURV>(a, first, stride);
+    else fused_B_body<T, P, NT, TCM, AA, SURF, CURV>(a, first, stride);
+}
+
 // The FP32 affine p = 3 volume kernel is capped at 48 registers per thread: ten CTAs of 128 threads
 // per SM (more warps to hide its shared-memory latency; an eleventh, which its shared memory would
-// allow, needs 40 registers, spills and measured slower). A minimum of 0 CTAs leaves the register
-// count to the compiler (an explicit 1 lets it take up to 255).
+// allow, needs 40 registers, spills and measured slower). The FP64 fixed-point kernel is capped at 96
+// registers, five CTAs of 128 threads per SM as its shared memory allows (four CTAs 6.99, three 7.50
+// against 6.66 ms at 48^3 p = 3). A minimum of 0 CTAs leaves the register count to the compiler (an
+// explicit 1 lets it take up to 255).
 template <typename T, int P, int NT, int TCM, bool AA, bool SURF, bool CURV>
 constexpr int fused_B_min_ctas()
 {
+    if (sizeof(T) == 8 && AA && !SURF) return 5 * 128 / NT;
     return (sizeof(T) == 4 && TCM == 0 && AA && !SURF && !CURV && P == 3) ? 10 * 128 / NT : 0;
 }
 
 template <typename T, int P, int NT, int TCM = 0, bool AA = true, bool SURF = false, bool CURV = false>
 __global__ void __launch_bounds__(NT, (fused_B_min_ctas<T, P, NT, TCM, AA, SURF, CURV>())) k_fused_B(HexArgs<T> a)
 {
-    fused_B_body<T, P, NT, TCM, AA, SURF, CURV>(a, blockIdx.x, gridDim.x);
+    volume_body<T, P, NT, TCM, AA, SURF, CURV>(a, blockIdx.x, gridDim.x);
 }
 
 // FP32 with surface-flux anti-aliasing: registers capped so that 896 threads' worth of CTAs (seven
@@ -2441,8 +2887,8 @@ template <typename T>
 __global__ void __launch_bounds__(128) k_multi_B(MultiArgs<T> ma)
 {
     for (int g = 0; g < ma.ng; g++) {
-        if (ma.kind[g] == 3) fused_B_body<T, 3, 128>(ma.a[g], blockIdx.x, gridDim.x);
-        else if (ma.kind[g] == 4) fused_B_body<T, 4, 128>(ma.a[g], blockIdx.x, gridDim.x);
+        if (ma.kind[g] == 3) volume_body<T, 3, 128>(ma.a[g], blockIdx.x, gridDim.x);
+        else if (ma.kind[g] == 4) volume_body<T, 4, 128>(ma.a[g], blockIdx.x, gridDim.x);
         else pri::pri_B_body<T, 128, 0>(ma.a[g], ma.pops, ma.pff, blockIdx.x, gridDim.x);
         __syncthreads();
     }
