@@ -734,6 +734,49 @@ static fr_status upload_priops(fr_mesh *m, void **dst)
     return FR_OK;
 }
 
+// The fixed-point copy of a dense element's FP64 tables. Scales: interpolation, traces and projection
+// end in 64-bit sums (row sums up to 4 after scaling), the gradient in limbs (row sums up to 1).
+template <typename OPS>
+static void fill_dense_fx(OPS &t)
+{
+    constexpr int NU = OPS::NU, NF = OPS::NF, NFACE = OPS::NFACE;
+    auto &x = t.fx;
+    // largest entry and absolute row sum of the operator whose outputs o read terms(o, add)
+    auto scale = [](int nout, auto terms, double limit) {
+        double big = 0, row = 0;
+        for (int o = 0; o < nout; o++) {
+            double s = 0;
+            terms(o, [&](double c) { s += std::fabs(c); big = std::fabs(c) > big ? std::fabs(c) : big; });
+            row = s > row ? s : row;
+        }
+        return fx_scale(big, row, limit);
+    };
+    x.kB = scale(FR_TQ, [&](int q, auto add) { for (int j = 0; j < NU; j++) add(t.Bt[j][q]); }, 4.0);
+    x.kM = scale(NF, [&](int s, auto add) { for (int j = 0; j < NU; j++) add(t.M0t[j][s]); }, 4.0);
+    x.kD = scale(3 * NU, [&](int o, auto add) {
+        const int d = o / NU, z = o % NU;
+        for (int j = 0; j < NU; j++) add(t.Dht[d][j][z]);
+        for (int s = 0; s < NF; s++) add(t.Lt[s][z]);   // times a normal's component, at most 1
+    }, 1.0);
+    x.kV = scale(NU, [&](int z, auto add) {
+        for (int d = 0; d < 3; d++)
+            for (int q = 0; q < FR_TQ; q++) add(t.Dvt[d][q][z]);
+    }, 4.0);
+    for (int j = 0; j < NU; j++) {
+        for (int q = 0; q < FR_TQ; q++) x.Bt[j][q] = fx_coef(t.Bt[j][q], x.kB);
+        for (int s = 0; s < NF; s++) x.M0t[j][s] = fx_coef(t.M0t[j][s], x.kM);
+        for (int d = 0; d < 3; d++)
+            for (int z = 0; z < NU; z++) x.Dht[d][j][z] = fx_coef(t.Dht[d][j][z], x.kD);
+    }
+    for (int s = 0; s < NF; s++)
+        for (int z = 0; z < NU; z++) x.Lt[s][z] = fx_coef(t.Lt[s][z], x.kD);
+    for (int f = 0; f < NFACE; f++)
+        for (int d = 0; d < 3; d++) x.nf[f][d] = fx_coef(t.nf[f][d], 0);
+    for (int d = 0; d < 3; d++)
+        for (int q = 0; q < FR_TQ; q++)
+            for (int z = 0; z < NU; z++) x.Dvt[d][q][z] = fx_coef(t.Dvt[d][q][z], x.kV);
+}
+
 // Transposed dense-element operator tables (DenseOps) from the host construction (DenseRef).
 template <typename T, typename REF, typename OPS>
 static fr_status upload_dense(fr_mesh *m, const REF &R, void **dst)
@@ -763,6 +806,7 @@ static fr_status upload_dense(fr_mesh *m, const REF &R, void **dst)
         t.foff[f] = R.foff[f];
         if (R.foff[f] != (f == NFACE ? NF : OPS::F0(f))) return fail(FR_EUNSUPPORTED, "dense-element face layout");
     }
+    if constexpr (std::is_same<T, double>::value) fill_dense_fx(t);
     fr_status st = dalloc(m, dst, sizeof(OPS));
     if (st) return st;
     CU(cudaMemcpy(*dst, o.data(), sizeof(OPS), cudaMemcpyHostToDevice));

@@ -591,6 +591,241 @@ __global__ void __launch_bounds__(NTH, sizeof(T) == 4 ? (TCM == 0 ? 8 : 6) : 0) 
 }
 
 // -------------------------------------------------------------------------------------------------
+// Phase B in FP64: the dense operators in block fixed point (fr_fx.cuh), one element per CTA
+// -------------------------------------------------------------------------------------------------
+// A dense element's operators are 0.85 (tetrahedron) to 0.9 (pyramid) of its FP64 arithmetic, which
+// bounds the kernel; on the integer multipliers they run beside the pointwise fluxes that stay on the
+// FP64 pipe. Blocks: each variable with its common solution; the three transformed flux components of
+// a variable, which the projection adds up. The quadrature-point fields never leave the registers: a
+// thread interpolates the 20 fields to its point, evaluates the flux there and keeps the 15 transformed
+// components until the CTA knows their largest magnitudes.
+template <typename OPS, int NTH>
+__global__ void __launch_bounds__(NTH, 4) k_dense_B_fx(HexArgs<double> a, const OPS *__restrict__ ops)
+{
+    constexpr int NU = OPS::NU, NF = OPS::NF, NFACE = OPS::NFACE, NUS = OPS::NUS;
+    constexpr int NCH = NTH / NU;                 // quadrature-point chunks of the projection
+    static_assert(NTH == 128 && NU + NF <= NTH, "one thread per quadrature point, state and flux point");
+    static_assert((3 * NQP + NCH - 1) / NCH <= 128, "terms of one 64-bit projection sum");
+    const auto &op = ops->fx;
+    __shared__ __align__(16) fx2 s_u[20 * NUS];          // state, then the physical gradient (5 + 3 alpha + d)
+    __shared__ fx2 s_c[5 * NF];                          // common solution
+    __shared__ __align__(16) fx2 s_w[15 * NQP];          // transformed flux; before it, the traces (FP64)
+    __shared__ long long s_red[NCH * 5 * NU];            // projection partial sums
+    __shared__ short s_plist[NF];
+    __shared__ int s_pcnt, s_mx[10];
+    double *s_tr = reinterpret_cast<double *>(s_w);      // [listed flux point][20]
+    static_assert(NF * 20 <= 15 * NQP, "traces over the flux");
+    const int tid = threadIdx.x;
+    const bool lane0 = (tid & 31) == 0;
+    if constexpr (NUS > NU)   // the pads meet zero operator rows
+        for (int it = tid; it < 20 * (NUS - NU); it += NTH) s_u[(it / (NUS - NU)) * NUS + NU + it % (NUS - NU)] = fx2{0, 0};
+    if (tid < 10) s_mx[tid] = 0;
+    if (tid == 0) s_pcnt = 0;
+    __syncthreads();
+    for (long long e = blockIdx.x; e < a.ne; e += gridDim.x) {
+        if (!fr_elem_ok(a, e, NU, NF)) continue;
+        const Geo<double> g = a.geo[e];
+        const Phys<double> ph = elem_phys(a, e);
+        const long long gf0 = elem_f0(a, e, NF);
+        // 1. state and common solution (one point per thread, five variables), largest magnitudes, and
+        //    the flux points whose side carries LDG weight
+        double val[5] = {0, 0, 0, 0, 0};
+        if (tid < NU) {
+            const double *U = a.U + elem_u0(a, e, NU) + tid;
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) val[alpha] = U[alpha * NU];
+        } else if (tid < NU + NF) {
+            const long long og = gf0 + (tid - NU);
+            const uint32_t pc = a.partner[og];
+            const bool isL = (pc & FR_LFLAG) != 0;
+            const long long pg = fr_partner(a, pc, og), gL = isL ? og : pg, gR = isL ? pg : og;
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++)
+                val[alpha] = (0.5 - ph.beta) * a.UF[alpha * a.nfpt + gL] + (0.5 + ph.beta) * a.UF[alpha * a.nfpt + gR];
+            if ((isL ? 0.5 + ph.beta : 0.5 - ph.beta) == 0.0) {
+#pragma unroll
+                for (int k = 0; k < 4; k++) a.FV[k * a.nfpt + og] = 0.0;
+            } else {
+                s_plist[atomicAdd(&s_pcnt, 1)] = (short)(tid - NU);
+            }
+        }
+#pragma unroll
+        for (int alpha = 0; alpha < 5; alpha++) {
+            const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx_mag(val[alpha]));
+            if (lane0) atomicMax(&s_mx[alpha], m >> 20);
+        }
+        __syncthreads();
+        int E[5];
+#pragma unroll
+        for (int alpha = 0; alpha < 5; alpha++) E[alpha] = s_mx[alpha];
+        if (tid < NU) {
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) s_u[alpha * NUS + tid] = fx_from(val[alpha], E[alpha]);
+        } else if (tid < NU + NF) {
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) s_c[alpha * NF + tid - NU] = fx_from(val[alpha], E[alpha]);
+        }
+        __syncthreads();
+        const int nplist = s_pcnt;
+        // 2. corrected gradient q~_d = Dh_d u + sum_f n_f,d (L_f c), then q = J^-T q~
+        int EJ = 0;
+#pragma unroll
+        for (int k = 0; k < 9; k++) EJ = max(EJ, fx_mag(g.Ji[k]) >> 20);
+        EJ += 2;   // three terms
+        const int qe = op.kD + EJ - 1022;   // gradient: value = X 2^(E - 1078 + qe)
+        for (int it = tid; it < 5 * NU; it += NTH) {
+            const int alpha = it / NU, z = it % NU;
+            const fx2 *u = s_u + alpha * NUS, *c = s_c + alpha * NF;
+            fxacc q[3] = {{FX_HALF, 0}, {FX_HALF, 0}, {FX_HALF, 0}};
+#pragma unroll 4
+            for (int j = 0; j < NU; j++) {
+                const fx2 uj = u[j];
+#pragma unroll
+                for (int d = 0; d < 3; d++) fx_mac(q[d], op.Dht[d][j][z], uj);
+            }
+#pragma unroll 1
+            for (int f = 0; f < NFACE; f++) {
+                fxacc l{FX_HALF, 0};
+                const int s1 = OPS::F0(f + 1);
+#pragma unroll 2
+                for (int s = OPS::F0(f); s < s1; s++) fx_mac(l, op.Lt[s][z], c[s]);
+                const fx2 lf = fx_limbs(fx_sum(l));
+#pragma unroll
+                for (int d = 0; d < 3; d++) fx_mac(q[d], op.nf[f][d], lf);
+            }
+            fx2 qr[3];
+#pragma unroll
+            for (int d = 0; d < 3; d++) qr[d] = fx_limbs(fx_sum(q[d]));
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                fxacc s{FX_HALF, 0};
+#pragma unroll
+                for (int d = 0; d < 3; d++) fx_mac(s, fx_factor(g.Ji[3 * d + k], EJ), qr[d]);
+                s_u[(5 + alpha * 3 + k) * NUS + z] = fx_limbs(fx_sum(s));
+            }
+        }
+        __syncthreads();
+        // 3. traces of the 20 fields at the listed flux points, four threads per point
+        for (int it = tid; it < 4 * nplist; it += NTH) {
+            const int li = it >> 2, fg = it & 3, s = s_plist[li];
+            fxacc t[5] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}, {0, 0}};
+#pragma unroll 2
+            for (int z = 0; z < NU; z++) {
+                const fx2 m = op.M0t[z][s];
+#pragma unroll
+                for (int k = 0; k < 5; k++) fx_mac(t[k], m, s_u[(5 * fg + k) * NUS + z]);
+            }
+#pragma unroll
+            for (int k = 0; k < 5; k++) {
+                const int f = 5 * fg + k, Ea = s_mx[f < 5 ? f : (f - 5) / 3];
+                s_tr[li * 20 + f] = fx_double(fx_sum(t[k]), Ea - 1080 + op.kM + (f < 5 ? 0 : qe), Ea >= 2047);
+            }
+        }
+        // 4. interpolation to this thread's quadrature point and the flux there
+        bool ok = true;
+        double f[3][5];
+        int fm[5] = {0, 0, 0, 0, 0};
+        if (tid < NQ) {
+            fxacc t[20];
+#pragma unroll
+            for (int i = 0; i < 20; i++) t[i] = fxacc{0, 0};
+#pragma unroll 1
+            for (int j = 0; j < NU; j++) {
+                const fx2 b = op.Bt[j][tid];
+#pragma unroll
+                for (int i = 0; i < 20; i++) fx_mac(t[i], b, s_u[i * NUS + j]);
+            }
+            double u[5], gq[5][3];
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) {
+                const int ex = E[alpha] - 1080 + op.kB;
+                u[alpha] = fx_double(fx_sum(t[alpha]), ex, E[alpha] >= 2047);
+#pragma unroll
+                for (int d = 0; d < 3; d++) gq[alpha][d] = fx_double(fx_sum(t[5 + alpha * 3 + d]), ex + qe, E[alpha] >= 2047);
+            }
+            ok = total_flux(ph, u, gq, f);
+            // det J J^-1 f, in place
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) {
+                const double f0 = f[0][alpha], f1 = f[1][alpha], f2 = f[2][alpha];
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    f[d][alpha] = g.det * (g.Ji[3 * d] * f0 + g.Ji[3 * d + 1] * f1 + g.Ji[3 * d + 2] * f2);
+                    fm[alpha] = max(fm[alpha], fx_mag(f[d][alpha]));
+                }
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < 15; c++) f[c % 3][c / 3] = 0.0;   // the pad rows meet zero operator rows
+        }
+        flag_status(a.status, ok);
+#pragma unroll
+        for (int alpha = 0; alpha < 5; alpha++) {
+            const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)fm[alpha]);
+            if (lane0) atomicMax(&s_mx[5 + alpha], m >> 20);
+        }
+        __syncthreads();
+        // 5. own-normal viscous flux at the listed flux points
+        for (int li = tid; li < nplist; li += NTH) {
+            const int s = s_plist[li];
+            const double *v = s_tr + li * 20;
+            double uf[5], qf[5][3];
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) {
+                uf[alpha] = v[alpha];
+#pragma unroll
+                for (int d = 0; d < 3; d++) qf[alpha][d] = v[5 + alpha * 3 + d];
+            }
+            const double *nt = a.fnrm + (e * 6 + OPS::FACE(s)) * 4;
+            const double n[3] = {nt[0], nt[1], nt[2]};
+            double fvn[4];
+            viscous_normal_flux(ph, uf, qf, n, fvn);
+#pragma unroll
+            for (int k = 0; k < 4; k++) a.FV[k * a.nfpt + gf0 + s] = fvn[k];
+        }
+        __syncthreads();
+        // 6. the flux in fixed point
+#pragma unroll
+        for (int alpha = 0; alpha < 5; alpha++) {
+            const int Ef = s_mx[5 + alpha];
+#pragma unroll
+            for (int d = 0; d < 3; d++) s_w[(alpha * 3 + d) * NQP + tid] = fx_from(f[d][alpha], Ef);
+        }
+        __syncthreads();
+        // 7. projection with the corrected divergence: R~[alpha][z] = sum_d sum_q Dv_d[z][q] f~_d[alpha][q],
+        //    thread (z, chunk) over its quadrature points, all variables; then the chunks' sums
+        if (tid < NU * NCH) {
+            const int z = tid % NU, c = tid / NU;
+            const int qb = c * NQP / NCH, qn = (c + 1) * NQP / NCH;
+            fxacc acc[5] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}, {0, 0}};
+#pragma unroll 1
+            for (int d = 0; d < 3; d++)
+#pragma unroll 2
+                for (int q = qb; q < qn; q++) {
+                    const fx2 m = op.Dvt[d][q][z];
+#pragma unroll
+                    for (int alpha = 0; alpha < 5; alpha++) fx_mac(acc[alpha], m, s_w[(alpha * 3 + d) * NQP + q]);
+                }
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) s_red[(c * 5 + alpha) * NU + z] = fx_sum(acc[alpha]);
+        }
+        __syncthreads();
+        double *R = a.R + elem_u0(a, e, NU);
+        for (int it = tid; it < 5 * NU; it += NTH) {
+            long long y = 0;
+#pragma unroll
+            for (int c = 0; c < NCH; c++) y += s_red[c * 5 * NU + it];
+            const int Ef = s_mx[5 + it / NU];
+            R[it] = fx_double(y, Ef - 1080 + op.kV, Ef >= 2047);
+        }
+        __syncthreads();
+        if (tid < 10) s_mx[tid] = 0;
+        if (tid == 0) s_pcnt = 0;
+        __syncthreads();
+    }
+}
+
+// -------------------------------------------------------------------------------------------------
 // Phase C: interface group (common flux at every own flux point, lift and scale)
 // -------------------------------------------------------------------------------------------------
 // FP32: registers capped for 1280 resident threads per SM (eight tetrahedral or five pyramidal CTAs):
@@ -765,7 +1000,9 @@ int dense_phase(int phase, const HexArgs<T> &a, const OPS *ops, const FFOf<OPS> 
                 kern<<<(int)g, NTH, smem, s>>>(a, ops, opsff);
             }
         }
-        if (!tcdone) {
+        if constexpr (sizeof(T) == 8) {
+            k_dense_B_fx<OPS, NTH><<<grid_elems(a.ne, 4), NTH, 0, s>>>(a, ops);
+        } else if (!tcdone) {
             static bool attr = false;
             if (!attr) {
                 cudaFuncSetAttribute(k_dense_B<T, NTH, OPS, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)base);

@@ -32,6 +32,15 @@ inline fx2 fx_coef(double c, int k)
     return fx2{(int)H, (int)(C - H * (1LL << 28))};
 }
 
+// The smallest scale k for which `largest` 2^-k < 1.9 (a coefficient's limb fits 32 bits) and
+// `rowsum` 2^-k <= limit (host).
+inline int fx_scale(double largest, double rowsum, double limit)
+{
+    int k = 0;
+    for (double s = 1.0; largest * s >= 1.9 || rowsum * s > limit; s *= 0.5) k++;
+    return k;
+}
+
 #ifdef __CUDACC__
 // A running product-sum.
 struct fxacc { long long hh, mm; };

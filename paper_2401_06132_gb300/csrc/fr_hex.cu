@@ -17,7 +17,6 @@
 #include <type_traits>
 
 #include "fr_internal.h"
-#include "fr_fx.cuh"
 #include "fr_physics.cuh"
 #include "fr_tcgen05.cuh"
 #include "fr_pri_body.cuh"   // the prism phase bodies, for the launches that serve several groups

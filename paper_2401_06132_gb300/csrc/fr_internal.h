@@ -3,9 +3,11 @@
 
 #include <cuda_runtime.h>
 #include <cstdint>
+#include <type_traits>
 
 #include "../../include/fr_gb300.h"
 #include "fr_ff.cuh"
+#include "fr_fx.cuh"
 
 #define FR_NV 5
 #define FR_MAXN 6          // max 1D solution points (p <= 5)
@@ -141,6 +143,19 @@ struct PriOps {
 // Dense-element (p = 3) operator tables, transposed so that the output index runs fastest (a warp's
 // lanes compute consecutive outputs and read consecutive entries). Rows of the solution-point index
 // are padded to NUS (a multiple of 4) for 16-byte vector loads; the pad rows are zero.
+// The FP64 tables carry them in block fixed point too (fr_fx.cuh), for the FP64 volume kernel.
+template <int NU, int NF, int NFACE>
+struct DenseFx {
+    static constexpr int NUS = (NU + 3) / 4 * 4;
+    fx2 Bt[NUS][FR_TQ];            // scale kB
+    fx2 M0t[NUS][NF];              // kM
+    fx2 Dht[3][NU][NU];            // kD, as the lift
+    fx2 Lt[NF][NU];
+    fx2 nf[NFACE][3];              // 0
+    fx2 Dvt[3][FR_TQP][NU];        // kV
+    int kB, kM, kD, kV;
+};
+struct NoFx {};
 template <typename T, int NU_, int NF_, int NFACE_>
 struct DenseOps {
     static constexpr int NU = NU_, NF = NF_, NFACE = NFACE_, NUS = (NU_ + 3) / 4 * 4;
@@ -156,6 +171,7 @@ struct DenseOps {
     T Dvt[3][FR_TQP][NU];          // (Dh_d Pj)^T: projection with the corrected divergence, [d][q][z]
     T nf[NFACE][3];
     int foff[NFACE + 1];           // F0(f), kept with the table
+    typename std::conditional<std::is_same<T, double>::value, DenseFx<NU, NF, NFACE>, NoFx>::type fx;
 };
 template <typename T> using TetOps = DenseOps<T, 20, 40, 4>;
 template <typename T> using PyrOps = DenseOps<T, 30, 56, 5>;
