@@ -718,15 +718,95 @@ static void fill_priops(const frb::Prism2D &P, PriOps<T> &o)
     }
 }
 
+// The fixed-point copy of the FP64 prism table: sums that end in limbs keep row sums of at most 1 (the
+// in-plane and line gradients, the triangle projection), sums that end in FP64 of at most 4.
+static void fill_prifx(const PriOps<double> &o, PriFx &table)
+{
+    PriFxS &x = table.s;
+    constexpr int NT = FR_PT, NQ = FR_PQ, NZ = FR_PE;
+    double PT[3][NT][NQ], PZ[3][NZ][5];
+    for (int t = 0; t < NT; t++)
+        for (int q = 0; q < NQ; q++) {
+            double vx = 0, vy = 0;
+            for (int j = 0; j < NT; j++) { vx += o.Dhx[t][j] * o.Pt[j][q]; vy += o.Dhy[t][j] * o.Pt[j][q]; }
+            PT[0][t][q] = vx; PT[1][t][q] = vy; PT[2][t][q] = o.Pt[t][q];
+        }
+    for (int k = 0; k < NZ; k++)
+        for (int c = 0; c < 5; c++) {
+            double v = 0;
+            for (int j = 0; j < NZ; j++) v += o.Dhz[k][j] * o.Pz[j][c];
+            PZ[0][k][c] = PZ[1][k][c] = o.Pz[k][c];
+            PZ[2][k][c] = v;
+        }
+    double big, row;
+    auto start = [&]() { big = row = 0; };
+    auto add = [&](double &s, double c) { s += std::fabs(c); big = std::fabs(c) > big ? std::fabs(c) : big; };
+    auto end = [&](double s) { row = s > row ? s : row; };
+    start();
+    for (int q = 0; q < NQ; q++) { double s = 0; for (int t = 0; t < NT; t++) add(s, o.Bt[q][t]); end(s); }
+    x.kB = fx_scale(big, row, 2.0);   // after the line interpolation (row sums below 1.6)
+    start();
+    for (int d = 0; d < 3; d++)
+        for (int t = 0; t < NT; t++) { double s = 0; for (int q = 0; q < NQ; q++) add(s, PT[d][t][q]); end(s); }
+    x.kT = fx_scale(big, row, 1.0);
+    start();
+    for (int k = 0; k < NZ; k++) { double s = 0; for (int d = 0; d < 3; d++) for (int c = 0; c < 5; c++) add(s, PZ[d][k][c]); end(s); }
+    x.kZ = fx_scale(big, row, 4.0);
+    start();
+    for (int t = 0; t < NT; t++) {
+        double s = 0, sy = 0;
+        for (int j = 0; j < NT; j++) { add(s, o.Dhx[t][j]); add(sy, o.Dhy[t][j]); }
+        s = s > sy ? s : sy;
+        for (int f = 0; f < 3; f++) for (int b = 0; b < NZ; b++) add(s, o.Lf[f][t][b]);   // times a normal's component, at most 1
+        end(s);
+    }
+    for (int k = 0; k < NZ; k++) {
+        double s = 0;
+        for (int j = 0; j < NZ; j++) add(s, o.Dhz[k][j]);
+        add(s, o.liftzL[k]); add(s, o.liftzR[k]);
+        end(s);
+    }
+    x.kD = fx_scale(big, row, 1.0);
+    start();
+    for (int f = 0; f < 3; f++) for (int a = 0; a < NZ; a++) { double s = 0; for (int t = 0; t < NT; t++) add(s, o.Ef[f][a][t]); end(s); }
+    { double s = 0, sr = 0; for (int k = 0; k < NZ; k++) { add(s, o.lzL[k]); add(sr, o.lzR[k]); } end(s); end(sr); }
+    x.kF = fx_scale(big, row, 4.0);
+    for (int t = 0; t < NT; t++) {
+        for (int q = 0; q < NQ; q++) {
+            table.Bt[q][t] = fx_coef(o.Bt[q][t], x.kB);
+            for (int d = 0; d < 3; d++) x.PT[d][t][q] = fx_coef(PT[d][t][q], x.kT);
+        }
+        for (int j = 0; j < NT; j++) { x.Dhx[t][j] = fx_coef(o.Dhx[t][j], x.kD); x.Dhy[t][j] = fx_coef(o.Dhy[t][j], x.kD); }
+    }
+    for (int k = 0; k < NZ; k++) {
+        for (int d = 0; d < 3; d++) for (int c = 0; c < 5; c++) x.PZ[d][k][c] = fx_coef(PZ[d][k][c], x.kZ);
+        for (int j = 0; j < NZ; j++) x.Dhz[k][j] = fx_coef(o.Dhz[k][j], x.kD);
+        for (int c = 0; c < 5; c++) x.Bz[c][k] = fx_coef(o.Bz[c][k], 0);
+        x.liftzL[k] = fx_coef(o.liftzL[k], x.kD); x.liftzR[k] = fx_coef(o.liftzR[k], x.kD);
+        x.lzL[k] = fx_coef(o.lzL[k], x.kF); x.lzR[k] = fx_coef(o.lzR[k], x.kF);
+    }
+    for (int f = 0; f < 3; f++) {
+        for (int d = 0; d < 2; d++) x.nf[f][d] = fx_coef(o.nf[f][d], 0);
+        for (int a = 0; a < NZ; a++)
+            for (int t = 0; t < NT; t++) { x.Ef[f][a][t] = fx_coef(o.Ef[f][a][t], x.kF); x.Lf[f][t][a] = fx_coef(o.Lf[f][t][a], x.kD); }
+    }
+}
+
 template <typename T>
 static fr_status upload_priops(fr_mesh *m, void **dst)
 {
     if (!m->has_pri) return FR_OK;
     PriOps<T> o;
     fill_priops<T>(m->pri, o);
-    fr_status st = dalloc(m, dst, sizeof(o));
+    constexpr bool FX = std::is_same<T, double>::value;   // the fixed-point copy follows the FP64 table
+    fr_status st = dalloc(m, dst, sizeof(o) + (FX ? sizeof(PriFx) : 0));
     if (st) return st;
     CU(cudaMemcpy(*dst, &o, sizeof(o), cudaMemcpyHostToDevice));
+    if constexpr (FX) {
+        PriFx x{};
+        fill_prifx(o, x);
+        CU(cudaMemcpy(static_cast<char *>(*dst) + sizeof(o), &x, sizeof(x), cudaMemcpyHostToDevice));
+    }
     if constexpr (sizeof(T) == 4) {
         // the FP32 volume kernels read the interpolation and projection blocks from constant memory
         if (pri_set_const_ops(&o) || multi_set_pri_const_ops(&o)) return fail(FR_ECUDA, "prism operator upload failed");

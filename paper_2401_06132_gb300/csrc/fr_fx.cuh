@@ -47,9 +47,13 @@ struct fxacc { long long hh, mm; };
 
 __device__ __forceinline__ void fx_mac(fxacc &s, fx2 c, fx2 x)
 {
-    s.hh += (long long)c.h * x.h;
-    s.mm += (long long)c.h * (int)x.l;
-    s.mm += (long long)c.l * x.h;
+    long long p, q, r;
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(p) : "r"(c.h), "r"(x.h));
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(q) : "r"(c.h), "r"(x.l));
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(r) : "r"(c.l), "r"(x.h));
+    asm("add.s64 %0, %0, %1;" : "+l"(s.hh) : "l"(p));
+    asm("add.s64 %0, %0, %1;" : "+l"(s.mm) : "l"(q));
+    asm("add.s64 %0, %0, %1;" : "+l"(s.mm) : "l"(r));
 }
 // The sum in units of 2^(k - 2) X.
 __device__ __forceinline__ long long fx_sum(const fxacc &s) { return s.hh + (s.mm >> 28); }

@@ -2888,6 +2888,7 @@ __global__ void __launch_bounds__(128) k_multi_B(MultiArgs<T> ma)
     for (int g = 0; g < ma.ng; g++) {
         if (ma.kind[g] == 3) volume_body<T, 3, 128>(ma.a[g], blockIdx.x, gridDim.x);
         else if (ma.kind[g] == 4) volume_body<T, 4, 128>(ma.a[g], blockIdx.x, gridDim.x);
+        else if constexpr (sizeof(T) == 8) pri::pri_B_fx_body<128>(ma.a[g], ma.pops, blockIdx.x, gridDim.x);
         else pri::pri_B_body<T, 128, 0>(ma.a[g], ma.pops, ma.pff, blockIdx.x, gridDim.x);
         __syncthreads();
     }
@@ -2914,9 +2915,9 @@ static size_t multi_B_smem(const MultiArgs<T> &ma)
         size_t v;
         if (ma.kind[g] == 3) v = HexSmem<T, 3>::SIZE * sizeof(T);
         else if (ma.kind[g] == 4) v = HexSmem<T, 4>::SIZE * sizeof(T);
-        else v = ((sizeof(PriOps<T>) + 15) / 16) * 16 +
-                 (size_t)(5 * pri::NU + 15 * pri::NU + 5 * pri::NF + 20 * pri::NQ) * sizeof(T) +
-                 (size_t)((sizeof(T) == 4 ? 20 : 5) * pri::NZ * pri::NQT) * sizeof(T);
+        else if constexpr (sizeof(T) == 8) v = pri::FX_SMEM;
+        else v = ((sizeof(PriOps<T>) + 15) / 16) * 16 + (size_t)(5 * pri::NU + 15 * pri::NU + 5 * pri::NF + 20 * pri::NQ) * sizeof(T) +
+                 (size_t)(20 * pri::NZ * pri::NQT) * sizeof(T);
         need = v > need ? v : need;
     }
     return need;

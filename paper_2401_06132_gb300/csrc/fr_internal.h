@@ -140,6 +140,25 @@ struct PriOps {
     T lzL[FR_PE], lzR[FR_PE], liftzL[FR_PE], liftzR[FR_PE];
 };
 
+// The prism operators in block fixed point (fr_fx.cuh), for the FP64 volume kernel; it follows the FP64
+// table in memory. The triangle projection carries the corrected in-plane derivatives (PT[0] = Dhx Pt,
+// PT[1] = Dhy Pt, PT[2] = Pt), the line projection the one along z (PZ[2] = Dhz Pz, else Pz).
+struct PriFxS {                                // copied to shared memory by every CTA
+    fx2 PT[3][FR_PT][FR_PQ];                   // scale kT
+    fx2 PZ[3][FR_PE][5];                       // kZ
+    fx2 Dhx[FR_PT][FR_PT], Dhy[FR_PT][FR_PT];  // kD, as Dhz and the lifts
+    fx2 Dhz[FR_PE][FR_PE];
+    fx2 Lf[3][FR_PT][FR_PE], liftzL[FR_PE], liftzR[FR_PE];
+    fx2 nf[3][2];                              // 0
+    fx2 Ef[3][FR_PE][FR_PT], lzL[FR_PE], lzR[FR_PE];   // kF
+    fx2 Bz[5][FR_PE];                          // 0
+    int kB, kT, kZ, kD, kF, pad;
+};
+struct PriFx {
+    fx2 Bt[FR_PQ][FR_PT];                      // kB
+    PriFxS s;
+};
+
 // Dense-element (p = 3) operator tables, transposed so that the output index runs fastest (a warp's
 // lanes compute consecutive outputs and read consecutive entries). Rows of the solution-point index
 // are padded to NUS (a multiple of 4) for 16-byte vector loads; the pad rows are zero.

@@ -35,9 +35,10 @@ __global__ void __launch_bounds__(256) k_pri_disu(HexArgs<T> a, const PriOps<T> 
 // shared memory allows (64 registers, a few spilled values in L1; 72 registers measured slower).
 // Otherwise (0) the compiler's own register count.
 template <typename T, int NTH, int TCM>
-__global__ void __launch_bounds__(NTH, sizeof(T) == 4 && TCM == 0 ? 8 : 0) k_pri_B(HexArgs<T> a, const PriOps<T> *gops, const PriOpsFF *opsff)
+__global__ void __launch_bounds__(NTH, sizeof(T) == 8 ? 5 : (TCM == 0 ? 8 : 0)) k_pri_B(HexArgs<T> a, const PriOps<T> *gops, const PriOpsFF *opsff)
 {
-    pri_B_body<T, NTH, TCM>(a, gops, opsff, blockIdx.x, gridDim.x);
+    if constexpr (sizeof(T) == 8) pri_B_fx_body<NTH>(a, gops, blockIdx.x, gridDim.x);
+    else pri_B_body<T, NTH, TCM>(a, gops, opsff, blockIdx.x, gridDim.x);
 }
 
 // FP32: registers capped for 960 resident threads per SM (ten CTAs of 96), as for the hexahedra
@@ -101,7 +102,7 @@ int pri_fused_phase(int phase, const HexArgs<T> &a, const PriOps<T> *ops, const 
         }
         if (!tcdone) {
             // FP32 interpolates all 20 fields per pass (staging 20 x 4 x 25 values)
-            const size_t smem = base + (size_t)((sizeof(T) == 4 ? 20 : 5) * NZ * NQT) * sizeof(T);
+            const size_t smem = sizeof(T) == 8 ? FX_SMEM : base + (size_t)(20 * NZ * NQT) * sizeof(T);
             static bool attr = false;
             if (!attr) {
                 cudaFuncSetAttribute(k_pri_B<T, NTH, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

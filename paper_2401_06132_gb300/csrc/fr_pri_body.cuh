@@ -315,6 +315,9 @@ __device__ __forceinline__ void pri_project_all_c(const float *src, float *tmp, 
     __syncthreads();
 }
 
+template <int NTH>
+__device__ __forceinline__ void pri_B_fx_body(const HexArgs<double> &a, const PriOps<double> *gops, long long first, long long stride);
+
 template <typename T, int NTH, int TCM>
 __device__ __forceinline__ void pri_B_body(const HexArgs<T> &a, const PriOps<T> *gops, const PriOpsFF *opsff, long long first, long long stride)
 {
@@ -647,6 +650,270 @@ __device__ __forceinline__ void pri_B_body(const HexArgs<T> &a, const PriOps<T> 
     }
 }
 
+
+// -------------------------------------------------------------------------------------------------
+// Phase B in FP64: the operators in block fixed point (fr_fx.cuh), one element per CTA
+// -------------------------------------------------------------------------------------------------
+// As the dense elements' kernel: the operators on the integer multipliers, the pointwise fluxes on the
+// FP64 pipe that bounded the kernel with every operator on it. The line interpolation comes first, so
+// that a thread then interpolates its own quadrature point's 20 fields in the triangle plane and holds
+// them and the flux in registers; the derivatives ride on the projection (Dhx Pt, Dhy Pt, Dhz Pz).
+constexpr int FX_TR = 20 * NF;                        // traces of the listed flux points
+constexpr int FX_S = 20 * MZ * NT_ + FX_TR;           // line-interpolated fields and traces, then the flux
+static_assert(FX_S >= 15 * NQ && 20 * NU + 5 * NF >= 15 * MZ * NT_, "staging fits over consumed buffers");
+constexpr size_t FX_SMEM = sizeof(PriFxS) + sizeof(fx2) * (20 * NU + 5 * NF + FX_S);
+
+template <int NTH>
+__device__ __forceinline__ void pri_B_fx_body(const HexArgs<double> &a, const PriOps<double> *gops, long long first, long long stride)
+{
+    static_assert(NTH == 128, "one thread per quadrature point, state and flux point");
+    static_assert(NU + NF <= NTH, "one thread per state and flux point");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ short s_plist[NF];
+    __shared__ int s_pcnt, s_mx[10];
+    const PriFx *gx = reinterpret_cast<const PriFx *>(gops + 1);
+    const PriFxS &op = *reinterpret_cast<const PriFxS *>(smem_raw);
+    const int tid = threadIdx.x;
+    const bool lane0 = (tid & 31) == 0;
+    {
+        const int *src = reinterpret_cast<const int *>(&gx->s);
+        int *dst = reinterpret_cast<int *>(smem_raw);
+        for (int i = tid; i < (int)(sizeof(PriFxS) / sizeof(int)); i += NTH) dst[i] = src[i];
+    }
+    fx2 *s_u = reinterpret_cast<fx2 *>(smem_raw + sizeof(PriFxS));   // state, then the physical gradient (5 + 3 alpha + d)
+    fx2 *s_c = s_u + 20 * NU;                                // common solution
+    fx2 *s_t = s_c + 5 * NF;                                 // [20][c][t] line-interpolated fields
+    double *s_tr = reinterpret_cast<double *>(s_t + 20 * MZ * NT_);
+    fx2 *s_w = s_t;                                          // [15][c][q] transformed flux
+    fx2 *s_p = s_u;                                          // [15][c][t] projected in the triangle plane
+    const int tq = tid < NQ ? tid % NQT : 0, tc_ = tid < NQ ? tid / NQT : 0;   // this thread's quadrature point
+    if (tid < 10) s_mx[tid] = 0;
+    if (tid == 0) s_pcnt = 0;
+    __syncthreads();
+    for (long long e = first; e < a.ne; e += stride) {
+        if (!fr_elem_ok(a, e, NU, NF)) continue;
+        const Geo<double> g = a.geo[e];
+        const Phys<double> ph = elem_phys(a, e);
+        const long long gf0 = elem_f0(a, e, NF);
+        // 1. state and common solution (one point per thread, five variables), largest magnitudes, and
+        //    the flux points whose side carries LDG weight
+        double val[5] = {0, 0, 0, 0, 0};
+        if (tid < NU) {
+            const double *U = a.U + elem_u0(a, e, NU) + tid;
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) val[alpha] = U[alpha * NU];
+        } else if (tid < NU + NF) {
+            const long long og = gf0 + (tid - NU);
+            const uint32_t pc = a.partner[og];
+            const bool isL = (pc & FR_LFLAG) != 0;
+            const long long pg = fr_partner(a, pc, og), gL = isL ? og : pg, gR = isL ? pg : og;
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++)
+                val[alpha] = (0.5 - ph.beta) * a.UF[alpha * a.nfpt + gL] + (0.5 + ph.beta) * a.UF[alpha * a.nfpt + gR];
+            if ((isL ? 0.5 + ph.beta : 0.5 - ph.beta) == 0.0) {
+#pragma unroll
+                for (int k = 0; k < 4; k++) a.FV[k * a.nfpt + og] = 0.0;
+            } else {
+                s_plist[atomicAdd(&s_pcnt, 1)] = (short)(tid - NU);
+            }
+        }
+#pragma unroll
+        for (int alpha = 0; alpha < 5; alpha++) {
+            const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx_mag(val[alpha]));
+            if (lane0) atomicMax(&s_mx[alpha], m >> 20);
+        }
+        __syncthreads();
+        int E[5];
+#pragma unroll
+        for (int alpha = 0; alpha < 5; alpha++) E[alpha] = s_mx[alpha];
+        if (tid < NU) {
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) s_u[alpha * NU + tid] = fx_from(val[alpha], E[alpha]);
+        } else if (tid < NU + NF) {
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) s_c[alpha * NF + tid - NU] = fx_from(val[alpha], E[alpha]);
+        }
+        __syncthreads();
+        const int nplist = s_pcnt;
+        // 2. corrected gradient: triangle planes and z lines, then q = J^-T q~
+        int EJ = 0;
+#pragma unroll
+        for (int k = 0; k < 9; k++) EJ = max(EJ, fx_mag(g.Ji[k]) >> 20);
+        EJ += 2;   // three terms
+        const int qe = op.kD + EJ - 1022;   // gradient: value = X 2^(E - 1078 + qe)
+        for (int it = tid; it < 5 * NU; it += NTH) {
+            const int alpha = it / NU, z = it % NU, k = z / NT_, t = z % NT_;
+            const fx2 *u = s_u + alpha * NU, *c = s_c + alpha * NF;
+            fxacc q[3] = {{FX_HALF, 0}, {FX_HALF, 0}, {FX_HALF, 0}};
+#pragma unroll
+            for (int j = 0; j < NT_; j++) {
+                fx_mac(q[0], op.Dhx[t][j], u[j + 10 * k]);
+                fx_mac(q[1], op.Dhy[t][j], u[j + 10 * k]);
+            }
+#pragma unroll 1
+            for (int f = 0; f < 3; f++) {
+                fxacc l{FX_HALF, 0};
+#pragma unroll
+                for (int b = 0; b < NZ; b++) fx_mac(l, op.Lf[f][t][b], c[20 + 16 * f + b + 4 * k]);
+                const fx2 lf = fx_limbs(fx_sum(l));
+                fx_mac(q[0], op.nf[f][0], lf);
+                fx_mac(q[1], op.nf[f][1], lf);
+            }
+#pragma unroll
+            for (int j = 0; j < NZ; j++) fx_mac(q[2], op.Dhz[k][j], u[t + 10 * j]);
+            fx_mac(q[2], op.liftzR[k], c[10 + t]);
+            fx_mac(q[2], op.liftzL[k], fx2{-c[t].h, -c[t].l});
+            fx2 qr[3];
+#pragma unroll
+            for (int d = 0; d < 3; d++) qr[d] = fx_limbs(fx_sum(q[d]));
+#pragma unroll
+            for (int kk = 0; kk < 3; kk++) {
+                fxacc s{FX_HALF, 0};
+#pragma unroll
+                for (int d = 0; d < 3; d++) fx_mac(s, fx_factor(g.Ji[3 * d + kk], EJ), qr[d]);
+                s_u[(5 + alpha * 3 + kk) * NU + z] = fx_limbs(fx_sum(s));
+            }
+        }
+        __syncthreads();
+        // 3. traces of the 20 fields at the listed flux points, four threads per point
+        for (int it = tid; it < 4 * nplist; it += NTH) {
+            const int li = it >> 2, fg = it & 3, s = s_plist[li];
+            fxacc t[5] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}, {0, 0}};
+            const fx2 *x = s_u + 5 * fg * NU;
+            if (s < 20) {
+                const fx2 *l = s < 10 ? op.lzL : op.lzR;
+                x += s % 10;
+#pragma unroll
+                for (int k = 0; k < NZ; k++)
+#pragma unroll
+                    for (int i = 0; i < 5; i++) fx_mac(t[i], l[k], x[i * NU + 10 * k]);
+            } else {
+                const int f = (s - 20) / 16, loc = (s - 20) % 16;
+                const fx2 *l = op.Ef[f][loc % 4];
+                x += 10 * (loc / 4);
+#pragma unroll 2
+                for (int j = 0; j < NT_; j++)
+#pragma unroll
+                    for (int i = 0; i < 5; i++) fx_mac(t[i], l[j], x[i * NU + j]);
+            }
+#pragma unroll
+            for (int i = 0; i < 5; i++) {
+                const int f = 5 * fg + i, Ea = s_mx[f < 5 ? f : (f - 5) / 3];
+                s_tr[li * 20 + f] = fx_double(fx_sum(t[i]), Ea - 1080 + op.kF + (f < 5 ? 0 : qe), Ea >= 2047);
+            }
+        }
+        // 4. interpolation: z lines, then this thread's quadrature point in the triangle plane; the flux there
+        for (int it = tid; it < 20 * NT_; it += NTH) {
+            const int f = it / NT_, t = it % NT_;
+            fx2 u[NZ];
+#pragma unroll
+            for (int k = 0; k < NZ; k++) u[k] = s_u[f * NU + t + 10 * k];
+#pragma unroll
+            for (int c = 0; c < MZ; c++) {
+                fxacc s{FX_HALF, 0};
+#pragma unroll
+                for (int k = 0; k < NZ; k++) fx_mac(s, op.Bz[c][k], u[k]);
+                s_t[(f * MZ + c) * NT_ + t] = fx_limbs(fx_sum(s));
+            }
+        }
+        __syncthreads();
+        bool ok = true;
+        double f[3][5];
+        int fm[5] = {0, 0, 0, 0, 0};
+        if (tid < NQ) {
+            fx2 b[NT_];
+#pragma unroll
+            for (int t = 0; t < NT_; t++) b[t] = gx->Bt[tq][t];
+            double u[5], gq[5][3];
+#pragma unroll
+            for (int i = 0; i < 20; i++) {
+                const fx2 *x = s_t + (i * MZ + tc_) * NT_;
+                fxacc s{0, 0};
+#pragma unroll
+                for (int t = 0; t < NT_; t++) fx_mac(s, b[t], x[t]);
+                const int alpha = i < 5 ? i : (i - 5) / 3;
+                const double v = fx_double(fx_sum(s), E[alpha] - 1080 + op.kB + (i < 5 ? 0 : qe), E[alpha] >= 2047);
+                if (i < 5) u[i] = v;
+                else gq[alpha][(i - 5) % 3] = v;
+            }
+            ok = total_flux(ph, u, gq, f);
+            // det J J^-1 f, in place
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) {
+                const double f0 = f[0][alpha], f1 = f[1][alpha], f2 = f[2][alpha];
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    f[d][alpha] = g.det * (g.Ji[3 * d] * f0 + g.Ji[3 * d + 1] * f1 + g.Ji[3 * d + 2] * f2);
+                    fm[alpha] = max(fm[alpha], fx_mag(f[d][alpha]));
+                }
+            }
+        }
+        flag_status(a.status, ok);
+#pragma unroll
+        for (int alpha = 0; alpha < 5; alpha++) {
+            const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)fm[alpha]);
+            if (lane0) atomicMax(&s_mx[5 + alpha], m >> 20);
+        }
+        // 5. own-normal viscous flux at the listed flux points
+        for (int li = tid; li < nplist; li += NTH) {
+            const int s = s_plist[li];
+            const double *v = s_tr + li * 20;
+            double uf[5], qf[5][3];
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) {
+                uf[alpha] = v[alpha];
+#pragma unroll
+                for (int d = 0; d < 3; d++) qf[alpha][d] = v[5 + alpha * 3 + d];
+            }
+            const double *nt = a.fnrm + (e * 6 + face_of(s)) * 4;
+            const double n[3] = {nt[0], nt[1], nt[2]};
+            double fvn[4];
+            viscous_normal_flux(ph, uf, qf, n, fvn);
+#pragma unroll
+            for (int k = 0; k < 4; k++) a.FV[k * a.nfpt + gf0 + s] = fvn[k];
+        }
+        __syncthreads();
+        // 6. the flux in fixed point, over the interpolated fields and the traces
+        if (tid < NQ) {
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) {
+                const int Ef = s_mx[5 + alpha];
+#pragma unroll
+                for (int d = 0; d < 3; d++) s_w[(alpha * 3 + d) * NQ + tid] = fx_from(f[d][alpha], Ef);
+            }
+        }
+        __syncthreads();
+        // 7. projection with the corrected divergence: triangle planes (Dhx Pt, Dhy Pt, Pt), then z and the
+        //    sum of the three components
+        for (int it = tid; it < 5 * MZ * NT_; it += NTH) {
+            const int alpha = it / (MZ * NT_), r = it % (MZ * NT_), c = r / NT_, t = r % NT_;
+#pragma unroll 1
+            for (int d = 0; d < 3; d++) {
+                const fx2 *x = s_w + (alpha * 3 + d) * NQ + NQT * c, *l = op.PT[d][t];
+                fxacc s{FX_HALF, 0};
+#pragma unroll 5
+                for (int q = 0; q < NQT; q++) fx_mac(s, l[q], x[q]);
+                s_p[(alpha * 3 + d) * MZ * NT_ + r] = fx_limbs(fx_sum(s));
+            }
+        }
+        __syncthreads();
+        double *R = a.R + elem_u0(a, e, NU);
+        for (int it = tid; it < 5 * NU; it += NTH) {
+            const int alpha = it / NU, z = it % NU, k = z / NT_, t = z % NT_;
+            fxacc s{0, 0};
+#pragma unroll
+            for (int d = 0; d < 3; d++)
+#pragma unroll
+                for (int c = 0; c < MZ; c++) fx_mac(s, op.PZ[d][k][c], s_p[(alpha * 3 + d) * MZ * NT_ + c * NT_ + t]);
+            const int Ef = s_mx[5 + alpha];
+            R[it] = fx_double(fx_sum(s), Ef - 1080 + op.kT + op.kZ, Ef >= 2047);
+        }
+        __syncthreads();
+        if (tid < 10) s_mx[tid] = 0;
+        if (tid == 0) s_pcnt = 0;
+        __syncthreads();
+    }
+}
 
 // -------------------------------------------------------------------------------------------------
 // Phase C: interface group
