@@ -1603,6 +1603,359 @@ __device__ __forceinline__ void fused_B_body(const HexArgs<T> &a, long long firs
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// Fused phase B of the low-Mach FP32 form (flux anti-aliasing, affine elements): planes and columns
+// ---------------------------------------------------------------------------------------------
+// The one-element form with a sweep per direction spends its issue slots and shared-memory cycles on the
+// sweeps' traffic: per element at p = 3, 8,500 warp instructions, 2,400 of them arithmetic, and 2,000
+// shared-memory wavefronts, 760 of them bank conflicts. Here a sweep's direction stays in registers
+// wherever one thread can hold it: the x and y factors of the interpolation are one thread's plane
+// (n^2 -> m^2 values), its z factor is formed by the quadrature point's own thread from 16-byte loads
+// that the points of a column share, and the projection is one thread's level (z, then x, then y,
+// streaming row by row). EPB elements per CTA fill the warps; the stages alternate between two buffers.
+// Measured: 5,800 warp instructions and 1,380 wavefronts per element; 48^3 p = 3 0.982 -> 0.781 ms,
+// 32^3 p = 4 0.633 -> 0.541 ms per launch.
+// Layouts: a plane of the state and the gradient starts PS words after the last and a field FS words,
+// which spreads a warp's (field, plane) threads over distinct banks; interpolated planes and fluxes put
+// the line through (a, b) in the 4 words of one 16-byte load, and its remaining values beside each other.
+template <int P, int EPB_>
+struct Hex32 {
+    static constexpr int EPB = EPB_, N = P + 1, M = P + 2, NU = N * N * N, NF = 6 * N * N, NQ = M * M * M, M2 = M * M;
+    static constexpr int PS = P == 3 ? 24 : 25, FS = P == 3 ? 100 : 131;   // solution-point fields
+    static constexpr int IS = P == 3 ? 100 : 184;          // interpolated planes: [field][ab][4], then [field][ab] for k = 4
+    static constexpr int S4 = P == 3 ? 100 : 148, S1 = M2 * (M - 4);       // fluxes: [12][ab][4], then [12][ab][M - 4]
+    static constexpr int W0 = (20 * FS > 12 * (S4 + S1) ? 20 * FS : 12 * (S4 + S1)) / 4 * 4 + 4;   // state and gradient, then the flux
+    static constexpr int W1 = 20 * IS;                     // interpolated planes, then the projected components
+    static constexpr int ES = (W0 + W1 + 5 * NF + 3) / 4 * 4;   // words per element (last the common solution, then the mass flux)
+    static_assert(12 * FS <= W1 && 3 * NU * 2 <= 5 * NF && N <= 5 && ES % 4 == 0, "buffers overlay");
+    static constexpr size_t SMEM = (size_t)EPB * ES * sizeof(float);
+};
+
+template <int P, int EPB, int NT>
+__device__ __forceinline__ void hex_B32_body(const HexArgs<float> &a, long long first, long long stride)
+{
+    using S = Hex32<P, EPB>;
+    constexpr int N = S::N, M = S::M, NU = S::NU, NF = S::NF, NQ = S::NQ, M2 = S::M2, PS = S::PS, FS = S::FS;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float *s_ws = reinterpret_cast<float *>(smem_raw);
+    __shared__ short s_list[EPB * NF];
+    __shared__ int s_cnt, s_full;
+    __shared__ long long s_u0[EPB], s_f0[EPB];
+    __shared__ float s_sc[EPB][3];                 // diagonal J^-1, or 1 (full metric)
+    __shared__ float s_cm[EPB][9];                 // det J J^-1
+    // operator rows selected at run time (a constant-memory load is serialised over a warp's distinct
+    // addresses): the projection's z rows (Pj, Dh Pj), the interpolation's, the traces, Dh in float-float
+    __shared__ float s_z[2][N][M], s_l[2][N];
+    __shared__ __align__(16) float s_b[M][(N + 3) / 4 * 4];
+    __shared__ ff s_dh[N][N];
+    const HexOps<float> &op = OPS<float>(P - 2);
+    const int tid = threadIdx.x;
+    for (int i = tid; i < 2 * N * M; i += NT) s_z[i / (N * M)][(i / M) % N][i % M] = i < N * M ? op.Pj[(i / M) % N][i % M] : op.DP[(i / M) % N][i % M];
+    for (int i = tid; i < M * N; i += NT) s_b[i / N][i % N] = op.B[i / N][i % N];
+    for (int i = tid; i < N * N; i += NT) s_dh[i / N][i % N] = c_hexff[P - 2].Dh[i / N][i % N];
+    for (int i = tid; i < 2 * N; i += NT) s_l[i / N][i % N] = i < N ? op.lL[i] : op.lR[i - N];
+    for (long long e0 = first * EPB; e0 < a.ne; e0 += stride * EPB) {
+        const int nb = (int)((a.ne - e0) < EPB ? (a.ne - e0) : EPB);
+        {
+            bool blk_ok = true;
+            for (int k = 0; k < nb; k++) blk_ok = blk_ok && fr_elem_ok(a, e0 + k, NU, NF);
+            if (!blk_ok) continue;
+        }
+        __syncthreads();   // the last elements' buffers are read
+        if (tid == 0) s_cnt = s_full = 0;
+        __syncthreads();
+        // 1. deviations of the state from the reference state, and the common solution
+        //    C = (1/2 - beta) uL + (1/2 + beta) uR, one point and five variables per thread; the flux
+        //    points whose side carries LDG weight (one side at beta = +-1/2), compacted
+        for (int it = tid; it < nb * (NU + NF); it += NT) {
+            const int el = it / (NU + NF), r = it % (NU + NF);
+            const Phys<float> ph = elem_phys(a, e0 + el);
+            float *w = s_ws + el * S::ES;
+            if (r < NU) {
+                const long long u0 = elem_u0(a, e0 + el, NU);
+                const float *U = a.U + u0 + r;
+                w += r % N + N * ((r / N) % N) + PS * (r / (N * N));
+                w[0] = U[0] - ph.rref;
+#pragma unroll
+                for (int alpha = 1; alpha < 4; alpha++) w[alpha * FS] = U[alpha * NU];
+                w[4 * FS] = U[4 * NU] - ph.eref;
+                if (r == 0) {
+                    const Geo<float> g = a.geo[e0 + el];
+                    const bool diag = g.Ji[1] == 0.f && g.Ji[2] == 0.f && g.Ji[3] == 0.f && g.Ji[5] == 0.f && g.Ji[6] == 0.f && g.Ji[7] == 0.f;
+#pragma unroll
+                    for (int d = 0; d < 3; d++) s_sc[el][d] = diag ? g.Ji[4 * d] : 1.f;
+#pragma unroll
+                    for (int k = 0; k < 9; k++) s_cm[el][k] = g.det * g.Ji[k];
+                    if (!diag) atomicOr(&s_full, 1 << el);
+                    s_u0[el] = u0;
+                    s_f0[el] = elem_f0(a, e0 + el, NF);
+                }
+            } else {
+                const int s = r - NU;
+                const long long og = elem_f0(a, e0 + el, NF) + s;
+                const uint32_t pc = a.partner[og];
+                const bool isL = (pc & FR_LFLAG) != 0;
+                const long long pg = fr_partner(a, pc, og);
+                const float *uL = a.UF + (isL ? og : pg), *uR = a.UF + (isL ? pg : og);
+                const float wl = 0.5f - ph.beta, wr = 0.5f + ph.beta;
+                w += S::W0 + S::W1 + s;
+#pragma unroll
+                for (int alpha = 0; alpha < 5; alpha++, uL += a.nfpt, uR += a.nfpt) w[alpha * NF] = wl * *uL + wr * *uR;
+                if ((isL ? wr : wl) == 0.f) {
+                    float *fv = a.FV + og;
+#pragma unroll
+                    for (int k = 0; k < 4; k++, fv += a.nfpt) *fv = 0.f;
+                } else {
+                    s_list[atomicAdd(&s_cnt, 1)] = (short)(el * NF + s);
+                }
+            }
+        }
+        __syncthreads();
+        const int nlist = s_cnt, fullm = s_full;
+        // 2. corrected gradient along lines, q~ = Dh u + liftR C_R - liftL C_L, and J^-T on diagonal
+        //    metrics (the other elements take the full J^-T in a pass of their own)
+        for (int it = tid; it < 3 * EPB * 5 * N * N; it += NT) {
+            const int g = it / (N * N), loc = it % (N * N), d = g / (EPB * 5), el = (g / 5) % EPB, alpha = g % 5;
+            int base, str;
+            face_line_p<N, N, PS>(2 * d, loc, base, str);
+            float *w = s_ws + el * S::ES + base;
+            const float *c = s_ws + el * S::ES + S::W0 + S::W1 + alpha * NF + 2 * d * N * N + loc;
+            const float sc = s_sc[el][d], cL = c[0], cR = c[N * N];
+            float u[N];
+#pragma unroll
+            for (int k = 0; k < N; k++) u[k] = w[alpha * FS + k * str];
+            w += (5 + alpha * 3 + d) * FS;
+#pragma unroll
+            for (int k = 0; k < N; k++) {
+                float v = op.liftR[k] * cR - op.liftL[k] * cL;
+#pragma unroll
+                for (int j = 0; j < N; j++) v += op.Dh[k][j] * u[j];
+                w[k * str] = v * sc;
+            }
+        }
+        __syncthreads();
+        if (fullm) {
+            for (int it = tid; it < nb * 5 * NU; it += NT) {
+                const int el = it / (5 * NU), r = it % (5 * NU), alpha = r / NU, z = r % NU;
+                if (!((fullm >> el) & 1)) continue;
+                const Geo<float> &g = a.geo[e0 + el];
+                float *q = s_ws + el * S::ES + (5 + alpha * 3) * FS + z % N + N * ((z / N) % N) + PS * (z / (N * N));
+                const float q0 = q[0], q1 = q[FS], q2 = q[2 * FS];
+#pragma unroll
+                for (int k = 0; k < 3; k++) q[k * FS] = g.Ji[k] * q0 + g.Ji[3 + k] * q1 + g.Ji[6 + k] * q2;
+            }
+            __syncthreads();
+        }
+        // 3. own-normal viscous flux at the listed flux points
+        for (int li = tid; li < nlist; li += NT) {
+            const int el = s_list[li] / NF, s = s_list[li] % NF, f = s / (N * N);
+            int base, str;
+            face_line_p<N, N, PS>(f, s % (N * N), base, str);
+            const float *w = s_ws + el * S::ES + base;
+            float lr[N], uf[5], qf[5][3];
+#pragma unroll
+            for (int k = 0; k < N; k++) lr[k] = s_l[f & 1][k];
+#pragma unroll
+            for (int fl = 0; fl < 20; fl++) {
+                float v = 0.f;
+#pragma unroll
+                for (int k = 0; k < N; k++) v += lr[k] * w[fl * FS + k * str];
+                if (fl < 5) uf[fl] = v;
+                else qf[(fl - 5) / 3][(fl - 5) % 3] = v;
+            }
+            const Phys<float> ph = elem_phys(a, e0 + el);
+            uf[0] += ph.rref;
+            uf[4] += ph.eref;
+            float n[3], mag;
+            face_nrm<float, float>(a.fnrm, e0 + el, f, n, mag);
+            float fvn[4];
+            viscous_normal_flux(ph, uf, qf, n, fvn);
+            float *fv = a.FV + s_f0[el] + s;
+#pragma unroll
+            for (int k = 0; k < 4; k++, fv += a.nfpt) *fv = fvn[k];
+        }
+        // 4. the volume part of R~_rho in float-float (rho v lies in the solution space: its L2 projection
+        //    is itself), Dh applied along each direction at the solution points; the transformed mass flux
+        //    over the common solution (consumed). The upper threads take the solution points while the
+        //    lower ones are on the flux-point list.
+        for (int it = NT - 1 - tid; it < nb * NU; it += NT) {
+            const int el = it / NU, z = it % NU;
+            const ff *cm = a.geo64[e0 + el].cm;
+            float *w = s_ws + el * S::ES;
+            const float *u = w + z % N + N * ((z / N) % N) + PS * (z / (N * N));
+            ff *mf = reinterpret_cast<ff *>(w + S::W0 + S::W1) + z;
+            const float m0 = u[FS], m1 = u[2 * FS], m2 = u[3 * FS];
+            if (!((fullm >> el) & 1)) {
+                mf[0] = ff_mul_f(cm[0], m0);
+                mf[NU] = ff_mul_f(cm[4], m1);
+                mf[2 * NU] = ff_mul_f(cm[8], m2);
+            } else {
+#pragma unroll
+                for (int d = 0; d < 3; d++)
+                    mf[d * NU] = ff_add(ff_add(ff_mul_f(cm[3 * d], m0), ff_mul_f(cm[3 * d + 1], m1)), ff_mul_f(cm[3 * d + 2], m2));
+            }
+        }
+        // 5. uqpts + gradcoru_qpts, x and y factors: one thread per (element, field, plane k)
+        for (int it = tid; it < EPB * 20 * N; it += NT) {
+            const int g = it / N, k = it % N, el = g / 20, fl = g % 20;
+            const float *x = s_ws + el * S::ES + fl * FS + PS * k;
+            float out[M2];   // [b][a]
+#pragma unroll
+            for (int q = 0; q < M2; q++) out[q] = 0.f;
+#pragma unroll
+            for (int j = 0; j < N; j++) {
+                float u[N];
+                if constexpr (N == 4) {
+                    const float4 v = *reinterpret_cast<const float4 *>(x + N * j);
+                    u[0] = v.x; u[1] = v.y; u[2] = v.z; u[3] = v.w;
+                } else {
+#pragma unroll
+                    for (int i = 0; i < N; i++) u[i] = x[N * j + i];
+                }
+#pragma unroll
+                for (int qa = 0; qa < M; qa++) {
+                    float v = 0.f;
+#pragma unroll
+                    for (int i = 0; i < N; i++) v += op.B[qa][i] * u[i];
+#pragma unroll
+                    for (int qb = 0; qb < M; qb++) out[qa + M * qb] += op.B[qb][j] * v;
+                }
+            }
+            float *y = s_ws + el * S::ES + S::W0 + fl * S::IS;
+            if (k < 4) {
+#pragma unroll
+                for (int q = 0; q < M2; q++) y[4 * q + k] = out[q];
+            } else {
+#pragma unroll
+                for (int q = 0; q < M2; q++) y[4 * M2 + q] = out[q];
+            }
+        }
+        __syncthreads();
+        for (int it = NT - 1 - tid; it < nb * NU; it += NT) {
+            const int el = it / NU, z = it % NU, i = z % N, j = (z / N) % N, k = z / (N * N);
+            const ff *mf = reinterpret_cast<const ff *>(s_ws + el * S::ES + S::W0 + S::W1);
+            float sh = 0.0f, c = 0.0f;   // compensated dot product (Dot2)
+#pragma unroll
+            for (int b = 0; b < N; b++) {
+                dot2ff_next(s_dh[i][b], mf[b + N * j + N * N * k], sh, c);
+                dot2ff_next(s_dh[j][b], mf[NU + i + N * b + N * N * k], sh, c);
+                dot2ff_next(s_dh[k][b], mf[2 * NU + i + N * j + N * N * b], sh, c);
+            }
+            a.RL[s_u0[el] / FR_NV + z] = two_sum(sh, c);
+        }
+        // 6. z factor and tdisf at each quadrature point (a, b, c), c fastest; the mass has no flux here
+        bool ok = true;
+        for (int it = tid; it < nb * NQ; it += NT) {
+            const int el = it / NQ, q = it % NQ, ab = q / M, c = q % M;
+            const float *y = s_ws + el * S::ES + S::W0 + 4 * ab;
+            float bz[N], u[5], gq[5][3], f[3][5];
+#pragma unroll
+            for (int k = 0; k < N; k++) bz[k] = s_b[c][k];
+#pragma unroll
+            for (int fl = 0; fl < 20; fl++) {
+                const float4 x = *reinterpret_cast<const float4 *>(y + fl * S::IS);
+                float v = bz[0] * x.x;
+                v += bz[1] * x.y;
+                v += bz[2] * x.z;
+                v += bz[3] * x.w;
+                if constexpr (N > 4) v += bz[4] * y[fl * S::IS + 4 * M2 - 3 * ab];
+                if (fl < 5) u[fl] = v;
+                else gq[(fl - 5) / 3][(fl - 5) % 3] = v;
+            }
+            const Phys<float> ph = elem_phys(a, e0 + el);
+            ok &= total_flux_dev(ph, u, gq, f);
+            float *F = s_ws + el * S::ES + (c < 4 ? 4 * ab + c : 12 * S::S4 + (M - 4) * ab + c - 4);
+            const int st = c < 4 ? S::S4 : S::S1;
+            const float *cm = s_cm[el];
+            if (!((fullm >> el) & 1)) {
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    const float s = cm[4 * d];
+#pragma unroll
+                    for (int alpha = 1; alpha < 5; alpha++) F[((alpha - 1) * 3 + d) * st] = s * f[d][alpha];
+                }
+            } else {
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    const float s0 = cm[3 * d], s1 = cm[3 * d + 1], s2 = cm[3 * d + 2];
+#pragma unroll
+                    for (int alpha = 1; alpha < 5; alpha++) F[((alpha - 1) * 3 + d) * st] = s0 * f[0][alpha] + s1 * f[1][alpha] + s2 * f[2][alpha];
+                }
+            }
+        }
+        flag_status(a.status, ok);
+        __syncthreads();
+        // 7. tdivtpcorf: one thread per (element, component (alpha, d), level k): z, then x and y row by
+        //    row, with Dh Pj along d and Pj along the others (the rows in registers and shared memory, one
+        //    code for the three directions: three copies with constant operands missed in the
+        //    instruction cache, 0.90 against 0.81 ms at 48^3 p = 3)
+        for (int t = tid; t < EPB * 12 * N; t += NT) {
+            const int g = t / N, k = t % N, el = g / 12, comp = g % 12, d = comp % 3;
+            const float *y4 = s_ws + el * S::ES + comp * S::S4, *y1 = s_ws + el * S::ES + 12 * S::S4 + comp * S::S1;
+            const float(&Y)[N][M] = s_z[d == 1];
+            float zr[M], X[N][M], out[N][N];   // out: [j][i]
+#pragma unroll
+            for (int c = 0; c < M; c++) zr[c] = s_z[d == 2][k][c];
+#pragma unroll
+            for (int i = 0; i < N; i++)
+#pragma unroll
+                for (int c = 0; c < M; c++) X[i][c] = s_z[d == 0][i][c];
+#pragma unroll
+            for (int j = 0; j < N; j++)
+#pragma unroll
+                for (int i = 0; i < N; i++) out[j][i] = 0.f;
+#pragma unroll 1
+            for (int b = 0; b < M; b++) {
+                float x[N];
+#pragma unroll
+                for (int i = 0; i < N; i++) x[i] = 0.f;
+#pragma unroll
+                for (int qa = 0; qa < M; qa++) {
+                    const int ab = qa + M * b;
+                    const float4 f = *reinterpret_cast<const float4 *>(y4 + 4 * ab);
+                    float v = zr[0] * f.x;
+                    v += zr[1] * f.y;
+                    v += zr[2] * f.z;
+                    v += zr[3] * f.w;
+#pragma unroll
+                    for (int c = 4; c < M; c++) v += zr[c] * y1[(M - 4) * ab + c - 4];
+#pragma unroll
+                    for (int i = 0; i < N; i++) x[i] += X[i][qa] * v;
+                }
+#pragma unroll
+                for (int j = 0; j < N; j++) {
+                    const float yj = Y[j][b];
+#pragma unroll
+                    for (int i = 0; i < N; i++) out[j][i] += yj * x[i];
+                }
+            }
+            float *o = s_ws + el * S::ES + S::W0 + comp * FS + PS * k;
+#pragma unroll
+            for (int j = 0; j < N; j++) {
+                if constexpr (N == 4) *reinterpret_cast<float4 *>(o + N * j) = make_float4(out[j][0], out[j][1], out[j][2], out[j][3]);
+                else {
+#pragma unroll
+                    for (int i = 0; i < N; i++) o[N * j + i] = out[j][i];
+                }
+            }
+        }
+        __syncthreads();
+        // R~[alpha] = the sum of its three components, written to R (finished in phase C, which forms the
+        // mass row from RL)
+        for (int it = tid; it < nb * 4 * NU; it += NT) {
+            const int g = it / NU, z = it % NU, el = g / 4, al = g % 4;
+            const float *y = s_ws + el * S::ES + S::W0 + al * 3 * FS + z % N + N * ((z / N) % N) + PS * (z / (N * N));
+            a.R[s_u0[el] + (al + 1) * NU + z] = (y[0] + y[FS]) + y[2 * FS];
+        }
+    }
+}
+
+template <int P, int EPB, int NT, int MB>
+__global__ void __launch_bounds__(NT, MB) k_hex_B32p(HexArgs<float> a)
+{
+    hex_B32_body<P, EPB, NT>(a, blockIdx.x, gridDim.x);
+}
+
 // The volume group of a precision and form: FP64 with flux anti-aliasing in block fixed point, the
 // other forms (FP32, collocation, surface-flux anti-aliasing) in their own arithmetic.
 template <typename T, int P, int NT, int TCM = 0, bool AA = true, bool SURF = false, bool CURV = false>
@@ -2804,6 +3157,18 @@ static int launch_B32(const HexArgs<float> &a, cudaStream_t s)
     return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
 }
 
+template <int P, int EPB, int NT, int MB>
+static void launch_B32p(const HexArgs<float> &a, cudaStream_t s)
+{
+    constexpr size_t smem = Hex32<P, EPB>::SMEM;
+    static bool attr = false;
+    if (!attr) {
+        cudaFuncSetAttribute(k_hex_B32p<P, EPB, NT, MB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        attr = true;
+    }
+    k_hex_B32p<P, EPB, NT, MB><<<grid_elems((a.ne + EPB - 1) / EPB, MB), NT, smem, s>>>(a);
+}
+
 template <typename T, int P>
 static int fused_phase(int phase, const HexArgs<T> &a, cudaStream_t s, int variant)
 {
@@ -2844,6 +3209,18 @@ static int fused_phase(int phase, const HexArgs<T> &a, cudaStream_t s, int varia
             if (variant == 3) return launch_B32<8, 160, 1>(a, s);
             if (variant == 4) return launch_B32<8, 160, 2>(a, s);
             if (variant == 5) return launch_B32<2, 224, 3, true>(a, s);
+        }
+        if constexpr (std::is_same<T, float>::value) {
+            // the low-Mach form (a handle's instances all carry it or none): planes and columns. Elements
+            // per CTA and CTAs per SM by measurement at 48^3 p = 3 (ms: one element of 96 threads at ten
+            // CTAs 0.798, two of 128 at six 0.781, two of 160 at six 0.806, two of 256 at four 0.867) and
+            // 32^3 p = 4 (one of 128 at six 0.541, at seven 0.554, one of 224 at four 0.607)
+            if (a.geo64 != nullptr) {
+                if (variant == 0) launch_B32p<P, 1, 96, P == 3 ? 10 : 7>(a, s);
+                else if (variant == 2) launch_B32p<P, P == 3 ? 2 : 1, P == 3 ? 160 : 224, P == 3 ? 6 : 4>(a, s);
+                else launch_B32p<P, P == 3 ? 2 : 1, 128, 6>(a, s);
+                return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
+            }
         }
         if (variant == 0) launch_B<T, P, 64>(a, s);
         else if (variant == 2) launch_B<T, P, 256>(a, s);
@@ -2886,6 +3263,14 @@ template <typename T>
 __global__ void __launch_bounds__(128) k_multi_B(MultiArgs<T> ma)
 {
     for (int g = 0; g < ma.ng; g++) {
+        if constexpr (sizeof(T) == 4) {
+            if (ma.a[g].geo64 != nullptr && ma.kind[g] != 1) {
+                if (ma.kind[g] == 3) hex_B32_body<3, 2, 128>(ma.a[g], blockIdx.x, gridDim.x);
+                else hex_B32_body<4, 1, 128>(ma.a[g], blockIdx.x, gridDim.x);
+                __syncthreads();
+                continue;
+            }
+        }
         if (ma.kind[g] == 3) volume_body<T, 3, 128>(ma.a[g], blockIdx.x, gridDim.x);
         else if (ma.kind[g] == 4) volume_body<T, 4, 128>(ma.a[g], blockIdx.x, gridDim.x);
         else if constexpr (sizeof(T) == 8) pri::pri_B_fx_body<128>(ma.a[g], ma.pops, blockIdx.x, gridDim.x);
@@ -2913,7 +3298,8 @@ static size_t multi_B_smem(const MultiArgs<T> &ma)
     size_t need = 0;
     for (int g = 0; g < ma.ng; g++) {
         size_t v;
-        if (ma.kind[g] == 3) v = HexSmem<T, 3>::SIZE * sizeof(T);
+        if (sizeof(T) == 4 && ma.a[g].geo64 != nullptr && ma.kind[g] != 1) v = ma.kind[g] == 3 ? Hex32<3, 2>::SMEM : Hex32<4, 1>::SMEM;
+        else if (ma.kind[g] == 3) v = HexSmem<T, 3>::SIZE * sizeof(T);
         else if (ma.kind[g] == 4) v = HexSmem<T, 4>::SIZE * sizeof(T);
         else if constexpr (sizeof(T) == 8) v = pri::FX_SMEM;
         else v = ((sizeof(PriOps<T>) + 15) / 16) * 16 + (size_t)(5 * pri::NU + 15 * pri::NU + 5 * pri::NF + 20 * pri::NQ) * sizeof(T) +
