@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(NTH, 4) k_dense_B_fx(HexArgs<double> a, const 
             const long long pg = fr_partner(a, pc, og), gL = isL ? og : pg, gR = isL ? pg : og;
 #pragma unroll
             for (int alpha = 0; alpha < 5; alpha++)
-                val[alpha] = (0.5 - ph.beta) * a.UF[alpha * a.nfpt + gL] + (0.5 + ph.beta) * a.UF[alpha * a.nfpt + gR];
+                val[alpha] = fr_common(0.5 - ph.beta, 0.5 + ph.beta, a.UF[alpha * a.nfpt + gL], a.UF[alpha * a.nfpt + gR]);
             if ((isL ? 0.5 + ph.beta : 0.5 - ph.beta) == 0.0) {
 #pragma unroll
                 for (int k = 0; k < 4; k++) a.FV[k * a.nfpt + og] = 0.0;

@@ -65,6 +65,14 @@ __device__ __forceinline__ fx2 fx_limbs(long long y)
     return fx2{(int)(y >> 30), (int)((unsigned)(y >> 2) & FX_MASK)};
 }
 
+// f x for one factor, at the scale of x (times 2^-k of the factor).
+__device__ __forceinline__ fx2 fx_mul(fx2 f, fx2 x)
+{
+    fxacc s{FX_HALF, 0};
+    fx_mac(s, f, x);
+    return fx_limbs(fx_sum(s));
+}
+
 // Exponent field of the largest magnitude is formed from the high words: abs(hi) of a value.
 __device__ __forceinline__ int fx_mag(double v) { return __double2hiint(v) & 0x7fffffff; }
 

@@ -622,7 +622,9 @@ __device__ __forceinline__ void project_5(const HexOps<T> &op, const T *src, T *
 // gradient) take static bounds from their operators. Values between the sweeps resolve 2^-56 of their
 // block, below the rounding (2^-53 per operation) of the FP64 sums; against an 80-bit evaluation the
 // RHS error is 0.99 of the FP64 sweeps' (4^3 and 3^3 boxes, diagonal, sheared and curved metrics).
-// Measured, 48^3 p = 3: 15.5 -> 6.66 ms per launch; 25^3 p = 4: 4.18 -> 1.84 ms.
+// What is left on the FP64 pipe: 80 operations per quadrature point and 70 per viscous flux point, 55% of
+// its cycles; the rest is latency (integer chains, barriers, instruction fetch) at 20 warps per SM.
+// Measured, 48^3 p = 3: 15.5 -> 5.48 ms per launch; 25^3 p = 4: 4.18 -> 1.60 ms.
 // y = A x along one line, rows to fixed-point limbs.
 template <int R, int C, int LD>
 __device__ __forceinline__ void line_fx(const fx2 (*A)[LD], const fx2 (&x)[C], fx2 (&y)[R])
@@ -636,29 +638,49 @@ __device__ __forceinline__ void line_fx(const fx2 (*A)[LD], const fx2 (&x)[C], f
     }
 }
 
+template <int P>
+struct HexFxSmem {
+    using S = HexSmem<double, P>;
+    static constexpr int TRC = S::NF / 2;                  // flux points whose traces are staged at a time
+    static constexpr int XO = 20 * S::M * S::N * S::N;     // the first sweep's output
+    // state, gradient and common solution, then the second sweep's output, then the projection's first
+    static constexpr int LOW = S::LOW;
+    // the first sweep's output and the traces, then the flux, then the projection's second sweep
+    static constexpr int W = XO + 20 * TRC > 15 * S::NQ ? XO + 20 * TRC : 15 * S::NQ;
+    static constexpr size_t SMEM = (size_t)(LOW + S::PF + W) * sizeof(double);
+};
+
 template <int P, int NT, bool CURV>
 __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long long first, long long stride)
 {
     using S = HexSmem<double, P>;
-    constexpr int N = S::N, M = S::M, NU = S::NU, NF = S::NF, NQ = S::NQ;
+    using X = HexFxSmem<P>;
+    constexpr int N = S::N, M = S::M, NU = S::NU, NF = S::NF, NQ = S::NQ, M2 = M * M;
     constexpr int XS = S::XS, PS = S::PS, FS = S::FS;
     constexpr int NV1 = NU + NF, IT = (NV1 + NT - 1) / NT;   // values of one variable: state, then common solution
     extern __shared__ __align__(16) unsigned char smem_raw[];
     fx2 *s_u = reinterpret_cast<fx2 *>(smem_raw);
     fx2 *s_q = s_u + 5 * FS;
     fx2 *s_c = s_q + 15 * FS;
-    double *s_pf = reinterpret_cast<double *>(s_u + S::LOW);   // prefetched state of the next element
+    double *s_pf = reinterpret_cast<double *>(s_u + X::LOW);   // prefetched state of the next element
     double *s_w = s_pf + S::PF;
     fx2 *s_wx = reinterpret_cast<fx2 *>(s_w);
+    double *s_tr = s_w + X::XO;                                // [listed flux point][20]
     __shared__ short s_list[NF];
     __shared__ int s_cnt;
     __shared__ int s_mx[21];   // exponent fields: 5 variables, 15 flux components, the metric (curved)
+    // operator rows selected at run time (a constant-memory load is serialised over distinct addresses)
+    __shared__ fx2 s_l[2][N], s_b[M][N], s_pj[2][N][M];   // (s_pj: Pj, Dh Pj)
     const HexFx &op = c_hexfx[P - 2];
     constexpr bool TMA_U = S::TMA;
     __shared__ uint64_t s_ubar;
     bool pending = false, first_wait = true;
     uint32_t uparity = 0;
     if (threadIdx.x < 21) s_mx[threadIdx.x] = 0;
+    for (int i = threadIdx.x; i < 2 * N; i += NT) s_l[i / N][i % N] = i < N ? op.lL[i] : op.lR[i - N];
+    for (int i = threadIdx.x; i < M * N; i += NT) s_b[i / N][i % N] = op.B[i / N][i % N];
+    for (int i = threadIdx.x; i < 2 * N * M; i += NT)
+        s_pj[i / (N * M)][(i / M) % N][i % M] = i < N * M ? op.Pj[(i / M) % N][i % M] : op.DP[(i / M) % N][i % M];
     if (threadIdx.x == 0) {
         s_cnt = 0;
         if constexpr (TMA_U) tc::mbar_init(&s_ubar, 1);
@@ -671,8 +693,7 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
         const Phys<double> ph = elem_phys(a, e);
         const long long gf0 = elem_f0(a, e, NF);
         const double *usrc = a.U + elem_u0(a, e, NU);
-        // 1. the element's state and common solution, C = (1/2 - beta) uL + (1/2 + beta) uR, in
-        //    registers, and each variable's largest magnitude
+        // 1. the element's state and common solution in registers, and each variable's largest magnitude
         if constexpr (TMA_U) {
             if (pending) {
                 const bool landed = tc::mbar_wait(&s_ubar, uparity, tc::first_limit(first_wait, a.dbg_wait0));
@@ -703,14 +724,14 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
                 const uint32_t pc = a.partner[og];
                 const bool isL = (pc & FR_LFLAG) != 0;
                 const long long pg = fr_partner(a, pc, og);
-                const long long gL = isL ? og : pg, gR = isL ? pg : og;
+                const double *uL = a.UF + (isL ? og : pg), *uR = a.UF + (isL ? pg : og);
 #pragma unroll
-                for (int alpha = 0; alpha < 5; alpha++)
-                    val[i][alpha] = (0.5 - ph.beta) * a.UF[alpha * a.nfpt + gL] + (0.5 + ph.beta) * a.UF[alpha * a.nfpt + gR];
+                for (int alpha = 0; alpha < 5; alpha++, uL += a.nfpt, uR += a.nfpt) val[i][alpha] = fr_common(0.5 - ph.beta, 0.5 + ph.beta, *uL, *uR);
                 // the flux points whose side carries LDG weight (one side at beta = +-1/2), compacted
                 if ((isL ? 0.5 + ph.beta : 0.5 - ph.beta) == 0.0) {
+                    double *fv = a.FV + og;
 #pragma unroll
-                    for (int k = 0; k < 4; k++) a.FV[k * a.nfpt + og] = 0.0;
+                    for (int k = 0; k < 4; k++, fv += a.nfpt) *fv = 0.0;
                 } else {
                     s_list[atomicAdd(&s_cnt, 1)] = (short)(r - NU);
                 }
@@ -759,13 +780,11 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
 #pragma unroll
         for (int i = 0; i < IT; i++) {
             const int r = threadIdx.x + i * NT;
-            if (r < NU) {
-                const int pz = r % N + XS * ((r / N) % N) + PS * (r / (N * N));
+            if (r < NV1) {
+                fx2 *d = r < NU ? s_u + r % N + XS * ((r / N) % N) + PS * (r / (N * N)) : s_c + r - NU;
+                const int st = r < NU ? FS : NF;
 #pragma unroll
-                for (int alpha = 0; alpha < 5; alpha++) s_u[alpha * FS + pz] = fx_from(val[i][alpha], E[alpha]);
-            } else if (r < NV1) {
-#pragma unroll
-                for (int alpha = 0; alpha < 5; alpha++) s_c[alpha * NF + r - NU] = fx_from(val[i][alpha], E[alpha]);
+                for (int alpha = 0; alpha < 5; alpha++) d[alpha * st] = fx_from(val[i][alpha], E[alpha]);
             }
         }
         __syncthreads();
@@ -809,11 +828,7 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
 #pragma unroll
                 for (int j = 0; j < N; j++) fx_mac(s, op.Dh[i][j], u[j]);
                 fx2 v = fx_limbs(fx_sum(s));
-                if (diagJ) {
-                    fxacc t{FX_HALF, 0};
-                    fx_mac(t, jf, v);
-                    v = fx_limbs(fx_sum(t));
-                }
+                if (diagJ) v = fx_mul(jf, v);
                 s_q[(alpha * 3 + d) * FS + base + i * str] = v;
             }
         }
@@ -826,7 +841,7 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
 #pragma unroll
                 for (int k = 0; k < 9; k++) J[k] = fx_factor(Ji[k], EJ);
                 fx2 *q = s_q + z % N + XS * ((z / N) % N) + PS * (z / (N * N));
-#pragma unroll
+#pragma unroll 1
                 for (int alpha = 0; alpha < 5; alpha++, q += 3 * FS) {
                     const fx2 q0 = q[0], q1 = q[FS], q2 = q[2 * FS];
 #pragma unroll
@@ -841,41 +856,58 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
             }
             __syncthreads();
         }
-        // 5. own-normal viscous flux n.f^v at the listed flux points
-        for (int li = threadIdx.x; li < nlist; li += NT) {
-            const int s = s_list[li];
-            const int f = s / (N * N), loc = s % (N * N);
-            int base, str;
-            face_line_p<N, XS, PS>(f, loc, base, str);
-            const fx2 *l = (f & 1) ? op.lR : op.lL;
-            fx2 lr[N];
+        // 5. own-normal viscous flux n.f^v at the listed flux points: the traces of the 20 fields (s_q
+        //    follows s_u) by four threads per point, TRC points at a time, then the flux per point
+        auto traces = [&](int c0) {
+            const int nt = min(nlist - c0, X::TRC);
+            for (int it = threadIdx.x; it < 4 * nt; it += NT) {
+                const int li = it >> 2, fg = it & 3, s = s_list[c0 + li], f = s / (N * N);
+                int base, str;
+                face_line_p<N, XS, PS>(f, s % (N * N), base, str);
+                const fx2 *x = s_u + 5 * fg * FS + base;
+#pragma unroll 1
+                for (int k = 0; k < 5; k++, x += FS) {
+                    const int fl = 5 * fg + k, alpha = fl < 5 ? fl : (fl - 5) / 3, d = (fl - 5) - 3 * alpha, Ef = s_mx[alpha];
+                    fxacc t{0, 0};
 #pragma unroll
-            for (int i = 0; i < N; i++) lr[i] = l[i];
-            double uf[5], qf[5][3];
-#pragma unroll
-            for (int fl = 0; fl < 20; fl++) {   // s_q follows s_u
-                fxacc t{0, 0};
-#pragma unroll
-                for (int i = 0; i < N; i++) fx_mac(t, lr[i], s_u[fl * FS + base + i * str]);
-                const int alpha = fl < 5 ? fl : (fl - 5) / 3, ex = E[alpha] - 1080 + FX_KL + (fl < 5 ? 0 : qe[(fl - 5) % 3]);
-                const double v = fx_double(fx_sum(t), ex, E[alpha] >= 2047);
-                if (fl < 5) uf[alpha] = v;
-                else qf[alpha][(fl - 5) % 3] = v;
+                    for (int i = 0; i < N; i++) fx_mac(t, s_l[f & 1][i], x[i * str]);
+                    s_tr[li * 20 + fl] = fx_double(fx_sum(t), Ef - 1080 + FX_KL + (fl < 5 ? 0 : (d == 0 ? qe[0] : (d == 1 ? qe[1] : qe[2]))), Ef >= 2047);
+                }
             }
-            double n[3], mg;
-            if constexpr (CURV) {   // the normal at this flux point
-                const double *t = a.mfn + (e * NF + s) * 4;
-                n[0] = t[0]; n[1] = t[1]; n[2] = t[2]; mg = t[3];
-            } else {
-                face_nrm<double, double>(a.fnrm, e, f, n, mg);
-            }
-            double fvn[4];
-            viscous_normal_flux(ph, uf, qf, n, fvn);
+        };
+        auto viscous = [&](int c0) {
+            const int nt = min(nlist - c0, X::TRC);
+            for (int li = threadIdx.x; li < nt; li += NT) {
+                const int s = s_list[c0 + li], f = s / (N * N);
+                const double *v = s_tr + li * 20;
+                double uf[5], qf[5][3], n[3], mg, fvn[4];
 #pragma unroll
-            for (int k = 0; k < 4; k++) a.FV[k * a.nfpt + gf0 + s] = fvn[k];
+                for (int alpha = 0; alpha < 5; alpha++) {
+                    uf[alpha] = v[alpha];
+#pragma unroll
+                    for (int d = 0; d < 3; d++) qf[alpha][d] = v[5 + alpha * 3 + d];
+                }
+                if constexpr (CURV) {   // the normal at this flux point
+                    const double *t = a.mfn + (e * NF + s) * 4;
+                    n[0] = t[0]; n[1] = t[1]; n[2] = t[2]; mg = t[3];
+                } else {
+                    face_nrm<double, double>(a.fnrm, e, f, n, mg);
+                }
+                viscous_normal_flux(ph, uf, qf, n, fvn);
+                double *fv = a.FV + gf0 + s;
+#pragma unroll
+                for (int k = 0; k < 4; k++, fv += a.nfpt) *fv = fvn[k];
+            }
+        };
+#pragma unroll 1
+        for (int c0 = X::TRC; c0 < nlist; c0 += X::TRC) {   // (elements whose every face is on the L side)
+            traces(c0);
+            __syncthreads();
+            viscous(c0);
+            __syncthreads();
         }
-        // 6. uqpts + gradcoru_qpts: 20 fields to the quadrature points, x then y then z; the last sweep
-        //    returns to FP64
+        traces(0);
+        // 6. uqpts + gradcoru_qpts, x and y sweeps of the 20 fields
         for (int it = threadIdx.x; it < 20 * N * N; it += NT) {
             const int f = it / (N * N), jk = it % (N * N);
             const int sb = f * FS + XS * (jk % N) + PS * (jk / N);
@@ -887,130 +919,130 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
             for (int q = 0; q < M; q++) s_wx[f * M * N * N + q + M * jk] = v[q];
         }
         __syncthreads();
-        for (int it = threadIdx.x; it < 20 * M * N; it += NT) {   // (f, qa, k), staged over the state and gradient
+        viscous(0);
+        for (int it = threadIdx.x; it < 20 * M * N; it += NT) {   // (f, qa, k) -> [f][ab][k], over the state and gradient
             const int f = it / (M * N), r = it % (M * N), qa = r % M, k = r / M;
             fx2 u[N], v[M];
 #pragma unroll
             for (int j = 0; j < N; j++) u[j] = s_wx[f * M * N * N + qa + M * j + M * N * k];
             line_fx(op.B, u, v);
 #pragma unroll
-            for (int q = 0; q < M; q++) s_u[f * M * M * N + qa + M * q + M * M * k] = v[q];
+            for (int q = 0; q < M; q++) s_u[(f * M2 + qa + M * q) * N + k] = v[q];
         }
         __syncthreads();
-        for (int it = threadIdx.x; it < 20 * M * M; it += NT) {   // (f, qa, qb)
-            const int f = it / (M * M), ab = it % (M * M);
-            const int alpha = f < 5 ? f : (f - 5) / 3, d = (f - 5) - 3 * alpha;
-            const int Ef = s_mx[alpha], ex = Ef - 1080 + (f < 5 ? 0 : (d == 0 ? qe[0] : (d == 1 ? qe[1] : qe[2])));
-            fx2 u[N];
-#pragma unroll
-            for (int k = 0; k < N; k++) u[k] = s_u[f * M * M * N + ab + M * M * k];
-#pragma unroll
-            for (int q = 0; q < M; q++) {
-                fxacc t{0, 0};
-#pragma unroll
-                for (int k = 0; k < N; k++) fx_mac(t, op.B[q][k], u[k]);
-                s_w[f * NQ + ab + M * M * q] = fx_double(fx_sum(t), ex, Ef >= 2047);
-            }
-        }
-        __syncthreads();
-        // 7. tdisf: flux at each quadrature point, in place (field alpha 3 + d); a diagonal metric's
-        //    three factors det J J^-1 are applied to the projected components instead
+        // 7. the z factor and tdisf at each quadrature point (ab, c), c fastest (the points of a column
+        //    share their loads); a diagonal metric's factors det J J^-1 are applied in the projection
         bool ok = true;
         int fm[15];
 #pragma unroll
         for (int c = 0; c < 15; c++) fm[c] = 0;
-        for (int q = threadIdx.x; q < NQ; q += NT) {
+        for (int it = threadIdx.x; it < NQ; it += NT) {
+            const int ab = it / M, c = it % M, q = ab + M2 * c;
+            fx2 bz[N];
+#pragma unroll
+            for (int k = 0; k < N; k++) bz[k] = s_b[c][k];
+            const fx2 *y = s_u + ab * N;
             double u[5], gq[5][3], f[3][5];
 #pragma unroll
-            for (int alpha = 0; alpha < 5; alpha++) {
-                u[alpha] = s_w[alpha * NQ + q];
+            for (int fl = 0; fl < 20; fl++) {
+                fxacc t{0, 0};
 #pragma unroll
-                for (int d = 0; d < 3; d++) gq[alpha][d] = s_w[(5 + alpha * 3 + d) * NQ + q];
+                for (int k = 0; k < N; k++) fx_mac(t, bz[k], y[fl * M2 * N + k]);
+                const int alpha = fl < 5 ? fl : (fl - 5) / 3, d = (fl - 5) % 3;
+                const double v = fx_double(fx_sum(t), E[alpha] - 1080 + (fl < 5 ? 0 : qe[fl < 5 ? 0 : d]), E[alpha] >= 2047);
+                if (fl < 5) u[fl] = v;
+                else gq[alpha][d] = v;
             }
             ok &= total_flux(ph, u, gq, f);
             if (diagJ) {
 #pragma unroll
-                for (int c = 0; c < 15; c++) {
-                    s_w[c * NQ + q] = f[c % 3][c / 3];
-                    fm[c] = max(fm[c], fx_mag(f[c % 3][c / 3]));
+                for (int i = 0; i < 15; i++) {
+                    s_w[i * NQ + q] = f[i % 3][i / 3];
+                    fm[i] = max(fm[i], fx_mag(f[i % 3][i / 3]));
                 }
             } else {
                 double cm[9];
                 if constexpr (CURV) {   // det J J^-1 at this quadrature point
-                    const double *c = a.mq + (e * NQ + q) * 9;
+                    const double *m = a.mq + (e * NQ + q) * 9;
 #pragma unroll
-                    for (int k = 0; k < 9; k++) cm[k] = c[k];
+                    for (int k = 0; k < 9; k++) cm[k] = m[k];
                 } else {
 #pragma unroll
                     for (int k = 0; k < 9; k++) cm[k] = g.det * g.Ji[k];
                 }
 #pragma unroll
-                for (int c = 0; c < 15; c++) {
-                    const int alpha = c / 3, d = c % 3;
+                for (int i = 0; i < 15; i++) {
+                    const int alpha = i / 3, d = i % 3;
                     const double v = cm[3 * d] * f[0][alpha] + cm[3 * d + 1] * f[1][alpha] + cm[3 * d + 2] * f[2][alpha];
-                    s_w[c * NQ + q] = v;
-                    fm[c] = max(fm[c], fx_mag(v));
+                    s_w[i * NQ + q] = v;
+                    fm[i] = max(fm[i], fx_mag(v));
                 }
             }
         }
         flag_status(a.status, ok);
 #pragma unroll
-        for (int c = 0; c < 15; c++) {
-            const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)fm[c]);
-            if (lane0) atomicMax(&s_mx[5 + c], m >> 20);
+        for (int i = 0; i < 15; i++) {
+            const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)fm[i]);
+            if (lane0) atomicMax(&s_mx[5 + i], m >> 20);
         }
         __syncthreads();
         // 8. tdivtpcorf: projection of the 15 components with the corrected divergence folded in
-        //    (Dh Pj along the component's own direction), z then y then x
+        //    (Dh Pj along the component's own direction), z then y then x. The three components of a
+        //    variable, each times its metric factor, are brought to one scale first, so that the x sweep
+        //    adds them up in its sums: component d is read at the exponent EC - es[d].
+        const double sd[3] = {g.det * g.Ji[0], g.det * g.Ji[4], g.det * g.Ji[8]};
+        int es[3];
 #pragma unroll
-        for (int d = 0; d < 3; d++) {
-            for (int it = threadIdx.x; it < 5 * M * M; it += NT) {   // z: (alpha, qa qb) -> k
-                const int alpha = it / (M * M), ab = it % (M * M), Ef = s_mx[5 + alpha * 3 + d];
-                fx2 u[M], v[N];
+        for (int d = 0; d < 3; d++) es[d] = diagJ ? (fx_mag(sd[d]) >> 20) - 1022 : 0;
+        auto common_exp = [&](int alpha) {
+            return max(max(s_mx[5 + alpha * 3] + es[0], s_mx[6 + alpha * 3] + es[1]), s_mx[7 + alpha * 3] + es[2]);
+        };
+        // (one code for the three directions, the operator rows from shared memory: three copies with
+        // constant operands missed in the instruction cache)
+        for (int it = threadIdx.x; it < 15 * M2; it += NT) {   // z: (d, alpha, qa qb) -> k
+            const int da = it / M2, ab = it % M2, d = da / 5, alpha = da % 5, comp = alpha * 3 + d;
+            const double sdd = d == 0 ? sd[0] : (d == 1 ? sd[1] : sd[2]);
+            const int Ef = common_exp(alpha) - (d == 0 ? es[0] : (d == 1 ? es[1] : es[2]));
+            const fx2 fd = fx_factor(sdd, fx_mag(sdd) >> 20);
+            fx2 u[M], v[N];
 #pragma unroll
-                for (int c = 0; c < M; c++) u[c] = fx_from(s_w[(alpha * 3 + d) * NQ + ab + M * M * c], Ef);
-                line_fx(d == 2 ? op.DP : op.Pj, u, v);
-#pragma unroll
-                for (int k = 0; k < N; k++) s_u[(d * 5 + alpha) * M * M * N + ab + M * M * k] = v[k];
+            for (int c = 0; c < M; c++) {
+                u[c] = fx_from(s_w[comp * NQ + ab + M2 * c], Ef);
+                if (diagJ) u[c] = fx_mul(fd, u[c]);
             }
+            line_fx(s_pj[d == 2], u, v);
+#pragma unroll
+            for (int k = 0; k < N; k++) s_u[da * M2 * N + ab + M2 * k] = v[k];
         }
         __syncthreads();
+        for (int it = threadIdx.x; it < 15 * M * N; it += NT) {   // y: (d, alpha, qa, k) -> j
+            const int da = it / (M * N), r2 = it % (M * N), d = da / 5, alpha = da % 5, qa = r2 % M, k = r2 / M;
+            fx2 u[M], v[N];
 #pragma unroll
-        for (int d = 0; d < 3; d++) {
-            for (int it = threadIdx.x; it < 5 * M * N; it += NT) {   // y: (alpha, qa, k) -> j
-                const int alpha = it / (M * N), r2 = it % (M * N), qa = r2 % M, k = r2 / M;
-                fx2 u[M], v[N];
+            for (int b = 0; b < M; b++) u[b] = s_u[da * M2 * N + qa + M * b + M2 * k];
+            line_fx(s_pj[d == 1], u, v);
 #pragma unroll
-                for (int b = 0; b < M; b++) u[b] = s_u[(d * 5 + alpha) * M * M * N + qa + M * b + M * M * k];
-                line_fx(d == 1 ? op.DP : op.Pj, u, v);
-#pragma unroll
-                for (int j = 0; j < N; j++) s_wx[(alpha * 3 + d) * NQ + qa + M * j + M * N * k] = v[j];
-            }
+            for (int j = 0; j < N; j++) s_wx[(alpha * 3 + d) * NQ + qa + M * j + M * N * k] = v[j];
         }
         __syncthreads();
         double *R = a.R + elem_u0(a, e, NU);
         for (int it = threadIdx.x; it < 5 * N * N; it += NT) {   // x: (alpha, j, k), sum over d -> i
             const int alpha = it / (N * N), jk = it % (N * N);
-            double v[N];
+            fxacc t[N];
 #pragma unroll
-            for (int i = 0; i < N; i++) v[i] = 0.0;
+            for (int i = 0; i < N; i++) t[i] = fxacc{0, 0};
+#pragma unroll 1
+            for (int d = 0; d < 3; d++)
 #pragma unroll
-            for (int d = 0; d < 3; d++) {
-                const int Ef = s_mx[5 + alpha * 3 + d];
-                const double sd = diagJ ? g.det * g.Ji[4 * d] : 1.0;
-                fx2 u[M];
+                for (int q = 0; q < M; q++) {
+                    const fx2 u = s_wx[(alpha * 3 + d) * NQ + q + M * jk];
 #pragma unroll
-                for (int q = 0; q < M; q++) u[q] = s_wx[(alpha * 3 + d) * NQ + q + M * jk];
-#pragma unroll
-                for (int i = 0; i < N; i++) {
-                    fxacc t{0, 0};
-#pragma unroll
-                    for (int q = 0; q < M; q++) fx_mac(t, d == 0 ? op.DP[i][q] : op.Pj[i][q], u[q]);
-                    v[i] += sd * fx_double(fx_sum(t), Ef - 1080 + FX_KP, Ef >= 2047);
+                    for (int i = 0; i < N; i++) fx_mac(t[i], s_pj[d == 0][i][q], u);
                 }
-            }
+            const int Ef = common_exp(alpha);
+            const bool bad = max(max(s_mx[5 + alpha * 3], s_mx[6 + alpha * 3]), s_mx[7 + alpha * 3]) >= 2047;
 #pragma unroll
-            for (int i = 0; i < N; i++) R[alpha * NU + i + N * jk] = v[i];
+            for (int i = 0; i < N; i++) R[alpha * NU + i + N * jk] = fx_double(fx_sum(t[i]), Ef - 1080 + FX_KP, bad);
         }
         __syncthreads();
         if (threadIdx.x < 21) s_mx[threadIdx.x] = 0;
@@ -1968,8 +2000,8 @@ __device__ __forceinline__ void volume_body(const HexArgs<T> &a, long long first
 // The FP32 affine p = 3 volume kernel is capped at 48 registers per thread: ten CTAs of 128 threads
 // per SM (more warps to hide its shared-memory latency; an eleventh, which its shared memory would
 // allow, needs 40 registers, spills and measured slower). The FP64 fixed-point kernel is capped at 96
-// registers, five CTAs of 128 threads per SM as its shared memory allows (four CTAs 6.99, three 7.50
-// against 6.66 ms at 48^3 p = 3). A minimum of 0 CTAs leaves the register count to the compiler (an
+// registers, five CTAs of 128 threads per SM as its shared memory allows (measured on its first form: four CTAs
+// 6.99, three 7.50, five 6.66 ms at 48^3 p = 3). A minimum of 0 CTAs leaves the register count to the compiler (an
 // explicit 1 lets it take up to 255).
 template <typename T, int P, int NT, int TCM, bool AA, bool SURF, bool CURV>
 constexpr int fused_B_min_ctas()
@@ -2077,9 +2109,12 @@ __device__ __forceinline__ void fused_C_body(const HexArgs<T> &a, long long firs
                 const int alpha = it / NU, z = it % NU, i = z % N, j = (z / N) % N, k = z / (N * N);
                 const T *D = s_d + alpha * NF;
                 T v = R[it];
-                v += liftL[i] * D[0 * N * N + j + N * k] + liftR[i] * D[1 * N * N + j + N * k];
-                v += liftL[j] * D[2 * N * N + i + N * k] + liftR[j] * D[3 * N * N + i + N * k];
-                v += liftL[k] * D[4 * N * N + i + N * j] + liftR[k] * D[5 * N * N + i + N * j];
+                v += liftL[i] * D[0 * N * N + j + N * k];
+                v += liftR[i] * D[1 * N * N + j + N * k];
+                v += liftL[j] * D[2 * N * N + i + N * k];
+                v += liftR[j] * D[3 * N * N + i + N * k];
+                v += liftL[k] * D[4 * N * N + i + N * j];
+                v += liftR[k] * D[5 * N * N + i + N * j];
                 // curved elements: det J at this solution point
                 const T sc = CURV ? T(-1) / a.mu[(e * NU + z) * 10 + 9] : idet;
                 if (a.rkstage == 0) R[it] = v * sc;
@@ -2095,9 +2130,12 @@ __device__ __forceinline__ void fused_C_body(const HexArgs<T> &a, long long firs
                 for (int alpha = 0; alpha < 5; alpha++) {
                     const T *D = s_d + alpha * NF;
                     T v = R[alpha * NU + z];
-                    v += liftL[i] * D[0 * N * N + j + N * k] + liftR[i] * D[1 * N * N + j + N * k];
-                    v += liftL[j] * D[2 * N * N + i + N * k] + liftR[j] * D[3 * N * N + i + N * k];
-                    v += liftL[k] * D[4 * N * N + i + N * j] + liftR[k] * D[5 * N * N + i + N * j];
+                    v += liftL[i] * D[0 * N * N + j + N * k];
+                    v += liftR[i] * D[1 * N * N + j + N * k];
+                    v += liftL[j] * D[2 * N * N + i + N * k];
+                    v += liftR[j] * D[3 * N * N + i + N * k];
+                    v += liftL[k] * D[4 * N * N + i + N * j];
+                    v += liftR[k] * D[5 * N * N + i + N * j];
                     out[alpha] = v * sc;
                 }
                 out[4] += ph.H0 * out[0];
@@ -2129,9 +2167,12 @@ __device__ __forceinline__ void fused_C_body(const HexArgs<T> &a, long long firs
                 for (int alpha = 1; alpha < 5; alpha++) {
                     const T *D = s_d + alpha * NF;
                     T v = R[alpha * NU + z];
-                    v += liftL[i] * D[0 * N * N + j + N * k] + liftR[i] * D[1 * N * N + j + N * k];
-                    v += liftL[j] * D[2 * N * N + i + N * k] + liftR[j] * D[3 * N * N + i + N * k];
-                    v += liftL[k] * D[4 * N * N + i + N * j] + liftR[k] * D[5 * N * N + i + N * j];
+                    v += liftL[i] * D[0 * N * N + j + N * k];
+                    v += liftR[i] * D[1 * N * N + j + N * k];
+                    v += liftL[j] * D[2 * N * N + i + N * k];
+                    v += liftR[j] * D[3 * N * N + i + N * k];
+                    v += liftL[k] * D[4 * N * N + i + N * j];
+                    v += liftR[k] * D[5 * N * N + i + N * j];
                     out[alpha] = v * idet;
                 }
                 const ff e4 = ff_fma(H0, Rrho, ff_of(out[4]));
@@ -2247,9 +2288,12 @@ __global__ void __launch_bounds__(NT) k_surf_lift(HexArgs<T> a)
                 const int alpha = it / NU, z = it % NU, i = z % N, j = (z / N) % N, k = z / (N * N);
                 const T *D = s_d + alpha * NF;
                 T v = R[it];
-                v += op.liftL[i] * D[0 * N * N + j + N * k] + op.liftR[i] * D[1 * N * N + j + N * k];
-                v += op.liftL[j] * D[2 * N * N + i + N * k] + op.liftR[j] * D[3 * N * N + i + N * k];
-                v += op.liftL[k] * D[4 * N * N + i + N * j] + op.liftR[k] * D[5 * N * N + i + N * j];
+                v += op.liftL[i] * D[0 * N * N + j + N * k];
+                v += op.liftR[i] * D[1 * N * N + j + N * k];
+                v += op.liftL[j] * D[2 * N * N + i + N * k];
+                v += op.liftR[j] * D[3 * N * N + i + N * k];
+                v += op.liftL[k] * D[4 * N * N + i + N * j];
+                v += op.liftR[k] * D[5 * N * N + i + N * j];
                 if (a.rkstage == 0) R[it] = v * idet;
                 else rk_fold(a, elem_u0(a, e, NU) + it, v * idet);
             }
@@ -2263,9 +2307,12 @@ __global__ void __launch_bounds__(NT) k_surf_lift(HexArgs<T> a)
                 for (int alpha = 0; alpha < 5; alpha++) {
                     const T *D = s_d + alpha * NF;
                     T v = R[alpha * NU + z];
-                    v += op.liftL[i] * D[0 * N * N + j + N * k] + op.liftR[i] * D[1 * N * N + j + N * k];
-                    v += op.liftL[j] * D[2 * N * N + i + N * k] + op.liftR[j] * D[3 * N * N + i + N * k];
-                    v += op.liftL[k] * D[4 * N * N + i + N * j] + op.liftR[k] * D[5 * N * N + i + N * j];
+                    v += op.liftL[i] * D[0 * N * N + j + N * k];
+                    v += op.liftR[i] * D[1 * N * N + j + N * k];
+                    v += op.liftL[j] * D[2 * N * N + i + N * k];
+                    v += op.liftR[j] * D[3 * N * N + i + N * k];
+                    v += op.liftL[k] * D[4 * N * N + i + N * j];
+                    v += op.liftR[k] * D[5 * N * N + i + N * j];
                     out[alpha] = v * idet;
                 }
                 out[4] += H0 * out[0];
@@ -2347,9 +2394,12 @@ __global__ void __launch_bounds__(NT) k_lift(HexArgs<T> a)
             const int alpha = it / NU, z = it % NU, i = z % N, j = (z / N) % N, k = z / (N * N);
             const T *D = s_d + alpha * NF;
             T v = R[it];
-            v += liftL[i] * D[0 * N * N + j + N * k] + liftR[i] * D[1 * N * N + j + N * k];
-            v += liftL[j] * D[2 * N * N + i + N * k] + liftR[j] * D[3 * N * N + i + N * k];
-            v += liftL[k] * D[4 * N * N + i + N * j] + liftR[k] * D[5 * N * N + i + N * j];
+            v += liftL[i] * D[0 * N * N + j + N * k];
+            v += liftR[i] * D[1 * N * N + j + N * k];
+            v += liftL[j] * D[2 * N * N + i + N * k];
+            v += liftR[j] * D[3 * N * N + i + N * k];
+            v += liftL[k] * D[4 * N * N + i + N * j];
+            v += liftR[k] * D[5 * N * N + i + N * j];
             // curved elements: det J at this solution point
             const T sc = CURV ? T(-1) / a.mu[(e * NU + z) * 10 + 9] : idet;
             if (a.rkstage == 0) R[it] = v * sc;
@@ -3089,7 +3139,8 @@ static void launch_B(const HexArgs<T> &a, cudaStream_t s)
     // the collocation form needs no quadrature-point buffers; surface-flux anti-aliasing stages its
     // in-plane interpolation (6 faces x 20 fields x m x n values) after the quadrature-point buffer
     constexpr int TI = 6 * 20 * S::M * S::N;
-    const size_t smem = (!AA ? S::LOW + S::PF : (SURF ? S::SIZE + TI : S::SIZE)) * sizeof(T);
+    constexpr bool FX = sizeof(T) == 8 && AA && !SURF;
+    const size_t smem = FX ? HexFxSmem<P>::SMEM : (!AA ? S::LOW + S::PF : (SURF ? S::SIZE + TI : S::SIZE)) * sizeof(T);
     static bool attr = false;
     if constexpr (SURF && sizeof(T) == 4) {
         if (!attr) {
@@ -3299,8 +3350,8 @@ static size_t multi_B_smem(const MultiArgs<T> &ma)
     for (int g = 0; g < ma.ng; g++) {
         size_t v;
         if (sizeof(T) == 4 && ma.a[g].geo64 != nullptr && ma.kind[g] != 1) v = ma.kind[g] == 3 ? Hex32<3, 2>::SMEM : Hex32<4, 1>::SMEM;
-        else if (ma.kind[g] == 3) v = HexSmem<T, 3>::SIZE * sizeof(T);
-        else if (ma.kind[g] == 4) v = HexSmem<T, 4>::SIZE * sizeof(T);
+        else if (ma.kind[g] == 3) v = sizeof(T) == 8 ? HexFxSmem<3>::SMEM : HexSmem<T, 3>::SIZE * sizeof(T);
+        else if (ma.kind[g] == 4) v = sizeof(T) == 8 ? HexFxSmem<4>::SMEM : HexSmem<T, 4>::SIZE * sizeof(T);
         else if constexpr (sizeof(T) == 8) v = pri::FX_SMEM;
         else v = ((sizeof(PriOps<T>) + 15) / 16) * 16 + (size_t)(5 * pri::NU + 15 * pri::NU + 5 * pri::NF + 20 * pri::NQ) * sizeof(T) +
                  (size_t)(20 * pri::NZ * pri::NQT) * sizeof(T);

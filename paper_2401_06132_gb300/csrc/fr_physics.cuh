@@ -8,6 +8,39 @@
 // Point physics (Sec. 2.1): total flux f = f^e - f^v, viscous normal flux, Rusanov common flux
 // ---------------------------------------------------------------------------------------------
 
+// 1/x and sqrt(x) of FP64: the hardware's approximations (about 20 bits; not on the FP64 pipe, which
+// bounds the FP64 kernels) with one third-order step, r (1 + e + e^2) with e = 1 - x r, and
+// s (1 + e/2 + 3 e^2/8) with s = x y, e = 1 - s y: the remainder e^3 is below 2^-58, so the final
+// rounding decides. 3 and 5 FP64 operations against 8 for the exactly rounded ones (measured by rate).
+// x = 0 and infinities give NaN.
+__device__ __forceinline__ double fr_inv(double x)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+__device__ __forceinline__ double fr_sqrt(double x)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double s = x * y, e = fma(-s, y, 1.0);
+    return fma(s, fma(0.375, e, 0.5) * e, s);
+}
+__device__ __forceinline__ float fr_inv(float x) { return 1.0f / x; }
+__device__ __forceinline__ float fr_sqrt(float x) { return sqrtf(x); }
+// Whether x is finite, from its exponent field (no FP64 operation).
+__device__ __forceinline__ bool fr_finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool fr_finite(float x) { return (__float_as_int(x) & 0x7f800000) != 0x7f800000; }
+
+// Common solution C = (1/2 - beta) uL + (1/2 + beta) uR with the weights wl, wr. At beta = 1/2 it is uR
+// (and not a number where uL is not finite, as 0 uL is): no FP64 operation.
+__device__ __forceinline__ double fr_common(double wl, double wr, double uL, double uR)
+{
+    if (wl == 0.0 && wr == 1.0) return fr_finite(uL) ? uR : __hiloint2double(0x7ff80000, 0);
+    return wl * uL + wr * uR;
+}
+
 // rho times the velocity gradient, w[i][d] = rho dv_i/dx_d = d(rho v_i)/dx_d - v_i d(rho)/dx_d; the
 // factor 1/rho is folded into the coefficients that multiply it (mu/rho, heat/rho).
 template <typename T>
@@ -33,12 +66,13 @@ __device__ __forceinline__ void viscous_stress(const T mr, const T (*w)[3], T (*
     tau[1][2] = tau[2][1] = mr * (w[1][2] + w[2][1]);
 }
 
-// Physical total flux f[d][alpha] from the state u and its physical gradient g[alpha][d].
-// Returns false for a non-physical state (rho <= 0, p <= 0 or non-finite).
+// Physical total flux f[d][alpha] from the state u and its physical gradient g[alpha][d]. The momentum
+// flux rho v v - tau is symmetric: six entries. Returns false for a non-physical state (rho <= 0, p <= 0
+// or non-finite).
 template <typename T>
 __device__ __forceinline__ bool total_flux(const Phys<T> &ph, const T *u, const T (*g)[3], T (*f)[5])
 {
-    const T rho = u[0], ir = T(1) / rho;
+    const T rho = u[0], ir = fr_inv(rho);
     const T v[3] = {u[1] * ir, u[2] * ir, u[3] * ir};
     const T E = u[4];
     const T p = ph.gm1 * (E - T(0.5) * (u[1] * v[0] + u[2] * v[1] + u[3] * v[2]));
@@ -46,24 +80,27 @@ __device__ __forceinline__ bool total_flux(const Phys<T> &ph, const T *u, const 
     rho_dv(v, g, w);
     viscous_stress(ph.mu * ir, w, tau);
     const T er = E * ir, hr = ph.heat * ir, pm = p - ph.pref, ep = E + p;
+    f[0][1] = u[1] * v[0] + (pm - tau[0][0]);
+    f[1][2] = u[2] * v[1] + (pm - tau[1][1]);
+    f[2][3] = u[3] * v[2] + (pm - tau[2][2]);
+    f[0][2] = f[1][1] = u[1] * v[1] - tau[0][1];
+    f[0][3] = f[2][1] = u[1] * v[2] - tau[0][2];
+    f[1][3] = f[2][2] = u[2] * v[2] - tau[1][2];
 #pragma unroll
     for (int d = 0; d < 3; d++) {
         // heat flux mu gamma/Pr [d(E/rho) - v.dv] = mu gamma/((gamma-1)Pr) d(p/rho)
-        const T phi = hr * ((g[4][d] - er * g[0][d]) - (v[0] * w[0][d] + v[1] * w[1][d] + v[2] * w[2][d]));
+        const T dh = g[4][d] - er * g[0][d] - v[0] * w[0][d] - v[1] * w[1][d] - v[2] * w[2][d];
         f[d][0] = u[1 + d];
-        f[d][1] = u[1] * v[d] + (d == 0 ? pm : T(0)) - tau[0][d];
-        f[d][2] = u[2] * v[d] + (d == 1 ? pm : T(0)) - tau[1][d];
-        f[d][3] = u[3] * v[d] + (d == 2 ? pm : T(0)) - tau[2][d];
-        f[d][4] = v[d] * ep - (v[0] * tau[0][d] + v[1] * tau[1][d] + v[2] * tau[2][d] + phi);
+        f[d][4] = v[d] * ep - (hr * dh + v[0] * tau[0][d] + v[1] * tau[1][d] + v[2] * tau[2][d]);
     }
-    return rho > T(0) && p > T(0) && isfinite(p) && isfinite(f[0][4] + f[1][4] + f[2][4]);
+    return rho > T(0) && p > T(0) && fr_finite(p) && fr_finite(f[0][4]) && fr_finite(f[1][4]) && fr_finite(f[2][4]);
 }
 
 // n . f^v for variables 1..4 (the mass component is zero).
 template <typename T>
 __device__ __forceinline__ void viscous_normal_flux(const Phys<T> &ph, const T *u, const T (*g)[3], const T *n, T *fvn)
 {
-    const T rho = u[0], ir = T(1) / rho;
+    const T rho = u[0], ir = fr_inv(rho);
     const T v[3] = {u[1] * ir, u[2] * ir, u[3] * ir};
     T w[3][3], tau[3][3];
     rho_dv(v, g, w);
@@ -74,7 +111,7 @@ __device__ __forceinline__ void viscous_normal_flux(const Phys<T> &ph, const T *
     // n . (tau v + phi) = v . (tau n) + n . phi
     T nphi = T(0);
 #pragma unroll
-    for (int d = 0; d < 3; d++) nphi += n[d] * ((g[4][d] - er * g[0][d]) - (v[0] * w[0][d] + v[1] * w[1][d] + v[2] * w[2][d]));
+    for (int d = 0; d < 3; d++) nphi += n[d] * (g[4][d] - er * g[0][d] - v[0] * w[0][d] - v[1] * w[1][d] - v[2] * w[2][d]);
     fvn[3] = v[0] * fvn[0] + v[1] * fvn[1] + v[2] * fvn[2] + ph.heat * ir * nphi;
 }
 
@@ -85,29 +122,27 @@ template <typename T>
 __device__ __forceinline__ bool common_flux(const Phys<T> &ph, const T *uL, const T *uR, const T *fvL, const T *fvR,
                                             const T *n, T *F)
 {
-    const T irL = T(1) / uL[0], irR = T(1) / uR[0];
-    const T vnL = (uL[1] * n[0] + uL[2] * n[1] + uL[3] * n[2]) * irL;
-    const T vnR = (uR[1] * n[0] + uR[2] * n[1] + uR[3] * n[2]) * irR;
+    const T irL = fr_inv(uL[0]), irR = fr_inv(uR[0]);
+    const T mL = uL[1] * n[0] + uL[2] * n[1] + uL[3] * n[2], mR = uR[1] * n[0] + uR[2] * n[1] + uR[3] * n[2];
+    const T vnL = mL * irL, vnR = mR * irR;
     const T pL = ph.gm1 * (uL[4] - T(0.5) * irL * (uL[1] * uL[1] + uL[2] * uL[2] + uL[3] * uL[3]));
     const T pR = ph.gm1 * (uR[4] - T(0.5) * irR * (uR[1] * uR[1] + uR[2] * uR[2] + uR[3] * uR[3]));
-    const T cL = sqrt(ph.gamma * pL * irL), cR = sqrt(ph.gamma * pR * irR);
+    const T cL = fr_sqrt(ph.gamma * pL * irL), cR = fr_sqrt(ph.gamma * pR * irR);
     const T s = fmax(fabs(vnL) + cL, fabs(vnR) + cR);
-    T fnL[5], fnR[5];
-    fnL[0] = uL[0] * vnL; fnR[0] = uR[0] * vnR;
+    // the two sides' normal fluxes added up, and the dissipation's factor s/2 + tau
+    const T pp = (pL - ph.pref) + (pR - ph.pref);
+    T fs[5];
+    fs[0] = mL + mR;
 #pragma unroll
-    for (int i = 0; i < 3; i++) {
-        fnL[1 + i] = uL[1 + i] * vnL + (pL - ph.pref) * n[i];
-        fnR[1 + i] = uR[1 + i] * vnR + (pR - ph.pref) * n[i];
-    }
-    fnL[4] = vnL * (uL[4] + pL); fnR[4] = vnR * (uR[4] + pR);
-    const T wl = T(0.5) + ph.beta, wr = T(0.5) - ph.beta;
+    for (int i = 0; i < 3; i++) fs[1 + i] = uL[1 + i] * vnL + uR[1 + i] * vnR + pp * n[i];
+    fs[4] = vnL * (uL[4] + pL) + vnR * (uR[4] + pR);
+    const T k = T(0.5) * s + ph.tau, wl = T(0.5) + ph.beta, wr = T(0.5) - ph.beta;
 #pragma unroll
     for (int a = 0; a < 5; a++) {
-        const T du = uL[a] - uR[a];
         const T fv = (a == 0) ? T(0) : (wl * fvL[a - 1] - wr * fvR[a - 1]);
-        F[a] = T(0.5) * (fnL[a] + fnR[a]) + T(0.5) * s * du - fv + ph.tau * du;
+        F[a] = T(0.5) * fs[a] + (k * (uL[a] - uR[a]) - fv);
     }
-    return pL > T(0) && pR > T(0) && uL[0] > T(0) && uR[0] > T(0) && isfinite(s);
+    return pL > T(0) && pR > T(0) && uL[0] > T(0) && uR[0] > T(0) && fr_finite(s);
 }
 
 
@@ -140,16 +175,19 @@ __device__ __forceinline__ bool total_flux_dev(const Phys<float> &ph, const floa
     rho_dv(v, g, rw);
     viscous_stress(ph.mu * ir, rw, tau);
     const float hred = w[4] + pd - ph.H0 * w[0];
+    f[0][1] = w[1] * v[0] + (pd - tau[0][0]);
+    f[1][2] = w[2] * v[1] + (pd - tau[1][1]);
+    f[2][3] = w[3] * v[2] + (pd - tau[2][2]);
+    f[0][2] = f[1][1] = w[1] * v[1] - tau[0][1];
+    f[0][3] = f[2][1] = w[1] * v[2] - tau[0][2];
+    f[1][3] = f[2][2] = w[2] * v[2] - tau[1][2];
 #pragma unroll
     for (int d = 0; d < 3; d++) {
-        const float phi = hr * ((g[4][d] - er * g[0][d]) - (v[0] * rw[0][d] + v[1] * rw[1][d] + v[2] * rw[2][d]));
+        const float dh = g[4][d] - er * g[0][d] - v[0] * rw[0][d] - v[1] * rw[1][d] - v[2] * rw[2][d];
         f[d][0] = mass ? w[1 + d] : 0.0f;
-        f[d][1] = w[1] * v[d] + (d == 0 ? pd : 0.0f) - tau[0][d];
-        f[d][2] = w[2] * v[d] + (d == 1 ? pd : 0.0f) - tau[1][d];
-        f[d][3] = w[3] * v[d] + (d == 2 ? pd : 0.0f) - tau[2][d];
-        f[d][4] = v[d] * hred - (v[0] * tau[0][d] + v[1] * tau[1][d] + v[2] * tau[2][d] + phi);
+        f[d][4] = v[d] * hred - (hr * dh + v[0] * tau[0][d] + v[1] * tau[1][d] + v[2] * tau[2][d]);
     }
-    return rho > 0.0f && ph.pref + pd > 0.0f && isfinite(pd) && isfinite(f[0][4] + f[1][4] + f[2][4]);
+    return rho > 0.0f && ph.pref + pd > 0.0f && fr_finite(pd) && fr_finite(f[0][4]) && fr_finite(f[1][4]) && fr_finite(f[2][4]);
 }
 
 // Common normal flux of (rho v, E - H0 rho) (F[1..4]) from deviation states, with the same Rusanov
