@@ -718,6 +718,61 @@ static void fill_priops(const frb::Prism2D &P, PriOps<T> &o)
     }
 }
 
+// The projections with the corrected derivatives: PT = Dhx Pt, Dhy Pt, Pt and PZ = Pz, Pz, Dhz Pz.
+static void pri_projections(const PriOps<double> &o, double (&PT)[3][FR_PT][FR_PQ], double (&PZ)[3][FR_PE][5])
+{
+    for (int t = 0; t < FR_PT; t++)
+        for (int q = 0; q < FR_PQ; q++) {
+            double vx = 0, vy = 0;
+            for (int j = 0; j < FR_PT; j++) { vx += o.Dhx[t][j] * o.Pt[j][q]; vy += o.Dhy[t][j] * o.Pt[j][q]; }
+            PT[0][t][q] = vx; PT[1][t][q] = vy; PT[2][t][q] = o.Pt[t][q];
+        }
+    for (int k = 0; k < FR_PE; k++)
+        for (int c = 0; c < 5; c++) {
+            double v = 0;
+            for (int j = 0; j < FR_PE; j++) v += o.Dhz[k][j] * o.Pz[j][c];
+            PZ[0][k][c] = PZ[1][k][c] = o.Pz[k][c];
+            PZ[2][k][c] = v;
+        }
+}
+
+static void fill_pric32(const PriOps<double> &o, PriC32 &x)
+{
+    double PT[3][FR_PT][FR_PQ], PZ[3][FR_PE][5];
+    pri_projections(o, PT, PZ);
+    for (int k = 0; k < FR_PE; k++) {
+        for (int j = 0; j < FR_PE; j++) x.Dhz[k][j] = (float)o.Dhz[k][j];
+        x.liftzL[k] = (float)o.liftzL[k]; x.liftzR[k] = (float)o.liftzR[k];
+        for (int c = 0; c < 5; c++) {
+            x.Bz[c][k] = (float)o.Bz[c][k];
+            for (int d = 0; d < 3; d++) x.PZ[d][k][c] = (float)PZ[d][k][c];
+        }
+    }
+}
+
+static void fill_pris32(const PriOps<double> &o, PriS32 &x)
+{
+    double PT[3][FR_PT][FR_PQ], PZ[3][FR_PE][5];
+    pri_projections(o, PT, PZ);
+    for (int t = 0; t < FR_PT; t++) {
+        for (int j = 0; j < FR_PT; j++) {
+            x.dl[0][t][j] = (float)o.Dhx[t][j]; x.dl[1][t][j] = (float)o.Dhy[t][j];
+            x.dx[t][j] = ff_from_double(o.Dhx[t][j]); x.dy[t][j] = ff_from_double(o.Dhy[t][j]);
+        }
+        for (int f = 0; f < 3; f++)
+            for (int b = 0; b < FR_PE; b++)
+                for (int d = 0; d < 2; d++) x.dl[d][t][FR_PT + 4 * f + b] = (float)(o.nf[f][d] * o.Lf[f][t][b]);
+        for (int d = 0; d < 3; d++)
+            for (int q = 0; q < FR_PQ; q++) x.pt[d][t][q] = (float)PT[d][t][q];
+        for (int f = 0; f < 3; f++)
+            for (int b = 0; b < FR_PE; b++) x.ef[f][b][t] = (float)o.Ef[f][b][t];
+    }
+    for (int k = 0; k < FR_PE; k++) {
+        x.lz[0][k] = (float)o.lzL[k]; x.lz[1][k] = (float)o.lzR[k];
+        for (int j = 0; j < FR_PE; j++) x.dz[k][j] = ff_from_double(o.Dhz[k][j]);
+    }
+}
+
 // The fixed-point copy of the FP64 prism table: sums that end in limbs keep row sums of at most 1 (the
 // in-plane and line gradients, the triangle projection), sums that end in FP64 of at most 4.
 static void fill_prifx(const PriOps<double> &o, PriFx &table)
@@ -725,19 +780,7 @@ static void fill_prifx(const PriOps<double> &o, PriFx &table)
     PriFxS &x = table.s;
     constexpr int NT = FR_PT, NQ = FR_PQ, NZ = FR_PE;
     double PT[3][NT][NQ], PZ[3][NZ][5];
-    for (int t = 0; t < NT; t++)
-        for (int q = 0; q < NQ; q++) {
-            double vx = 0, vy = 0;
-            for (int j = 0; j < NT; j++) { vx += o.Dhx[t][j] * o.Pt[j][q]; vy += o.Dhy[t][j] * o.Pt[j][q]; }
-            PT[0][t][q] = vx; PT[1][t][q] = vy; PT[2][t][q] = o.Pt[t][q];
-        }
-    for (int k = 0; k < NZ; k++)
-        for (int c = 0; c < 5; c++) {
-            double v = 0;
-            for (int j = 0; j < NZ; j++) v += o.Dhz[k][j] * o.Pz[j][c];
-            PZ[0][k][c] = PZ[1][k][c] = o.Pz[k][c];
-            PZ[2][k][c] = v;
-        }
+    pri_projections(o, PT, PZ);
     double big, row;
     auto start = [&]() { big = row = 0; };
     auto add = [&](double &s, double c) { s += std::fabs(c); big = std::fabs(c) > big ? std::fabs(c) : big; };
@@ -808,8 +851,12 @@ static fr_status upload_priops(fr_mesh *m, void **dst)
         CU(cudaMemcpy(static_cast<char *>(*dst) + sizeof(o), &x, sizeof(x), cudaMemcpyHostToDevice));
     }
     if constexpr (sizeof(T) == 4) {
-        // the FP32 volume kernels read the interpolation and projection blocks from constant memory
-        if (pri_set_const_ops(&o) || multi_set_pri_const_ops(&o)) return fail(FR_ECUDA, "prism operator upload failed");
+        // the FP32 volume kernels read their operators from constant memory
+        PriOps<double> o64;
+        fill_priops<double>(m->pri, o64);
+        PriC32 c{};
+        fill_pric32(o64, c);
+        if (pri_set_const_ops(&c) || multi_set_pri_const_ops(&c)) return fail(FR_ECUDA, "prism operator upload failed");
     }
     return FR_OK;
 }
@@ -1208,8 +1255,11 @@ static fr_status finish_create(fr_mesh *m, std::vector<uint32_t> &partner, fr_me
         float *l = reinterpret_cast<float *>(&pff.lo);
         static_assert(sizeof(PriOps<double>) == 2 * sizeof(PriOps<float>), "same member layout in both precisions");
         for (size_t i = 0; i < sizeof(PriOps<float>) / sizeof(float); i++) l[i] = (float)(src[i] - (double)h[i]);
-        st = dalloc(m, &m->d_priops64, sizeof(pff));
-        if (!st && cudaMemcpy(m->d_priops64, &pff, sizeof(pff), cudaMemcpyHostToDevice) != cudaSuccess)
+        PriS32 ps{};
+        fill_pris32(o64, ps);
+        st = dalloc(m, &m->d_priops64, sizeof(pff) + sizeof(ps));
+        if (!st && (cudaMemcpy(m->d_priops64, &pff, sizeof(pff), cudaMemcpyHostToDevice) != cudaSuccess ||
+                    cudaMemcpy(static_cast<char *>(m->d_priops64) + sizeof(pff), &ps, sizeof(ps), cudaMemcpyHostToDevice) != cudaSuccess))
             st = fail(FR_ECUDA, "prism operator upload failed");
     }
     // float-float dense tables: the compensated face values of every reduced precision, and the

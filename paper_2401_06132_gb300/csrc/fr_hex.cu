@@ -3297,7 +3297,7 @@ static int fused_phase(int phase, const HexArgs<T> &a, cudaStream_t s, int varia
 // every CTA runs each group's phase body on its share of that group's elements in turn. The
 // dynamic shared memory is the largest group's; each body uses it from the start.
 // ---------------------------------------------------------------------------------------------
-int multi_set_pri_const_ops(const PriOps<float> *h) { return pri::set_const_ops(*h); }
+int multi_set_pri_const_ops(const PriC32 *h) { return pri::set_const_ops(*h); }
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_multi_A(MultiArgs<T> ma)
@@ -3325,7 +3325,7 @@ __global__ void __launch_bounds__(128) k_multi_B(MultiArgs<T> ma)
         if (ma.kind[g] == 3) volume_body<T, 3, 128>(ma.a[g], blockIdx.x, gridDim.x);
         else if (ma.kind[g] == 4) volume_body<T, 4, 128>(ma.a[g], blockIdx.x, gridDim.x);
         else if constexpr (sizeof(T) == 8) pri::pri_B_fx_body<128>(ma.a[g], ma.pops, blockIdx.x, gridDim.x);
-        else pri::pri_B_body<T, 128, 0>(ma.a[g], ma.pops, ma.pff, blockIdx.x, gridDim.x);
+        else pri::pri_B32_body<128>(ma.a[g], ma.pff, blockIdx.x, gridDim.x);
         __syncthreads();
     }
 }
@@ -3352,9 +3352,7 @@ static size_t multi_B_smem(const MultiArgs<T> &ma)
         if (sizeof(T) == 4 && ma.a[g].geo64 != nullptr && ma.kind[g] != 1) v = ma.kind[g] == 3 ? Hex32<3, 2>::SMEM : Hex32<4, 1>::SMEM;
         else if (ma.kind[g] == 3) v = sizeof(T) == 8 ? HexFxSmem<3>::SMEM : HexSmem<T, 3>::SIZE * sizeof(T);
         else if (ma.kind[g] == 4) v = sizeof(T) == 8 ? HexFxSmem<4>::SMEM : HexSmem<T, 4>::SIZE * sizeof(T);
-        else if constexpr (sizeof(T) == 8) v = pri::FX_SMEM;
-        else v = ((sizeof(PriOps<T>) + 15) / 16) * 16 + (size_t)(5 * pri::NU + 15 * pri::NU + 5 * pri::NF + 20 * pri::NQ) * sizeof(T) +
-                 (size_t)(20 * pri::NZ * pri::NQT) * sizeof(T);
+        else v = sizeof(T) == 8 ? pri::FX_SMEM : pri::P32_SMEM;
         need = v > need ? v : need;
     }
     return need;

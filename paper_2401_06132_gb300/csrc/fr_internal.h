@@ -159,6 +159,25 @@ struct PriFx {
     PriFxS s;
 };
 
+// The FP32 prism operators as the CUDA-core volume kernel applies them. In constant memory, the line
+// operators (PZ: the projection with the corrected derivative, Pz, Pz, Dhz Pz).
+struct PriC32 {
+    float Dhz[FR_PE][FR_PE], liftzL[FR_PE], liftzR[FR_PE];
+    float Bz[5][FR_PE];
+    float PZ[3][FR_PE][5];
+};
+// Copied to shared memory by every CTA (it follows PriOpsFF in memory; whole 16-byte rows): the plane
+// gradients with their lifts, [x, y][t] = Dh (10 entries) and the three quadrilateral faces' lifts times
+// the face normal's component (4 f + b); the triangle projections with the corrected derivatives (formed
+// in FP64), [Dhx Pt, Dhy Pt, Pt][t]; the traces; the corrected derivatives in float-float.
+struct PriS32 {
+    float dl[2][FR_PT][24];
+    float pt[3][FR_PT][28];
+    float ef[3][FR_PE][FR_PT], lz[2][FR_PE];
+    ff dx[FR_PT][FR_PT], dy[FR_PT][FR_PT], dz[FR_PE][FR_PE];
+};
+static_assert(sizeof(PriS32) % 16 == 0, "copied in 16-byte units");
+
 // Dense-element (p = 3) operator tables, transposed so that the output index runs fastest (a warp's
 // lanes compute consecutive outputs and read consecutive entries). Rows of the solution-point index
 // are padded to NUS (a multiple of 4) for 16-byte vector loads; the pad rows are zero.
@@ -432,10 +451,10 @@ int hex_upload_ops(int p, int m, const frb::Hex1D &h);
 // Prism kernels (fr_pri.cu); the operator tables are passed by device pointer (opsff: the
 // float-float table of the low-Mach FP32 form's mass channel; null otherwise).
 template <typename T> int pri_fused_phase(int phase, const HexArgs<T> &a, const PriOps<T> *ops, const PriOpsFF *opsff, cudaStream_t s);
-// The FP32 prism operator table in the constant memory of the current device, for the prism kernels
+// The FP32 prism operators in the constant memory of the current device, for the prism kernels
 // (fr_pri.cu) and the launches that serve several element groups (fr_hex.cu); 0 on success.
-int pri_set_const_ops(const PriOps<float> *h);
-int multi_set_pri_const_ops(const PriOps<float> *h);
+int pri_set_const_ops(const PriC32 *h);
+int multi_set_pri_const_ops(const PriC32 *h);
 // Dense-element kernels (fr_dense.cu): tetrahedra and pyramids, operator table by device pointer.
 // (opsff: the float-float FP32 table of the low-Mach form's mass channel; null otherwise).
 template <typename T>

@@ -38,6 +38,7 @@ template <typename T, int NTH, int TCM>
 __global__ void __launch_bounds__(NTH, sizeof(T) == 8 ? 5 : (TCM == 0 ? 8 : 0)) k_pri_B(HexArgs<T> a, const PriOps<T> *gops, const PriOpsFF *opsff)
 {
     if constexpr (sizeof(T) == 8) pri_B_fx_body<NTH>(a, gops, blockIdx.x, gridDim.x);
+    else if constexpr (TCM == 0) pri_B32_body<NTH>(a, opsff, blockIdx.x, gridDim.x);
     else pri_B_body<T, NTH, TCM>(a, gops, opsff, blockIdx.x, gridDim.x);
 }
 
@@ -60,7 +61,7 @@ int grid_elems(long long ne, int per_sm)
 
 using namespace pri;
 
-int pri_set_const_ops(const PriOps<float> *h) { return pri::set_const_ops(*h); }
+int pri_set_const_ops(const PriC32 *h) { return pri::set_const_ops(*h); }
 
 template <typename T>
 int pri_fused_phase(int phase, const HexArgs<T> &a, const PriOps<T> *ops, const PriOpsFF *ops64, cudaStream_t s)
@@ -101,8 +102,7 @@ int pri_fused_phase(int phase, const HexArgs<T> &a, const PriOps<T> *ops, const 
           }
         }
         if (!tcdone) {
-            // FP32 interpolates all 20 fields per pass (staging 20 x 4 x 25 values)
-            const size_t smem = sizeof(T) == 8 ? FX_SMEM : base + (size_t)(20 * NZ * NQT) * sizeof(T);
+            const size_t smem = sizeof(T) == 8 ? FX_SMEM : P32_SMEM;
             static bool attr = false;
             if (!attr) {
                 cudaFuncSetAttribute(k_pri_B<T, NTH, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

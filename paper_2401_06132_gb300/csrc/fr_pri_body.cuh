@@ -20,14 +20,14 @@ constexpr int NQ = NQT * MZ;                  // 125
 
 __device__ __forceinline__ int face_of(int s) { return s < 10 ? 0 : s < 20 ? 1 : 2 + (s - 20) / 16; }
 
-// The FP32 operator table in constant memory (one copy per translation unit that includes this
+// The FP32 volume kernel's operators in constant memory (one copy per translation unit that includes this
 // file, filled by set_const_ops on each device): read with compile-time indices, its entries are
 // constant-bank operands of the multiply-adds instead of a shared-memory load per coefficient.
-__constant__ PriOps<float> c_pri32;
+__constant__ PriC32 c_prib32;
 
-inline int set_const_ops(const PriOps<float> &h)
+inline int set_const_ops(const PriC32 &h)
 {
-    return cudaMemcpyToSymbol(c_pri32, &h, sizeof(h)) == cudaSuccess ? 0 : -1;
+    return cudaMemcpyToSymbol(c_prib32, &h, sizeof(h)) == cudaSuccess ? 0 : -1;
 }
 
 template <typename T>
@@ -198,131 +198,11 @@ __device__ __forceinline__ void pri_disu_body(const HexArgs<T> &a, const PriOps<
 // -------------------------------------------------------------------------------------------------
 // Phase B: volume group
 // -------------------------------------------------------------------------------------------------
-template <typename T, int NTH>
-__device__ __forceinline__ void pri_interp_5(const PriOps<T> &op, const T *src, T *tmp, T *dst)
-{
-    for (int it = threadIdx.x; it < 5 * NZ * NQT; it += NTH) {   // triangle plane: (fc, k, q)
-        const int fc = it / (NZ * NQT), r = it % (NZ * NQT), k = r / NQT, q = r % NQT;
-        T v = T(0);
-#pragma unroll
-        for (int t = 0; t < NT_; t++) v += op.Bt[q][t] * src[fc * NU + t + 10 * k];
-        tmp[fc * NZ * NQT + q + NQT * k] = v;
-    }
-    __syncthreads();
-    for (int it = threadIdx.x; it < 5 * MZ * NQT; it += NTH) {   // z: (fc, c, q)
-        const int fc = it / (MZ * NQT), r = it % (MZ * NQT), c = r / NQT, q = r % NQT;
-        T v = T(0);
-#pragma unroll
-        for (int k = 0; k < NZ; k++) v += op.Bz[c][k] * tmp[fc * NZ * NQT + q + NQT * k];
-        dst[fc * NQ + q + NQT * c] = v;
-    }
-    __syncthreads();
-}
-
-template <typename T, int NTH>
-__device__ __forceinline__ void pri_project_5(const PriOps<T> &op, const T *src, T *tmp, T *dst)
-{
-    for (int it = threadIdx.x; it < 5 * NZ * NQT; it += NTH) {   // z: (fc, k, q)
-        const int fc = it / (NZ * NQT), r = it % (NZ * NQT), k = r / NQT, q = r % NQT;
-        T v = T(0);
-#pragma unroll
-        for (int c = 0; c < MZ; c++) v += op.Pz[k][c] * src[fc * NQ + q + NQT * c];
-        tmp[fc * NZ * NQT + q + NQT * k] = v;
-    }
-    __syncthreads();
-    for (int it = threadIdx.x; it < 5 * NU; it += NTH) {          // triangle plane: (fc, k, t)
-        const int fc = it / NU, r = it % NU, k = r / NT_, t = r % NT_;
-        T v = T(0);
-#pragma unroll
-        for (int q = 0; q < NQT; q++) v += op.Pt[t][q] * tmp[fc * NZ * NQT + q + NQT * k];
-        dst[fc * NU + t + 10 * k] = v;
-    }
-    __syncthreads();
-}
-
-// FP32 without tensor cores, all 20 fields: the triangle-plane factor with one thread per (field, z
-// level) line, its 10 values in registers and all 25 quadrature points formed from them, then z with
-// one thread per (field, triangle quadrature point); the operators from the constant-memory table
-// with compile-time indices.
-template <int NTH>
-__device__ __forceinline__ void pri_interp_all_c(const float *src, float *tmp, float *dst)
-{
-    for (int it = threadIdx.x; it < 20 * NZ; it += NTH) {   // triangle plane: (f, k)
-        const float *s = src + (it / NZ) * NU + 10 * (it % NZ);
-        float u[NT_];
-#pragma unroll
-        for (int t = 0; t < NT_; t++) u[t] = s[t];
-        float *d = tmp + it * NQT;   // (f NZ + k) NQT + q
-#pragma unroll
-        for (int q = 0; q < NQT; q++) {
-            float v = 0.f;
-#pragma unroll
-            for (int t = 0; t < NT_; t++) v += c_pri32.Bt[q][t] * u[t];
-            d[q] = v;
-        }
-    }
-    __syncthreads();
-    for (int it = threadIdx.x; it < 20 * NQT; it += NTH) {   // z: (f, q)
-        const int f = it / NQT, q = it % NQT;
-        float u[NZ];
-#pragma unroll
-        for (int k = 0; k < NZ; k++) u[k] = tmp[(f * NZ + k) * NQT + q];
-#pragma unroll
-        for (int c = 0; c < MZ; c++) {
-            float v = 0.f;
-#pragma unroll
-            for (int k = 0; k < NZ; k++) v += c_pri32.Bz[c][k] * u[k];
-            dst[f * NQ + q + NQT * c] = v;
-        }
-    }
-    __syncthreads();
-}
-
-// The projection of the 15 flux fields in the same form: z with one thread per (field, triangle
-// quadrature point), then the triangle plane with one thread per (field, z level) line, its 25
-// values in registers.
-template <int NTH>
-__device__ __forceinline__ void pri_project_all_c(const float *src, float *tmp, float *dst)
-{
-    for (int it = threadIdx.x; it < 15 * NQT; it += NTH) {   // z: (f, q)
-        const int f = it / NQT, q = it % NQT;
-        float u[MZ];
-#pragma unroll
-        for (int c = 0; c < MZ; c++) u[c] = src[f * NQ + q + NQT * c];
-#pragma unroll
-        for (int k = 0; k < NZ; k++) {
-            float v = 0.f;
-#pragma unroll
-            for (int c = 0; c < MZ; c++) v += c_pri32.Pz[k][c] * u[c];
-            tmp[(f * NZ + k) * NQT + q] = v;
-        }
-    }
-    __syncthreads();
-    for (int it = threadIdx.x; it < 15 * NZ; it += NTH) {   // triangle plane: (f, k)
-        const float *s = tmp + it * NQT;
-        float u[NQT];
-#pragma unroll
-        for (int q = 0; q < NQT; q++) u[q] = s[q];
-        float *d = dst + (it / NZ) * NU + 10 * (it % NZ);
-#pragma unroll
-        for (int t = 0; t < NT_; t++) {
-            float v = 0.f;
-#pragma unroll
-            for (int q = 0; q < NQT; q++) v += c_pri32.Pt[t][q] * u[q];
-            d[t] = v;
-        }
-    }
-    __syncthreads();
-}
-
-template <int NTH>
-__device__ __forceinline__ void pri_B_fx_body(const HexArgs<double> &a, const PriOps<double> *gops, long long first, long long stride);
-
 template <typename T, int NTH, int TCM>
 __device__ __forceinline__ void pri_B_body(const HexArgs<T> &a, const PriOps<T> *gops, const PriOpsFF *opsff, long long first, long long stride)
 {
-    static_assert(TCM == 0 || (NTH == 128 && sizeof(T) == 4), "tensor-core form: FP32, one warpgroup per element");
-    using PT = PriTC<TCM == 0 ? 1 : TCM>;
+    static_assert(TCM != 0 && NTH == 128 && sizeof(T) == 4, "tensor-core form: FP32, one warpgroup per element");
+    using PT = PriTC<TCM>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ ff s_mf[sizeof(T) == 4 ? 3 * NU : 1];   // low-Mach form: transformed mass flux
     __shared__ short s_plist[NF];                         // flux points that need the viscous flux
@@ -430,7 +310,6 @@ __device__ __forceinline__ void pri_B_body(const HexArgs<T> &a, const PriOps<T> 
                 }
             }
         };
-        if constexpr (TCM == 0) mass_channel();
         // corrected gradient: z lines (alpha, t) and triangle planes (alpha, k, t)
         for (int it = threadIdx.x; it < 5 * NT_; it += NTH) {
             const int alpha = it / NT_, t = it % NT_;
@@ -506,14 +385,7 @@ __device__ __forceinline__ void pri_B_body(const HexArgs<T> &a, const PriOps<T> 
                 for (int k = 0; k < 4; k++) a.FV[k * a.nfpt + gf0 + s] = fvn[k];
             }
         };
-        if constexpr (TCM == 0) viscous_faces();
-        if constexpr (TCM == 0 && sizeof(T) == 4) {
-            pri_interp_all_c<NTH>(s_u, s_t, s_w);   // s_q follows s_u
-        } else if constexpr (TCM == 0) {
-            pri_interp_5<T, NTH>(op, s_u, s_t, s_w);
-#pragma unroll 1
-            for (int c = 0; c < 3; c++) pri_interp_5<T, NTH>(op, s_q + 5 * c * NU, s_t, s_w + (5 + 5 * c) * NQ);
-        } else {
+        {
             // z first (CUDA cores): row r = 5 f + c holds field f (s_q follows s_u) at z level c on
             // the 10 triangle points; then the triangle interpolation of all 100 rows on the tensor core.
             const int r = threadIdx.x;
@@ -581,12 +453,7 @@ __device__ __forceinline__ void pri_B_body(const HexArgs<T> &a, const PriOps<T> 
         }
         flag_status(a.status, ok);
         __syncthreads();
-        if constexpr (TCM == 0 && sizeof(T) == 4) {
-            pri_project_all_c<NTH>(s_w, s_t, s_q);
-        } else if constexpr (TCM == 0) {
-#pragma unroll 1
-            for (int c = 0; c < 3; c++) pri_project_5<T, NTH>(op, s_w + 5 * c * NQ, s_t, s_q + 5 * c * NU);
-        } else {
+        {
             // triangle projection of the 75 rows (flux component f, quadrature level c) on the tensor
             // core, then z (CUDA cores)
             const int r = threadIdx.x;
@@ -650,6 +517,300 @@ __device__ __forceinline__ void pri_B_body(const HexArgs<T> &a, const PriOps<T> 
     }
 }
 
+
+constexpr int P32_TS = 12, P32_WS = 28;   // padded triangle rows: whole 16-byte vectors
+static_assert(sizeof(PriOpsFF) % 16 == 0, "PriS32 follows at a 16-byte boundary");
+constexpr size_t P32_SMEM = sizeof(float) * (20 * NU + 5 * NF + 20 * MZ * P32_TS + 20 * NF);
+static_assert(20 * MZ * P32_TS + 20 * NF >= 15 * MZ * P32_WS && 20 * NU + 5 * NF >= 15 * MZ * NT_ && (20 * NU + 5 * NF) % 4 == 0,
+              "staging fits over consumed buffers, in 16-byte rows");
+
+// -------------------------------------------------------------------------------------------------
+// Phase B in FP32 on the CUDA cores, one element per CTA
+// -------------------------------------------------------------------------------------------------
+// A line, a triangle plane or a quadrature point per thread wherever it can be held in registers, with
+// the operators as constant-bank operands: the gradient's planes and lines on their own warps, the line
+// interpolation first so that a thread interpolates its own quadrature point's 20 fields in the triangle
+// plane and keeps them in registers through the flux, the corrected derivatives on the projection
+// (Dhx Pt, Dhy Pt, Dhz Pz), one warp per component direction, with the mass channel beside them. With a
+// pass per operator the kernel issued 11,000 warp instructions per element behind 18 barriers; now 7,900
+// behind 9. Measured, 24^3 mixed box (13,824 prisms): 202 -> 148 us per launch.
+template <int NTH>
+__device__ __forceinline__ void pri_B32_body(const HexArgs<float> &a, const PriOpsFF *opsff, long long first, long long stride)
+{
+    static_assert(NTH == 128 && NU + NF <= NTH, "four warps; one thread per quadrature point, state and flux point");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float *s_u = reinterpret_cast<float *>(smem_raw);        // state, then the physical gradient (5 + 3 alpha + d)
+    float *s_c = s_u + 20 * NU;                              // common solution
+    float *s_t = s_c + 5 * NF;                               // [20][c][12] line-interpolated fields
+    float *s_tr = s_t + 20 * MZ * P32_TS;                    // [listed flux point][20] traces
+    float *s_w = s_t;                                        // [15][c][28] transformed flux
+    float *s_p = s_u;                                        // [15][c][t] projected in the triangle plane
+    __shared__ ff s_mf[3 * NU];                              // low-Mach form: transformed mass flux
+    // plane operators and traces, read by loops over their outputs or rows selected at run time
+    // (unrolled with constant operands, the planes missed in the instruction cache)
+    __shared__ __align__(16) PriS32 so;
+    __shared__ short s_plist[NF];
+    __shared__ int s_pcnt;
+    const PriC32 &op = c_prib32;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    {
+        const float4 *src = reinterpret_cast<const float4 *>(opsff + 1);
+        float4 *dst = reinterpret_cast<float4 *>(&so);
+        for (int i = tid; i < (int)(sizeof(PriS32) / 16); i += NTH) dst[i] = src[i];
+    }
+    float bt[NT_];   // this thread's row of the triangle interpolation
+    const int tq = tid % NQT, tc_ = tid / NQT;
+#pragma unroll
+    for (int t = 0; t < NT_; t++) bt[t] = opsff->hi.Bt[tq][t];
+    if (tid == 0) s_pcnt = 0;
+    __syncthreads();
+    for (long long e = first; e < a.ne; e += stride) {
+        if (!fr_elem_ok(a, e, NU, NF)) continue;
+        const Geo<float> g = a.geo[e];
+        const Phys<float> ph = elem_phys(a, e);
+        const bool dev = ph.dev != 0;
+        const int a0 = dev ? 1 : 0;   // low-Mach form: the mass has no flux on this path
+        const long long u0 = elem_u0(a, e, NU), gf0 = elem_f0(a, e, NF);
+        // 1. state (deviations in the low-Mach form; with the transformed mass flux) and common solution, one
+        //    point and five variables per thread, and the flux points whose side carries LDG weight
+        if (tid < NU) {
+            const float *U = a.U + u0 + tid;
+            const float m0 = U[NU], m1 = U[2 * NU], m2 = U[3 * NU];
+            s_u[tid] = U[0] - (dev ? ph.rref : 0.f);
+            s_u[NU + tid] = m0; s_u[2 * NU + tid] = m1; s_u[3 * NU + tid] = m2;
+            s_u[4 * NU + tid] = U[4 * NU] - (dev ? ph.eref : 0.f);
+            if (dev) {
+                const ff *cm = a.geo64[e].cm;   // det J J^-1
+#pragma unroll
+                for (int d = 0; d < 3; d++)
+                    s_mf[d * NU + tid] = ff_add(ff_add(ff_mul_f(cm[3 * d], m0), ff_mul_f(cm[3 * d + 1], m1)), ff_mul_f(cm[3 * d + 2], m2));
+            }
+        } else if (tid < NU + NF) {
+            const int s = tid - NU;
+            const long long og = gf0 + s;
+            const uint32_t pc = a.partner[og];
+            const bool isL = (pc & FR_LFLAG) != 0;
+            const long long pg = fr_partner(a, pc, og);
+            const float *uL = a.UF + (isL ? og : pg), *uR = a.UF + (isL ? pg : og);
+            const float wl = 0.5f - ph.beta, wr = 0.5f + ph.beta;
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++, uL += a.nfpt, uR += a.nfpt) s_c[alpha * NF + s] = wl * *uL + wr * *uR;
+            if ((isL ? wr : wl) == 0.f) {
+                float *fv = a.FV + og;
+#pragma unroll
+                for (int k = 0; k < 4; k++, fv += a.nfpt) *fv = 0.f;
+            } else {
+                s_plist[atomicAdd(&s_pcnt, 1)] = (short)s;
+            }
+        }
+        __syncthreads();
+        const int nplist = s_pcnt;
+        // 2. corrected gradient: x and y of the triangle planes (alpha, k) on warps 0 and 1, z lines
+        //    (alpha, t) on warps 2 and 3
+        if (warp < 2) {
+            if (lane < 5 * NZ) {
+                const int alpha = lane / NZ, k = lane % NZ;
+                const float *x = s_u + alpha * NU + 10 * k, *c = s_c + alpha * NF + 20 + 4 * k;
+                float u[NT_], cf[12];
+#pragma unroll
+                for (int t = 0; t < NT_; t++) u[t] = x[t];
+#pragma unroll
+                for (int b = 0; b < 12; b++) cf[b] = c[16 * (b / 4) + b % 4];
+                float *q = s_u + (5 + alpha * 3 + warp) * NU + 10 * k;
+#pragma unroll 1
+                for (int t = 0; t < NT_; t++) {
+                    float L[24];
+#pragma unroll
+                    for (int i = 0; i < 6; i++) {
+                        const float4 y = *reinterpret_cast<const float4 *>(&so.dl[warp][t][4 * i]);
+                        L[4 * i] = y.x; L[4 * i + 1] = y.y; L[4 * i + 2] = y.z; L[4 * i + 3] = y.w;
+                    }
+                    float v = 0.f;
+#pragma unroll
+                    for (int j = 0; j < NT_; j++) v += L[j] * u[j];
+#pragma unroll
+                    for (int b = 0; b < 12; b++) v += L[NT_ + b] * cf[b];
+                    q[t] = v;
+                }
+            }
+        } else {
+            const int l = tid - 64;
+            if (l < 5 * NT_) {
+                const int alpha = l / NT_, t = l % NT_;
+                float u[NZ];
+#pragma unroll
+                for (int k = 0; k < NZ; k++) u[k] = s_u[alpha * NU + t + 10 * k];
+                const float cB = s_c[alpha * NF + t], cT = s_c[alpha * NF + 10 + t];
+#pragma unroll
+                for (int k = 0; k < NZ; k++) {
+                    float v = op.liftzR[k] * cT - op.liftzL[k] * cB;
+#pragma unroll
+                    for (int j = 0; j < NZ; j++) v += op.Dhz[k][j] * u[j];
+                    s_u[(5 + alpha * 3 + 2) * NU + t + 10 * k] = v;
+                }
+            }
+        }
+        __syncthreads();
+        for (int it = tid; it < 5 * NU; it += NTH) {   // q = J^-T q~
+            float *q = s_u + (5 + it / NU * 3) * NU + it % NU;
+            const float q0 = q[0], q1 = q[NU], q2 = q[2 * NU];
+#pragma unroll
+            for (int k = 0; k < 3; k++) q[k * NU] = g.Ji[k] * q0 + g.Ji[3 + k] * q1 + g.Ji[6 + k] * q2;
+        }
+        __syncthreads();
+        // 3. traces of the 20 fields at the listed flux points, four threads per point; z lines of the
+        //    interpolation
+        for (int it = tid; it < 4 * nplist; it += NTH) {
+            const int li = it >> 2, fg = it & 3, s = s_plist[li];
+            const float *x = s_u + 5 * fg * NU;
+            float v[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+            if (s < 20) {
+                const float *l = so.lz[s / 10];
+                x += s % 10;
+#pragma unroll
+                for (int k = 0; k < NZ; k++)
+#pragma unroll
+                    for (int i = 0; i < 5; i++) v[i] += l[k] * x[i * NU + 10 * k];
+            } else {
+                const int f = (s - 20) / 16, loc = (s - 20) % 16;
+                const float *l = so.ef[f][loc % 4];
+                x += 10 * (loc / 4);
+#pragma unroll
+                for (int j = 0; j < NT_; j++)
+#pragma unroll
+                    for (int i = 0; i < 5; i++) v[i] += l[j] * x[i * NU + j];
+            }
+#pragma unroll
+            for (int i = 0; i < 5; i++) s_tr[li * 20 + 5 * fg + i] = v[i];
+        }
+        for (int it = tid; it < 20 * NT_; it += NTH) {
+            const int f = it / NT_, t = it % NT_;
+            float u[NZ];
+#pragma unroll
+            for (int k = 0; k < NZ; k++) u[k] = s_u[f * NU + t + 10 * k];
+#pragma unroll
+            for (int c = 0; c < MZ; c++) {
+                float v = 0.f;
+#pragma unroll
+                for (int k = 0; k < NZ; k++) v += op.Bz[c][k] * u[k];
+                s_t[(f * MZ + c) * P32_TS + t] = v;
+            }
+        }
+        __syncthreads();
+        // 4. own-normal viscous flux at the listed flux points (from the upper warps down)
+        for (int li = NTH - 1 - tid; li < nplist; li += NTH) {
+            const int s = s_plist[li];
+            const float *v = s_tr + li * 20;
+            float uf[5], qf[5][3];
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) {
+                uf[alpha] = v[alpha];
+#pragma unroll
+                for (int d = 0; d < 3; d++) qf[alpha][d] = v[5 + alpha * 3 + d];
+            }
+            const float *nt = a.fnrm + (e * 6 + face_of(s)) * 4;
+            const float n[3] = {nt[0], nt[1], nt[2]};
+            if (dev) { uf[0] += ph.rref; uf[4] += ph.eref; }
+            float fvn[4];
+            viscous_normal_flux(ph, uf, qf, n, fvn);
+            float *fv = a.FV + gf0 + s;
+#pragma unroll
+            for (int k = 0; k < 4; k++, fv += a.nfpt) *fv = fvn[k];
+        }
+        // 5. this thread's quadrature point: triangle-plane interpolation, flux and its transformation
+        bool ok = true;
+        float f[3][5];
+        if (tid < NQ) {
+            float u[5], gq[5][3];
+#pragma unroll
+            for (int i = 0; i < 20; i++) {
+                const float *x = s_t + (i * MZ + tc_) * P32_TS;
+                const float4 x0 = *reinterpret_cast<const float4 *>(x), x1 = *reinterpret_cast<const float4 *>(x + 4);
+                const float2 x2 = *reinterpret_cast<const float2 *>(x + 8);
+                float v = bt[0] * x0.x;
+                v += bt[1] * x0.y; v += bt[2] * x0.z; v += bt[3] * x0.w;
+                v += bt[4] * x1.x; v += bt[5] * x1.y; v += bt[6] * x1.z; v += bt[7] * x1.w;
+                v += bt[8] * x2.x; v += bt[9] * x2.y;
+                if (i < 5) u[i] = v;
+                else gq[(i - 5) / 3][(i - 5) % 3] = v;
+            }
+            if (dev) ok = total_flux_dev(ph, u, gq, f);
+            else ok = total_flux(ph, u, gq, f);
+        }
+        flag_status(a.status, ok);
+        __syncthreads();   // the interpolated fields and the traces are read
+        if (tid < NQ) {
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++)
+                if (alpha >= a0) {
+#pragma unroll
+                    for (int d = 0; d < 3; d++)
+                        s_w[(alpha * 3 + d) * MZ * P32_WS + tc_ * P32_WS + tq] =
+                            g.det * (g.Ji[3 * d] * f[0][alpha] + g.Ji[3 * d + 1] * f[1][alpha] + g.Ji[3 * d + 2] * f[2][alpha]);
+                }
+        }
+        __syncthreads();
+        // 6. projection with the corrected divergence in the triangle planes (alpha, c), one direction per
+        //    warp; the fourth warp forms the low-Mach form's volume part of R~_rho in float-float (rho v lies
+        //    in the solution space, so its projection is itself)
+        if (warp < 3) {
+            const int alpha = a0 + lane / MZ, c = lane % MZ;
+            if (alpha < 5 && lane < 25) {
+                const float *x = s_w + (alpha * 3 + warp) * MZ * P32_WS + c * P32_WS;
+                float *p = s_p + (alpha * 3 + warp) * MZ * NT_ + c * NT_;
+                float w[NQT];
+                w[24] = x[24];
+#pragma unroll
+                for (int i = 0; i < 6; i++) {
+                    const float4 y = *reinterpret_cast<const float4 *>(x + 4 * i);
+                    w[4 * i] = y.x; w[4 * i + 1] = y.y; w[4 * i + 2] = y.z; w[4 * i + 3] = y.w;
+                }
+#pragma unroll 1
+                for (int t = 0; t < NT_; t++) {
+                    float v = so.pt[warp][t][24] * w[24];
+#pragma unroll
+                    for (int i = 0; i < 6; i++) {
+                        const float4 y = *reinterpret_cast<const float4 *>(&so.pt[warp][t][4 * i]);
+                        v += y.x * w[4 * i]; v += y.y * w[4 * i + 1]; v += y.z * w[4 * i + 2]; v += y.w * w[4 * i + 3];
+                    }
+                    p[t] = v;
+                }
+            }
+        } else if (dev) {
+            for (int z = lane; z < NU; z += 32) {
+                const int k = z / NT_, t = z % NT_;
+                float sh = 0.0f, c = 0.0f;   // compensated dot product (Dot2)
+#pragma unroll
+                for (int j = 0; j < NT_; j++) {
+                    dot2ff_next(so.dx[t][j], s_mf[j + 10 * k], sh, c);
+                    dot2ff_next(so.dy[t][j], s_mf[NU + j + 10 * k], sh, c);
+                }
+#pragma unroll
+                for (int j = 0; j < NZ; j++) dot2ff_next(so.dz[k][j], s_mf[2 * NU + t + 10 * j], sh, c);
+                a.RL[u0 / FR_NV + z] = two_sum(sh, c);
+            }
+        }
+        if (tid == 0) s_pcnt = 0;
+        __syncthreads();
+        // 7. z lines (alpha, t) and the sum of the three components
+        if (tid < (5 - a0) * NT_) {
+            const int alpha = a0 + tid / NT_, t = tid % NT_;
+            float v[NZ] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int d = 0; d < 3; d++)
+#pragma unroll
+                for (int c = 0; c < MZ; c++) {
+                    const float x = s_p[(alpha * 3 + d) * MZ * NT_ + c * NT_ + t];
+#pragma unroll
+                    for (int k = 0; k < NZ; k++) v[k] += op.PZ[d][k][c] * x;
+                }
+            float *R = a.R + u0 + alpha * NU + t;
+#pragma unroll
+            for (int k = 0; k < NZ; k++) R[10 * k] = v[k];
+        }
+        __syncthreads();
+    }
+}
 
 // -------------------------------------------------------------------------------------------------
 // Phase B in FP64: the operators in block fixed point (fr_fx.cuh), one element per CTA
