@@ -204,6 +204,58 @@ k_dense_disu(HexArgs<T> a, const OPS *__restrict__ op, const FFOf<OPS> *__restri
     }
 }
 
+// The same in FP64, with the face values in block fixed point (fr_fx.cuh): on the FP64 pipe the 5 NU
+// multiply-adds per flux point bounded the kernel. A thread keeps its column of M0 in registers.
+template <typename OPS, int EPB>
+__global__ void __launch_bounds__(OPS::NF * EPB) k_dense_disu_fx(HexArgs<double> a, const OPS *__restrict__ ops)
+{
+    constexpr int NU = OPS::NU, NF = OPS::NF, NUS = OPS::NUS, NTH = NF * EPB;
+    static_assert(NU <= 32 && NTH % 32 == 0, "one variable of one element per warp pass");
+    const auto &op = ops->fx;
+    __shared__ __align__(16) fx2 s_u[EPB][FR_NV * NUS];
+    __shared__ int s_E[EPB * FR_NV];
+    const int el = threadIdx.x / NF, s = threadIdx.x % NF, kM = op.kM;
+    fx2 col[NUS];
+#pragma unroll
+    for (int z = 0; z < NUS; z++) col[z] = op.M0t[z][s];   // pad rows are zero
+    if constexpr (NUS > NU) {
+        for (int i = threadIdx.x; i < EPB * FR_NV * (NUS - NU); i += NTH) {
+            const int l = i / (FR_NV * (NUS - NU)), r = i % (FR_NV * (NUS - NU));
+            s_u[l][(r / (NUS - NU)) * NUS + NU + r % (NUS - NU)] = fx2{0, 0};
+        }
+    }
+    const long long ng = (a.ne + EPB - 1) / EPB;
+    for (long long g = blockIdx.x; g < ng; g += gridDim.x) {
+        const long long e0 = g * EPB;
+        const int nel = (int)(a.ne - e0 < EPB ? a.ne - e0 : EPB);
+        {
+            bool blk_ok = true;
+            for (int k = 0; k < nel; k++) blk_ok = blk_ok && fr_elem_ok(a, e0 + k, NU, NF);
+            if (!blk_ok) continue;
+        }
+        for (int b = threadIdx.x / 32; b < nel * FR_NV; b += NTH / 32)
+            fx_warp_block<1>(a.U + elem_u0(a, e0 + b / FR_NV, NU) + (b % FR_NV) * NU, NU, s_u[b / FR_NV] + (b % FR_NV) * NUS, s_E + b);
+        __syncthreads();
+        if (el < nel) {
+            double *o = a.UF + elem_f0(a, e0 + el, NF) + s;
+#pragma unroll 1
+            for (int alpha = 0; alpha < FR_NV; alpha++, o += a.nfpt) {
+                const fx2 *u = s_u[el] + alpha * NUS;
+                const int E = s_E[el * FR_NV + alpha];
+                fxacc t{0, 0};
+#pragma unroll
+                for (int z = 0; z < NUS; z += 2) {
+                    const int4 y = *reinterpret_cast<const int4 *>(u + z);
+                    fx_mac(t, col[z], fx2{y.x, y.y});
+                    fx_mac(t, col[z + 1], fx2{y.z, y.w});
+                }
+                *o = fx_double(fx_sum(t), E - 1080 + kM, E >= 2047);
+            }
+        }
+        __syncthreads();
+    }
+}
+
 // -------------------------------------------------------------------------------------------------
 // Phase B: volume group, one element per CTA of NTH threads (persistent over elements)
 // -------------------------------------------------------------------------------------------------
@@ -605,7 +657,7 @@ __global__ void __launch_bounds__(NTH, 4) k_dense_B_fx(HexArgs<double> a, const 
     constexpr int NU = OPS::NU, NF = OPS::NF, NFACE = OPS::NFACE, NUS = OPS::NUS;
     constexpr int NCH = NTH / NU;                 // quadrature-point chunks of the projection
     static_assert(NTH == 128 && NU + NF <= NTH, "one thread per quadrature point, state and flux point");
-    static_assert((3 * NQP + NCH - 1) / NCH <= 128, "terms of one 64-bit projection sum");
+    static_assert((3 * NQP + NCH - 1) / NCH + 6 <= 128 && NQP % 2 == 0 && NUS % 2 == 0, "terms of one 64-bit projection sum");
     const auto &op = ops->fx;
     __shared__ __align__(16) fx2 s_u[20 * NUS];          // state, then the physical gradient (5 + 3 alpha + d)
     __shared__ fx2 s_c[5 * NF];                          // common solution
@@ -729,11 +781,19 @@ __global__ void __launch_bounds__(NTH, 4) k_dense_B_fx(HexArgs<double> a, const 
             fxacc t[20];
 #pragma unroll
             for (int i = 0; i < 20; i++) t[i] = fxacc{0, 0};
+            // two solution points per step (16-byte loads of a field's values), their operator entries
+            // fetched a step ahead
+            fx2 n0 = op.Bt[0][tid], n1 = op.Bt[1][tid];
 #pragma unroll 1
-            for (int j = 0; j < NU; j++) {
-                const fx2 b = op.Bt[j][tid];
+            for (int j = 0; j < NUS; j += 2) {
+                const fx2 b0 = n0, b1 = n1;
+                if (j + 2 < NUS) { n0 = op.Bt[j + 2][tid]; n1 = op.Bt[j + 3][tid]; }   // (pad rows are zero)
 #pragma unroll
-                for (int i = 0; i < 20; i++) fx_mac(t[i], b, s_u[i * NUS + j]);
+                for (int i = 0; i < 20; i++) {
+                    const int4 y = *reinterpret_cast<const int4 *>(s_u + i * NUS + j);
+                    fx_mac(t[i], b0, fx2{y.x, y.y});
+                    fx_mac(t[i], b1, fx2{y.z, y.w});
+                }
             }
             double u[5], gq[5][3];
 #pragma unroll
@@ -796,15 +856,19 @@ __global__ void __launch_bounds__(NTH, 4) k_dense_B_fx(HexArgs<double> a, const 
         //    thread (z, chunk) over its quadrature points, all variables; then the chunks' sums
         if (tid < NU * NCH) {
             const int z = tid % NU, c = tid / NU;
-            const int qb = c * NQP / NCH, qn = (c + 1) * NQP / NCH;
+            const int qb = c * (NQP / 2) / NCH * 2, qn = (c + 1) * (NQP / 2) / NCH * 2;
             fxacc acc[5] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}, {0, 0}};
 #pragma unroll 1
             for (int d = 0; d < 3; d++)
 #pragma unroll 2
-                for (int q = qb; q < qn; q++) {
-                    const fx2 m = op.Dvt[d][q][z];
+                for (int q = qb; q < qn; q += 2) {
+                    const fx2 m0 = op.Dvt[d][q][z], m1 = op.Dvt[d][q + 1][z];
 #pragma unroll
-                    for (int alpha = 0; alpha < 5; alpha++) fx_mac(acc[alpha], m, s_w[(alpha * 3 + d) * NQP + q]);
+                    for (int alpha = 0; alpha < 5; alpha++) {
+                        const int4 y = *reinterpret_cast<const int4 *>(s_w + (alpha * 3 + d) * NQP + q);
+                        fx_mac(acc[alpha], m0, fx2{y.x, y.y});
+                        fx_mac(acc[alpha], m1, fx2{y.z, y.w});
+                    }
                 }
 #pragma unroll
             for (int alpha = 0; alpha < 5; alpha++) s_red[(c * 5 + alpha) * NU + z] = fx_sum(acc[alpha]);
@@ -836,8 +900,11 @@ __global__ void __launch_bounds__(OPS::NF * EPB, sizeof(T) == 4 ? 1280 / (OPS::N
     constexpr int NU = OPS::NU, NF = OPS::NF, NTH = NF * EPB;
     constexpr bool F32 = sizeof(T) == 4;
     constexpr int VN = V16<T>::n;
-    static_assert(NF % VN == 0, "flux-point rows are whole 16-byte vectors");
-    __shared__ __align__(16) T s_d[EPB][FR_NV * NF];
+    static_assert(NF % VN == 0 && NF % 2 == 0 && NTH % 32 == 0, "flux-point rows are whole 16-byte vectors; whole warps");
+    __shared__ __align__(16) T s_d[F32 ? EPB : 1][F32 ? FR_NV * NF : 1];
+    // FP64: the lift in block fixed point (fr_fx.cuh)
+    __shared__ __align__(16) fx2 s_dx[F32 ? 1 : EPB][F32 ? 2 : FR_NV * NF];
+    __shared__ int s_mx[F32 ? 1 : EPB][FR_NV];
     __shared__ ff s_dff[F32 ? EPB : 1][F32 ? NF : 1];    // low-Mach form: scaled common mass flux (float-float)
     __shared__ ff s_rr[F32 ? EPB : 1][F32 ? NU : 1];     // low-Mach form: R_rho (float-float)
     __shared__ ff s_idet[F32 ? EPB : 1];                 // low-Mach form: -1 / det J (float-float)
@@ -851,6 +918,11 @@ __global__ void __launch_bounds__(OPS::NF * EPB, sizeof(T) == 4 ? 1280 / (OPS::N
             for (int k = 0; k < nel; k++) blk_ok = blk_ok && fr_elem_ok(a, e0 + k, NU, NF);
             if (!blk_ok) continue;
         }
+        if constexpr (!F32) {
+            for (int i = threadIdx.x; i < EPB * FR_NV; i += NTH) s_mx[i / FR_NV][i % FR_NV] = 0;
+            __syncthreads();
+        }
+        T dv[5] = {T(0), T(0), T(0), T(0), T(0)};
         bool ok = true;
         if (el < nel) {
             const long long e = e0 + el;
@@ -859,39 +931,81 @@ __global__ void __launch_bounds__(OPS::NF * EPB, sizeof(T) == 4 ? 1280 / (OPS::N
             const uint32_t pc = a.partner[og];
             const bool isL = (pc & FR_LFLAG) != 0;
             const long long pg = fr_partner(a, pc, og);
-            T uo[5], up[5], fvo[4], fvp[4];
+            // own and partner values (the own ones do not wait for the partner's index), then the pair's L and
+            // R states: one flux evaluation per warp, whatever roles its points have
+            T uL[5], uR[5], fvL[4], fvR[4];
 #pragma unroll
-            for (int k = 0; k < 5; k++) { uo[k] = a.UF[k * a.nfpt + og]; up[k] = a.UF[k * a.nfpt + pg]; }
+            for (int k = 0; k < 5; k++) { uL[k] = a.UF[k * a.nfpt + og]; uR[k] = a.UF[k * a.nfpt + pg]; }
 #pragma unroll
-            for (int k = 0; k < 4; k++) { fvo[k] = a.FV[k * a.nfpt + og]; fvp[k] = a.FV[k * a.nfpt + pg]; }
+            for (int k = 0; k < 4; k++) { fvL[k] = a.FV[k * a.nfpt + og]; fvR[k] = a.FV[k * a.nfpt + pg]; }
+#pragma unroll
+            for (int k = 0; k < 5; k++) { const T o = uL[k]; uL[k] = isL ? o : uR[k]; uR[k] = isL ? uR[k] : o; }
+#pragma unroll
+            for (int k = 0; k < 4; k++) { const T o = fvL[k]; fvL[k] = isL ? o : fvR[k]; fvR[k] = isL ? fvR[k] : o; }
             const T *nt = a.fnrm + (e * 6 + OPS::FACE(s)) * 4;
             const T mag = nt[3];
-            T nL[3] = {isL ? nt[0] : -nt[0], isL ? nt[1] : -nt[1], isL ? nt[2] : -nt[2]};
+            const T nL[3] = {isL ? nt[0] : -nt[0], isL ? nt[1] : -nt[1], isL ? nt[2] : -nt[2]};
             T F[5];
             bool dev = false;
             if constexpr (F32) dev = ph.dev != 0;
             if (dev) {
                 if constexpr (F32) {
                     float sw;
-                    ok = isL ? common_flux_dev(ph, uo, up, fvo, fvp, nL, F, sw) : common_flux_dev(ph, up, uo, fvp, fvo, nL, F, sw);
+                    ok = common_flux_dev(ph, uL, uR, fvL, fvR, nL, F, sw);
                     // mass flux in float-float: 1/2 (mL - mR) + (s/2 + tau)(rho_L - rho_R), mX = own-normal n.(rho v)
                     const ff mo = a.MF[og], mp = a.MF[pg];
                     const ff mL = isL ? mo : mp, mR = isL ? mp : mo;
-                    const float rL = isL ? uo[0] : up[0], rR = isL ? up[0] : uo[0];
-                    const ff Fr = ff_add(ff_mul_f(ff_sub(mL, mR), 0.5f), ff_mul_f(two_sum(rL, -rR), 0.5f * sw + ph.tau));
-                    const ff magf = a.fnrm64[(e * 6 + OPS::FACE(s)) * 4 + 3];
-                    s_dff[el][s] = isL ? ff_mul(magf, Fr) : ff_neg(ff_mul(magf, Fr));
+                    const ff Fr = ff_add(ff_mul_f(ff_sub(mL, mR), 0.5f), ff_mul_f(two_sum(uL[0], -uR[0]), 0.5f * sw + ph.tau));
+                    const ff magf = a.fnrm64[(e * 6 + OPS::FACE(s)) * 4 + 3], Dr = ff_mul(magf, Fr);
+                    s_dff[el][s] = isL ? Dr : ff_neg(Dr);
                     if (s == 0) s_idet[el] = a.geo64[e].idet;
                 }
             } else {
-                ok = isL ? common_flux(ph, uo, up, fvo, fvp, nL, F) : common_flux(ph, up, uo, fvp, fvo, nL, F);
+                ok = common_flux(ph, uL, uR, fvL, fvR, nL, F);
             }
             const T sc = isL ? mag : -mag;
 #pragma unroll
-            for (int k = 0; k < 5; k++) s_d[el][k * NF + s] = sc * F[k];
+            for (int k = 0; k < 5; k++) {
+                if constexpr (F32) s_d[el][k * NF + s] = sc * F[k];
+                else dv[k] = sc * F[k];
+            }
         }
         flag_status(a.status, ok);
+        if constexpr (!F32) {
+            // each variable of each element scaled by its largest magnitude (a warp holds points of up to
+            // two elements)
+            const unsigned mask = __match_any_sync(0xffffffffu, el);
+#pragma unroll
+            for (int k = 0; k < 5; k++) {
+                const int m = (int)__reduce_max_sync(mask, (unsigned)fx_mag(dv[k])) >> 20;
+                if ((threadIdx.x & 31) == __ffs(mask) - 1) atomicMax(&s_mx[el][k], m);
+            }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < 5; k++) s_dx[el][k * NF + s] = fx_from(dv[k], s_mx[el][k]);
+        }
         __syncthreads();
+        if constexpr (!F32) {
+            const auto &fx = op->fx;
+            const int kD = fx.kD;
+            for (int i = threadIdx.x; i < nel * FR_NV * NU; i += NTH) {
+                const int l = i / (FR_NV * NU), alpha = (i / NU) % FR_NV, z = i % NU, E = s_mx[l][alpha];
+                const long long ui = elem_u0(a, e0 + l, NU) + alpha * NU + z;
+                const fx2 *D = s_dx[l] + alpha * NF;
+                fxacc t{0, 0};
+#pragma unroll 4
+                for (int s2 = 0; s2 < NF; s2 += 2) {
+                    const int4 y = *reinterpret_cast<const int4 *>(D + s2);
+                    fx_mac(t, fx.Lt[s2][z], fx2{y.x, y.y});
+                    fx_mac(t, fx.Lt[s2 + 1][z], fx2{y.z, y.w});
+                }
+                const double v = (a.R[ui] + fx_double(fx_sum(t), E - 1080 + kD, E >= 2047)) * a.geo[e0 + l].nidet;
+                if (a.rkstage == 0) a.R[ui] = v;
+                else rk_fold(a, ui, v);
+            }
+            __syncthreads();
+            continue;
+        }
         // lift and scale: R += L D, R *= -1/det; the mass rows of low-Mach elements in float-float,
         // then the energy rows, which add H0 R_rho
         for (int pass = 0; pass < 2; pass++) {
@@ -971,7 +1085,8 @@ int dense_phase(int phase, const HexArgs<T> &a, const OPS *ops, const FFOf<OPS> 
     constexpr int NU = OPS::NU, NF = OPS::NF, NUS = OPS::NUS;
     if (a.ne == 0) return 0;
     if (phase == 0) {
-        k_dense_disu<T, OPS, 4><<<grid_groups(a.ne, 4, 8), NF * 4, 0, s>>>(a, ops, opsff);
+        if constexpr (sizeof(T) == 8) k_dense_disu_fx<OPS, 4><<<grid_groups(a.ne, 4, 8), NF * 4, 0, s>>>(a, ops);
+        else k_dense_disu<T, OPS, 4><<<grid_groups(a.ne, 4, 8), NF * 4, 0, s>>>(a, ops, opsff);
     } else if (phase == 1) {
         constexpr int NTH = 128;
         const size_t base = (size_t)(20 * NUS + 5 * NF + 20 * NQP) * sizeof(T);

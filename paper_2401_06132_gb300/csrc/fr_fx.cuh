@@ -102,6 +102,56 @@ __device__ __forceinline__ double fx_double(long long y, int e2, bool bad)
     return __hiloint2double(hi, (int)(unsigned)b);
 }
 
+// One warp: the n values at src (n <= 32 KR) to limbs at dst, scaled by their largest magnitude; its
+// exponent field goes to *E (by lane 0).
+template <int KR>
+__device__ __forceinline__ void fx_warp_block(const double *src, int n, fx2 *dst, int *E)
+{
+    const int lane = threadIdx.x & 31;
+    double v[KR];
+    int m = 0;
+#pragma unroll
+    for (int k = 0; k < KR; k++) {
+        v[k] = lane + 32 * k < n ? src[lane + 32 * k] : 0.0;
+        m = max(m, fx_mag(v[k]));
+    }
+    const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)m) >> 20;
+    if (lane == 0) *E = e;
+#pragma unroll
+    for (int k = 0; k < KR; k++)
+        if (lane + 32 * k < n) dst[lane + 32 * k] = fx_from(v[k], e);
+}
+
+// A CTA of one element: the values v[rd][alpha] of flux points threadIdx.x + rd NT (below NF) to limbs at
+// dst[alpha NF + s], each variable scaled by its largest magnitude (exponent fields in E). mx: two sets of
+// five words, zero at first, used in turn (par). Two barriers.
+template <int NF, int NT, int RD>
+__device__ __forceinline__ void fx_stage5(const double (&v)[RD][5], fx2 *dst, int (*mx)[5], int &par, int (&E)[5])
+{
+#pragma unroll
+    for (int a = 0; a < 5; a++) {
+        int m = 0;
+#pragma unroll
+        for (int rd = 0; rd < RD; rd++) m = max(m, fx_mag(v[rd][a]));
+        m = (int)__reduce_max_sync(0xffffffffu, (unsigned)m) >> 20;
+        if ((threadIdx.x & 31) == 0) atomicMax(&mx[par][a], m);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < 5; a++) E[a] = mx[par][a];
+    if (threadIdx.x < 5) mx[par ^ 1][threadIdx.x] = 0;
+    par ^= 1;
+#pragma unroll
+    for (int rd = 0; rd < RD; rd++) {
+        const int s = threadIdx.x + rd * NT;
+        if (s < NF) {
+#pragma unroll
+            for (int a = 0; a < 5; a++) dst[a * NF + s] = fx_from(v[rd][a], E[a]);
+        }
+    }
+    __syncthreads();
+}
+
 // A run-time factor c (of an element's metric) in limbs for the common exponent E of its block:
 // c 2^(1080 - E), below 2^58.
 __device__ __forceinline__ fx2 fx_factor(double c, int E)

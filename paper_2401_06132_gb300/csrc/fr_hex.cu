@@ -223,16 +223,9 @@ __device__ __forceinline__ void disu_blk_body(const HexArgs<T> &a, long long fir
     __shared__ T s_u[EB * FR_NV * NU];
     // the trace rows, selected by each flux point's run-time face side, from shared memory (a
     // constant-memory load is serialised over the distinct addresses of a warp)
-    __shared__ T s_l[2 * N];
-    __shared__ ff s_lff[std::is_same<T, float>::value ? 2 * N : 1];
-    {
-        const HexOps<T> &op = OPS<T>(P - 2);
-        for (int i = threadIdx.x; i < 2 * N; i += NT) {
-            s_l[i] = i < N ? op.lL[i] : op.lR[i - N];
-            if constexpr (std::is_same<T, float>::value) s_lff[i] = i < N ? c_hexff[P - 2].lL[i] : c_hexff[P - 2].lR[i - N];
-        }
-        __syncthreads();
-    }
+    __shared__ ff s_lff[2 * N];
+    for (int i = threadIdx.x; i < 2 * N; i += NT) s_lff[i] = i < N ? c_hexff[P - 2].lL[i] : c_hexff[P - 2].lR[i - N];
+    __syncthreads();
     for (long long e0 = (long long)first * EB; e0 < a.ne; e0 += (long long)stride * EB) {
         const int nb = (int)((a.ne - e0) < EB ? (a.ne - e0) : EB);
         {
@@ -289,16 +282,49 @@ __device__ __forceinline__ void disu_blk_body(const HexArgs<T> &a, long long fir
                     }
                     a.MF[fo] = mf;
                 }
-            } else {
-                const T *l = s_l + (f & 1) * N;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// The same in FP64, with the traces in block fixed point (fr_fx.cuh): on the FP64 pipe the 20 multiply-adds
+// per flux point bounded the kernel.
+template <int P, int EB, int NT>
+__device__ __forceinline__ void disu_fx_body(const HexArgs<double> &a, long long first, long long stride)
+{
+    constexpr int N = P + 1, NU = N * N * N, NF = 6 * N * N;
+    __shared__ fx2 s_u[EB * FR_NV * NU];
+    __shared__ int s_E[EB * FR_NV];
+    __shared__ fx2 s_l[2][N];
+    for (int i = threadIdx.x; i < 2 * N; i += NT) s_l[i / N][i % N] = i < N ? c_hexfx[P - 2].lL[i] : c_hexfx[P - 2].lR[i - N];
+    __syncthreads();
+    for (long long e0 = (long long)first * EB; e0 < a.ne; e0 += (long long)stride * EB) {
+        const int nb = (int)((a.ne - e0) < EB ? (a.ne - e0) : EB);
+        {
+            bool blk_ok = true;
+            for (int k = 0; k < nb; k++) blk_ok = blk_ok && fr_elem_ok(a, e0 + k, NU, NF);
+            if (!blk_ok) continue;
+        }
+        for (int b = threadIdx.x / 32; b < nb * FR_NV; b += NT / 32)   // one variable of one element per warp
+            fx_warp_block<(NU + 31) / 32>(a.U + elem_u0(a, e0 + b / FR_NV, NU) + (b % FR_NV) * NU, NU, s_u + b * NU, s_E + b);
+        __syncthreads();
+        for (int it = threadIdx.x; it < nb * NF; it += NT) {
+            const int el = it / NF, sp = it % NF, f = sp / (N * N);
+            int base, str;
+            face_line<N>(f, sp % (N * N), base, str);
+            double *o = a.UF + elem_f0(a, e0 + el, NF) + sp;
+            fx2 l[N];
 #pragma unroll
-                for (int alpha = 0; alpha < FR_NV; alpha++) {
-                    const T *u = s_u + (el * FR_NV + alpha) * NU + base;
-                    T v = T(0);
+            for (int i = 0; i < N; i++) l[i] = s_l[f & 1][i];
 #pragma unroll
-                    for (int i = 0; i < N; i++) v += l[i] * u[i * stride];
-                    a.UF[alpha * a.nfpt + fo] = v;
-                }
+            for (int alpha = 0; alpha < FR_NV; alpha++, o += a.nfpt) {
+                const fx2 *u = s_u + (el * FR_NV + alpha) * NU + base;
+                const int E = s_E[el * FR_NV + alpha];
+                fxacc t{0, 0};
+#pragma unroll
+                for (int i = 0; i < N; i++) fx_mac(t, l[i], u[i * str]);
+                *o = fx_double(fx_sum(t), E - 1080 + FX_KL, E >= 2047);
             }
         }
         __syncthreads();
@@ -306,9 +332,16 @@ __device__ __forceinline__ void disu_blk_body(const HexArgs<T> &a, long long fir
 }
 
 template <typename T, int P, int EB, int NT>
+__device__ __forceinline__ void face_body(const HexArgs<T> &a, long long first, long long stride)
+{
+    if constexpr (sizeof(T) == 8) disu_fx_body<P, EB, NT>(a, first, stride);
+    else disu_blk_body<T, P, EB, NT>(a, first, stride);
+}
+
+template <typename T, int P, int EB, int NT>
 __global__ void __launch_bounds__(NT) k_disu_blk(HexArgs<T> a)
 {
-    disu_blk_body<T, P, EB, NT>(a, blockIdx.x, gridDim.x);
+    face_body<T, P, EB, NT>(a, blockIdx.x, gridDim.x);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2027,11 +2060,40 @@ __global__ void __launch_bounds__(NT, 896 / NT) k_fused_B_surf32(HexArgs<float> 
 // ---------------------------------------------------------------------------------------------
 // Fused phase C: comm_flux + tdivtconf + negdivconf per element
 // ---------------------------------------------------------------------------------------------
+// FP64: R += lift of the common flux held in block fixed point (D: [variable][flux point], exponent fields
+// E), R *= -1/det J, and the RK4 stage update. On the FP64 pipe the six multiply-adds per value were half
+// of the lift kernel's operations.
+template <int P, int NT, bool CURV>
+__device__ __forceinline__ void lift_fx(const HexArgs<double> &a, long long e, const fx2 *Dx, const fx2 *l, const int *E, double *R, double idet)
+{
+    constexpr int N = P + 1, NU = N * N * N, NF = 6 * N * N, N2 = N * N;
+    for (int it = threadIdx.x; it < 5 * NU; it += NT) {
+        const int alpha = it / NU, z = it % NU, i = z % N, j = (z / N) % N, k = z / N2;
+        const fx2 *D = Dx + alpha * NF;
+        fxacc t{0, 0};
+        fx_mac(t, l[i], D[j + N * k]);
+        fx_mac(t, l[N + i], D[N2 + j + N * k]);
+        fx_mac(t, l[j], D[2 * N2 + i + N * k]);
+        fx_mac(t, l[N + j], D[3 * N2 + i + N * k]);
+        fx_mac(t, l[k], D[4 * N2 + i + N * j]);
+        fx_mac(t, l[N + k], D[5 * N2 + i + N * j]);
+        // curved elements: det J at this solution point
+        const double sc = CURV ? -fr_inv(a.mu[(e * NU + z) * 10 + 9]) : idet;
+        const double v = (R[it] + fx_double(fx_sum(t), E[alpha] - 1080 + FX_KD, E[alpha] >= 2047)) * sc;
+        if (a.rkstage == 0) R[it] = v;
+        else rk_fold(a, elem_u0(a, e, NU) + it, v);
+    }
+}
+
 template <typename T, int P, int NT, bool CURV = false>
 __device__ __forceinline__ void fused_C_body(const HexArgs<T> &a, long long first, long long stride)
 {
     constexpr int N = P + 1, NU = N * N * N, NF = 6 * N * N;
-    __shared__ T s_d[5 * NF];
+    constexpr bool FX = sizeof(T) == 8;   // FP64: the lift in block fixed point (fr_fx.cuh)
+    constexpr int RD = (NF + NT - 1) / NT;
+    __shared__ T s_d[FX ? 1 : 5 * NF];
+    __shared__ fx2 s_dx[FX ? 5 * NF : 1], s_lx[2 * N];
+    __shared__ int s_mx[2][5];
     __shared__ ff s_dff[std::is_same<T, float>::value ? NF : 1];   // low-Mach form: transformed mass flux
     // the lift rows, read with each solution point's run-time (i, j, k), from shared memory: a
     // constant-memory load is serialised over the distinct addresses of a warp
@@ -2042,10 +2104,13 @@ __device__ __forceinline__ void fused_C_body(const HexArgs<T> &a, long long firs
         for (int i = threadIdx.x; i < 2 * N; i += NT) {
             s_lift[i] = i < N ? op.liftL[i] : op.liftR[i - N];
             if constexpr (std::is_same<T, float>::value) s_liftff[i] = i < N ? c_hexff[P - 2].liftL[i] : c_hexff[P - 2].liftR[i - N];
+            if constexpr (FX) s_lx[i] = i < N ? c_hexfx[P - 2].liftL[i] : c_hexfx[P - 2].liftR[i - N];
         }
+        if (threadIdx.x < 10) s_mx[threadIdx.x / 5][threadIdx.x % 5] = 0;
         __syncthreads();
     }
     const T *liftL = s_lift, *liftR = s_lift + N;
+    int par = 0;
     for (long long e = first; e < a.ne; e += stride) {
         if (!fr_elem_ok(a, e, (P + 1) * (P + 1) * (P + 1), 6 * (P + 1) * (P + 1))) continue;
         const Geo<T> g = a.geo[e];
@@ -2054,16 +2119,28 @@ __device__ __forceinline__ void fused_C_body(const HexArgs<T> &a, long long firs
         if constexpr (std::is_same<T, float>::value) dev = ph.dev != 0;
         const long long gf0 = elem_f0(a, e, NF);
         bool ok = true;
-        for (int s = threadIdx.x; s < NF; s += NT) {
+        T dv[RD][5];
+#pragma unroll
+        for (int rd = 0; rd < RD; rd++) {
+            const int s = threadIdx.x + rd * NT;
+#pragma unroll
+            for (int k = 0; k < 5; k++) dv[rd][k] = T(0);
+            if (s >= NF) continue;
             const int f = s / (N * N);
             const uint32_t pc = a.partner[gf0 + s];
             const bool isL = (pc & FR_LFLAG) != 0;
             const long long og = gf0 + s, pg = fr_partner(a, pc, og);
-            T uo[5], up[5], fvo[4], fvp[4];
+            // own and partner values (the own ones do not wait for the partner's index), then the pair's L and
+            // R states: one flux evaluation per warp, whatever roles its points have
+            T uL[5], uR[5], fvL[4], fvR[4];
 #pragma unroll
-            for (int k = 0; k < 5; k++) { uo[k] = a.UF[k * a.nfpt + og]; up[k] = a.UF[k * a.nfpt + pg]; }
+            for (int k = 0; k < 5; k++) { uL[k] = a.UF[k * a.nfpt + og]; uR[k] = a.UF[k * a.nfpt + pg]; }
 #pragma unroll
-            for (int k = 0; k < 4; k++) { fvo[k] = a.FV[k * a.nfpt + og]; fvp[k] = a.FV[k * a.nfpt + pg]; }
+            for (int k = 0; k < 4; k++) { fvL[k] = a.FV[k * a.nfpt + og]; fvR[k] = a.FV[k * a.nfpt + pg]; }
+#pragma unroll
+            for (int k = 0; k < 5; k++) { const T o = uL[k]; uL[k] = isL ? o : uR[k]; uR[k] = isL ? uR[k] : o; }
+#pragma unroll
+            for (int k = 0; k < 4; k++) { const T o = fvL[k]; fvL[k] = isL ? o : fvR[k]; fvR[k] = isL ? fvR[k] : o; }
             T n[3], mag;
             if constexpr (CURV) {   // curved elements: the normal at this flux point
                 const T *t = a.mfn + (e * NF + s) * 4;
@@ -2071,40 +2148,47 @@ __device__ __forceinline__ void fused_C_body(const HexArgs<T> &a, long long firs
             } else {
                 face_nrm<T, T>(a.fnrm, e, f, n, mag);
             }
-            T nL[3] = {isL ? n[0] : -n[0], isL ? n[1] : -n[1], isL ? n[2] : -n[2]};
+            const T nL[3] = {isL ? n[0] : -n[0], isL ? n[1] : -n[1], isL ? n[2] : -n[2]};
             T F[5];
-            if constexpr (std::is_same<T, float>::value) {
-                if (dev) {
+            if (dev) {
+                if constexpr (std::is_same<T, float>::value) {
                     float sw;
-                    ok &= isL ? common_flux_dev(ph, uo, up, fvo, fvp, nL, F, sw) : common_flux_dev(ph, up, uo, fvp, fvo, nL, F, sw);
+                    ok &= common_flux_dev(ph, uL, uR, fvL, fvR, nL, F, sw);
                     if constexpr (CURV) {
                         // curved elements: the mass equation runs through the FP32 flux path
-                        F[0] = isL ? common_mass_flux_dev(ph, uo, up, nL, sw) : common_mass_flux_dev(ph, up, uo, nL, sw);
+                        F[0] = common_mass_flux_dev(ph, uL, uR, nL, sw);
                     } else {
                         // mass flux in float-float: 1/2 (mL - mR) + (s/2 + tau)(rho_L - rho_R),
                         // mX = own-normal n.(rho v)
                         const ff mo = a.MF[og], mp = a.MF[pg];
                         const ff mL = isL ? mo : mp, mR = isL ? mp : mo;
-                        const float rL = isL ? uo[0] : up[0], rR = isL ? up[0] : uo[0];
-                        const ff Fr = ff_add(ff_mul_f(ff_sub(mL, mR), 0.5f), ff_mul_f(two_sum(rL, -rR), 0.5f * sw + ph.tau));
-                        const ff mag = a.fnrm64[(e * 6 + f) * 4 + 3];
-                        s_dff[s] = isL ? ff_mul(mag, Fr) : ff_neg(ff_mul(mag, Fr));
+                        const ff Fr = ff_add(ff_mul_f(ff_sub(mL, mR), 0.5f), ff_mul_f(two_sum(uL[0], -uR[0]), 0.5f * sw + ph.tau));
+                        const ff magf = a.fnrm64[(e * 6 + f) * 4 + 3], Dr = ff_mul(magf, Fr);
+                        s_dff[s] = isL ? Dr : ff_neg(Dr);
                     }
-                } else {
-                    ok &= isL ? common_flux(ph, uo, up, fvo, fvp, nL, F) : common_flux(ph, up, uo, fvp, fvo, nL, F);
                 }
             } else {
-                ok &= isL ? common_flux(ph, uo, up, fvo, fvp, nL, F) : common_flux(ph, up, uo, fvp, fvo, nL, F);
+                ok &= common_flux(ph, uL, uR, fvL, fvR, nL, F);
             }
             const T sc = isL ? mag : -mag;
 #pragma unroll
-            for (int k = 0; k < 5; k++) s_d[k * NF + s] = sc * F[k];
+            for (int k = 0; k < 5; k++) {
+                if constexpr (FX) dv[rd][k] = sc * F[k];
+                else s_d[k * NF + s] = sc * F[k];
+            }
         }
         flag_status(a.status, ok);
-        __syncthreads();
         T *R = a.R + elem_u0(a, e, NU);
         const T idet = g.nidet;
-        if (!dev) {
+        if constexpr (FX) {
+            int E[5];
+            fx_stage5<NF, NT, RD>(dv, s_dx, s_mx, par, E);
+            lift_fx<P, NT, CURV>(a, e, s_dx, s_lx, s_mx[par ^ 1], R, idet);
+        } else {
+            __syncthreads();
+        }
+        if constexpr (FX) {
+        } else if (!dev) {
             for (int it = threadIdx.x; it < 5 * NU; it += NT) {
                 const int alpha = it / NU, z = it % NU, i = z % N, j = (z / N) % N, k = z / (N * N);
                 const T *D = s_d + alpha * NF;
@@ -2116,7 +2200,7 @@ __device__ __forceinline__ void fused_C_body(const HexArgs<T> &a, long long firs
                 v += liftL[k] * D[4 * N * N + i + N * j];
                 v += liftR[k] * D[5 * N * N + i + N * j];
                 // curved elements: det J at this solution point
-                const T sc = CURV ? T(-1) / a.mu[(e * NU + z) * 10 + 9] : idet;
+                const T sc = CURV ? -fr_inv(a.mu[(e * NU + z) * 10 + 9]) : idet;
                 if (a.rkstage == 0) R[it] = v * sc;
                 else rk_fold(a, elem_u0(a, e, NU) + it, v * sc);
             }
@@ -2362,49 +2446,39 @@ __global__ void __launch_bounds__(128) k_pair_flux(HexArgs<T> a)
     flag_status(a.status, ok);
 }
 
-template <typename T, int P, int NT, bool CURV = false>
-__global__ void __launch_bounds__(NT) k_lift(HexArgs<T> a)
+template <int P, int NT, bool CURV = false>
+__global__ void __launch_bounds__(NT) k_lift(HexArgs<double> a)
 {
-    constexpr int N = P + 1, NU = N * N * N, NF = 6 * N * N;
-    __shared__ T s_d[5 * NF];
-    __shared__ T s_lift[2 * N];   // liftL | liftR, read with run-time (i, j, k)
-    {
-        const HexOps<T> &op = OPS<T>(P - 2);
-        for (int i = threadIdx.x; i < 2 * N; i += NT) s_lift[i] = i < N ? op.liftL[i] : op.liftR[i - N];
-        __syncthreads();
-    }
-    const T *liftL = s_lift, *liftR = s_lift + N;
+    constexpr int N = P + 1, NU = N * N * N, NF = 6 * N * N, RD = (NF + NT - 1) / NT;
+    __shared__ fx2 s_dx[5 * NF], s_lx[2 * N];   // s_lx: liftL | liftR, read with run-time (i, j, k)
+    __shared__ int s_mx[2][5];
+    for (int i = threadIdx.x; i < 2 * N; i += NT) s_lx[i] = i < N ? c_hexfx[P - 2].liftL[i] : c_hexfx[P - 2].liftR[i - N];
+    if (threadIdx.x < 10) s_mx[threadIdx.x / 5][threadIdx.x % 5] = 0;
+    __syncthreads();
+    int par = 0;
     for (long long e = blockIdx.x; e < a.ne; e += gridDim.x) {
         if (!fr_elem_ok(a, e, (P + 1) * (P + 1) * (P + 1), 6 * (P + 1) * (P + 1))) continue;
-        const Geo<T> g = a.geo[e];
+        const Geo<double> g = a.geo[e];
         const long long gf0 = elem_f0(a, e, NF);
-        for (int s = threadIdx.x; s < NF; s += NT) {
-            const uint32_t pc = a.partner[gf0 + s];
-            const bool isL = (pc & FR_LFLAG) != 0;
-            const long long src = isL ? gf0 + s : fr_partner(a, pc, gf0 + s);
-            const T mag = CURV ? a.mfn[(e * NF + s) * 4 + 3] : a.fnrm[(e * 6 + s / (N * N)) * 4 + 3];
-            const T sc = isL ? mag : -mag;
+        double dv[RD][5];
 #pragma unroll
-            for (int k = 0; k < 5; k++) s_d[k * NF + s] = sc * a.DF[k * a.nfpt + src];
+        for (int rd = 0; rd < RD; rd++) {
+            const int s = threadIdx.x + rd * NT;
+#pragma unroll
+            for (int k = 0; k < 5; k++) dv[rd][k] = 0.0;
+            if (s < NF) {
+                const uint32_t pc = a.partner[gf0 + s];
+                const bool isL = (pc & FR_LFLAG) != 0;
+                const double *D = a.DF + (isL ? gf0 + s : fr_partner(a, pc, gf0 + s));
+                const double mag = CURV ? a.mfn[(e * NF + s) * 4 + 3] : a.fnrm[(e * 6 + s / (N * N)) * 4 + 3];
+                const double sc = isL ? mag : -mag;
+#pragma unroll
+                for (int k = 0; k < 5; k++, D += a.nfpt) dv[rd][k] = sc * *D;
+            }
         }
-        __syncthreads();
-        T *R = a.R + elem_u0(a, e, NU);
-        const T idet = g.nidet;
-        for (int it = threadIdx.x; it < 5 * NU; it += NT) {
-            const int alpha = it / NU, z = it % NU, i = z % N, j = (z / N) % N, k = z / (N * N);
-            const T *D = s_d + alpha * NF;
-            T v = R[it];
-            v += liftL[i] * D[0 * N * N + j + N * k];
-            v += liftR[i] * D[1 * N * N + j + N * k];
-            v += liftL[j] * D[2 * N * N + i + N * k];
-            v += liftR[j] * D[3 * N * N + i + N * k];
-            v += liftL[k] * D[4 * N * N + i + N * j];
-            v += liftR[k] * D[5 * N * N + i + N * j];
-            // curved elements: det J at this solution point
-            const T sc = CURV ? T(-1) / a.mu[(e * NU + z) * 10 + 9] : idet;
-            if (a.rkstage == 0) R[it] = v * sc;
-            else rk_fold(a, elem_u0(a, e, NU) + it, v * sc);
-        }
+        int E[5];
+        fx_stage5<NF, NT, RD>(dv, s_dx, s_mx, par, E);
+        lift_fx<P, NT, CURV>(a, e, s_dx, s_lx, s_mx[par ^ 1], a.R + elem_u0(a, e, NU), g.nidet);
         __syncthreads();
     }
 }
@@ -3286,8 +3360,10 @@ static int fused_phase(int phase, const HexArgs<T> &a, cudaStream_t s, int varia
         else if (a.nlpts > 0) k_pair_flux<T, P><<<grid_for(a.nlpts, 128), 128, 0, s>>>(a);
     } else {
         if (a.surf) k_surf_lift<T, P, 128><<<grid_elems(a.ne, 8), 128, 0, s>>>(a);
-        else if (a.mu) k_lift<T, P, 128, true><<<grid_elems(a.ne, 8), 128, 0, s>>>(a);
-        else k_lift<T, P, 128><<<grid_elems(a.ne, 8), 128, 0, s>>>(a);
+        else if constexpr (sizeof(T) == 8) {   // (only FP64 hexahedral handles split the interface phase)
+            if (a.mu) k_lift<P, 128, true><<<grid_elems(a.ne, 8), 128, 0, s>>>(a);
+            else k_lift<P, 128><<<grid_elems(a.ne, 8), 128, 0, s>>>(a);
+        } else return -1;
     }
     return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
 }
@@ -3303,9 +3379,10 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_multi_A(MultiArgs<T> ma)
 {
     for (int g = 0; g < ma.ng; g++) {
-        if (ma.kind[g] == 3) disu_blk_body<T, 3, 8, 256>(ma.a[g], blockIdx.x, gridDim.x);
-        else if (ma.kind[g] == 4) disu_blk_body<T, 4, 8, 256>(ma.a[g], blockIdx.x, gridDim.x);
-        else pri::pri_disu_body<T>(ma.a[g], ma.pops, ma.pff, blockIdx.x, gridDim.x);
+        if (ma.kind[g] == 3) face_body<T, 3, 8, 256>(ma.a[g], blockIdx.x, gridDim.x);
+        else if (ma.kind[g] == 4) face_body<T, 4, 8, 256>(ma.a[g], blockIdx.x, gridDim.x);
+        else if constexpr (sizeof(T) == 8) pri::pri_disu_fx_body(ma.a[g], ma.pops, blockIdx.x, gridDim.x);
+        else pri::pri_disu_body(ma.a[g], ma.pff, blockIdx.x, gridDim.x);
         __syncthreads();
     }
 }

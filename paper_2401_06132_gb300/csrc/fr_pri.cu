@@ -28,7 +28,8 @@ namespace {
 template <typename T>
 __global__ void __launch_bounds__(256) k_pri_disu(HexArgs<T> a, const PriOps<T> *gops, const PriOpsFF *opsff)
 {
-    pri_disu_body<T>(a, gops, opsff, blockIdx.x, gridDim.x);
+    if constexpr (sizeof(T) == 8) pri_disu_fx_body(a, gops, blockIdx.x, gridDim.x);
+    else pri_disu_body(a, opsff, blockIdx.x, gridDim.x);
 }
 
 // FP32 on the CUDA cores: registers capped for eight CTAs of 128 threads per SM, as many as its
@@ -68,8 +69,9 @@ int pri_fused_phase(int phase, const HexArgs<T> &a, const PriOps<T> *ops, const 
 {
     if (a.ne == 0) return 0;
     if (phase == 0) {
-        long long work = a.ne * NF;
-        long long g = (work + 255) / 256;
+        // FP64: groups of three elements; FP32: flux points over whole CTAs
+        const long long g0 = sizeof(T) == 8 ? (a.ne + 2) / 3 : (a.ne * NF + 255) / 256;
+        long long g = g0;
         if (g > fr_sms() * 64) g = fr_sms() * 64;
         k_pri_disu<T><<<(int)g, 256, 0, s>>>(a, ops, ops64);
     } else if (phase == 1) {

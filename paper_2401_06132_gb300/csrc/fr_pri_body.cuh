@@ -138,17 +138,14 @@ struct PriTC {
 // the Rusanov dissipation (1/2)(|v.n| + c)(u_L - u_R), with c about 10 |v|, lifts any rounding of a
 // face value into R. Low-Mach form (ph.dev): the face solution of the deviations from the reference
 // state, and the own-normal mass flux n.(rho v) at every flux point in float-float.
-template <typename T>
-__device__ __forceinline__ void pri_disu_body(const HexArgs<T> &a, const PriOps<T> *gops, const PriOpsFF *opsff, long long first, long long stride)
+__device__ __forceinline__ void pri_disu_body(const HexArgs<float> &a, const PriOpsFF *opsff, long long first, long long stride)
 {
-    constexpr bool F32 = sizeof(T) == 4;
-    __shared__ __align__(16) unsigned char raw[F32 ? sizeof(PriOpsFF) : sizeof(PriOps<T>)];
-    if constexpr (F32) {
+    using T = float;
+    __shared__ __align__(16) unsigned char raw[sizeof(PriOpsFF)];
+    {
         const float *src = reinterpret_cast<const float *>(opsff);
         float *dst = reinterpret_cast<float *>(raw);
         for (int i = threadIdx.x; i < (int)(sizeof(PriOpsFF) / sizeof(float)); i += 256) dst[i] = src[i];
-    } else {
-        load_ops<T, 256>(gops, *reinterpret_cast<PriOps<T> *>(raw));
     }
     __syncthreads();
     const long long total = a.ne * NF;
@@ -167,7 +164,7 @@ __device__ __forceinline__ void pri_disu_body(const HexArgs<T> &a, const PriOps<
 #endif
         const T *u = a.U + elem_u0(a, e, NU);
         const long long fo = elem_f0(a, e, NF) + s;
-        if constexpr (F32) {
+        {
             const PriOpsFF &o = *reinterpret_cast<const PriOpsFF *>(raw);
             const Phys<T> ph = elem_phys(a, e);
             const bool dev = ph.dev != 0;
@@ -186,14 +183,55 @@ __device__ __forceinline__ void pri_disu_body(const HexArgs<T> &a, const PriOps<
                     if (nt[k].hi != 0.0f) mf = ff_fma(nt[k], v[1 + k], mf);
                 a.MF[fo] = mf;
             }
-        } else {
-            const PriOps<T> &op = *reinterpret_cast<const PriOps<T> *>(raw);
-#pragma unroll
-            for (int alpha = 0; alpha < FR_NV; alpha++) a.UF[alpha * a.nfpt + fo] = face_value(op, u + alpha * NU, s);
         }
     }
 }
 
+
+// The same in FP64, with the traces in block fixed point (fr_fx.cuh): EB elements per CTA of 256 threads.
+__device__ __forceinline__ void pri_disu_fx_body(const HexArgs<double> &a, const PriOps<double> *gops, long long first, long long stride)
+{
+    constexpr int EB = 3, NTH = 256;   // 204 flux points
+    __shared__ fx2 s_u[EB * FR_NV * NU], s_ef[3][NZ][NT_], s_lz[2][NZ];
+    __shared__ int s_E[EB * FR_NV];
+    const PriFxS &op = reinterpret_cast<const PriFx *>(gops + 1)->s;
+    for (int i = threadIdx.x; i < 3 * NZ * NT_; i += NTH) (&s_ef[0][0][0])[i] = (&op.Ef[0][0][0])[i];
+    for (int i = threadIdx.x; i < 2 * NZ; i += NTH) s_lz[i / NZ][i % NZ] = i < NZ ? op.lzL[i] : op.lzR[i - NZ];
+    const int kF = op.kF;
+    __syncthreads();
+    for (long long e0 = first * EB; e0 < a.ne; e0 += stride * EB) {
+        const int nb = (int)(a.ne - e0 < EB ? a.ne - e0 : EB);
+        {
+            bool blk_ok = true;
+            for (int k = 0; k < nb; k++) blk_ok = blk_ok && fr_elem_ok(a, e0 + k, NU, NF);
+            if (!blk_ok) continue;
+        }
+        for (int b = threadIdx.x / 32; b < nb * FR_NV; b += NTH / 32)   // one variable of one element per warp
+            fx_warp_block<(NU + 31) / 32>(a.U + elem_u0(a, e0 + b / FR_NV, NU) + (b % FR_NV) * NU, NU, s_u + b * NU, s_E + b);
+        __syncthreads();
+        for (int it = threadIdx.x; it < nb * NF; it += NTH) {
+            const int el = it / NF, s = it % NF;
+            double *o = a.UF + elem_f0(a, e0 + el, NF) + s;
+            const int f = (s - 20) / 16, loc = (s - 20) % 16;
+            const fx2 *l = s < 20 ? s_lz[s / 10] : s_ef[f][loc % 4];
+            const fx2 *u = s_u + el * FR_NV * NU + (s < 20 ? s % 10 : 10 * (loc / 4));
+            const int n = s < 20 ? NZ : NT_, str = s < 20 ? 10 : 1;
+            fxacc t[FR_NV] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}, {0, 0}};
+#pragma unroll 2
+            for (int j = 0; j < n; j++) {
+                const fx2 c = l[j];
+#pragma unroll
+                for (int alpha = 0; alpha < FR_NV; alpha++) fx_mac(t[alpha], c, u[alpha * NU + j * str]);
+            }
+#pragma unroll
+            for (int alpha = 0; alpha < FR_NV; alpha++, o += a.nfpt) {
+                const int E = s_E[el * FR_NV + alpha];
+                *o = fx_double(fx_sum(t[alpha]), E - 1080 + kF, E >= 2047);
+            }
+        }
+        __syncthreads();
+    }
+}
 
 // -------------------------------------------------------------------------------------------------
 // Phase B: volume group
@@ -1082,10 +1120,24 @@ __device__ __forceinline__ void pri_B_fx_body(const HexArgs<double> &a, const Pr
 template <typename T, int NTH>
 __device__ __forceinline__ void pri_C_body(const HexArgs<T> &a, const PriOps<T> *gops, const PriOpsFF *opsff, long long first, long long stride)
 {
-    __shared__ PriOps<T> op;
-    __shared__ T s_d[5 * NF];
+    constexpr bool FX = sizeof(T) == 8;   // FP64: the lift in block fixed point (fr_fx.cuh)
+    static_assert(!FX || NF <= NTH, "one flux point per thread");
+    __shared__ PriOps<typename std::conditional<FX, float, T>::type> op_;
+    __shared__ T s_d[FX ? 1 : 5 * NF];
+    __shared__ fx2 s_dx[FX ? 5 * NF : 1], s_lf[FX ? 3 * NT_ * NZ : 1], s_lz[FX ? 2 * NZ : 1];
+    __shared__ int s_mx[2][5];
     __shared__ ff s_dff[sizeof(T) == 4 ? NF : 1];   // low-Mach form: transformed mass flux (float-float)
-    load_ops<T, NTH>(gops, op);
+    const auto &op = op_;
+    int par = 0, kD = 0;
+    if constexpr (FX) {
+        const PriFxS &ox = reinterpret_cast<const PriFx *>(gops + 1)->s;
+        for (int i = threadIdx.x; i < 3 * NT_ * NZ; i += NTH) s_lf[i] = (&ox.Lf[0][0][0])[i];
+        for (int i = threadIdx.x; i < 2 * NZ; i += NTH) s_lz[i] = i < NZ ? ox.liftzL[i] : ox.liftzR[i - NZ];
+        if (threadIdx.x < 10) s_mx[threadIdx.x / 5][threadIdx.x % 5] = 0;
+        kD = ox.kD;
+    } else {
+        load_ops<T, NTH>(gops, op_);
+    }
     __syncthreads();
     for (long long e = first; e < a.ne; e += stride) {
         if (!fr_elem_ok(a, e, NU, NF)) continue;
@@ -1095,47 +1147,73 @@ __device__ __forceinline__ void pri_C_body(const HexArgs<T> &a, const PriOps<T> 
         bool dev = false;
         if constexpr (sizeof(T) == 4) dev = ph.dev != 0;
         bool ok = true;
+        T dv[1][5] = {{T(0), T(0), T(0), T(0), T(0)}};
         for (int s = threadIdx.x; s < NF; s += NTH) {
             const uint32_t pc = a.partner[gf0 + s];
             const bool isL = (pc & FR_LFLAG) != 0;
             const long long og = gf0 + s, pg = fr_partner(a, pc, og);
-            T uo[5], up[5], fvo[4], fvp[4];
+            // own and partner values (the own ones do not wait for the partner's index), then the pair's L and
+            // R states: one flux evaluation per warp, whatever roles its points have
+            T uL[5], uR[5], fvL[4], fvR[4];
 #pragma unroll
-            for (int k = 0; k < 5; k++) { uo[k] = a.UF[k * a.nfpt + og]; up[k] = a.UF[k * a.nfpt + pg]; }
+            for (int k = 0; k < 5; k++) { uL[k] = a.UF[k * a.nfpt + og]; uR[k] = a.UF[k * a.nfpt + pg]; }
 #pragma unroll
-            for (int k = 0; k < 4; k++) { fvo[k] = a.FV[k * a.nfpt + og]; fvp[k] = a.FV[k * a.nfpt + pg]; }
+            for (int k = 0; k < 4; k++) { fvL[k] = a.FV[k * a.nfpt + og]; fvR[k] = a.FV[k * a.nfpt + pg]; }
+#pragma unroll
+            for (int k = 0; k < 5; k++) { const T o = uL[k]; uL[k] = isL ? o : uR[k]; uR[k] = isL ? uR[k] : o; }
+#pragma unroll
+            for (int k = 0; k < 4; k++) { const T o = fvL[k]; fvL[k] = isL ? o : fvR[k]; fvR[k] = isL ? fvR[k] : o; }
             const T *nt = a.fnrm + (e * 6 + face_of(s)) * 4;
-            T n[3] = {nt[0], nt[1], nt[2]};
             const T mag = nt[3];
-            T nL[3] = {isL ? n[0] : -n[0], isL ? n[1] : -n[1], isL ? n[2] : -n[2]};
+            const T nL[3] = {isL ? nt[0] : -nt[0], isL ? nt[1] : -nt[1], isL ? nt[2] : -nt[2]};
             T F[5];
-            if constexpr (sizeof(T) == 4) {
-                if (dev) {
+            if (dev) {
+                if constexpr (sizeof(T) == 4) {
                     float sw;
-                    ok &= isL ? common_flux_dev(ph, uo, up, fvo, fvp, nL, F, sw) : common_flux_dev(ph, up, uo, fvp, fvo, nL, F, sw);
+                    ok &= common_flux_dev(ph, uL, uR, fvL, fvR, nL, F, sw);
                     // mass flux in float-float: 1/2 (mL - mR) + (s/2 + tau)(rho_L - rho_R),
                     // mX = own-normal n.(rho v)
                     const ff mo = a.MF[og], mp = a.MF[pg];
                     const ff mL = isL ? mo : mp, mR = isL ? mp : mo;
-                    const float rL = isL ? uo[0] : up[0], rR = isL ? up[0] : uo[0];
-                    const ff Fr = ff_add(ff_mul_f(ff_sub(mL, mR), 0.5f), ff_mul_f(two_sum(rL, -rR), 0.5f * sw + ph.tau));
-                    const ff magf = a.fnrm64[(e * 6 + face_of(s)) * 4 + 3];
-                    s_dff[s] = isL ? ff_mul(magf, Fr) : ff_neg(ff_mul(magf, Fr));
-                } else {
-                    ok &= isL ? common_flux(ph, uo, up, fvo, fvp, nL, F) : common_flux(ph, up, uo, fvp, fvo, nL, F);
+                    const ff Fr = ff_add(ff_mul_f(ff_sub(mL, mR), 0.5f), ff_mul_f(two_sum(uL[0], -uR[0]), 0.5f * sw + ph.tau));
+                    const ff magf = a.fnrm64[(e * 6 + face_of(s)) * 4 + 3], Dr = ff_mul(magf, Fr);
+                    s_dff[s] = isL ? Dr : ff_neg(Dr);
                 }
             } else {
-                ok &= isL ? common_flux(ph, uo, up, fvo, fvp, nL, F) : common_flux(ph, up, uo, fvp, fvo, nL, F);
+                ok &= common_flux(ph, uL, uR, fvL, fvR, nL, F);
             }
             const T sc = isL ? mag : -mag;
 #pragma unroll
-            for (int k = 0; k < 5; k++) s_d[k * NF + s] = sc * F[k];
+            for (int k = 0; k < 5; k++) {
+                if constexpr (FX) dv[0][k] = sc * F[k];
+                else s_d[k * NF + s] = sc * F[k];
+            }
         }
         flag_status(a.status, ok);
-        __syncthreads();
         T *R = a.R + elem_u0(a, e, NU);
         const T idet = g.nidet;
-        if (!dev) {
+        if constexpr (FX) {
+            int E[5];
+            fx_stage5<NF, NTH, 1>(dv, s_dx, s_mx, par, E);
+            for (int it = threadIdx.x; it < 5 * NU; it += NTH) {
+                const int alpha = it / NU, r = it % NU, k = r / NT_, t = r % NT_, Ea = s_mx[par ^ 1][alpha];
+                const fx2 *D = s_dx + alpha * NF;
+                fxacc x{0, 0};
+                fx_mac(x, s_lz[k], D[t]);
+                fx_mac(x, s_lz[NZ + k], D[10 + t]);
+#pragma unroll
+                for (int f = 0; f < 3; f++)
+#pragma unroll
+                    for (int b = 0; b < NZ; b++) fx_mac(x, s_lf[(f * NT_ + t) * NZ + b], D[20 + 16 * f + b + 4 * k]);
+                const double v = (R[it] + fx_double(fx_sum(x), Ea - 1080 + kD, Ea >= 2047)) * idet;
+                if (a.rkstage == 0) R[it] = v;
+                else rk_fold(a, elem_u0(a, e, NU) + it, v);
+            }
+        } else {
+            __syncthreads();
+        }
+        if constexpr (FX) {
+        } else if (!dev) {
             for (int it = threadIdx.x; it < 5 * NU; it += NTH) {
                 const int alpha = it / NU, r = it % NU, k = r / NT_, t = r % NT_;
                 const T *D = s_d + alpha * NF;
