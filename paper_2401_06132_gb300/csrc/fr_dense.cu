@@ -643,6 +643,327 @@ __global__ void __launch_bounds__(NTH, sizeof(T) == 4 ? (TCM == 0 ? 8 : 6) : 0) 
 }
 
 // -------------------------------------------------------------------------------------------------
+// Phase B in FP32 on the CUDA cores: four elements per CTA
+// -------------------------------------------------------------------------------------------------
+// The dense products re-read their operators per element (the projection alone 30 KB) and were bound by
+// the shared-memory and L1 data path (77% busy, FMA pipe 26%). Here an operator entry serves several
+// products: the gradient's all five variables, the interpolation's two quadrature points per thread (a
+// field value feeds both), and the projection is a register-tiled product, NU x 375 times 375 x (elements
+// times variables), a thread holding NU/5 rows by 4 columns of one slice of the quadrature points. The
+// interpolated fields stay in registers through the flux.
+template <typename OPS>
+struct Dense32 {
+    static constexpr int EPB = 4, NTH = 128, NUS = OPS::NUS, NF = OPS::NF, NU = OPS::NU;
+    static constexpr int ZT = NU / 5;                      // rows of a projection tile
+    static constexpr int LOWF = EPB * (20 * NUS + 5 * NF); // state, gradient and common solution; then the partial sums
+    static constexpr int SL(int ncol) { return NTH / (5 * (ncol / 4)); }   // slices of the projection's sum
+    static_assert(NU % 5 == 0 && ZT % 2 == 0 && SL(16) * 16 * NU <= LOWF && SL(20) * 20 * NU <= LOWF && LOWF % 4 == 0, "tiles");
+    static constexpr size_t SMEM = (size_t)(LOWF + 3 * NQ * EPB * 5) * sizeof(float);
+};
+
+template <typename OPS>
+__global__ void __launch_bounds__(128, OPS::NU <= 20 ? 5 : 4) k_dense_B32(HexArgs<float> a, const OPS *__restrict__ op, const FFOf<OPS> *__restrict__ opsff)
+{
+    using D = Dense32<OPS>;
+    constexpr int NU = OPS::NU, NF = OPS::NF, NFACE = OPS::NFACE, NUS = OPS::NUS, EPB = D::EPB, NTH = D::NTH, ZT = D::ZT;
+    extern __shared__ __align__(16) float s_low[];
+    float *s_c = s_low + EPB * 20 * NUS;          // [el][5][NF] common solution
+    float *s_F = s_low + D::LOWF;                 // [d][q][el][variable] transformed flux
+    __shared__ short s_plist[EPB * NF];
+    __shared__ int s_pcnt;
+    __shared__ __align__(8) double s_mfb[EPB * 3 * NU];   // low-Mach form: transformed mass flux
+    __shared__ __align__(8) double s_rlb[EPB * 3 * NU];   // low-Mach form: Dh_d of it, per d
+    const int tid = threadIdx.x;
+    if (tid == 0) s_pcnt = 0;
+    const long long ng = (a.ne + EPB - 1) / EPB;
+    for (long long grp = blockIdx.x; grp < ng; grp += gridDim.x) {
+        const long long e0 = grp * EPB;
+        const int nb = (int)(a.ne - e0 < EPB ? a.ne - e0 : EPB);
+        {
+            bool blk_ok = true;
+            for (int k = 0; k < nb; k++) blk_ok = blk_ok && fr_elem_ok(a, e0 + k, NU, NF);
+            if (!blk_ok) continue;
+        }
+        const bool dev = elem_phys(a, e0).dev != 0;   // a handle's instances all carry the low-Mach form or none
+        const int nv = dev ? 4 : 5, ncol = EPB * nv;  // low-Mach form: the mass has no flux on this path
+        __syncthreads();
+        // 1. state (deviations in the low-Mach form), common solution and, in the low-Mach form, the
+        //    transformed mass flux (in FP64 on the tetrahedron, where the otherwise idle FP64 pipe does its
+        //    products faster; in float-float on the pyramid); the flux points whose side carries LDG weight
+        for (int it = tid; it < nb * (NU + NF); it += NTH) {
+            const int el = it / (NU + NF), r = it % (NU + NF);
+            const Phys<float> ph = elem_phys(a, e0 + el);
+            if (r < NU) {
+                const float *U = a.U + elem_u0(a, e0 + el, NU) + r;
+                float *u = s_low + el * 20 * NUS + r;
+                const float m0 = U[NU], m1 = U[2 * NU], m2 = U[3 * NU];
+                u[0] = U[0] - (dev ? ph.rref : 0.f);
+                u[NUS] = m0; u[2 * NUS] = m1; u[3 * NUS] = m2;
+                u[4 * NUS] = U[4 * NU] - (dev ? ph.eref : 0.f);
+                if (dev) {
+                    const GeoLM &g64 = a.geo64[e0 + el];
+#pragma unroll
+                    for (int d = 0; d < 3; d++) {
+                        if constexpr (NU <= 20) {
+                            s_mfb[(el * 3 + d) * NU + r] = g64.det * (g64.Ji[3 * d] * (double)m0 + g64.Ji[3 * d + 1] * (double)m1 + g64.Ji[3 * d + 2] * (double)m2);
+                        } else {
+                            reinterpret_cast<ff *>(s_mfb)[(el * 3 + d) * NU + r] =
+                                ff_add(ff_add(ff_mul_f(g64.cm[3 * d], m0), ff_mul_f(g64.cm[3 * d + 1], m1)), ff_mul_f(g64.cm[3 * d + 2], m2));
+                        }
+                    }
+                }
+            } else {
+                const int s = r - NU;
+                const long long og = elem_f0(a, e0 + el, NF) + s;
+                const uint32_t pc = a.partner[og];
+                const bool isL = (pc & FR_LFLAG) != 0;
+                const long long pg = fr_partner(a, pc, og);
+                const float *uL = a.UF + (isL ? og : pg), *uR = a.UF + (isL ? pg : og);
+                const float wl = 0.5f - ph.beta, wr = 0.5f + ph.beta;
+                float *c = s_c + el * 5 * NF + s;
+#pragma unroll
+                for (int alpha = 0; alpha < 5; alpha++, uL += a.nfpt, uR += a.nfpt) c[alpha * NF] = wl * *uL + wr * *uR;
+                if ((isL ? wr : wl) == 0.f) {
+                    float *fv = a.FV + og;
+#pragma unroll
+                    for (int k = 0; k < 4; k++, fv += a.nfpt) *fv = 0.f;
+                } else {
+                    s_plist[atomicAdd(&s_pcnt, 1)] = (short)(el * NF + s);
+                }
+            }
+        }
+        if constexpr (NUS > NU) {   // the pads meet zero operator rows
+            for (int it = tid; it < EPB * 20 * (NUS - NU); it += NTH) s_low[(it / (NUS - NU)) * NUS + NU + it % (NUS - NU)] = 0.f;
+        }
+        __syncthreads();
+        const int nplist = s_pcnt;
+        // 2. corrected gradient q~_d = Dh_d u + sum_f n_f,d (L_f c), then q = J^-T q~: one thread per
+        //    (element, point), all variables
+        for (int it = tid; it < nb * NU; it += NTH) {
+            const int el = it / NU, z = it % NU;
+            const float *u = s_low + el * 20 * NUS, *c = s_c + el * 5 * NF;
+            float q[5][3];
+#pragma unroll
+            for (int i = 0; i < 15; i++) q[i / 3][i % 3] = 0.f;
+#pragma unroll 5
+            for (int j = 0; j < NU; j++) {
+                const float d0 = op->Dht[0][j][z], d1 = op->Dht[1][j][z], d2 = op->Dht[2][j][z];
+#pragma unroll
+                for (int alpha = 0; alpha < 5; alpha++) {
+                    const float x = u[alpha * NUS + j];
+                    q[alpha][0] += d0 * x; q[alpha][1] += d1 * x; q[alpha][2] += d2 * x;
+                }
+            }
+#pragma unroll 1
+            for (int f = 0; f < NFACE; f++) {
+                float l[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+                const int s1 = OPS::F0(f + 1);
+#pragma unroll 5
+                for (int s = OPS::F0(f); s < s1; s++) {
+                    const float w = op->Lt[s][z];
+#pragma unroll
+                    for (int alpha = 0; alpha < 5; alpha++) l[alpha] += w * c[alpha * NF + s];
+                }
+                const float n0 = op->nf[f][0], n1 = op->nf[f][1], n2 = op->nf[f][2];
+#pragma unroll
+                for (int alpha = 0; alpha < 5; alpha++) { q[alpha][0] += n0 * l[alpha]; q[alpha][1] += n1 * l[alpha]; q[alpha][2] += n2 * l[alpha]; }
+            }
+            const Geo<float> g = a.geo[e0 + el];
+            float *o = s_low + el * 20 * NUS + 5 * NUS + z;
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++)
+#pragma unroll
+                for (int k = 0; k < 3; k++) o[(alpha * 3 + k) * NUS] = g.Ji[k] * q[alpha][0] + g.Ji[3 + k] * q[alpha][1] + g.Ji[6 + k] * q[alpha][2];
+        }
+        // 3. low-Mach form: (Dh_d m_d)[z], the volume part of R~_rho (rho v lies in the solution space, so
+        //    its L2 projection is itself and the corrected divergence applies at the solution points); from
+        //    the upper threads down
+        if (dev) {
+            for (int it = NTH - 1 - tid; it < nb * 3 * NU; it += NTH) {
+                const int el = it / (3 * NU), d = (it / NU) % 3, z = it % NU;
+                const FFOf<OPS> &o = *opsff;
+                if constexpr (NU <= 20) {
+                    const double *m = s_mfb + (el * 3 + d) * NU;
+                    double v = 0.0;
+#pragma unroll 5
+                    for (int j = 0; j < NU; j++) v += o.Dht64[d][j][z] * m[j];
+                    s_rlb[it] = v;
+                } else {
+                    // compensated dot product (Dot2) of the float-float operator row and m_d
+                    const ff *m = reinterpret_cast<const ff *>(s_mfb) + (el * 3 + d) * NU;
+                    float sh = 0.0f, c = 0.0f;
+#pragma unroll 5
+                    for (int j = 0; j < NU; j++) dot2ff_next(ff{o.hi.Dht[d][j][z], o.lo.Dht[d][j][z]}, m[j], sh, c);
+                    reinterpret_cast<ff *>(s_rlb)[it] = two_sum(sh, c);
+                }
+            }
+        }
+        __syncthreads();
+        if (dev) {
+            for (int it = NTH - 1 - tid; it < nb * NU; it += NTH) {
+                const int el = it / NU, z = it % NU;
+                const long long pbase = elem_u0(a, e0 + el, NU) / FR_NV;
+                if constexpr (NU <= 20) {
+                    const double *r = s_rlb + el * 3 * NU + z;
+                    a.RL[pbase + z] = ff_from_double(r[0] + r[NU] + r[2 * NU]);
+                } else {
+                    const ff *r = reinterpret_cast<const ff *>(s_rlb) + el * 3 * NU + z;
+                    a.RL[pbase + z] = ff_add(ff_add(r[0], r[NU]), r[2 * NU]);
+                }
+            }
+        }
+        // 4. own-normal viscous flux at the listed flux points
+        for (int li = tid; li < nplist; li += NTH) {
+            const int el = s_plist[li] / NF, s = s_plist[li] % NF;
+            const float *x = s_low + el * 20 * NUS;
+            float v[20];
+#pragma unroll
+            for (int f = 0; f < 20; f++) v[f] = 0.f;
+            float mn[4];   // (fetched a step ahead)
+#pragma unroll
+            for (int k = 0; k < 4; k++) mn[k] = op->M0t[k][s];
+#pragma unroll 1
+            for (int z0 = 0; z0 < NUS; z0 += 4) {
+                float m[4];
+#pragma unroll
+                for (int k = 0; k < 4; k++) m[k] = mn[k];
+                if (z0 + 4 < NUS) {
+#pragma unroll
+                    for (int k = 0; k < 4; k++) mn[k] = op->M0t[z0 + 4 + k][s];
+                }
+#pragma unroll
+                for (int f = 0; f < 20; f++) {
+                    const float4 y = *reinterpret_cast<const float4 *>(x + f * NUS + z0);
+                    v[f] += m[0] * y.x; v[f] += m[1] * y.y; v[f] += m[2] * y.z; v[f] += m[3] * y.w;
+                }
+            }
+            float uf[5], qf[5][3];
+#pragma unroll
+            for (int alpha = 0; alpha < 5; alpha++) {
+                uf[alpha] = v[alpha];
+#pragma unroll
+                for (int d = 0; d < 3; d++) qf[alpha][d] = v[5 + alpha * 3 + d];
+            }
+            const Phys<float> ph = elem_phys(a, e0 + el);
+            const float *nt = a.fnrm + ((e0 + el) * 6 + OPS::FACE(s)) * 4;
+            const float n[3] = {nt[0], nt[1], nt[2]};
+            if (dev) { uf[0] += ph.rref; uf[4] += ph.eref; }
+            float fvn[4];
+            viscous_normal_flux(ph, uf, qf, n, fvn);
+            float *fv = a.FV + elem_f0(a, e0 + el, NF) + s;
+#pragma unroll
+            for (int k = 0; k < 4; k++, fv += a.nfpt) *fv = fvn[k];
+        }
+        // 5. interpolation of the 20 fields to two quadrature points, q and q + H, and the flux there
+        constexpr int H = (NQ + 1) / 2;
+        bool ok = true;
+        for (int it = tid; it < nb * H; it += NTH) {
+            const int el = it / H, q = it % H;
+            const bool two = q + H < NQ;
+            const float *x = s_low + el * 20 * NUS;
+            float v[2][20];
+#pragma unroll
+            for (int f = 0; f < 20; f++) v[0][f] = v[1][f] = 0.f;
+            // (operator entries fetched a step ahead)
+            float n0[4], n1[4];
+            const int q1 = two ? q + H : q;
+#pragma unroll
+            for (int k = 0; k < 4; k++) { n0[k] = op->Bt[k][q]; n1[k] = op->Bt[k][q1]; }
+#pragma unroll 1
+            for (int j0 = 0; j0 < NUS; j0 += 4) {
+                float b0[4], b1[4];
+#pragma unroll
+                for (int k = 0; k < 4; k++) { b0[k] = n0[k]; b1[k] = n1[k]; }
+                if (j0 + 4 < NUS) {
+#pragma unroll
+                    for (int k = 0; k < 4; k++) { n0[k] = op->Bt[j0 + 4 + k][q]; n1[k] = op->Bt[j0 + 4 + k][q1]; }
+                }
+#pragma unroll
+                for (int f = 0; f < 20; f++) {
+                    const float4 y = *reinterpret_cast<const float4 *>(x + f * NUS + j0);
+                    v[0][f] += b0[0] * y.x; v[0][f] += b0[1] * y.y; v[0][f] += b0[2] * y.z; v[0][f] += b0[3] * y.w;
+                    v[1][f] += b1[0] * y.x; v[1][f] += b1[1] * y.y; v[1][f] += b1[2] * y.z; v[1][f] += b1[3] * y.w;
+                }
+            }
+            const Phys<float> ph = elem_phys(a, e0 + el);
+            const Geo<float> g = a.geo[e0 + el];
+#pragma unroll
+            for (int p = 0; p < 2; p++) {
+                if (p == 1 && !two) break;
+                float u[5], gq[5][3], f[3][5];
+#pragma unroll
+                for (int alpha = 0; alpha < 5; alpha++) {
+                    u[alpha] = v[p][alpha];
+#pragma unroll
+                    for (int d = 0; d < 3; d++) gq[alpha][d] = v[p][5 + alpha * 3 + d];
+                }
+                if (dev) ok &= total_flux_dev(ph, u, gq, f);
+                else ok &= total_flux(ph, u, gq, f);
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    const float c0 = g.det * g.Ji[3 * d], c1 = g.det * g.Ji[3 * d + 1], c2 = g.det * g.Ji[3 * d + 2];
+                    float *F = s_F + (d * NQ + q + p * H) * ncol + el * nv;
+                    float t[5];
+#pragma unroll
+                    for (int alpha = 0; alpha < 5; alpha++) t[alpha] = c0 * f[0][alpha] + c1 * f[1][alpha] + c2 * f[2][alpha];
+                    if (dev) *reinterpret_cast<float4 *>(F) = make_float4(t[1], t[2], t[3], t[4]);
+                    else {
+#pragma unroll
+                        for (int alpha = 0; alpha < 5; alpha++) F[alpha] = t[alpha];
+                    }
+                }
+            }
+        }
+        flag_status(a.status, ok);
+        __syncthreads();
+        // 6. projection with the corrected divergence, R~[z][column] = sum_k Dv[z][k] F[k][column], k = (d, q):
+        //    thread (slice of k, row group of ZT, column group of 4)
+        {
+            const int ncg = ncol / 4, per = 5 * ncg, nsl = NTH / per;
+            const int sl = tid / per, zg = (tid % per) / ncg, cg = tid % ncg;
+            float acc[ZT][4];
+#pragma unroll
+            for (int i = 0; i < ZT; i++)
+#pragma unroll
+                for (int j = 0; j < 4; j++) acc[i][j] = 0.f;
+            if (sl < nsl) {
+#pragma unroll 1
+                for (int d = 0; d < 3; d++) {
+                    const int qb = sl * NQ / nsl, qe = (sl + 1) * NQ / nsl;
+                    const float *w = &op->Dvt[d][qb][zg * ZT];
+                    const float *F = s_F + (d * NQ + qb) * ncol + 4 * cg;
+#pragma unroll 4
+                    for (int q = qb; q < qe; q++, w += NU, F += ncol) {
+                        float m[ZT];
+#pragma unroll
+                        for (int i = 0; i < ZT; i += 2) {
+                            const float2 y = *reinterpret_cast<const float2 *>(w + i);
+                            m[i] = y.x; m[i + 1] = y.y;
+                        }
+                        const float4 x = *reinterpret_cast<const float4 *>(F);
+#pragma unroll
+                        for (int i = 0; i < ZT; i++) { acc[i][0] += m[i] * x.x; acc[i][1] += m[i] * x.y; acc[i][2] += m[i] * x.z; acc[i][3] += m[i] * x.w; }
+                    }
+                }
+                // partial sums [slice][row][column] over the consumed state, gradient and common solution
+                float *o = s_low + (sl * NU + zg * ZT) * ncol + 4 * cg;
+#pragma unroll
+                for (int i = 0; i < ZT; i++) *reinterpret_cast<float4 *>(o + i * ncol) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+            }
+            if (tid == 0) s_pcnt = 0;
+            __syncthreads();
+            for (int it = tid; it < nb * nv * NU; it += NTH) {
+                const int el = it / (nv * NU), r = it % (nv * NU), al = r / NU, z = r % NU;
+                const float *p = s_low + z * ncol + el * nv + al;
+                float v = 0.f;
+                for (int k = 0; k < nsl; k++) v += p[k * NU * ncol];
+                a.R[elem_u0(a, e0 + el, NU) + (al + 5 - nv) * NU + z] = v;
+            }
+        }
+    }
+}
+
+// -------------------------------------------------------------------------------------------------
 // Phase B in FP64: the dense operators in block fixed point (fr_fx.cuh), one element per CTA
 // -------------------------------------------------------------------------------------------------
 // A dense element's operators are 0.85 (tetrahedron) to 0.9 (pyramid) of its FP64 arithmetic, which
@@ -1118,12 +1439,13 @@ int dense_phase(int phase, const HexArgs<T> &a, const OPS *ops, const FFOf<OPS> 
         if constexpr (sizeof(T) == 8) {
             k_dense_B_fx<OPS, NTH><<<grid_elems(a.ne, 4), NTH, 0, s>>>(a, ops);
         } else if (!tcdone) {
+            using D = Dense32<OPS>;
             static bool attr = false;
             if (!attr) {
-                cudaFuncSetAttribute(k_dense_B<T, NTH, OPS, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)base);
+                cudaFuncSetAttribute(k_dense_B32<OPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D::SMEM);
                 attr = true;
             }
-            k_dense_B<T, NTH, OPS, 0><<<grid_elems(a.ne, 8), NTH, base, s>>>(a, ops, opsff);
+            k_dense_B32<OPS><<<grid_groups(a.ne, D::EPB, 5), D::NTH, D::SMEM, s>>>(a, ops, opsff);
         }
     } else {
         k_dense_C<T, OPS, 4><<<grid_groups(a.ne, 4, 8), NF * 4, 0, s>>>(a, ops, opsff);
