@@ -80,33 +80,32 @@ __device__ __forceinline__ ff ffat(const FF &o, const float &hi)
 // state, and the own-normal mass flux n.(rho v) at every flux point in float-float: first
 // m_f = n_f . (rho v) at the solution points per face (the face normal is constant on an affine
 // element), then the same compensated dot product with m_f.
-// FP32 pyramids (224 threads per CTA): registers capped for five CTAs per SM, up from two at the
+// Pyramids (224 threads per CTA): registers capped for five CTAs per SM, up from two at the
 // compiler's 112 (a few spilled values; the tetrahedral form is faster uncapped). Otherwise (0) the
 // compiler's own register count.
-template <typename T, typename OPS, int EPB>
-__global__ void __launch_bounds__(OPS::NF * EPB, (sizeof(T) == 4 && OPS::NF * EPB > 192) ? 1280 / (OPS::NF * EPB) : 0)
-k_dense_disu(HexArgs<T> a, const OPS *__restrict__ op, const FFOf<OPS> *__restrict__ opsff)
+template <typename OPS, int EPB>
+__global__ void __launch_bounds__(OPS::NF * EPB, OPS::NF * EPB > 192 ? 1280 / (OPS::NF * EPB) : 0)
+k_dense_disu(HexArgs<float> a, const OPS *__restrict__ op, const FFOf<OPS> *__restrict__ opsff)
 {
     constexpr int NU = OPS::NU, NF = OPS::NF, NUS = OPS::NUS, NFACE = OPS::NFACE, NTH = NF * EPB;
-    constexpr bool F32 = sizeof(T) == 4;
+    using T = float;
     constexpr int VN = V16<T>::n;
     __shared__ __align__(16) T s_u[EPB][FR_NV * NUS];
-    __shared__ __align__(16) ff s_m[F32 ? EPB : 1][F32 ? NFACE * NUS : 1];
+    __shared__ __align__(16) ff s_m[EPB][NFACE * NUS];
     const int el = threadIdx.x / NF, s = threadIdx.x % NF;
     T col[NUS];
 #pragma unroll
     for (int z = 0; z < NUS; z++) col[z] = op->M0t[z][s];   // pad rows are zero
-    float col_lo[F32 ? NUS : 1];                              // lo parts of the FP32 column
-    if constexpr (F32) {
+    float col_lo[NUS];                              // lo parts of the FP32 column
 #pragma unroll
-        for (int z = 0; z < NUS; z++) col_lo[z] = opsff->lo.M0t[z][s];
-    }
+    for (int z = 0; z < NUS; z++) col_lo[z] = opsff->lo.M0t[z][s];
     if constexpr (NUS > NU) {
         for (int i = threadIdx.x; i < EPB * FR_NV * (NUS - NU); i += NTH) {
             const int l = i / (FR_NV * (NUS - NU)), r = i % (FR_NV * (NUS - NU));
             s_u[l][(r / (NUS - NU)) * NUS + NU + r % (NUS - NU)] = T(0);
         }
     }
+    fr_grid_wait();
     const long long ng = (a.ne + EPB - 1) / EPB;
     for (long long g = blockIdx.x; g < ng; g += gridDim.x) {
         const long long e0 = g * EPB;
@@ -120,88 +119,66 @@ k_dense_disu(HexArgs<T> a, const OPS *__restrict__ op, const FFOf<OPS> *__restri
             const int l = i / (FR_NV * NU), r = i % (FR_NV * NU), alpha = r / NU;
             const long long e = e0 + l;
             T v = a.U[elem_u0(a, e, NU) + r];
-            if constexpr (F32) {
-                const Phys<T> ph = elem_phys(a, e);
-                if (ph.dev) v -= alpha == 0 ? ph.rref : (alpha == 4 ? ph.eref : T(0));
-            }
+            const Phys<T> ph = elem_phys(a, e);
+            if (ph.dev) v -= alpha == 0 ? ph.rref : (alpha == 4 ? ph.eref : T(0));
             s_u[l][alpha * NUS + r % NU] = v;
         }
-        if constexpr (F32) {
-            __syncthreads();
-            for (int i = threadIdx.x; i < nel * NFACE * NU; i += NTH) {
-                const int l = i / (NFACE * NU), r = i % (NFACE * NU), f = r / NU, z = r % NU;
-                const long long e = e0 + l;
-                if (!elem_phys(a, e).dev) continue;
-                const ff *nt = a.fnrm64 + (e * 6 + f) * 4;
-                const float *u = s_u[l];
-                ff m = ff_mul_f(nt[0], u[NUS + z]);
-                m = ff_add(m, ff_mul_f(nt[1], u[2 * NUS + z]));
-                s_m[l][f * NUS + z] = ff_add(m, ff_mul_f(nt[2], u[3 * NUS + z]));
-            }
+        __syncthreads();
+        for (int i = threadIdx.x; i < nel * NFACE * NU; i += NTH) {
+            const int l = i / (NFACE * NU), r = i % (NFACE * NU), f = r / NU, z = r % NU;
+            const long long e = e0 + l;
+            if (!elem_phys(a, e).dev) continue;
+            const ff *nt = a.fnrm64 + (e * 6 + f) * 4;
+            const float *u = s_u[l];
+            ff m = ff_mul_f(nt[0], u[NUS + z]);
+            m = ff_add(m, ff_mul_f(nt[1], u[2 * NUS + z]));
+            s_m[l][f * NUS + z] = ff_add(m, ff_mul_f(nt[2], u[3 * NUS + z]));
         }
         __syncthreads();
         if (el < nel) {
             const long long e = e0 + el;
             const long long f0 = elem_f0(a, e, NF);
             const T *u = s_u[el];
-            if constexpr (F32) {
-                // sh + c = sum_z (col + col_lo)[z] x[z]: exact products (one FMA each), TwoSum
-                // accumulation of the high parts, the errors summed in c
-                float sh[FR_NV], c[FR_NV];
+            // sh + c = sum_z (col + col_lo)[z] x[z]: exact products (one FMA each), TwoSum
+            // accumulation of the high parts, the errors summed in c
+            float sh[FR_NV], c[FR_NV];
 #pragma unroll
-                for (int alpha = 0; alpha < FR_NV; alpha++) { sh[alpha] = 0.0f; c[alpha] = 0.0f; }
+            for (int alpha = 0; alpha < FR_NV; alpha++) { sh[alpha] = 0.0f; c[alpha] = 0.0f; }
 #pragma unroll
-                for (int z = 0; z < NUS; z += VN) {
+            for (int z = 0; z < NUS; z += VN) {
 #pragma unroll
-                    for (int alpha = 0; alpha < FR_NV; alpha++) {
-                        const V16<T> x = ld16(u + alpha * NUS + z);
+                for (int alpha = 0; alpha < FR_NV; alpha++) {
+                    const V16<T> x = ld16(u + alpha * NUS + z);
 #pragma unroll
-                        for (int j = 0; j < VN; j++) {
-                            const float pr = col[z + j] * x.v[j];
-                            const float er = __fmaf_rn(col_lo[z + j], x.v[j], __fmaf_rn(col[z + j], x.v[j], -pr));
-                            const ff t = two_sum(sh[alpha], pr);
-                            sh[alpha] = t.hi;
-                            c[alpha] += t.lo + er;
-                        }
+                    for (int j = 0; j < VN; j++) {
+                        const float pr = col[z + j] * x.v[j];
+                        const float er = __fmaf_rn(col_lo[z + j], x.v[j], __fmaf_rn(col[z + j], x.v[j], -pr));
+                        const ff t = two_sum(sh[alpha], pr);
+                        sh[alpha] = t.hi;
+                        c[alpha] += t.lo + er;
                     }
                 }
-#pragma unroll
-                for (int alpha = 0; alpha < FR_NV; alpha++) a.UF[alpha * a.nfpt + f0 + s] = sh[alpha] + c[alpha];
-            } else {
-                T v[FR_NV];
-#pragma unroll
-                for (int alpha = 0; alpha < FR_NV; alpha++) v[alpha] = T(0);
-#pragma unroll
-                for (int z = 0; z < NUS; z += VN) {
-#pragma unroll
-                    for (int alpha = 0; alpha < FR_NV; alpha++) {
-                        const V16<T> x = ld16(u + alpha * NUS + z);
-#pragma unroll
-                        for (int j = 0; j < VN; j++) v[alpha] += col[z + j] * x.v[j];
-                    }
-                }
-#pragma unroll
-                for (int alpha = 0; alpha < FR_NV; alpha++) a.UF[alpha * a.nfpt + f0 + s] = v[alpha];
             }
-            if constexpr (F32) {
-                if (elem_phys(a, e).dev) {
-                    const ff *m = s_m[el] + OPS::FACE(s) * NUS;
-                    float sh = 0.0f, c = 0.0f;
 #pragma unroll
-                    for (int z = 0; z < NU; z++) {
-                        const ff mz = m[z];
-                        const float pr = col[z] * mz.hi;
-                        const float er = __fmaf_rn(opsff->lo.M0t[z][s], mz.hi, __fmaf_rn(col[z], mz.lo, __fmaf_rn(col[z], mz.hi, -pr)));
-                        const ff t = two_sum(sh, pr);
-                        sh = t.hi;
-                        c += t.lo + er;
-                    }
-                    a.MF[f0 + s] = two_sum(sh, c);
+            for (int alpha = 0; alpha < FR_NV; alpha++) a.UF[alpha * a.nfpt + f0 + s] = sh[alpha] + c[alpha];
+            if (elem_phys(a, e).dev) {
+                const ff *m = s_m[el] + OPS::FACE(s) * NUS;
+                float sh = 0.0f, c = 0.0f;
+#pragma unroll
+                for (int z = 0; z < NU; z++) {
+                    const ff mz = m[z];
+                    const float pr = col[z] * mz.hi;
+                    const float er = __fmaf_rn(opsff->lo.M0t[z][s], mz.hi, __fmaf_rn(col[z], mz.lo, __fmaf_rn(col[z], mz.hi, -pr)));
+                    const ff t = two_sum(sh, pr);
+                    sh = t.hi;
+                    c += t.lo + er;
                 }
+                a.MF[f0 + s] = two_sum(sh, c);
             }
         }
         __syncthreads();
     }
+    fr_grid_done();
 }
 
 // The same in FP64, with the face values in block fixed point (fr_fx.cuh): on the FP64 pipe the 5 NU
@@ -224,6 +201,7 @@ __global__ void __launch_bounds__(OPS::NF * EPB) k_dense_disu_fx(HexArgs<double>
             s_u[l][(r / (NUS - NU)) * NUS + NU + r % (NUS - NU)] = fx2{0, 0};
         }
     }
+    fr_grid_wait();
     const long long ng = (a.ne + EPB - 1) / EPB;
     for (long long g = blockIdx.x; g < ng; g += gridDim.x) {
         const long long e0 = g * EPB;
@@ -254,24 +232,26 @@ __global__ void __launch_bounds__(OPS::NF * EPB) k_dense_disu_fx(HexArgs<double>
         }
         __syncthreads();
     }
+    fr_grid_done();
 }
 
 // -------------------------------------------------------------------------------------------------
 // Phase B: volume group, one element per CTA of NTH threads (persistent over elements)
 // -------------------------------------------------------------------------------------------------
-template <typename T, int NTH, typename OPS, int TCM>
-__global__ void __launch_bounds__(NTH, sizeof(T) == 4 ? (TCM == 0 ? 8 : 6) : 0) k_dense_B(HexArgs<T> a, const OPS *__restrict__ op, const FFOf<OPS> *__restrict__ opsff)
+template <int NTH, typename OPS, int TCM>
+__global__ void __launch_bounds__(NTH, TCM == 0 ? 8 : 6) k_dense_B(HexArgs<float> a, const OPS *__restrict__ op, const FFOf<OPS> *__restrict__ opsff)
 {
+    using T = float;
     constexpr int NU = OPS::NU, NF = OPS::NF, NFACE = OPS::NFACE, NUS = OPS::NUS;
     static_assert(NTH >= NQ, "one thread per quadrature point");
-    static_assert(TCM == 0 || (NTH == 128 && sizeof(T) == 4), "tensor-core form: FP32, one warpgroup per element");
+    static_assert(TCM == 0 || NTH == 128, "tensor-core form: one warpgroup per element");
     using TC = DenseTC<OPS, TCM == 0 ? 1 : TCM>;
     using SF = tc::SplitForm<TCM == 0 ? 1 : TCM>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ short s_plist[NF];
     __shared__ int s_pcnt;
-    __shared__ __align__(8) double s_mfb[sizeof(T) == 4 ? 3 * NU : 1];   // low-Mach form: transformed mass flux
-    __shared__ __align__(8) double s_rlb[sizeof(T) == 4 ? 3 * NU : 1];   // low-Mach form: Dh_d of it, per d
+    __shared__ __align__(8) double s_mfb[3 * NU];   // low-Mach form: transformed mass flux
+    __shared__ __align__(8) double s_rlb[3 * NU];   // low-Mach form: Dh_d of it, per d
     constexpr int VW = V16<T>::n;
     constexpr int NCH = NTH / NU;                 // quadrature-point chunks of the projection
     unsigned char *arr = smem_raw;
@@ -317,41 +297,39 @@ __global__ void __launch_bounds__(NTH, sizeof(T) == 4 ? (TCM == 0 ? 8 : 6) : 0) 
     for (int it = threadIdx.x; it < 20 * (NQP - NQ); it += NTH) s_w[(it / (NQP - NQ)) * NQP + NQ + it % (NQP - NQ)] = T(0);
     if constexpr (NUS > NU)
         for (int it = threadIdx.x; it < 20 * (NUS - NU); it += NTH) s_u[(it / (NUS - NU)) * NUS + NU + it % (NUS - NU)] = T(0);
+    fr_grid_wait();
     for (long long e = blockIdx.x; e < a.ne; e += gridDim.x) {
         if (!fr_elem_ok(a, e, NU, NF)) continue;
         const Geo<T> g = a.geo[e];
         const Phys<T> ph = elem_phys(a, e);
         const T *U = a.U + elem_u0(a, e, NU);
         const long long gf0 = elem_f0(a, e, NF);
-        bool dev = false;
-        if constexpr (sizeof(T) == 4) dev = ph.dev != 0;
+        const bool dev = ph.dev != 0;
         for (int it = threadIdx.x; it < 5 * NU; it += NTH) {
             T v = U[it];
             if (dev) v -= it < NU ? ph.rref : (it >= 4 * NU ? ph.eref : T(0));
             s_u[(it / NU) * NUS + it % NU] = v;
         }
-        if constexpr (sizeof(T) == 4) {
-            // low-Mach form: the volume part of R~_rho, sum_d Dh_d (det J J^-1 rho v)_d, in about 48
-            // bits or better (rho v lies in the solution space, so its L2 projection is itself and
-            // the corrected divergence Dh applies at the solution points). First the transformed
-            // mass flux (read from the state in global memory, so that it is ready at the first
-            // barrier); the 3 NU products Dh_d m_d then ride along with the gradient items below.
-            // The dense product costs 3 NU^2 multiply-adds per element: on the tetrahedron (NU = 20)
-            // the FP64 pipe, idle in this kernel, does them faster than float-float arithmetic on
-            // the busy FP32 pipe; on the pyramid (NU = 30) the FP64 pipe would become the limit, so
-            // it stays in float-float.
-            if (dev) {
-                const GeoLM &g64 = a.geo64[e];
-                for (int z = threadIdx.x; z < NU; z += NTH) {
-                    const float m0 = U[NU + z], m1 = U[2 * NU + z], m2 = U[3 * NU + z];
+        // low-Mach form: the volume part of R~_rho, sum_d Dh_d (det J J^-1 rho v)_d, in about 48
+        // bits or better (rho v lies in the solution space, so its L2 projection is itself and
+        // the corrected divergence Dh applies at the solution points). First the transformed
+        // mass flux (read from the state in global memory, so that it is ready at the first
+        // barrier); the 3 NU products Dh_d m_d then ride along with the gradient items below.
+        // The dense product costs 3 NU^2 multiply-adds per element: on the tetrahedron (NU = 20)
+        // the FP64 pipe, idle in this kernel, does them faster than float-float arithmetic on
+        // the busy FP32 pipe; on the pyramid (NU = 30) the FP64 pipe would become the limit, so
+        // it stays in float-float.
+        if (dev) {
+            const GeoLM &g64 = a.geo64[e];
+            for (int z = threadIdx.x; z < NU; z += NTH) {
+                const float m0 = U[NU + z], m1 = U[2 * NU + z], m2 = U[3 * NU + z];
 #pragma unroll
-                    for (int d = 0; d < 3; d++) {
-                        if constexpr (NU <= 20) {
-                            s_mfb[d * NU + z] = g64.det * (g64.Ji[3 * d] * (double)m0 + g64.Ji[3 * d + 1] * (double)m1 + g64.Ji[3 * d + 2] * (double)m2);
-                        } else {
-                            ff *s_mf = reinterpret_cast<ff *>(s_mfb);
-                            s_mf[d * NU + z] = ff_add(ff_add(ff_mul_f(g64.cm[3 * d], m0), ff_mul_f(g64.cm[3 * d + 1], m1)), ff_mul_f(g64.cm[3 * d + 2], m2));
-                        }
+                for (int d = 0; d < 3; d++) {
+                    if constexpr (NU <= 20) {
+                        s_mfb[d * NU + z] = g64.det * (g64.Ji[3 * d] * (double)m0 + g64.Ji[3 * d + 1] * (double)m1 + g64.Ji[3 * d + 2] * (double)m2);
+                    } else {
+                        ff *s_mf = reinterpret_cast<ff *>(s_mfb);
+                        s_mf[d * NU + z] = ff_add(ff_add(ff_mul_f(g64.cm[3 * d], m0), ff_mul_f(g64.cm[3 * d + 1], m1)), ff_mul_f(g64.cm[3 * d + 2], m2));
                     }
                 }
             }
@@ -370,33 +348,31 @@ __global__ void __launch_bounds__(NTH, sizeof(T) == 4 ? (TCM == 0 ? 8 : 6) : 0) 
         // corrected gradient q~_d = Dh_d u + sum_f n_f,d (L_f c), then q = J^-T q~
         const int ngrad = 5 * NU + (dev ? 3 * NU : 0);
         for (int it = threadIdx.x; it < ngrad; it += NTH) {
-            if constexpr (sizeof(T) == 4) {
-                if (it >= 5 * NU) {   // low-Mach mass channel: (Dh_d m_d)[z]
-                    const int d = (it - 5 * NU) / NU, z = (it - 5 * NU) % NU;
-                    const FFOf<OPS> &o = *opsff;
-                    if constexpr (NU <= 20) {
-                        double v = 0.0;
+            if (it >= 5 * NU) {   // low-Mach mass channel: (Dh_d m_d)[z]
+                const int d = (it - 5 * NU) / NU, z = (it - 5 * NU) % NU;
+                const FFOf<OPS> &o = *opsff;
+                if constexpr (NU <= 20) {
+                    double v = 0.0;
 #pragma unroll 5
-                        for (int j = 0; j < NU; j++) v += o.Dht64[d][j][z] * s_mfb[d * NU + j];
-                        s_rlb[d * NU + z] = v;
-                    } else {
-                        // compensated dot product (Dot2) of the float-float operator row and m_d
-                        const ff *m = reinterpret_cast<const ff *>(s_mfb) + d * NU;
-                        float sh = 0.0f, c = 0.0f;
+                    for (int j = 0; j < NU; j++) v += o.Dht64[d][j][z] * s_mfb[d * NU + j];
+                    s_rlb[d * NU + z] = v;
+                } else {
+                    // compensated dot product (Dot2) of the float-float operator row and m_d
+                    const ff *m = reinterpret_cast<const ff *>(s_mfb) + d * NU;
+                    float sh = 0.0f, c = 0.0f;
 #pragma unroll 5
-                        for (int j = 0; j < NU; j++) {
-                            const float h = o.hi.Dht[d][j][z], l = o.lo.Dht[d][j][z];
-                            const ff mj = m[j];
-                            const float pr = h * mj.hi;
-                            const float er = __fmaf_rn(l, mj.hi, __fmaf_rn(h, mj.lo, __fmaf_rn(h, mj.hi, -pr)));
-                            const ff t = two_sum(sh, pr);
-                            sh = t.hi;
-                            c += t.lo + er;
-                        }
-                        reinterpret_cast<ff *>(s_rlb)[d * NU + z] = two_sum(sh, c);
+                    for (int j = 0; j < NU; j++) {
+                        const float h = o.hi.Dht[d][j][z], l = o.lo.Dht[d][j][z];
+                        const ff mj = m[j];
+                        const float pr = h * mj.hi;
+                        const float er = __fmaf_rn(l, mj.hi, __fmaf_rn(h, mj.lo, __fmaf_rn(h, mj.hi, -pr)));
+                        const ff t = two_sum(sh, pr);
+                        sh = t.hi;
+                        c += t.lo + er;
                     }
-                    continue;
+                    reinterpret_cast<ff *>(s_rlb)[d * NU + z] = two_sum(sh, c);
                 }
+                continue;
             }
             const int alpha = it / NU, z = it % NU;
             const T *u = s_u + alpha * NUS;
@@ -422,16 +398,14 @@ __global__ void __launch_bounds__(NTH, sizeof(T) == 4 ? (TCM == 0 ? 8 : 6) : 0) 
             for (int k = 0; k < 3; k++) s_q[(alpha * 3 + k) * NUS + z] = g.Ji[k] * q0 + g.Ji[3 + k] * q1 + g.Ji[6 + k] * q2;
         }
         __syncthreads();
-        if constexpr (sizeof(T) == 4) {
-            if (dev) {
-                const long long pbase = elem_u0(a, e, NU) / FR_NV;
-                for (int z = threadIdx.x; z < NU; z += NTH) {
-                    if constexpr (NU <= 20) {
-                        a.RL[pbase + z] = ff_from_double(s_rlb[z] + s_rlb[NU + z] + s_rlb[2 * NU + z]);
-                    } else {
-                        const ff *r = reinterpret_cast<const ff *>(s_rlb);
-                        a.RL[pbase + z] = ff_add(ff_add(r[z], r[NU + z]), r[2 * NU + z]);
-                    }
+        if (dev) {
+            const long long pbase = elem_u0(a, e, NU) / FR_NV;
+            for (int z = threadIdx.x; z < NU; z += NTH) {
+                if constexpr (NU <= 20) {
+                    a.RL[pbase + z] = ff_from_double(s_rlb[z] + s_rlb[NU + z] + s_rlb[2 * NU + z]);
+                } else {
+                    const ff *r = reinterpret_cast<const ff *>(s_rlb);
+                    a.RL[pbase + z] = ff_add(ff_add(r[z], r[NU + z]), r[2 * NU + z]);
                 }
             }
         }
@@ -581,12 +555,8 @@ __global__ void __launch_bounds__(NTH, sizeof(T) == 4 ? (TCM == 0 ? 8 : 6) : 0) 
 #pragma unroll
                 for (int d = 0; d < 3; d++) gq[alpha][d] = s_w[(5 + alpha * 3 + d) * NQP + q];
             }
-            if constexpr (sizeof(T) == 4) {
-                if (dev) ok &= total_flux_dev(ph, u, gq, f);
-                else ok &= total_flux(ph, u, gq, f);
-            } else {
-                ok &= total_flux(ph, u, gq, f);
-            }
+            if (dev) ok &= total_flux_dev(ph, u, gq, f);
+            else ok &= total_flux(ph, u, gq, f);
 #pragma unroll
             for (int alpha = 0; alpha < 5; alpha++)
 #pragma unroll
@@ -635,6 +605,7 @@ __global__ void __launch_bounds__(NTH, sizeof(T) == 4 ? (TCM == 0 ? 8 : 6) : 0) 
         }
         __syncthreads();
     }
+    fr_grid_done();
     if constexpr (TCM != 0) {
         // a chain that did not complete within the bound is reported; the tensor memory is released
         if (tc_fail && threadIdx.x == 0) atomicOr(a.status, 2);
@@ -675,6 +646,7 @@ __global__ void __launch_bounds__(128, OPS::NU <= 20 ? 5 : 4) k_dense_B32(HexArg
     __shared__ __align__(8) double s_rlb[EPB * 3 * NU];   // low-Mach form: Dh_d of it, per d
     const int tid = threadIdx.x;
     if (tid == 0) s_pcnt = 0;
+    fr_grid_wait();
     const long long ng = (a.ne + EPB - 1) / EPB;
     for (long long grp = blockIdx.x; grp < ng; grp += gridDim.x) {
         const long long e0 = grp * EPB;
@@ -961,6 +933,7 @@ __global__ void __launch_bounds__(128, OPS::NU <= 20 ? 5 : 4) k_dense_B32(HexArg
             }
         }
     }
+    fr_grid_done();
 }
 
 // -------------------------------------------------------------------------------------------------
@@ -995,6 +968,7 @@ __global__ void __launch_bounds__(NTH, 4) k_dense_B_fx(HexArgs<double> a, const 
     if (tid < 10) s_mx[tid] = 0;
     if (tid == 0) s_pcnt = 0;
     __syncthreads();
+    fr_grid_wait();
     for (long long e = blockIdx.x; e < a.ne; e += gridDim.x) {
         if (!fr_elem_ok(a, e, NU, NF)) continue;
         const Geo<double> g = a.geo[e];
@@ -1208,6 +1182,7 @@ __global__ void __launch_bounds__(NTH, 4) k_dense_B_fx(HexArgs<double> a, const 
         if (tid == 0) s_pcnt = 0;
         __syncthreads();
     }
+    fr_grid_done();
 }
 
 // -------------------------------------------------------------------------------------------------
@@ -1230,6 +1205,7 @@ __global__ void __launch_bounds__(OPS::NF * EPB, sizeof(T) == 4 ? 1280 / (OPS::N
     __shared__ ff s_rr[F32 ? EPB : 1][F32 ? NU : 1];     // low-Mach form: R_rho (float-float)
     __shared__ ff s_idet[F32 ? EPB : 1];                 // low-Mach form: -1 / det J (float-float)
     const int el = threadIdx.x / NF, s = threadIdx.x % NF;
+    fr_grid_wait();
     const long long ng = (a.ne + EPB - 1) / EPB;
     for (long long g = blockIdx.x; g < ng; g += gridDim.x) {
         const long long e0 = g * EPB;
@@ -1324,65 +1300,64 @@ __global__ void __launch_bounds__(OPS::NF * EPB, sizeof(T) == 4 ? 1280 / (OPS::N
                 if (a.rkstage == 0) a.R[ui] = v;
                 else rk_fold(a, ui, v);
             }
-            __syncthreads();
-            continue;
-        }
-        // lift and scale: R += L D, R *= -1/det; the mass rows of low-Mach elements in float-float,
-        // then the energy rows, which add H0 R_rho
-        for (int pass = 0; pass < 2; pass++) {
-            const int nrow = pass == 0 ? 4 : 1;
-            for (int i = threadIdx.x; i < nel * nrow * NU; i += NTH) {
-                const int l = i / (nrow * NU), alpha = pass == 0 ? (i / NU) % 4 : 4, z = i % NU;
-                const long long e = e0 + l;
-                const long long ui = elem_u0(a, e, NU) + alpha * NU + z;
-                bool dev = false;
-                if constexpr (F32) dev = elem_phys(a, e).dev != 0;
-                float outf = 0.0f;
-                T out;
-                if (F32 && dev && alpha == 0) {
-                    if constexpr (F32) {
-                        const ff r0 = a.RL[elem_u0(a, e, NU) / FR_NV + z];
-                        float sh = r0.hi, c = r0.lo;
-                        const ff *d = s_dff[l];
+        } else {
+            // lift and scale: R += L D, R *= -1/det; the mass rows of low-Mach elements in float-float,
+            // then the energy rows, which add H0 R_rho
+            for (int pass = 0; pass < 2; pass++) {
+                const int nrow = pass == 0 ? 4 : 1;
+                for (int i = threadIdx.x; i < nel * nrow * NU; i += NTH) {
+                    const int l = i / (nrow * NU), alpha = pass == 0 ? (i / NU) % 4 : 4, z = i % NU;
+                    const long long e = e0 + l;
+                    const long long ui = elem_u0(a, e, NU) + alpha * NU + z;
+                    const bool dev = elem_phys(a, e).dev != 0;
+                    float outf = 0.0f;
+                    T out;
+                    if (dev && alpha == 0) {
+                        if constexpr (F32) {
+                            const ff r0 = a.RL[elem_u0(a, e, NU) / FR_NV + z];
+                            float sh = r0.hi, c = r0.lo;
+                            const ff *d = s_dff[l];
 #pragma unroll 8
-                        for (int s2 = 0; s2 < NF; s2++) {
-                            const float lh = op->Lt[s2][z], ll = opsff->lo.Lt[s2][z];
-                            const ff ds = d[s2];
-                            const float pr = lh * ds.hi;
-                            const float er = __fmaf_rn(ll, ds.hi, __fmaf_rn(lh, ds.lo, __fmaf_rn(lh, ds.hi, -pr)));
-                            const ff t = two_sum(sh, pr);
-                            sh = t.hi;
-                            c += t.lo + er;
+                            for (int s2 = 0; s2 < NF; s2++) {
+                                const float lh = op->Lt[s2][z], ll = opsff->lo.Lt[s2][z];
+                                const ff ds = d[s2];
+                                const float pr = lh * ds.hi;
+                                const float er = __fmaf_rn(ll, ds.hi, __fmaf_rn(lh, ds.lo, __fmaf_rn(lh, ds.hi, -pr)));
+                                const ff t = two_sum(sh, pr);
+                                sh = t.hi;
+                                c += t.lo + er;
+                            }
+                            const ff Rrho = ff_mul(two_sum(sh, c), s_idet[l]);
+                            s_rr[l][z] = Rrho;
+                            outf = Rrho.hi + Rrho.lo;
                         }
-                        const ff Rrho = ff_mul(two_sum(sh, c), s_idet[l]);
-                        s_rr[l][z] = Rrho;
-                        outf = Rrho.hi + Rrho.lo;
-                    }
-                    out = (T)outf;
-                } else {
-                    const T *D = s_d[l] + alpha * NF;
-                    T v = a.R[ui];
+                        out = (T)outf;
+                    } else {
+                        const T *D = s_d[l] + alpha * NF;
+                        T v = a.R[ui];
 #pragma unroll 2
-                    for (int s2 = 0; s2 < NF; s2 += VN) {
-                        const V16<T> x = ld16(D + s2);
+                        for (int s2 = 0; s2 < NF; s2 += VN) {
+                            const V16<T> x = ld16(D + s2);
 #pragma unroll
-                        for (int j = 0; j < VN; j++) v += op->Lt[s2 + j][z] * x.v[j];
-                    }
-                    out = v * a.geo[e].nidet;
-                    if constexpr (F32) {
-                        if (dev && alpha == 4) {
-                            const ff e4 = ff_fma(elem_phys(a, e).H0ff, s_rr[l][z], ff_of(out));
-                            out = e4.hi + e4.lo;
+                            for (int j = 0; j < VN; j++) v += op->Lt[s2 + j][z] * x.v[j];
+                        }
+                        out = v * a.geo[e].nidet;
+                        if constexpr (F32) {
+                            if (dev && alpha == 4) {
+                                const ff e4 = ff_fma(elem_phys(a, e).H0ff, s_rr[l][z], ff_of(out));
+                                out = e4.hi + e4.lo;
+                            }
                         }
                     }
+                    if (a.rkstage == 0) a.R[ui] = out;
+                    else rk_fold(a, ui, out);
                 }
-                if (a.rkstage == 0) a.R[ui] = out;
-                else rk_fold(a, ui, out);
+                if (pass == 0) __syncthreads();
             }
-            if (F32 && pass == 0) __syncthreads();
         }
         __syncthreads();
     }
+    fr_grid_done();
 }
 
 // persistent grid over groups of epb elements: at most per_sm CTAs per SM, 8 waves
@@ -1406,8 +1381,8 @@ int dense_phase(int phase, const HexArgs<T> &a, const OPS *ops, const FFOf<OPS> 
     constexpr int NU = OPS::NU, NF = OPS::NF, NUS = OPS::NUS;
     if (a.ne == 0) return 0;
     if (phase == 0) {
-        if constexpr (sizeof(T) == 8) k_dense_disu_fx<OPS, 4><<<grid_groups(a.ne, 4, 8), NF * 4, 0, s>>>(a, ops);
-        else k_dense_disu<T, OPS, 4><<<grid_groups(a.ne, 4, 8), NF * 4, 0, s>>>(a, ops, opsff);
+        if constexpr (sizeof(T) == 8) fr_launch(k_dense_disu_fx<OPS, 4>, grid_groups(a.ne, 4, 8), NF * 4, 0, s, a, ops);
+        else fr_launch(k_dense_disu<OPS, 4>, grid_groups(a.ne, 4, 8), NF * 4, 0, s, a, ops, opsff);
     } else if (phase == 1) {
         constexpr int NTH = 128;
         const size_t base = (size_t)(20 * NUS + 5 * NF + 20 * NQP) * sizeof(T);
@@ -1418,7 +1393,7 @@ int dense_phase(int phase, const HexArgs<T> &a, const OPS *ops, const FFOf<OPS> 
                 const size_t smem = base + (a.tcmode == 1 ? DenseTC<OPS, 1>::BYTES : DenseTC<OPS, 2>::BYTES);
                 // persistent: as many CTAs as fit on the SMs (shared memory, registers, and the 512
                 // tensor-memory columns at 32 per CTA)
-                auto kern = a.tcmode == 1 ? k_dense_B<T, NTH, OPS, 1> : k_dense_B<T, NTH, OPS, 2>;
+                auto kern = a.tcmode == 1 ? k_dense_B<NTH, OPS, 1> : k_dense_B<NTH, OPS, 2>;
                 static int occ[3] = {-1, -1, -1};
                 int &o = occ[a.tcmode];
                 if (o < 0) {
@@ -1437,7 +1412,17 @@ int dense_phase(int phase, const HexArgs<T> &a, const OPS *ops, const FFOf<OPS> 
             }
         }
         if constexpr (sizeof(T) == 8) {
-            k_dense_B_fx<OPS, NTH><<<grid_elems(a.ne, 4), NTH, 0, s>>>(a, ops);
+            fr_launch(k_dense_B_fx<OPS, NTH>, grid_elems(a.ne, 4), NTH, 0, s, a, ops);
+        } else if (!tcdone && a.ne < 8 * fr_sms()) {
+            // fewer elements than resident CTAs of one element: a small handle waits for one element's chain
+            // (B at 750 elements: tetrahedra 20.4 against 28.0 us with four per CTA, pyramids 29.2 against
+            // 37.4; at 1,296 tetrahedra 34.9 against 31.0)
+            static bool attr = false;
+            if (!attr) {
+                cudaFuncSetAttribute(k_dense_B<NTH, OPS, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)base);
+                attr = true;
+            }
+            fr_launch(k_dense_B<NTH, OPS, 0>, grid_elems(a.ne, 8), NTH, base, s, a, ops, opsff);
         } else if (!tcdone) {
             using D = Dense32<OPS>;
             static bool attr = false;
@@ -1445,10 +1430,10 @@ int dense_phase(int phase, const HexArgs<T> &a, const OPS *ops, const FFOf<OPS> 
                 cudaFuncSetAttribute(k_dense_B32<OPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D::SMEM);
                 attr = true;
             }
-            k_dense_B32<OPS><<<grid_groups(a.ne, D::EPB, 5), D::NTH, D::SMEM, s>>>(a, ops, opsff);
+            fr_launch(k_dense_B32<OPS>, grid_groups(a.ne, D::EPB, 5), D::NTH, D::SMEM, s, a, ops, opsff);
         }
     } else {
-        k_dense_C<T, OPS, 4><<<grid_groups(a.ne, 4, 8), NF * 4, 0, s>>>(a, ops, opsff);
+        fr_launch(k_dense_C<T, OPS, 4>, grid_groups(a.ne, 4, 8), NF * 4, 0, s, a, ops, opsff);
     }
     (void)NU;
     return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;

@@ -226,6 +226,7 @@ __device__ __forceinline__ void disu_blk_body(const HexArgs<T> &a, long long fir
     __shared__ ff s_lff[2 * N];
     for (int i = threadIdx.x; i < 2 * N; i += NT) s_lff[i] = i < N ? c_hexff[P - 2].lL[i] : c_hexff[P - 2].lR[i - N];
     __syncthreads();
+    fr_grid_wait();
     for (long long e0 = (long long)first * EB; e0 < a.ne; e0 += (long long)stride * EB) {
         const int nb = (int)((a.ne - e0) < EB ? (a.ne - e0) : EB);
         {
@@ -286,6 +287,7 @@ __device__ __forceinline__ void disu_blk_body(const HexArgs<T> &a, long long fir
         }
         __syncthreads();
     }
+    fr_grid_done();
 }
 
 // The same in FP64, with the traces in block fixed point (fr_fx.cuh): on the FP64 pipe the 20 multiply-adds
@@ -299,6 +301,7 @@ __device__ __forceinline__ void disu_fx_body(const HexArgs<double> &a, long long
     __shared__ fx2 s_l[2][N];
     for (int i = threadIdx.x; i < 2 * N; i += NT) s_l[i / N][i % N] = i < N ? c_hexfx[P - 2].lL[i] : c_hexfx[P - 2].lR[i - N];
     __syncthreads();
+    fr_grid_wait();
     for (long long e0 = (long long)first * EB; e0 < a.ne; e0 += (long long)stride * EB) {
         const int nb = (int)((a.ne - e0) < EB ? (a.ne - e0) : EB);
         {
@@ -329,6 +332,7 @@ __device__ __forceinline__ void disu_fx_body(const HexArgs<double> &a, long long
         }
         __syncthreads();
     }
+    fr_grid_done();
 }
 
 template <typename T, int P, int EB, int NT>
@@ -719,6 +723,7 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
         if constexpr (TMA_U) tc::mbar_init(&s_ubar, 1);
     }
     __syncthreads();
+    fr_grid_wait();
     const bool lane0 = (threadIdx.x & 31) == 0;
 
     for (long long e = first; e < a.ne; e += stride) {
@@ -1082,6 +1087,7 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
         if (threadIdx.x == 0) s_cnt = 0;
         __syncthreads();
     }
+    fr_grid_done();
 }
 
 template <typename T, int P, int NT, int TCM = 0, bool AA = true, bool SURF = false, bool CURV = false>
@@ -1166,6 +1172,7 @@ __device__ __forceinline__ void fused_B_body(const HexArgs<T> &a, long long firs
         tmem = s_tmem[0];
     }
 
+    fr_grid_wait();
     for (long long e = first; e < a.ne; e += stride) {
         const Geo<T> g = a.geo[e];
         const Phys<T> ph = elem_phys(a, e);
@@ -1666,6 +1673,7 @@ __device__ __forceinline__ void fused_B_body(const HexArgs<T> &a, long long firs
         if (tc_fail && threadIdx.x == 0) atomicOr(a.status, 2);
         tc::teardown(s_mbar, parity, tc_fail, tmem, TC::COLS);
     }
+    fr_grid_done();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1719,6 +1727,7 @@ __device__ __forceinline__ void hex_B32_body(const HexArgs<float> &a, long long 
     for (int i = tid; i < M * N; i += NT) s_b[i / N][i % N] = op.B[i / N][i % N];
     for (int i = tid; i < N * N; i += NT) s_dh[i / N][i % N] = c_hexff[P - 2].Dh[i / N][i % N];
     for (int i = tid; i < 2 * N; i += NT) s_l[i / N][i % N] = i < N ? op.lL[i] : op.lR[i - N];
+    fr_grid_wait();
     for (long long e0 = first * EPB; e0 < a.ne; e0 += stride * EPB) {
         const int nb = (int)((a.ne - e0) < EPB ? (a.ne - e0) : EPB);
         {
@@ -2013,6 +2022,7 @@ __device__ __forceinline__ void hex_B32_body(const HexArgs<float> &a, long long 
             a.R[s_u0[el] + (al + 1) * NU + z] = (y[0] + y[FS]) + y[2 * FS];
         }
     }
+    fr_grid_done();
 }
 
 template <int P, int EPB, int NT, int MB>
@@ -2111,6 +2121,7 @@ __device__ __forceinline__ void fused_C_body(const HexArgs<T> &a, long long firs
     }
     const T *liftL = s_lift, *liftR = s_lift + N;
     int par = 0;
+    fr_grid_wait();
     for (long long e = first; e < a.ne; e += stride) {
         if (!fr_elem_ok(a, e, (P + 1) * (P + 1) * (P + 1), 6 * (P + 1) * (P + 1))) continue;
         const Geo<T> g = a.geo[e];
@@ -2270,6 +2281,7 @@ __device__ __forceinline__ void fused_C_body(const HexArgs<T> &a, long long firs
         }
         __syncthreads();
     }
+    fr_grid_done();
 }
 
 // FP32: registers capped for 960 resident threads per SM (ten CTAs of 96, one thread per flux point
@@ -2292,6 +2304,7 @@ template <typename T, int P>
 __global__ void __launch_bounds__(128) k_surf_pair(HexArgs<T> a)
 {
     constexpr int M = P + 2, NQF = 6 * M * M;
+    fr_grid_wait();
     bool ok = true;
     for (long long it = blockIdx.x * (long long)blockDim.x + threadIdx.x; it < a.nqlpts; it += (long long)gridDim.x * blockDim.x) {
         const long long gl = a.qlpts[it];
@@ -2327,6 +2340,7 @@ __global__ void __launch_bounds__(128) k_surf_pair(HexArgs<T> a)
         }
     }
     flag_status(a.status, ok);
+    fr_grid_done();
 }
 
 template <typename T, int P, int NT>
@@ -2337,6 +2351,7 @@ __global__ void __launch_bounds__(NT) k_surf_lift(HexArgs<T> a)
     __shared__ T s_t[5 * 6 * N * M];
     __shared__ T s_d[5 * NF];
     const HexOps<T> &op = OPS<T>(P - 2);
+    fr_grid_wait();
     for (long long e = blockIdx.x; e < a.ne; e += gridDim.x) {
         if (!fr_elem_ok(a, e, (P + 1) * (P + 1) * (P + 1), 6 * (P + 1) * (P + 1))) continue;
         const Geo<T> g = a.geo[e];
@@ -2409,6 +2424,7 @@ __global__ void __launch_bounds__(NT) k_surf_lift(HexArgs<T> a)
         }
         __syncthreads();
     }
+    fr_grid_done();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2418,6 +2434,7 @@ template <typename T, int P, bool CURV = false>
 __global__ void __launch_bounds__(128) k_pair_flux(HexArgs<T> a)
 {
     constexpr int N = P + 1, NF = 6 * N * N;
+    fr_grid_wait();
     bool ok = true;
     for (long long it = blockIdx.x * (long long)blockDim.x + threadIdx.x; it < a.nlpts; it += (long long)gridDim.x * blockDim.x) {
         const uint32_t code = a.lpts[it];
@@ -2444,6 +2461,7 @@ __global__ void __launch_bounds__(128) k_pair_flux(HexArgs<T> a)
         for (int k = 0; k < 5; k++) a.DF[k * a.nfpt + gl] = F[k];
     }
     flag_status(a.status, ok);
+    fr_grid_done();
 }
 
 template <int P, int NT, bool CURV = false>
@@ -2455,6 +2473,7 @@ __global__ void __launch_bounds__(NT) k_lift(HexArgs<double> a)
     for (int i = threadIdx.x; i < 2 * N; i += NT) s_lx[i] = i < N ? c_hexfx[P - 2].liftL[i] : c_hexfx[P - 2].liftR[i - N];
     if (threadIdx.x < 10) s_mx[threadIdx.x / 5][threadIdx.x % 5] = 0;
     __syncthreads();
+    fr_grid_wait();
     int par = 0;
     for (long long e = blockIdx.x; e < a.ne; e += gridDim.x) {
         if (!fr_elem_ok(a, e, (P + 1) * (P + 1) * (P + 1), 6 * (P + 1) * (P + 1))) continue;
@@ -2481,6 +2500,7 @@ __global__ void __launch_bounds__(NT) k_lift(HexArgs<double> a)
         lift_fx<P, NT, CURV>(a, e, s_dx, s_lx, s_mx[par ^ 1], a.R + elem_u0(a, e, NU), g.nidet);
         __syncthreads();
     }
+    fr_grid_done();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2786,6 +2806,7 @@ __global__ void __launch_bounds__(NT, MB) k_hex_B32(HexArgs<float> a)
     __shared__ int s_cnt;
     const HexOps<float> &op = OPS<float>(1);
     const int tid = threadIdx.x;
+    fr_grid_wait();
     for (long long e0 = (long long)blockIdx.x * EPB; e0 < a.ne; e0 += (long long)gridDim.x * EPB) {
         const int nb = (int)((a.ne - e0) < EPB ? (a.ne - e0) : EPB);
         {
@@ -3187,6 +3208,7 @@ __global__ void __launch_bounds__(NT, MB) k_hex_B32(HexArgs<float> a)
         }
         __syncthreads();
     }
+    fr_grid_done();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -3221,13 +3243,13 @@ static void launch_B(const HexArgs<T> &a, cudaStream_t s)
             cudaFuncSetAttribute(k_fused_B_surf32<P, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             attr = true;
         }
-        k_fused_B_surf32<P, NT><<<grid_elems(a.ne, 8), NT, smem, s>>>(a);
+        fr_launch(k_fused_B_surf32<P, NT>, grid_elems(a.ne, 8), NT, smem, s, a);
     } else {
         if (!attr) {
             cudaFuncSetAttribute(k_fused_B<T, P, NT, 0, AA, SURF, CURV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             attr = true;
         }
-        k_fused_B<T, P, NT, 0, AA, SURF, CURV><<<grid_elems(a.ne, 8), NT, smem, s>>>(a);
+        fr_launch(k_fused_B<T, P, NT, 0, AA, SURF, CURV>, grid_elems(a.ne, 8), NT, smem, s, a);
     }
 }
 
@@ -3278,7 +3300,7 @@ static int launch_B32(const HexArgs<float> &a, cudaStream_t s)
     }
     long long g = (a.ne + EPB - 1) / EPB;   // persistent: at most the resident CTAs
     if (g > (long long)nsm * occ) g = (long long)nsm * occ;
-    k_hex_B32<EPB, NT, MB, SPLIT><<<(int)g, NT, smem, s>>>(a);
+    fr_launch(k_hex_B32<EPB, NT, MB, SPLIT>, g, NT, smem, s, a);
     return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -3291,7 +3313,7 @@ static void launch_B32p(const HexArgs<float> &a, cudaStream_t s)
         cudaFuncSetAttribute(k_hex_B32p<P, EPB, NT, MB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         attr = true;
     }
-    k_hex_B32p<P, EPB, NT, MB><<<grid_elems((a.ne + EPB - 1) / EPB, MB), NT, smem, s>>>(a);
+    fr_launch(k_hex_B32p<P, EPB, NT, MB>, grid_elems((a.ne + EPB - 1) / EPB, MB), NT, smem, s, a);
 }
 
 template <typename T, int P>
@@ -3299,10 +3321,16 @@ static int fused_phase(int phase, const HexArgs<T> &a, cudaStream_t s, int varia
 {
     if (a.ne == 0) return 0;
     if (phase == 0) {
-        constexpr int EB = 8;
-        long long g = (a.ne + EB - 1) / EB;
-        if (g > fr_sms() * 16) g = fr_sms() * 16;
-        k_disu_blk<T, P, EB, 256><<<(int)g, 256, 0, s>>>(a);
+        // fewer elements than one CTA of eight per SM: one element per CTA (the latency of eight elements'
+        // points in one CTA is what a small handle waits for)
+        if (a.ne < 8 * fr_sms()) {
+            fr_launch(k_disu_blk<T, P, 1, 128>, a.ne, 128, 0, s, a);
+        } else {
+            constexpr int EB = 8;
+            long long g = (a.ne + EB - 1) / EB;
+            if (g > fr_sms() * 16) g = fr_sms() * 16;
+            fr_launch(k_disu_blk<T, P, EB, 256>, g, 256, 0, s, a);
+        }
     } else if (phase == 1) {
         if constexpr (std::is_same<T, float>::value) {
             if (a.tcmode != 0) {
@@ -3343,6 +3371,7 @@ static int fused_phase(int phase, const HexArgs<T> &a, cudaStream_t s, int varia
             if (a.geo64 != nullptr) {
                 if (variant == 0) launch_B32p<P, 1, 96, P == 3 ? 10 : 7>(a, s);
                 else if (variant == 2) launch_B32p<P, P == 3 ? 2 : 1, P == 3 ? 160 : 224, P == 3 ? 6 : 4>(a, s);
+                else if (a.ne <= 2 * fr_sms()) launch_B32p<P, 1, 256, 2>(a, s);   // a small handle waits for one element's chain
                 else launch_B32p<P, P == 3 ? 2 : 1, 128, 6>(a, s);
                 return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
             }
@@ -3351,18 +3380,18 @@ static int fused_phase(int phase, const HexArgs<T> &a, cudaStream_t s, int varia
         else if (variant == 2) launch_B<T, P, 256>(a, s);
         else launch_B<T, P, 128>(a, s);
     } else if (phase == 2) {
-        if (a.mu) k_fused_C<T, P, 128, true><<<grid_elems(a.ne, 8), 128, 0, s>>>(a);
-        else if (P == 3) k_fused_C<T, P, 96><<<grid_elems(a.ne, 10), 96, 0, s>>>(a);
-        else k_fused_C<T, P, 128><<<grid_elems(a.ne, 8), 128, 0, s>>>(a);
+        if (a.mu) fr_launch(k_fused_C<T, P, 128, true>, grid_elems(a.ne, 8), 128, 0, s, a);
+        else if (P == 3) fr_launch(k_fused_C<T, P, 96>, grid_elems(a.ne, 10), 96, 0, s, a);
+        else fr_launch(k_fused_C<T, P, 128>, grid_elems(a.ne, 8), 128, 0, s, a);
     } else if (phase == 3) {
-        if (a.surf) { if (a.nqlpts > 0) k_surf_pair<T, P><<<grid_for(a.nqlpts, 128), 128, 0, s>>>(a); }
-        else if (a.nlpts > 0 && a.mu) k_pair_flux<T, P, true><<<grid_for(a.nlpts, 128), 128, 0, s>>>(a);
-        else if (a.nlpts > 0) k_pair_flux<T, P><<<grid_for(a.nlpts, 128), 128, 0, s>>>(a);
+        if (a.surf) { if (a.nqlpts > 0) fr_launch(k_surf_pair<T, P>, grid_for(a.nqlpts, 128), 128, 0, s, a); }
+        else if (a.nlpts > 0 && a.mu) fr_launch(k_pair_flux<T, P, true>, grid_for(a.nlpts, 128), 128, 0, s, a);
+        else if (a.nlpts > 0) fr_launch(k_pair_flux<T, P>, grid_for(a.nlpts, 128), 128, 0, s, a);
     } else {
-        if (a.surf) k_surf_lift<T, P, 128><<<grid_elems(a.ne, 8), 128, 0, s>>>(a);
+        if (a.surf) fr_launch(k_surf_lift<T, P, 128>, grid_elems(a.ne, 8), 128, 0, s, a);
         else if constexpr (sizeof(T) == 8) {   // (only FP64 hexahedral handles split the interface phase)
-            if (a.mu) k_lift<P, 128, true><<<grid_elems(a.ne, 8), 128, 0, s>>>(a);
-            else k_lift<P, 128><<<grid_elems(a.ne, 8), 128, 0, s>>>(a);
+            if (a.mu) fr_launch(k_lift<P, 128, true>, grid_elems(a.ne, 8), 128, 0, s, a);
+            else fr_launch(k_lift<P, 128>, grid_elems(a.ne, 8), 128, 0, s, a);
         } else return -1;
     }
     return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;

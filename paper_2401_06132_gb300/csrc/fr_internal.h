@@ -358,6 +358,32 @@ inline long long fr_sms()
 }
 
 #ifdef __CUDACC__
+// The phase kernels of an RHS are launched so that the next one may be set up while the last one's final
+// CTAs finish: every CTA of a phase kernel sets up its tables, then waits in fr_grid_wait, before it touches
+// the state or the face arrays, until the kernels before it have completed and their writes are visible (a
+// kernel completes only after the ones before it have, so the order is that of the stream), and lets the
+// next kernel in with fr_grid_done once its own work is done. (Let in at the start, waiting CTAs of later
+// kernels crowd the SMs: a 5^3 FP64 box with full anti-aliasing took 0.120 instead of 0.081 ms.)
+__device__ __forceinline__ void fr_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void fr_grid_done() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Launches a phase kernel that calls fr_grid_wait.
+template <typename... P, typename... A>
+inline void fr_launch(void (*kernel)(P...), long long grid, int block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3((unsigned)block);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = at;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
 template <typename T>
 __device__ __forceinline__ void rk_fold(const HexArgs<T> &a, long long i, T val)
 {

@@ -73,7 +73,7 @@ int pri_fused_phase(int phase, const HexArgs<T> &a, const PriOps<T> *ops, const 
         const long long g0 = sizeof(T) == 8 ? (a.ne + 2) / 3 : (a.ne * NF + 255) / 256;
         long long g = g0;
         if (g > fr_sms() * 64) g = fr_sms() * 64;
-        k_pri_disu<T><<<(int)g, 256, 0, s>>>(a, ops, ops64);
+        fr_launch(k_pri_disu<T>, (int)g, 256, 0, s, a, ops, ops64);
     } else if (phase == 1) {
         constexpr int NTH = 128;
         const size_t base = ((sizeof(PriOps<T>) + 15) / 16) * 16 + (size_t)(5 * NU + 15 * NU + 5 * NF + 20 * NQ) * sizeof(T);
@@ -110,11 +110,11 @@ int pri_fused_phase(int phase, const HexArgs<T> &a, const PriOps<T> *ops, const 
                 cudaFuncSetAttribute(k_pri_B<T, NTH, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
                 attr = true;
             }
-            k_pri_B<T, NTH, 0><<<grid_elems(a.ne, 8), NTH, smem, s>>>(a, ops, ops64);
+            fr_launch(k_pri_B<T, NTH, 0>, grid_elems(a.ne, 8), NTH, smem, s, a, ops, ops64);
         }
     } else {
-        if constexpr (sizeof(T) == 4) k_pri_C<T, 96><<<grid_elems(a.ne, 10), 96, 0, s>>>(a, ops, ops64);
-        else k_pri_C<T, 128><<<grid_elems(a.ne, 8), 128, 0, s>>>(a, ops, ops64);
+        if constexpr (sizeof(T) == 4) fr_launch(k_pri_C<T, 96>, grid_elems(a.ne, 10), 96, 0, s, a, ops, ops64);
+        else fr_launch(k_pri_C<T, 128>, grid_elems(a.ne, 8), 128, 0, s, a, ops, ops64);
     }
     return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
 }

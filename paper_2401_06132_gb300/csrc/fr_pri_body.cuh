@@ -148,6 +148,7 @@ __device__ __forceinline__ void pri_disu_body(const HexArgs<float> &a, const Pri
         for (int i = threadIdx.x; i < (int)(sizeof(PriOpsFF) / sizeof(float)); i += 256) dst[i] = src[i];
     }
     __syncthreads();
+    fr_grid_wait();
     const long long total = a.ne * NF;
     for (long long it = first * (long long)blockDim.x + threadIdx.x; it < total; it += (long long)stride * blockDim.x) {
         // one thread per (element, flux point), all five variables
@@ -185,6 +186,7 @@ __device__ __forceinline__ void pri_disu_body(const HexArgs<float> &a, const Pri
             }
         }
     }
+    fr_grid_done();
 }
 
 
@@ -199,6 +201,7 @@ __device__ __forceinline__ void pri_disu_fx_body(const HexArgs<double> &a, const
     for (int i = threadIdx.x; i < 2 * NZ; i += NTH) s_lz[i / NZ][i % NZ] = i < NZ ? op.lzL[i] : op.lzR[i - NZ];
     const int kF = op.kF;
     __syncthreads();
+    fr_grid_wait();
     for (long long e0 = first * EB; e0 < a.ne; e0 += stride * EB) {
         const int nb = (int)(a.ne - e0 < EB ? a.ne - e0 : EB);
         {
@@ -231,6 +234,7 @@ __device__ __forceinline__ void pri_disu_fx_body(const HexArgs<double> &a, const
         }
         __syncthreads();
     }
+    fr_grid_done();
 }
 
 // -------------------------------------------------------------------------------------------------
@@ -602,6 +606,7 @@ __device__ __forceinline__ void pri_B32_body(const HexArgs<float> &a, const PriO
     for (int t = 0; t < NT_; t++) bt[t] = opsff->hi.Bt[tq][t];
     if (tid == 0) s_pcnt = 0;
     __syncthreads();
+    fr_grid_wait();
     for (long long e = first; e < a.ne; e += stride) {
         if (!fr_elem_ok(a, e, NU, NF)) continue;
         const Geo<float> g = a.geo[e];
@@ -848,6 +853,7 @@ __device__ __forceinline__ void pri_B32_body(const HexArgs<float> &a, const PriO
         }
         __syncthreads();
     }
+    fr_grid_done();
 }
 
 // -------------------------------------------------------------------------------------------------
@@ -889,6 +895,7 @@ __device__ __forceinline__ void pri_B_fx_body(const HexArgs<double> &a, const Pr
     if (tid < 10) s_mx[tid] = 0;
     if (tid == 0) s_pcnt = 0;
     __syncthreads();
+    fr_grid_wait();
     for (long long e = first; e < a.ne; e += stride) {
         if (!fr_elem_ok(a, e, NU, NF)) continue;
         const Geo<double> g = a.geo[e];
@@ -1112,6 +1119,7 @@ __device__ __forceinline__ void pri_B_fx_body(const HexArgs<double> &a, const Pr
         if (tid == 0) s_pcnt = 0;
         __syncthreads();
     }
+    fr_grid_done();
 }
 
 // -------------------------------------------------------------------------------------------------
@@ -1139,6 +1147,7 @@ __device__ __forceinline__ void pri_C_body(const HexArgs<T> &a, const PriOps<T> 
         load_ops<T, NTH>(gops, op_);
     }
     __syncthreads();
+    fr_grid_wait();
     for (long long e = first; e < a.ne; e += stride) {
         if (!fr_elem_ok(a, e, NU, NF)) continue;
         const Geo<T> g = a.geo[e];
@@ -1264,6 +1273,7 @@ __device__ __forceinline__ void pri_C_body(const HexArgs<T> &a, const PriOps<T> 
         }
         __syncthreads();
     }
+    fr_grid_done();
 }
 
 
