@@ -1,7 +1,8 @@
 // fr_fx.cuh -- 64-bit block fixed-point arithmetic for the linear operators of the FP64 kernels.
 //
-// GB300 issues 1.6 FP64 multiply-adds per clock and SM, but 54 wide integer multiply-adds
-// (32 x 32 + 64 -> 64 bits; both measured, dependent-free streams). The interpolation, projection,
+// GB300 issues 1.6 FP64 multiply-adds per clock and SM, but 32 wide integer multiplications
+// (32 x 32 -> 64 bits; both measured, dependent-free streams), so about ten terms of a fixed-point
+// sum (eight in the kernels' loops). The interpolation, projection,
 // differentiation and trace operators are constant matrices applied to a block of values (one field of
 // one element), so they run in fixed point: the block is scaled by one power of two, taken from its
 // largest magnitude, to integers below 2^56, and every product-sum is exact in 64-bit integers down
@@ -10,7 +11,7 @@
 //
 // A value X is held as two limbs X = h 2^28 + l (0 <= l < 2^28), a coefficient C = round(c 2^(58-k))
 // as C = H 2^28 + L (|L| <= 2^27; k is the operator's scale, FX_KD, FX_KP or FX_KL). A term of a sum
-// takes three wide multiply-adds: hh += H h, mm += H l + L h; the dropped L l is below 2^-57 of the
+// takes three wide products, each added to a 64-bit sum: hh += H h, mm += H l + L h; the dropped L l is below 2^-57 of the
 // term's bound. The sum is Y = hh + (mm >> 28), in units of X 2^(k - 2). Bounds, for operators whose
 // absolute row sums are at most 2 after scaling and |X| < 2^59: |h| < 2^31, |hh| < 2^62, |mm| < 2^62.
 #pragma once

@@ -2040,7 +2040,7 @@ __device__ __forceinline__ void volume_body(const HexArgs<T> &a, long long first
     else fused_B_body<T, P, NT, TCM, AA, SURF, CURV>(a, first, stride);
 }
 
-// The FP32 affine p = 3 volume kernel is capped at 48 registers per thread: ten CTAs of 128 threads
+// The FP32 affine p = 3 volume kernel without a reference state is capped at 48 registers per thread: ten CTAs of 128 threads
 // per SM (more warps to hide its shared-memory latency; an eleventh, which its shared memory would
 // allow, needs 40 registers, spills and measured slower). The FP64 fixed-point kernel is capped at 96
 // registers, five CTAs of 128 threads per SM as its shared memory allows (measured on its first form: four CTAs
@@ -2073,11 +2073,36 @@ __global__ void __launch_bounds__(NT, 896 / NT) k_fused_B_surf32(HexArgs<float> 
 // FP64: R += lift of the common flux held in block fixed point (D: [variable][flux point], exponent fields
 // E), R *= -1/det J, and the RK4 stage update. On the FP64 pipe the six multiply-adds per value were half
 // of the lift kernel's operations.
+// p = 3 loads R and the stage sums of its three values per thread before the common flux arrives (the
+// kernel waits on memory: 0.404 to 0.375 ms at 48^3 elements); the five of p = 4 would cost too many
+// registers (0.103 to 0.145 ms at 25^3) and are loaded one by one.
+template <int P, int NT>
+struct LiftIn {
+    static constexpr int M = (5 * (P + 1) * (P + 1) * (P + 1) + NT - 1) / NT;
+    static constexpr bool EARLY = M <= 3;
+    double r[EARLY ? M : 1];
+    RkIn rk[EARLY ? M : 1];
+    __device__ __forceinline__ LiftIn(const HexArgs<double> &a, long long u0)
+    {
+#pragma unroll
+        for (int m = 0; m < (EARLY ? M : 0); m++) {
+            const int it = threadIdx.x + m * NT;
+            const bool in = it < 5 * (P + 1) * (P + 1) * (P + 1);
+            r[m] = in ? a.R[u0 + it] : 0.0;
+            rk[m] = in && a.rkstage != 0 ? rk_load(a, u0 + it) : RkIn{0.0, 0.0};
+        }
+    }
+};
+
 template <int P, int NT, bool CURV>
-__device__ __forceinline__ void lift_fx(const HexArgs<double> &a, long long e, const fx2 *Dx, const fx2 *l, const int *E, double *R, double idet)
+__device__ __forceinline__ void lift_fx(const HexArgs<double> &a, long long e, const LiftIn<P, NT> &in, const fx2 *Dx, const fx2 *l, const int *E, double *R, double idet)
 {
-    constexpr int N = P + 1, NU = N * N * N, NF = 6 * N * N, N2 = N * N;
-    for (int it = threadIdx.x; it < 5 * NU; it += NT) {
+    constexpr int N = P + 1, NU = N * N * N, NF = 6 * N * N, N2 = N * N, M = LiftIn<P, NT>::M;
+    constexpr bool EARLY = LiftIn<P, NT>::EARLY;
+#pragma unroll(EARLY ? M : 1)
+    for (int m = 0; m < M; m++) {
+        const int it = threadIdx.x + m * NT;
+        if (it >= 5 * NU) break;
         const int alpha = it / NU, z = it % NU, i = z % N, j = (z / N) % N, k = z / N2;
         const fx2 *D = Dx + alpha * NF;
         fxacc t{0, 0};
@@ -2089,8 +2114,9 @@ __device__ __forceinline__ void lift_fx(const HexArgs<double> &a, long long e, c
         fx_mac(t, l[N + k], D[5 * N2 + i + N * j]);
         // curved elements: det J at this solution point
         const double sc = CURV ? -fr_inv(a.mu[(e * NU + z) * 10 + 9]) : idet;
-        const double v = (R[it] + fx_double(fx_sum(t), E[alpha] - 1080 + FX_KD, E[alpha] >= 2047)) * sc;
+        const double v = ((EARLY ? in.r[EARLY ? m : 0] : R[it]) + fx_double(fx_sum(t), E[alpha] - 1080 + FX_KD, E[alpha] >= 2047)) * sc;
         if (a.rkstage == 0) R[it] = v;
+        else if constexpr (EARLY) rk_store(a, elem_u0(a, e, NU) + it, v, in.rk[m]);
         else rk_fold(a, elem_u0(a, e, NU) + it, v);
     }
 }
@@ -2193,8 +2219,9 @@ __device__ __forceinline__ void fused_C_body(const HexArgs<T> &a, long long firs
         const T idet = g.nidet;
         if constexpr (FX) {
             int E[5];
+            const LiftIn<P, NT> in(a, elem_u0(a, e, NU));
             fx_stage5<NF, NT, RD>(dv, s_dx, s_mx, par, E);
-            lift_fx<P, NT, CURV>(a, e, s_dx, s_lx, s_mx[par ^ 1], R, idet);
+            lift_fx<P, NT, CURV>(a, e, in, s_dx, s_lx, s_mx[par ^ 1], R, idet);
         } else {
             __syncthreads();
         }
@@ -2479,6 +2506,7 @@ __global__ void __launch_bounds__(NT) k_lift(HexArgs<double> a)
         if (!fr_elem_ok(a, e, (P + 1) * (P + 1) * (P + 1), 6 * (P + 1) * (P + 1))) continue;
         const Geo<double> g = a.geo[e];
         const long long gf0 = elem_f0(a, e, NF);
+        const LiftIn<P, NT> in(a, elem_u0(a, e, NU));
         double dv[RD][5];
 #pragma unroll
         for (int rd = 0; rd < RD; rd++) {
@@ -2497,7 +2525,7 @@ __global__ void __launch_bounds__(NT) k_lift(HexArgs<double> a)
         }
         int E[5];
         fx_stage5<NF, NT, RD>(dv, s_dx, s_mx, par, E);
-        lift_fx<P, NT, CURV>(a, e, s_dx, s_lx, s_mx[par ^ 1], a.R + elem_u0(a, e, NU), g.nidet);
+        lift_fx<P, NT, CURV>(a, e, in, s_dx, s_lx, s_mx[par ^ 1], a.R + elem_u0(a, e, NU), g.nidet);
         __syncthreads();
     }
     fr_grid_done();
@@ -3322,7 +3350,8 @@ static int fused_phase(int phase, const HexArgs<T> &a, cudaStream_t s, int varia
     if (a.ne == 0) return 0;
     if (phase == 0) {
         // fewer elements than one CTA of eight per SM: one element per CTA (the latency of eight elements'
-        // points in one CTA is what a small handle waits for)
+        // points in one CTA is what a small handle waits for: FP32 p = 3, 27 elements 12.4 to 8.6 us, 512
+        // elements 11.7 to 8.8; p = 4, 512 elements 15.1 to 11.3)
         if (a.ne < 8 * fr_sms()) {
             fr_launch(k_disu_blk<T, P, 1, 128>, a.ne, 128, 0, s, a);
         } else {
@@ -3371,7 +3400,9 @@ static int fused_phase(int phase, const HexArgs<T> &a, cudaStream_t s, int varia
             if (a.geo64 != nullptr) {
                 if (variant == 0) launch_B32p<P, 1, 96, P == 3 ? 10 : 7>(a, s);
                 else if (variant == 2) launch_B32p<P, P == 3 ? 2 : 1, P == 3 ? 160 : 224, P == 3 ? 6 : 4>(a, s);
-                else if (a.ne <= 2 * fr_sms()) launch_B32p<P, 1, 256, 2>(a, s);   // a small handle waits for one element's chain
+                // a small handle waits for one element's chain: twice the threads per element (p = 3, 27
+                // elements: 12.2 to 10.0 us, 216: 12.2 to 10.8, but 343: 13.5 to 14.3)
+                else if (a.ne <= 2 * fr_sms()) launch_B32p<P, 1, 256, 2>(a, s);
                 else launch_B32p<P, P == 3 ? 2 : 1, 128, 6>(a, s);
                 return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
             }

@@ -384,19 +384,33 @@ inline void fr_launch(void (*kernel)(P...), long long grid, int block, size_t sm
     cudaLaunchKernelEx(&c, kernel, P(args)...);
 }
 
+// The RK4 stage sums at a value: their operands, and the update.
+struct RkIn {
+    double u, acc;
+};
 template <typename T>
-__device__ __forceinline__ void rk_fold(const HexArgs<T> &a, long long i, T val)
+__device__ __forceinline__ RkIn rk_load(const HexArgs<T> &a, long long i)
+{
+    return {a.rkU[i], a.rkstage == 1 ? 0.0 : a.rkacc[i]};
+}
+template <typename T>
+__device__ __forceinline__ void rk_store(const HexArgs<T> &a, long long i, T val, const RkIn &in)
 {
     const double kv = (double)val;
     const int st = a.rkstage - 1;
     if (st == 3) {
-        a.rkU[i] += a.rkdt * (a.rkacc[i] + (1.0 / 6.0) * kv);
+        a.rkU[i] = in.u + a.rkdt * (in.acc + (1.0 / 6.0) * kv);
     } else {
         const double b = st == 0 ? 1.0 / 6.0 : 1.0 / 3.0;
         const double c = st == 2 ? 1.0 : 0.5;
-        a.rkacc[i] = (st == 0 ? 0.0 : a.rkacc[i]) + b * kv;
-        a.rkus[i] = (T)(a.rkU[i] + c * a.rkdt * kv);
+        a.rkacc[i] = in.acc + b * kv;
+        a.rkus[i] = (T)(in.u + c * a.rkdt * kv);
     }
+}
+template <typename T>
+__device__ __forceinline__ void rk_fold(const HexArgs<T> &a, long long i, T val)
+{
+    rk_store(a, i, val, rk_load(a, i));
 }
 #endif
 
