@@ -652,7 +652,7 @@ __device__ __forceinline__ void project_5(const HexOps<T> &op, const T *src, T *
 // ---------------------------------------------------------------------------------------------
 // With every operator on the FP64 pipe (1.6 multiply-adds per clock and SM) that pipe bounds the
 // kernel: 69,000 FP64 operations per element at p = 3, two thirds of them in the line operators. Those
-// run on the integer multipliers instead (three wide multiply-adds per term at 54 per clock and SM),
+// run on the integer multipliers instead (three wide products per term, 32 per clock and SM),
 // which leaves the FP64 pipe the pointwise fluxes; the two overlap across the CTAs of an SM. Every
 // block (one conserved variable of one element with its common solution; one flux component) is
 // scaled by the power of two of its largest magnitude, found with warp reductions; derived fields (the
@@ -661,7 +661,8 @@ __device__ __forceinline__ void project_5(const HexOps<T> &op, const T *src, T *
 // RHS error is 0.99 of the FP64 sweeps' (4^3 and 3^3 boxes, diagonal, sheared and curved metrics).
 // What is left on the FP64 pipe: 80 operations per quadrature point and 70 per viscous flux point, 55% of
 // its cycles; the rest is latency (integer chains, barriers, instruction fetch) at 20 warps per SM.
-// Measured, 48^3 p = 3: 15.5 -> 5.48 ms per launch; 25^3 p = 4: 4.18 -> 1.60 ms.
+// Measured, 48^3 p = 3: 15.5 -> 5.48 ms per launch; 25^3 p = 4: 4.18 -> 1.60 ms. Collocation, per RHS:
+// 48^3 p = 3 7.72 -> 4.80 ms (this kernel 3.33), 25^3 p = 4 with every other kernel 2.42 -> 1.23 ms.
 // y = A x along one line, rows to fixed-point limbs.
 template <int R, int C, int LD>
 __device__ __forceinline__ void line_fx(const fx2 (*A)[LD], const fx2 (&x)[C], fx2 (&y)[R])
@@ -675,23 +676,26 @@ __device__ __forceinline__ void line_fx(const fx2 (*A)[LD], const fx2 (&x)[C], f
     }
 }
 
-template <int P>
+// AA = false, collocation: the quadrature points are the solution points. No interpolation; the flux of
+// the solution points, then R = sum_d Dh_d f~_d in fixed point too.
+template <int P, bool AA = true>
 struct HexFxSmem {
     using S = HexSmem<double, P>;
     static constexpr int TRC = S::NF / 2;                  // flux points whose traces are staged at a time
-    static constexpr int XO = 20 * S::M * S::N * S::N;     // the first sweep's output
+    static constexpr int XO = AA ? 20 * S::M * S::N * S::N : 15 * S::NU;   // the first sweep's output; the flux
     // state, gradient and common solution, then the second sweep's output, then the projection's first
     static constexpr int LOW = S::LOW;
     // the first sweep's output and the traces, then the flux, then the projection's second sweep
-    static constexpr int W = XO + 20 * TRC > 15 * S::NQ ? XO + 20 * TRC : 15 * S::NQ;
+    static constexpr int W = !AA || XO + 20 * TRC > 15 * S::NQ ? XO + 20 * TRC : 15 * S::NQ;
     static constexpr size_t SMEM = (size_t)(LOW + S::PF + W) * sizeof(double);
 };
 
-template <int P, int NT, bool CURV>
+template <int P, int NT, bool CURV, bool AA>
 __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long long first, long long stride)
 {
+    static_assert(AA || !CURV, "curved elements run with flux anti-aliasing");
     using S = HexSmem<double, P>;
-    using X = HexFxSmem<P>;
+    using X = HexFxSmem<P, AA>;
     constexpr int N = S::N, M = S::M, NU = S::NU, NF = S::NF, NQ = S::NQ, M2 = M * M;
     constexpr int XS = S::XS, PS = S::PS, FS = S::FS;
     constexpr int NV1 = NU + NF, IT = (NV1 + NT - 1) / NT;   // values of one variable: state, then common solution
@@ -707,7 +711,7 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
     __shared__ int s_cnt;
     __shared__ int s_mx[21];   // exponent fields: 5 variables, 15 flux components, the metric (curved)
     // operator rows selected at run time (a constant-memory load is serialised over distinct addresses)
-    __shared__ fx2 s_l[2][N], s_b[M][N], s_pj[2][N][M];   // (s_pj: Pj, Dh Pj)
+    __shared__ fx2 s_l[2][N], s_b[M][N], s_pj[2][N][M];   // (s_pj: Pj, Dh Pj; AA = false: Dh)
     const HexFx &op = c_hexfx[P - 2];
     constexpr bool TMA_U = S::TMA;
     __shared__ uint64_t s_ubar;
@@ -716,8 +720,12 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
     if (threadIdx.x < 21) s_mx[threadIdx.x] = 0;
     for (int i = threadIdx.x; i < 2 * N; i += NT) s_l[i / N][i % N] = i < N ? op.lL[i] : op.lR[i - N];
     for (int i = threadIdx.x; i < M * N; i += NT) s_b[i / N][i % N] = op.B[i / N][i % N];
-    for (int i = threadIdx.x; i < 2 * N * M; i += NT)
-        s_pj[i / (N * M)][(i / M) % N][i % M] = i < N * M ? op.Pj[(i / M) % N][i % M] : op.DP[(i / M) % N][i % M];
+    if constexpr (AA) {
+        for (int i = threadIdx.x; i < 2 * N * M; i += NT)
+            s_pj[i / (N * M)][(i / M) % N][i % M] = i < N * M ? op.Pj[(i / M) % N][i % M] : op.DP[(i / M) % N][i % M];
+    } else {
+        for (int i = threadIdx.x; i < N * N; i += NT) s_pj[0][i / N][i % N] = op.Dh[i / N][i % N];
+    }
     if (threadIdx.x == 0) {
         s_cnt = 0;
         if constexpr (TMA_U) tc::mbar_init(&s_ubar, 1);
@@ -945,49 +953,63 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
             __syncthreads();
         }
         traces(0);
-        // 6. uqpts + gradcoru_qpts, x and y sweeps of the 20 fields
-        for (int it = threadIdx.x; it < 20 * N * N; it += NT) {
-            const int f = it / (N * N), jk = it % (N * N);
-            const int sb = f * FS + XS * (jk % N) + PS * (jk / N);
-            fx2 u[N], v[M];
+        if constexpr (AA) {
+            // 6. uqpts + gradcoru_qpts, x and y sweeps of the 20 fields
+            for (int it = threadIdx.x; it < 20 * N * N; it += NT) {
+                const int f = it / (N * N), jk = it % (N * N);
+                const int sb = f * FS + XS * (jk % N) + PS * (jk / N);
+                fx2 u[N], v[M];
 #pragma unroll
-            for (int i = 0; i < N; i++) u[i] = s_u[sb + i];
-            line_fx(op.B, u, v);
+                for (int i = 0; i < N; i++) u[i] = s_u[sb + i];
+                line_fx(op.B, u, v);
 #pragma unroll
-            for (int q = 0; q < M; q++) s_wx[f * M * N * N + q + M * jk] = v[q];
+                for (int q = 0; q < M; q++) s_wx[f * M * N * N + q + M * jk] = v[q];
+            }
         }
         __syncthreads();
         viscous(0);
-        for (int it = threadIdx.x; it < 20 * M * N; it += NT) {   // (f, qa, k) -> [f][ab][k], over the state and gradient
-            const int f = it / (M * N), r = it % (M * N), qa = r % M, k = r / M;
-            fx2 u[N], v[M];
+        if constexpr (AA) {
+            for (int it = threadIdx.x; it < 20 * M * N; it += NT) {   // (f, qa, k) -> [f][ab][k], over the state and gradient
+                const int f = it / (M * N), r = it % (M * N), qa = r % M, k = r / M;
+                fx2 u[N], v[M];
 #pragma unroll
-            for (int j = 0; j < N; j++) u[j] = s_wx[f * M * N * N + qa + M * j + M * N * k];
-            line_fx(op.B, u, v);
+                for (int j = 0; j < N; j++) u[j] = s_wx[f * M * N * N + qa + M * j + M * N * k];
+                line_fx(op.B, u, v);
 #pragma unroll
-            for (int q = 0; q < M; q++) s_u[(f * M2 + qa + M * q) * N + k] = v[q];
+                for (int q = 0; q < M; q++) s_u[(f * M2 + qa + M * q) * N + k] = v[q];
+            }
+            __syncthreads();
         }
-        __syncthreads();
         // 7. the z factor and tdisf at each quadrature point (ab, c), c fastest (the points of a column
         //    share their loads); a diagonal metric's factors det J J^-1 are applied in the projection
         bool ok = true;
         int fm[15];
 #pragma unroll
         for (int c = 0; c < 15; c++) fm[c] = 0;
-        for (int it = threadIdx.x; it < NQ; it += NT) {
-            const int ab = it / M, c = it % M, q = ab + M2 * c;
-            fx2 bz[N];
+        constexpr int NP = AA ? NQ : NU;   // points of the flux
+        for (int it = threadIdx.x; it < NP; it += NT) {
+            const int ab = it / M, c = it % M, q = AA ? ab + M2 * c : it;
+            fx2 bz[AA ? N : 1];
+            const fx2 *y = AA ? s_u + ab * N : s_u + it % N + XS * ((it / N) % N) + PS * (it / (N * N));
+            if constexpr (AA) {
 #pragma unroll
-            for (int k = 0; k < N; k++) bz[k] = s_b[c][k];
-            const fx2 *y = s_u + ab * N;
+                for (int k = 0; k < N; k++) bz[k] = s_b[c][k];
+            }
             double u[5], gq[5][3], f[3][5];
 #pragma unroll
             for (int fl = 0; fl < 20; fl++) {
-                fxacc t{0, 0};
-#pragma unroll
-                for (int k = 0; k < N; k++) fx_mac(t, bz[k], y[fl * M2 * N + k]);
                 const int alpha = fl < 5 ? fl : (fl - 5) / 3, d = (fl - 5) % 3;
-                const double v = fx_double(fx_sum(t), E[alpha] - 1080 + (fl < 5 ? 0 : qe[fl < 5 ? 0 : d]), E[alpha] >= 2047);
+                const int ex = E[alpha] + (fl < 5 ? 0 : qe[fl < 5 ? 0 : d]);
+                double v;
+                if constexpr (AA) {
+                    fxacc t{0, 0};
+#pragma unroll
+                    for (int k = 0; k < N; k++) fx_mac(t, bz[k], y[fl * M2 * N + k]);
+                    v = fx_double(fx_sum(t), ex - 1080, E[alpha] >= 2047);
+                } else {
+                    const fx2 x = y[fl * FS];
+                    v = fx_double((long long)x.h * (1LL << 28) + x.l, ex - 1078, E[alpha] >= 2047);
+                }
                 if (fl < 5) u[fl] = v;
                 else gq[alpha][d] = v;
             }
@@ -995,7 +1017,7 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
             if (diagJ) {
 #pragma unroll
                 for (int i = 0; i < 15; i++) {
-                    s_w[i * NQ + q] = f[i % 3][i / 3];
+                    s_w[i * NP + q] = f[i % 3][i / 3];
                     fm[i] = max(fm[i], fx_mag(f[i % 3][i / 3]));
                 }
             } else {
@@ -1012,7 +1034,7 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
                 for (int i = 0; i < 15; i++) {
                     const int alpha = i / 3, d = i % 3;
                     const double v = cm[3 * d] * f[0][alpha] + cm[3 * d + 1] * f[1][alpha] + cm[3 * d + 2] * f[2][alpha];
-                    s_w[i * NQ + q] = v;
+                    s_w[i * NP + q] = v;
                     fm[i] = max(fm[i], fx_mag(v));
                 }
             }
@@ -1035,52 +1057,77 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
         auto common_exp = [&](int alpha) {
             return max(max(s_mx[5 + alpha * 3] + es[0], s_mx[6 + alpha * 3] + es[1]), s_mx[7 + alpha * 3] + es[2]);
         };
-        // (one code for the three directions, the operator rows from shared memory: three copies with
-        // constant operands missed in the instruction cache)
-        for (int it = threadIdx.x; it < 15 * M2; it += NT) {   // z: (d, alpha, qa qb) -> k
-            const int da = it / M2, ab = it % M2, d = da / 5, alpha = da % 5, comp = alpha * 3 + d;
-            const double sdd = d == 0 ? sd[0] : (d == 1 ? sd[1] : sd[2]);
-            const int Ef = common_exp(alpha) - (d == 0 ? es[0] : (d == 1 ? es[1] : es[2]));
-            const fx2 fd = fx_factor(sdd, fx_mag(sdd) >> 20);
-            fx2 u[M], v[N];
-#pragma unroll
-            for (int c = 0; c < M; c++) {
-                u[c] = fx_from(s_w[comp * NQ + ab + M2 * c], Ef);
-                if (diagJ) u[c] = fx_mul(fd, u[c]);
-            }
-            line_fx(s_pj[d == 2], u, v);
-#pragma unroll
-            for (int k = 0; k < N; k++) s_u[da * M2 * N + ab + M2 * k] = v[k];
-        }
-        __syncthreads();
-        for (int it = threadIdx.x; it < 15 * M * N; it += NT) {   // y: (d, alpha, qa, k) -> j
-            const int da = it / (M * N), r2 = it % (M * N), d = da / 5, alpha = da % 5, qa = r2 % M, k = r2 / M;
-            fx2 u[M], v[N];
-#pragma unroll
-            for (int b = 0; b < M; b++) u[b] = s_u[da * M2 * N + qa + M * b + M2 * k];
-            line_fx(s_pj[d == 1], u, v);
-#pragma unroll
-            for (int j = 0; j < N; j++) s_wx[(alpha * 3 + d) * NQ + qa + M * j + M * N * k] = v[j];
-        }
-        __syncthreads();
         double *R = a.R + elem_u0(a, e, NU);
-        for (int it = threadIdx.x; it < 5 * N * N; it += NT) {   // x: (alpha, j, k), sum over d -> i
-            const int alpha = it / (N * N), jk = it % (N * N);
-            fxacc t[N];
+        if constexpr (AA) {
+            // (one code for the three directions, the operator rows from shared memory: three copies with
+            // constant operands missed in the instruction cache)
+            for (int it = threadIdx.x; it < 15 * M2; it += NT) {   // z: (d, alpha, qa qb) -> k
+                const int da = it / M2, ab = it % M2, d = da / 5, alpha = da % 5, comp = alpha * 3 + d;
+                const double sdd = d == 0 ? sd[0] : (d == 1 ? sd[1] : sd[2]);
+                const int Ef = common_exp(alpha) - (d == 0 ? es[0] : (d == 1 ? es[1] : es[2]));
+                const fx2 fd = fx_factor(sdd, fx_mag(sdd) >> 20);
+                fx2 u[M], v[N];
 #pragma unroll
-            for (int i = 0; i < N; i++) t[i] = fxacc{0, 0};
-#pragma unroll 1
-            for (int d = 0; d < 3; d++)
-#pragma unroll
-                for (int q = 0; q < M; q++) {
-                    const fx2 u = s_wx[(alpha * 3 + d) * NQ + q + M * jk];
-#pragma unroll
-                    for (int i = 0; i < N; i++) fx_mac(t[i], s_pj[d == 0][i][q], u);
+                for (int c = 0; c < M; c++) {
+                    u[c] = fx_from(s_w[comp * NQ + ab + M2 * c], Ef);
+                    if (diagJ) u[c] = fx_mul(fd, u[c]);
                 }
-            const int Ef = common_exp(alpha);
-            const bool bad = max(max(s_mx[5 + alpha * 3], s_mx[6 + alpha * 3]), s_mx[7 + alpha * 3]) >= 2047;
+                line_fx(s_pj[d == 2], u, v);
 #pragma unroll
-            for (int i = 0; i < N; i++) R[alpha * NU + i + N * jk] = fx_double(fx_sum(t[i]), Ef - 1080 + FX_KP, bad);
+                for (int k = 0; k < N; k++) s_u[da * M2 * N + ab + M2 * k] = v[k];
+            }
+            __syncthreads();
+            for (int it = threadIdx.x; it < 15 * M * N; it += NT) {   // y: (d, alpha, qa, k) -> j
+                const int da = it / (M * N), r2 = it % (M * N), d = da / 5, alpha = da % 5, qa = r2 % M, k = r2 / M;
+                fx2 u[M], v[N];
+#pragma unroll
+                for (int b = 0; b < M; b++) u[b] = s_u[da * M2 * N + qa + M * b + M2 * k];
+                line_fx(s_pj[d == 1], u, v);
+#pragma unroll
+                for (int j = 0; j < N; j++) s_wx[(alpha * 3 + d) * NQ + qa + M * j + M * N * k] = v[j];
+            }
+            __syncthreads();
+            for (int it = threadIdx.x; it < 5 * N * N; it += NT) {   // x: (alpha, j, k), sum over d -> i
+                const int alpha = it / (N * N), jk = it % (N * N);
+                fxacc t[N];
+#pragma unroll
+                for (int i = 0; i < N; i++) t[i] = fxacc{0, 0};
+#pragma unroll 1
+                for (int d = 0; d < 3; d++)
+#pragma unroll
+                    for (int q = 0; q < M; q++) {
+                        const fx2 u = s_wx[(alpha * 3 + d) * NQ + q + M * jk];
+#pragma unroll
+                        for (int i = 0; i < N; i++) fx_mac(t[i], s_pj[d == 0][i][q], u);
+                    }
+                const int Ef = common_exp(alpha);
+                const bool bad = max(max(s_mx[5 + alpha * 3], s_mx[6 + alpha * 3]), s_mx[7 + alpha * 3]) >= 2047;
+#pragma unroll
+                for (int i = 0; i < N; i++) R[alpha * NU + i + N * jk] = fx_double(fx_sum(t[i]), Ef - 1080 + FX_KP, bad);
+            }
+        } else {
+            // the components in fixed point, over the state and gradient, then three line products per value
+            for (int it = threadIdx.x; it < 15 * NU; it += NT) {
+                const int comp = it / NU, z = it % NU, alpha = comp / 3, d = comp % 3;
+                const double sdd = d == 0 ? sd[0] : (d == 1 ? sd[1] : sd[2]);
+                fx2 u = fx_from(s_w[it], common_exp(alpha) - (d == 0 ? es[0] : (d == 1 ? es[1] : es[2])));
+                if (diagJ) u = fx_mul(fx_factor(sdd, fx_mag(sdd) >> 20), u);
+                s_u[comp * FS + z % N + XS * ((z / N) % N) + PS * (z / (N * N))] = u;
+            }
+            __syncthreads();
+            for (int it = threadIdx.x; it < 5 * NU; it += NT) {
+                const int alpha = it / NU, z = it % NU, i = z % N, j = (z / N) % N, k = z / (N * N);
+                const fx2 *x = s_u + alpha * 3 * FS;
+                fxacc t{0, 0};
+#pragma unroll
+                for (int c = 0; c < N; c++) {
+                    fx_mac(t, s_pj[0][i][c], x[c + XS * j + PS * k]);
+                    fx_mac(t, s_pj[0][j][c], x[FS + i + XS * c + PS * k]);
+                    fx_mac(t, s_pj[0][k][c], x[2 * FS + i + XS * j + PS * c]);
+                }
+                const bool bad = max(max(s_mx[5 + alpha * 3], s_mx[6 + alpha * 3]), s_mx[7 + alpha * 3]) >= 2047;
+                R[it] = fx_double(fx_sum(t), common_exp(alpha) - 1080 + FX_KD, bad);
+            }
         }
         __syncthreads();
         if (threadIdx.x < 21) s_mx[threadIdx.x] = 0;
@@ -2031,12 +2078,12 @@ __global__ void __launch_bounds__(NT, MB) k_hex_B32p(HexArgs<float> a)
     hex_B32_body<P, EPB, NT>(a, blockIdx.x, gridDim.x);
 }
 
-// The volume group of a precision and form: FP64 with flux anti-aliasing in block fixed point, the
-// other forms (FP32, collocation, surface-flux anti-aliasing) in their own arithmetic.
+// The volume group of a precision and form: FP64 in block fixed point but for surface-flux
+// anti-aliasing, the other forms in their own arithmetic.
 template <typename T, int P, int NT, int TCM = 0, bool AA = true, bool SURF = false, bool CURV = false>
 __device__ __forceinline__ void volume_body(const HexArgs<T> &a, long long first, long long stride)
 {
-    if constexpr (sizeof(T) == 8 && AA && !SURF) fused_B_fx_body<P, NT, CURV>(a, first, stride);
+    if constexpr (sizeof(T) == 8 && !SURF) fused_B_fx_body<P, NT, CURV, AA>(a, first, stride);
     else fused_B_body<T, P, NT, TCM, AA, SURF, CURV>(a, first, stride);
 }
 
@@ -2049,7 +2096,7 @@ __device__ __forceinline__ void volume_body(const HexArgs<T> &a, long long first
 template <typename T, int P, int NT, int TCM, bool AA, bool SURF, bool CURV>
 constexpr int fused_B_min_ctas()
 {
-    if (sizeof(T) == 8 && AA && !SURF) return 5 * 128 / NT;
+    if (sizeof(T) == 8 && !SURF) return 5 * 128 / NT;
     return (sizeof(T) == 4 && TCM == 0 && AA && !SURF && !CURV && P == 3) ? 10 * 128 / NT : 0;
 }
 
@@ -3263,8 +3310,8 @@ static void launch_B(const HexArgs<T> &a, cudaStream_t s)
     // the collocation form needs no quadrature-point buffers; surface-flux anti-aliasing stages its
     // in-plane interpolation (6 faces x 20 fields x m x n values) after the quadrature-point buffer
     constexpr int TI = 6 * 20 * S::M * S::N;
-    constexpr bool FX = sizeof(T) == 8 && AA && !SURF;
-    const size_t smem = FX ? HexFxSmem<P>::SMEM : (!AA ? S::LOW + S::PF : (SURF ? S::SIZE + TI : S::SIZE)) * sizeof(T);
+    constexpr bool FX = sizeof(T) == 8 && !SURF;
+    const size_t smem = FX ? HexFxSmem<P, AA>::SMEM : (!AA ? S::LOW + S::PF : (SURF ? S::SIZE + TI : S::SIZE)) * sizeof(T);
     static bool attr = false;
     if constexpr (SURF && sizeof(T) == 4) {
         if (!attr) {

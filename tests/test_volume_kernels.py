@@ -116,3 +116,34 @@ def test_fp32_dense_matches_oracle_on_both_sides_of_the_line(mesh, lowmach, beta
     f.sync_status()
     err = np.abs(r.cpu().numpy().reshape(ne, 5, nu) - Ro).max(axis=(0, 2)) / np.abs(Ro).max(axis=(0, 2))
     assert err.max() <= (2e-5 if lowmach else 1e-3), err
+
+
+@pytest.mark.parametrize("mesh", ["stretched", "sheared"])
+@pytest.mark.parametrize("p", [3, 4])
+@pytest.mark.parametrize("kind", ["jumps", "decades", "units"])
+@pytest.mark.parametrize("beta", [0.5, 0.2])
+def test_fp64_collocation_matches_oracle_on_extreme_states(mesh, p, kind, beta):
+    """Hexahedra without anti-aliasing, at the bound of the first test (chains are shorter)."""
+    m = W.sheared_box_mesh(3) if mesh == "sheared" else W.box_hex_mesh(3)
+    s = np.array([1.0, 7.0, 50.0]) if mesh == "stretched" else np.ones(3)
+    m = dict(m, verts=m["verts"] * s, period=tuple(np.array(m["period"]) * s))
+    mu, ne, nu = 1e-5 if kind == "units" else 1e-3, 27, (p + 1) ** 3
+    o = O.Oracle(m, p, p + 1, mu=mu, beta=beta, threads=NCPU)
+    amp = _state(kind, ne * nu, np.random.default_rng(7))
+    Uf = np.moveaxis(amp.reshape(5, ne, nu), 0, 1).reshape(-1).copy()
+    Ro = o.rhs(Uf)
+    f = fr.FRMesh(m, fr.make_params(p=p, nq1d=p + 1, beta=beta, mu=mu))
+    u = torch.from_numpy(Uf).cuda()
+    r = torch.empty_like(u)
+    f.rhs(u, r)
+    f.sync_status()
+    d = np.abs(r.cpu().numpy() - Ro).reshape(ne, 5, nu).max(axis=(0, 2))
+    G = max(np.abs(o.geometry(e)[1]).sum() for e in range(ne))
+    S = (np.abs(o.op(0, "Adiv")).sum(axis=(1, 2)) + np.abs(o.op(0, "lift")) @ np.linalg.norm(o.op(0, "nref"), axis=1)).max()
+    L = np.abs(o.op(0, "M0")).sum(1).max()
+    amp = np.abs(amp)
+    pr = 0.4 * amp[4].max()
+    w = ((amp[1:4] / amp[0]).max() + np.sqrt(1.4 * pr / amp[0].min())) * L
+    for a in range(5):
+        F = w * amp[a].max() * L + (pr if 1 <= a <= 3 else 0) + (w * pr if a == 4 else 0)
+        assert d[a] <= 2 * 500 * 2.0 ** -53 * F * S * G, (a, d[a])
