@@ -797,11 +797,15 @@ static void fill_prifx(const PriOps<double> &o, PriFx &table)
     x.kZ = fx_scale(big, row, 4.0);
     start();
     for (int t = 0; t < NT; t++) {
-        double s = 0, sy = 0;
-        for (int j = 0; j < NT; j++) { add(s, o.Dhx[t][j]); add(sy, o.Dhy[t][j]); }
-        s = s > sy ? s : sy;
-        for (int f = 0; f < 3; f++) for (int b = 0; b < NZ; b++) add(s, o.Lf[f][t][b]);   // times a normal's component, at most 1
-        end(s);
+        double s[2] = {0, 0}, l = 0;
+        for (int j = 0; j < NT; j++) { add(s[0], o.Dhx[t][j]); add(s[1], o.Dhy[t][j]); }
+        for (int f = 0; f < 3; f++)
+            for (int b = 0; b < NZ; b++) {
+                add(l, o.Lf[f][t][b]);   // (their largest entry; in a row, times the normal's components)
+                for (int d = 0; d < 2; d++) s[d] += std::fabs(o.nf[f][d] * o.Lf[f][t][b]);
+            }
+        end(s[0]);
+        end(s[1]);
     }
     for (int k = 0; k < NZ; k++) {
         double s = 0;
@@ -883,8 +887,12 @@ static void fill_dense_fx(OPS &t)
     x.kD = scale(3 * NU, [&](int o, auto add) {
         const int d = o / NU, z = o % NU;
         for (int j = 0; j < NU; j++) add(t.Dht[d][j][z]);
-        for (int s = 0; s < NF; s++) add(t.Lt[s][z]);   // times a normal's component, at most 1
+        for (int f = 0; f < NFACE; f++)
+            for (int s = OPS::F0(f); s < OPS::F0(f + 1); s++) add(t.nf[f][d] * t.Lt[s][z]);
     }, 1.0);
+    // (the lift alone too: its entries in limbs, its rows in a 64-bit sum)
+    const int kL = scale(NU, [&](int z, auto add) { for (int s = 0; s < NF; s++) add(t.Lt[s][z]); }, 4.0);
+    x.kD = x.kD > kL ? x.kD : kL;
     x.kV = scale(NU, [&](int z, auto add) {
         for (int d = 0; d < 3; d++)
             for (int q = 0; q < FR_TQ; q++) add(t.Dvt[d][q][z]);

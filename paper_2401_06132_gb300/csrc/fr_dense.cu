@@ -1007,19 +1007,20 @@ __global__ void __launch_bounds__(NTH, 4) k_dense_B_fx(HexArgs<double> a, const 
         for (int alpha = 0; alpha < 5; alpha++) E[alpha] = s_mx[alpha];
         if (tid < NU) {
 #pragma unroll
-            for (int alpha = 0; alpha < 5; alpha++) s_u[alpha * NUS + tid] = fx_from(val[alpha], E[alpha]);
+            for (int alpha = 0; alpha < 5; alpha++) s_u[alpha * NUS + tid] = fx_from<FX_WS>(val[alpha], E[alpha]);
         } else if (tid < NU + NF) {
 #pragma unroll
-            for (int alpha = 0; alpha < 5; alpha++) s_c[alpha * NF + tid - NU] = fx_from(val[alpha], E[alpha]);
+            for (int alpha = 0; alpha < 5; alpha++) s_c[alpha * NF + tid - NU] = fx_from<FX_WS>(val[alpha], E[alpha]);
         }
         __syncthreads();
         const int nplist = s_pcnt;
         // 2. corrected gradient q~_d = Dh_d u + sum_f n_f,d (L_f c), then q = J^-T q~
-        int EJ = 0;
+        int EJ[3], qe[3];   // gradient component k: value = X 2^(E - 1078 - FX_WS + qe[k])
 #pragma unroll
-        for (int k = 0; k < 9; k++) EJ = max(EJ, fx_mag(g.Ji[k]) >> 20);
-        EJ += 2;   // three terms
-        const int qe = op.kD + EJ - 1022;   // gradient: value = X 2^(E - 1078 + qe)
+        for (int k = 0; k < 3; k++) {
+            EJ[k] = fx_column_exp(g.Ji, k);
+            qe[k] = op.kD + EJ[k] - 1022;
+        }
         for (int it = tid; it < 5 * NU; it += NTH) {
             const int alpha = it / NU, z = it % NU;
             const fx2 *u = s_u + alpha * NUS, *c = s_c + alpha * NF;
@@ -1047,7 +1048,7 @@ __global__ void __launch_bounds__(NTH, 4) k_dense_B_fx(HexArgs<double> a, const 
             for (int k = 0; k < 3; k++) {
                 fxacc s{FX_HALF, 0};
 #pragma unroll
-                for (int d = 0; d < 3; d++) fx_mac(s, fx_factor(g.Ji[3 * d + k], EJ), qr[d]);
+                for (int d = 0; d < 3; d++) fx_mac(s, fx_factor(g.Ji[3 * d + k], EJ[k]), qr[d]);
                 s_u[(5 + alpha * 3 + k) * NUS + z] = fx_limbs(fx_sum(s));
             }
         }
@@ -1065,7 +1066,7 @@ __global__ void __launch_bounds__(NTH, 4) k_dense_B_fx(HexArgs<double> a, const 
 #pragma unroll
             for (int k = 0; k < 5; k++) {
                 const int f = 5 * fg + k, Ea = s_mx[f < 5 ? f : (f - 5) / 3];
-                s_tr[li * 20 + f] = fx_double(fx_sum(t[k]), Ea - 1080 + op.kM + (f < 5 ? 0 : qe), Ea >= 2047);
+                s_tr[li * 20 + f] = fx_double(fx_sum(t[k]), Ea - 1080 - FX_WS + op.kM + fx_field_exp(f, qe), Ea >= 2047);
             }
         }
         // 4. interpolation to this thread's quadrature point and the flux there
@@ -1093,10 +1094,10 @@ __global__ void __launch_bounds__(NTH, 4) k_dense_B_fx(HexArgs<double> a, const 
             double u[5], gq[5][3];
 #pragma unroll
             for (int alpha = 0; alpha < 5; alpha++) {
-                const int ex = E[alpha] - 1080 + op.kB;
+                const int ex = E[alpha] - 1080 - FX_WS + op.kB;
                 u[alpha] = fx_double(fx_sum(t[alpha]), ex, E[alpha] >= 2047);
 #pragma unroll
-                for (int d = 0; d < 3; d++) gq[alpha][d] = fx_double(fx_sum(t[5 + alpha * 3 + d]), ex + qe, E[alpha] >= 2047);
+                for (int d = 0; d < 3; d++) gq[alpha][d] = fx_double(fx_sum(t[5 + alpha * 3 + d]), ex + qe[d], E[alpha] >= 2047);
             }
             ok = total_flux(ph, u, gq, f);
             // det J J^-1 f, in place

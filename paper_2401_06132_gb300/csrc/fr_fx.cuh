@@ -14,11 +14,18 @@
 // takes three wide products, each added to a 64-bit sum: hh += H h, mm += H l + L h; the dropped L l is below 2^-57 of the
 // term's bound. The sum is Y = hh + (mm >> 28), in units of X 2^(k - 2). Bounds, for operators whose
 // absolute row sums are at most 2 after scaling and |X| < 2^59: |h| < 2^31, |hh| < 2^62, |mm| < 2^62.
+//
+// The state blocks of the prismatic, tetrahedral and pyramidal volume kernels are held FX_WS bits wider,
+// |X| < 2^58: with operators of at most 30 terms, scaled to row sums of at most 1 where a sum ends in limbs
+// and of 4 where it ends in FP64, |hh| < 2^62 and |mm| < 2^60 + 30 2^57 < 2^63. Their gradients take a
+// scale of 2^5 or 2^6 and then the room of the metric's three terms. (The prisms' line interpolation, row sums
+// below 1.6, ends in limbs below 1.6 2^58 and meets row sums of at most 2.)
 #pragma once
 
 #include <cstdint>
 
 #define FX_MASK 0x0fffffffu
+#define FX_WS 2
 
 // One coefficient or value in two limbs.
 struct fx2 { int h, l; };
@@ -77,17 +84,19 @@ __device__ __forceinline__ fx2 fx_mul(fx2 f, fx2 x)
 // Exponent field of the largest magnitude is formed from the high words: abs(hi) of a value.
 __device__ __forceinline__ int fx_mag(double v) { return __double2hiint(v) & 0x7fffffff; }
 
-// v of a block with biased exponent E (of its largest magnitude) as X = v 2^(1078 - E), |X| < 2^56.
+// v of a block with biased exponent E (of its largest magnitude) as X = v 2^(1078 + W - E), |X| < 2^(56 + W).
+template <int W = 0>
 __device__ __forceinline__ long long fx_int(double v, int E)
 {
     const int hi = __double2hiint(v), e = (hi >> 20) & 0x7ff;
     const unsigned mh = e ? ((unsigned)(hi & 0xfffff) | 0x100000u) : 0u;   // subnormal values count as zero
     unsigned long long m = ((unsigned long long)mh << 32) | (e ? (unsigned)__double2loint(v) : 0u);
-    m = (m << 3) >> min(E - e, 63);
+    m = (m << (3 + W)) >> min(E - e, 63);
     return hi < 0 ? -(long long)m : (long long)m;
 }
 __device__ __forceinline__ fx2 fx_split(long long x) { return fx2{(int)(x >> 28), (int)((unsigned)x & FX_MASK)}; }
-__device__ __forceinline__ fx2 fx_from(double v, int E) { return fx_split(fx_int(v, E)); }
+template <int W = 0>
+__device__ __forceinline__ fx2 fx_from(double v, int E) { return fx_split(fx_int<W>(v, E)); }
 
 // y 2^e2 rounded to FP64; NaN for a block that held a non-finite value.
 __device__ __forceinline__ double fx_double(long long y, int e2, bool bad)
@@ -160,5 +169,19 @@ __device__ __forceinline__ fx2 fx_factor(double c, int E)
     const long long C = fx_int(c, E) << 2;
     const int H = (int)((C + (1LL << 27)) >> 28);
     return fx2{H, (int)(C - ((long long)H << 28))};
+}
+
+// Exponent of the factors J^-1[d][k], d = 0..2, that form component k of a gradient (Ji: [3 d + k]), with the
+// room of three terms. Each component has its own: on an element of aspect ratio A the columns differ by A, and
+// at the largest one's exponent the gradient along the long direction would lose log2(A) bits.
+__device__ __forceinline__ int fx_column_exp(const double *Ji, int k)
+{
+    return (max(max(fx_mag(Ji[k]), fx_mag(Ji[3 + k])), fx_mag(Ji[6 + k])) >> 20) + 2;
+}
+// Exponent of field f (5 variables, then the gradients 5 + 3 alpha + d) relative to its variable's.
+__device__ __forceinline__ int fx_field_exp(int f, const int (&qe)[3])
+{
+    const int d = (f - 5) % 3;
+    return f < 5 ? 0 : (d == 0 ? qe[0] : (d == 1 ? qe[1] : qe[2]));
 }
 #endif

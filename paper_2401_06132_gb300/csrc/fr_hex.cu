@@ -657,8 +657,13 @@ __device__ __forceinline__ void project_5(const HexOps<T> &op, const T *src, T *
 // block (one conserved variable of one element with its common solution; one flux component) is
 // scaled by the power of two of its largest magnitude, found with warp reductions; derived fields (the
 // gradient) take static bounds from their operators. Values between the sweeps resolve 2^-56 of their
-// block, below the rounding (2^-53 per operation) of the FP64 sums; against an 80-bit evaluation the
-// RHS error is 0.99 of the FP64 sweeps' (4^3 and 3^3 boxes, diagonal, sheared and curved metrics).
+// block; a gradient component resolves 2^-52 of its variable's largest value (FX_KD bits of room) times the
+// largest entry of its own column of J^-1 (2^-50 on a full metric, three terms), where the FP64 sums round
+// terms of up to 2^3 of that value at 2^-53 each. A value far below its block's largest one holds fewer bits
+// than FP64 gives it; the element's results do not show it, as their sums run over the block. Against an 80-bit
+// evaluation the RHS error is 0.99 of the FP64 sweeps' (4^3 and 3^3 boxes, diagonal, sheared and curved
+// metrics), and per variable at most 1.4 times theirs on elements stretched by 10^4 and on velocities over
+// twelve decades inside an element.
 // What is left on the FP64 pipe: 80 operations per quadrature point and 70 per viscous flux point, 55% of
 // its cycles; the rest is latency (integer chains, barriers, instruction fetch) at 20 warps per SM.
 // Measured, 48^3 p = 3: 15.5 -> 5.48 ms per launch; 25^3 p = 4: 4.18 -> 1.60 ms. Collocation, per RHS:
@@ -709,7 +714,7 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
     double *s_tr = s_w + X::XO;                                // [listed flux point][20]
     __shared__ short s_list[NF];
     __shared__ int s_cnt;
-    __shared__ int s_mx[21];   // exponent fields: 5 variables, 15 flux components, the metric (curved)
+    __shared__ int s_mx[23];   // exponent fields: 5 variables, 15 flux components, the metric's columns (curved)
     // operator rows selected at run time (a constant-memory load is serialised over distinct addresses)
     __shared__ fx2 s_l[2][N], s_b[M][N], s_pj[2][N][M];   // (s_pj: Pj, Dh Pj; AA = false: Dh)
     const HexFx &op = c_hexfx[P - 2];
@@ -717,7 +722,7 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
     __shared__ uint64_t s_ubar;
     bool pending = false, first_wait = true;
     uint32_t uparity = 0;
-    if (threadIdx.x < 21) s_mx[threadIdx.x] = 0;
+    if (threadIdx.x < 23) s_mx[threadIdx.x] = 0;
     for (int i = threadIdx.x; i < 2 * N; i += NT) s_l[i / N][i % N] = i < N ? op.lL[i] : op.lR[i - N];
     for (int i = threadIdx.x; i < M * N; i += NT) s_b[i / N][i % N] = op.B[i / N][i % N];
     if constexpr (AA) {
@@ -794,10 +799,17 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
             if (lane0) atomicMax(&s_mx[alpha], m >> 20);
         }
         if constexpr (CURV) {
-            int m = 0;
-            for (int it = threadIdx.x; it < NU * 9; it += NT) m = max(m, fx_mag(a.mu[(e * NU + it / 9) * 10 + it % 9]));
-            m = (int)__reduce_max_sync(0xffffffffu, (unsigned)m);
-            if (lane0) atomicMax(&s_mx[20], m >> 20);
+            int m[3] = {0, 0, 0};
+            for (int it = threadIdx.x; it < NU * 3; it += NT) {
+                const double *Ji = a.mu + (e * NU + it / 3) * 10 + 3 * (it % 3);
+#pragma unroll
+                for (int k = 0; k < 3; k++) m[k] = max(m[k], fx_mag(Ji[k]));
+            }
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                m[k] = (int)__reduce_max_sync(0xffffffffu, (unsigned)m[k]);
+                if (lane0) atomicMax(&s_mx[20 + k], m[k] >> 20);
+            }
         }
         if constexpr (TMA_U) tc::fence_async_smem();   // this element's reads of s_pf before the copy that overwrites it
         __syncthreads();
@@ -840,20 +852,16 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
         const bool diagJ = !CURV && g.Ji[1] == 0.0 && g.Ji[2] == 0.0 && g.Ji[3] == 0.0 && g.Ji[5] == 0.0 &&
                            g.Ji[6] == 0.0 && g.Ji[7] == 0.0;
         // exponents of the physical gradient relative to the variable's: value = X 2^(E - 1078 + qe[d])
-        int qe[3], EJ = 0;
+        int qe[3], EJ[3] = {0, 0, 0};
         if (diagJ) {
 #pragma unroll
             for (int d = 0; d < 3; d++) qe[d] = FX_KD + (fx_mag(g.Ji[4 * d]) >> 20) - 1022;
         } else {
-            if constexpr (CURV) EJ = s_mx[20] + 2;
-            else {
-                int m = 0;
 #pragma unroll
-                for (int k = 0; k < 9; k++) m = max(m, fx_mag(g.Ji[k]));
-                EJ = (m >> 20) + 2;   // three terms
+            for (int k = 0; k < 3; k++) {
+                EJ[k] = CURV ? s_mx[20 + k] + 2 : fx_column_exp(g.Ji, k);
+                qe[k] = FX_KD + EJ[k] - 1022;
             }
-#pragma unroll
-            for (int d = 0; d < 3; d++) qe[d] = FX_KD + EJ - 1022;
         }
         for (int it = threadIdx.x; it < 15 * N * N; it += NT) {
             const int alpha = it / (3 * N * N), r = it % (3 * N * N), d = r / (N * N), loc = r % (N * N);
@@ -885,7 +893,7 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
                 const double *Ji = CURV ? a.mu + (e * NU + z) * 10 : g.Ji;
                 fx2 J[9];
 #pragma unroll
-                for (int k = 0; k < 9; k++) J[k] = fx_factor(Ji[k], EJ);
+                for (int k = 0; k < 9; k++) J[k] = fx_factor(Ji[k], EJ[k % 3]);
                 fx2 *q = s_q + z % N + XS * ((z / N) % N) + PS * (z / (N * N));
 #pragma unroll 1
                 for (int alpha = 0; alpha < 5; alpha++, q += 3 * FS) {
@@ -913,11 +921,11 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
                 const fx2 *x = s_u + 5 * fg * FS + base;
 #pragma unroll 1
                 for (int k = 0; k < 5; k++, x += FS) {
-                    const int fl = 5 * fg + k, alpha = fl < 5 ? fl : (fl - 5) / 3, d = (fl - 5) - 3 * alpha, Ef = s_mx[alpha];
+                    const int fl = 5 * fg + k, Ef = s_mx[fl < 5 ? fl : (fl - 5) / 3];
                     fxacc t{0, 0};
 #pragma unroll
                     for (int i = 0; i < N; i++) fx_mac(t, s_l[f & 1][i], x[i * str]);
-                    s_tr[li * 20 + fl] = fx_double(fx_sum(t), Ef - 1080 + FX_KL + (fl < 5 ? 0 : (d == 0 ? qe[0] : (d == 1 ? qe[1] : qe[2]))), Ef >= 2047);
+                    s_tr[li * 20 + fl] = fx_double(fx_sum(t), Ef - 1080 + FX_KL + fx_field_exp(fl, qe), Ef >= 2047);
                 }
             }
         };
@@ -999,7 +1007,7 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
 #pragma unroll
             for (int fl = 0; fl < 20; fl++) {
                 const int alpha = fl < 5 ? fl : (fl - 5) / 3, d = (fl - 5) % 3;
-                const int ex = E[alpha] + (fl < 5 ? 0 : qe[fl < 5 ? 0 : d]);
+                const int ex = E[alpha] + fx_field_exp(fl, qe);
                 double v;
                 if constexpr (AA) {
                     fxacc t{0, 0};
@@ -1130,7 +1138,7 @@ __device__ __forceinline__ void fused_B_fx_body(const HexArgs<double> &a, long l
             }
         }
         __syncthreads();
-        if (threadIdx.x < 21) s_mx[threadIdx.x] = 0;
+        if (threadIdx.x < 23) s_mx[threadIdx.x] = 0;
         if (threadIdx.x == 0) s_cnt = 0;
         __syncthreads();
     }

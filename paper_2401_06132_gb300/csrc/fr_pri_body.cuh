@@ -934,19 +934,20 @@ __device__ __forceinline__ void pri_B_fx_body(const HexArgs<double> &a, const Pr
         for (int alpha = 0; alpha < 5; alpha++) E[alpha] = s_mx[alpha];
         if (tid < NU) {
 #pragma unroll
-            for (int alpha = 0; alpha < 5; alpha++) s_u[alpha * NU + tid] = fx_from(val[alpha], E[alpha]);
+            for (int alpha = 0; alpha < 5; alpha++) s_u[alpha * NU + tid] = fx_from<FX_WS>(val[alpha], E[alpha]);
         } else if (tid < NU + NF) {
 #pragma unroll
-            for (int alpha = 0; alpha < 5; alpha++) s_c[alpha * NF + tid - NU] = fx_from(val[alpha], E[alpha]);
+            for (int alpha = 0; alpha < 5; alpha++) s_c[alpha * NF + tid - NU] = fx_from<FX_WS>(val[alpha], E[alpha]);
         }
         __syncthreads();
         const int nplist = s_pcnt;
         // 2. corrected gradient: triangle planes and z lines, then q = J^-T q~
-        int EJ = 0;
+        int EJ[3], qe[3];   // gradient component k: value = X 2^(E - 1078 - FX_WS + qe[k])
 #pragma unroll
-        for (int k = 0; k < 9; k++) EJ = max(EJ, fx_mag(g.Ji[k]) >> 20);
-        EJ += 2;   // three terms
-        const int qe = op.kD + EJ - 1022;   // gradient: value = X 2^(E - 1078 + qe)
+        for (int k = 0; k < 3; k++) {
+            EJ[k] = fx_column_exp(g.Ji, k);
+            qe[k] = op.kD + EJ[k] - 1022;
+        }
         for (int it = tid; it < 5 * NU; it += NTH) {
             const int alpha = it / NU, z = it % NU, k = z / NT_, t = z % NT_;
             const fx2 *u = s_u + alpha * NU, *c = s_c + alpha * NF;
@@ -976,7 +977,7 @@ __device__ __forceinline__ void pri_B_fx_body(const HexArgs<double> &a, const Pr
             for (int kk = 0; kk < 3; kk++) {
                 fxacc s{FX_HALF, 0};
 #pragma unroll
-                for (int d = 0; d < 3; d++) fx_mac(s, fx_factor(g.Ji[3 * d + kk], EJ), qr[d]);
+                for (int d = 0; d < 3; d++) fx_mac(s, fx_factor(g.Ji[3 * d + kk], EJ[kk]), qr[d]);
                 s_u[(5 + alpha * 3 + kk) * NU + z] = fx_limbs(fx_sum(s));
             }
         }
@@ -1005,7 +1006,7 @@ __device__ __forceinline__ void pri_B_fx_body(const HexArgs<double> &a, const Pr
 #pragma unroll
             for (int i = 0; i < 5; i++) {
                 const int f = 5 * fg + i, Ea = s_mx[f < 5 ? f : (f - 5) / 3];
-                s_tr[li * 20 + f] = fx_double(fx_sum(t[i]), Ea - 1080 + op.kF + (f < 5 ? 0 : qe), Ea >= 2047);
+                s_tr[li * 20 + f] = fx_double(fx_sum(t[i]), Ea - 1080 - FX_WS + op.kF + fx_field_exp(f, qe), Ea >= 2047);
             }
         }
         // 4. interpolation: z lines, then this thread's quadrature point in the triangle plane; the flux there
@@ -1038,7 +1039,7 @@ __device__ __forceinline__ void pri_B_fx_body(const HexArgs<double> &a, const Pr
 #pragma unroll
                 for (int t = 0; t < NT_; t++) fx_mac(s, b[t], x[t]);
                 const int alpha = i < 5 ? i : (i - 5) / 3;
-                const double v = fx_double(fx_sum(s), E[alpha] - 1080 + op.kB + (i < 5 ? 0 : qe), E[alpha] >= 2047);
+                const double v = fx_double(fx_sum(s), E[alpha] - 1080 - FX_WS + op.kB + fx_field_exp(i, qe), E[alpha] >= 2047);
                 if (i < 5) u[i] = v;
                 else gq[alpha][(i - 5) % 3] = v;
             }
