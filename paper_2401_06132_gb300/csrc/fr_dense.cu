@@ -1395,10 +1395,11 @@ int dense_phase(int phase, const HexArgs<T> &a, const OPS *ops, const FFOf<OPS> 
                 // persistent: as many CTAs as fit on the SMs (shared memory, registers, and the 512
                 // tensor-memory columns at 32 per CTA)
                 auto kern = a.tcmode == 1 ? k_dense_B<NTH, OPS, 1> : k_dense_B<NTH, OPS, 2>;
+                static SmemOptIn optin[3];
+                optin[a.tcmode](kern, smem);
                 static int occ[3] = {-1, -1, -1};
                 int &o = occ[a.tcmode];
                 if (o < 0) {
-                    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
                     cudaFuncAttributes fa{};
                     if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return -1;
                     const int by_smem = (int)(232448 / (smem + fa.sharedSizeBytes + 1024));
@@ -1418,19 +1419,13 @@ int dense_phase(int phase, const HexArgs<T> &a, const OPS *ops, const FFOf<OPS> 
             // fewer elements than resident CTAs of one element: a small handle waits for one element's chain
             // (B at 750 elements: tetrahedra 20.4 against 28.0 us with four per CTA, pyramids 29.2 against
             // 37.4; at 1,296 tetrahedra 34.9 against 31.0)
-            static bool attr = false;
-            if (!attr) {
-                cudaFuncSetAttribute(k_dense_B<NTH, OPS, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)base);
-                attr = true;
-            }
+            static SmemOptIn optin;
+            optin(k_dense_B<NTH, OPS, 0>, base);
             fr_launch(k_dense_B<NTH, OPS, 0>, grid_elems(a.ne, 8), NTH, base, s, a, ops, opsff);
         } else if (!tcdone) {
             using D = Dense32<OPS>;
-            static bool attr = false;
-            if (!attr) {
-                cudaFuncSetAttribute(k_dense_B32<OPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D::SMEM);
-                attr = true;
-            }
+            static SmemOptIn optin;
+            optin(k_dense_B32<OPS>, D::SMEM);
             fr_launch(k_dense_B32<OPS>, grid_groups(a.ne, D::EPB, 5), D::NTH, D::SMEM, s, a, ops, opsff);
         }
     } else {

@@ -3320,18 +3320,12 @@ static void launch_B(const HexArgs<T> &a, cudaStream_t s)
     constexpr int TI = 6 * 20 * S::M * S::N;
     constexpr bool FX = sizeof(T) == 8 && !SURF;
     const size_t smem = FX ? HexFxSmem<P, AA>::SMEM : (!AA ? S::LOW + S::PF : (SURF ? S::SIZE + TI : S::SIZE)) * sizeof(T);
-    static bool attr = false;
+    static SmemOptIn optin;
     if constexpr (SURF && sizeof(T) == 4) {
-        if (!attr) {
-            cudaFuncSetAttribute(k_fused_B_surf32<P, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            attr = true;
-        }
+        optin(k_fused_B_surf32<P, NT>, smem);
         fr_launch(k_fused_B_surf32<P, NT>, grid_elems(a.ne, 8), NT, smem, s, a);
     } else {
-        if (!attr) {
-            cudaFuncSetAttribute(k_fused_B<T, P, NT, 0, AA, SURF, CURV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            attr = true;
-        }
+        optin(k_fused_B<T, P, NT, 0, AA, SURF, CURV>, smem);
         fr_launch(k_fused_B<T, P, NT, 0, AA, SURF, CURV>, grid_elems(a.ne, 8), NT, smem, s, a);
     }
 }
@@ -3348,12 +3342,13 @@ static int launch_B_tc(const HexArgs<float> &a, cudaStream_t s)
     // the staged rows of the plane contractions sit after the quadrature-point buffer
     const size_t tt = (size_t)TC::TT;
     const size_t smem = TC::HEAD + (HexSmem<float, P>::SIZE + tt) * sizeof(float);
+    static SmemOptIn optin;
+    optin(k_fused_B<float, P, 128, TCM>, smem);
     static int occ = -1;
     if (occ < 0) {
         // resident CTAs per SM from the kernel's shared memory and registers (232,448 B of shared
         // memory and 64K registers per SM, 1 KB reserved per CTA); each CTA holds COLS of the 512
         // tensor-memory columns, which bounds the count too
-        cudaFuncSetAttribute(k_fused_B<float, P, 128, TCM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         cudaFuncAttributes fa{};
         if (cudaFuncGetAttributes(&fa, k_fused_B<float, P, 128, TCM>) != cudaSuccess) return -1;
         const int by_smem = (int)(232448 / (smem + fa.sharedSizeBytes + 1024));
@@ -3372,9 +3367,10 @@ template <int EPB, int NT, int MB, bool SPLIT = false>
 static int launch_B32(const HexArgs<float> &a, cudaStream_t s)
 {
     const size_t smem = (size_t)EPB * b32::ES * sizeof(float);
+    static SmemOptIn optin;
+    optin(k_hex_B32<EPB, NT, MB, SPLIT>, smem);
     static int occ = -1, nsm = 0;
     if (occ < 0) {
-        cudaFuncSetAttribute(k_hex_B32<EPB, NT, MB, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             return -1;
@@ -3391,11 +3387,8 @@ template <int P, int EPB, int NT, int MB>
 static void launch_B32p(const HexArgs<float> &a, cudaStream_t s)
 {
     constexpr size_t smem = Hex32<P, EPB>::SMEM;
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k_hex_B32p<P, EPB, NT, MB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr = true;
-    }
+    static SmemOptIn optin;
+    optin(k_hex_B32p<P, EPB, NT, MB>, smem);
     fr_launch(k_hex_B32p<P, EPB, NT, MB>, grid_elems((a.ne + EPB - 1) / EPB, MB), NT, smem, s, a);
 }
 

@@ -8,6 +8,7 @@
 #include "../../include/fr_gb300.h"
 #include "fr_ff.cuh"
 #include "fr_fx.cuh"
+#include "fr_smem.h"
 
 #define FR_NV 5
 #define FR_MAXN 6          // max 1D solution points (p <= 5)

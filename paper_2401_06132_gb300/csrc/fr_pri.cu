@@ -86,10 +86,11 @@ int pri_fused_phase(int phase, const HexArgs<T> &a, const PriOps<T> *ops, const 
             // persistent: as many CTAs as fit on the SMs (shared memory, registers, and the 512
             // tensor-memory columns at 32 per CTA)
             auto kern = a.tcmode == 1 ? k_pri_B<T, NTH, 1> : k_pri_B<T, NTH, 2>;
+            static SmemOptIn optin[3];
+            optin[a.tcmode](kern, smem);
             static int occ[3] = {-1, -1, -1};
             int &o = occ[a.tcmode];
             if (o < 0) {
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
                 cudaFuncAttributes fa{};
                 if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return -1;
                 const int by_smem = (int)(232448 / (smem + fa.sharedSizeBytes + 1024));
@@ -105,11 +106,8 @@ int pri_fused_phase(int phase, const HexArgs<T> &a, const PriOps<T> *ops, const 
         }
         if (!tcdone) {
             const size_t smem = sizeof(T) == 8 ? FX_SMEM : P32_SMEM;
-            static bool attr = false;
-            if (!attr) {
-                cudaFuncSetAttribute(k_pri_B<T, NTH, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                attr = true;
-            }
+            static SmemOptIn optin;
+            optin(k_pri_B<T, NTH, 0>, smem);
             fr_launch(k_pri_B<T, NTH, 0>, grid_elems(a.ne, 8), NTH, smem, s, a, ops, ops64);
         }
     } else {
