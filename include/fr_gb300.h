@@ -186,7 +186,10 @@ fr_status fr_rk4_step_host(fr_mesh *m, void *U_host, double dt, int nsteps, void
 
 /* Autotuner: times every launch shape of the volume kernel of each hexahedral group (one element
  * type and order) on the given device state U_dev (R_dev is scratch output) and keeps the fastest
- * for later calls. Shapes: 0, 1, 2 = one element per CTA of 64, 128 or 256 threads; for FP32 (and
+ * for later calls. Shapes: 0, 1, 2 = one element per CTA of 64, 128 or 256 threads; in the low-Mach form
+ * with flux anti-aliasing on affine elements (CUDA cores) instead 0 = one element per CTA of 96 threads, 1 = two
+ * elements (p = 4: one) of 128, or one of 256 in a group of up to two elements per SM, 2 = two elements of 160
+ * (p = 4: one of 224); for FP32 (and
  * the mixed forms without hexahedral tensor cores) at p = 3 with flux anti-aliasing on affine
  * elements also 3, 4 = eight elements per CTA of 160 threads, each sum-factorised operator applied
  * to a whole field by one thread from registers (one CTA per SM with up to 255 registers, or two).

@@ -1909,7 +1909,8 @@ extern "C" fr_status fr_rhs_phase(fr_mesh *m, int phase, const void *U_dev, void
 }
 
 // Launch shapes of a hexahedral group's volume kernel: 0, 1, 2 = one element per CTA of 64, 128,
-// 256 threads; FP32 p = 3 with flux anti-aliasing on the CUDA cores also 3, 4 = eight elements per
+// 256 threads (the low-Mach form with flux anti-aliasing: one or two elements of 96 to 256, fused_phase in
+// fr_hex.cu); FP32 p = 3 with flux anti-aliasing on the CUDA cores also 3, 4 = eight elements per
 // CTA with register-resident line sweeps (one or two CTAs per SM).
 static int volume_shapes(const fr_mesh *m, const Block &b)
 {

@@ -19,8 +19,9 @@ FR_OK, FR_EINVAL, FR_ENOMEM, FR_ECUDA, FR_EMESH, FR_ETIMEOUT, FR_ENONPHYS, FR_EU
 STATUS_NAMES = ["FR_OK", "FR_EINVAL", "FR_ENOMEM", "FR_ECUDA", "FR_EMESH", "FR_ETIMEOUT", "FR_ENONPHYS",
                 "FR_EUNSUPPORTED", "FR_EBOUNDS"]
 PRECISIONS = {"fp64": 0, "fp32": 1, "mixed_bf16": 2, "mixed_fp16": 3}
-# volume-kernel launch shapes (fr_autotune, fr_set_volume_shape): threads per element, or elements per
-# CTA with register-resident sweeps and the CTAs per SM
+# volume-kernel launch shapes by index (fr_autotune, fr_set_volume_shape): threads per element, or elements per
+# CTA with register-resident sweeps and the CTAs per SM. (64, 128 and 256 name the indices 0, 1 and 2 in the
+# low-Mach form with flux anti-aliasing too, whose kernels take other threads and elements per CTA.)
 SHAPES = (64, 128, 256, "8/CTA x1", "8/CTA x2", "2/CTA split")
 FORMS = {"fused": 0, "unfused": 1}
 
@@ -170,6 +171,7 @@ class FRMesh:
         self.h = h
         self.prec = params[0].prec
         self.n_inst = len(meshes)
+        self._lowmach = self._is_lowmach(params)
 
     @classmethod
     def part(cls, mesh: dict, params: Params, nparts: int, part: int) -> "FRMesh":
@@ -182,7 +184,13 @@ class FRMesh:
         self.h = h
         self.prec = params.prec
         self.n_inst = 1
+        self._lowmach = cls._is_lowmach([params])
         return self
+
+    @staticmethod
+    def _is_lowmach(params) -> bool:
+        """Whether a handle takes the low-Mach form: reduced precision, a reference state in every instance."""
+        return params[0].prec != PRECISIONS["fp64"] and all(p.p_ref > 0 and p.rho_ref > 0 for p in params)
 
     def halo_info(self) -> dict:
         info = (C.c_longlong * 7)()
@@ -304,8 +312,8 @@ class FRMesh:
 
     def autotune(self, U, R, stream=None, cache: str | None = None):
         """Pick the fastest volume-kernel launch shape per group on this state; returns the choices.
-        With `cache` (a JSON file), a choice stored there for the same device, precision, element type
-        and order is applied without timing, and new choices are added to it."""
+        With `cache` (a JSON file), a choice stored there for the same device, precision, element type,
+        order and, in the low-Mach form, size class is applied without timing, and new choices are added to it."""
         self._check_tensor(U)
         self._check_tensor(R)
         keys = self._shape_keys() if cache else None
@@ -334,11 +342,21 @@ class FRMesh:
         return [SHAPES[v] for v in out if v >= 0]
 
     def _shape_keys(self):
-        """Cache key of each group's volume-kernel shape (None for groups without a choice)."""
+        """Cache key of each group's volume-kernel shape (None for groups without a choice). The low-Mach form
+        with flux anti-aliasing runs kernels of its own, and other ones up to two elements per SM, so a choice
+        for one says nothing about the others."""
         import torch
         dev = torch.cuda.get_device_name()
         prec = {v: k for k, v in PRECISIONS.items()}[self.prec]
-        return [f"{dev}|{prec}|type{g['type']}|p{g['p']}|m{g['m']}" if g["shapes"] > 1 else None for g in self.groups()]
+        small = 2 * torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+
+        def key(g):
+            k = f"{dev}|{prec}|type{g['type']}|p{g['p']}|m{g['m']}"
+            if self._lowmach and g["m"] == g["p"] + 2:
+                k += "|lowmach" + ("|small" if g["elements"] <= small else "")
+            return k
+
+        return [key(g) if g["shapes"] > 1 else None for g in self.groups()]
 
     def set_merged(self, on: bool):
         """fr_set_merged: one launch per phase over all element groups."""
