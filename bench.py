@@ -41,10 +41,9 @@ def workload_name(n=N_EDGE, p=P, m=MQ):
 # FP64 peak of the chip from its unit counts and clock: 152 SMs x 2 FP64 FMA/clock x 2 FLOP x 2.07 GHz
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # DRAM bytes (read + written) per element of one FP64 volume-kernel launch, from one Nsight Compute
-# capture on the 40^3 p = 3 box (859.1 MB / 64,000 elements; the 164 MB state is larger than L2; taken
-# with the operators in FP64 arithmetic, which reads and writes the same arrays); the kernel touches each element's inputs and outputs once, so a launch's traffic
-# scales with its element count
-VOLUME_FP64_DRAM_BYTES_PER_ELEMENT = 859.063808e6 / 64000
+# capture on the 40^3 p = 3 box (861.8 MB / 64,000 elements; the 164 MB state is larger than L2); the
+# kernel touches each element's inputs and outputs once, so a launch's traffic scales with its element count
+VOLUME_FP64_DRAM_BYTES_PER_ELEMENT = 861.812224e6 / 64000
 
 # ---------------------------------------------------------------------------------------------
 # FLOP model of the fused volume kernel (phase B), FMA = 2 FLOP; counted from its arithmetic
@@ -73,18 +72,21 @@ def phase_b_flops_per_element(p=P, m=MQ, one_sided=True, diagonal_metric=True, d
     return con_u + grad + jt + face + interp + tdisf + proj + div
 
 
+# FP64 operations that total_flux and viscous_normal_flux run per point (a reciprocal is three multiply-adds)
+POINT_FLUX_FP64_FLOPS, VISC_NORMAL_FP64_FLOPS = 123, 99
+
+
 def phase_b_fp64_pipe_flops_per_element(p=P, m=MQ):
-    """The part of phase_b_flops_per_element that the FP64 kernel runs on the FP64 pipe: common solution,
-    J^-T, viscous normal flux and point flux. Its linear operators (interpolation, projection, gradient,
-    traces) run in block fixed point on the integer multipliers."""
-    n = p + 1
-    nu, nf, nq = n ** 3, 6 * n * n, m ** 3
-    return 5 * nf * 3 + 5 * nu * 3 + nf // 2 * VISC_NORMAL_FLOPS + nq * (POINT_FLUX_FLOPS + TRANSFORM_FLOPS)
+    """What the FP64 kernel runs on the FP64 pipe on an axis-aligned element at beta = 1/2: the viscous normal
+    flux and the point flux. Its linear operators (interpolation, projection, gradient, traces) and the
+    diagonal metric's factors run in block fixed point on the integer multipliers, and the common solution
+    is a copy."""
+    return 6 * (p + 1) ** 2 // 2 * VISC_NORMAL_FP64_FLOPS + m ** 3 * POINT_FLUX_FP64_FLOPS
 
 
-def tet_phase_b_fp64_pipe_flops_per_element(nu=20, nf=40):
-    """The same part of tet_phase_b_flops_per_element."""
-    return 5 * nf * 3 + 5 * nu * 15 + nf // 2 * VISC_NORMAL_FLOPS + 125 * (POINT_FLUX_FLOPS + 90)
+def dense_phase_b_fp64_pipe_flops_per_element(nf=40):
+    """The same of a tetrahedron (nf = 40) or pyramid (56): det J J^-1 f is on the FP64 pipe too."""
+    return nf // 2 * VISC_NORMAL_FP64_FLOPS + 125 * (POINT_FLUX_FP64_FLOPS + 90)
 
 
 def tet_phase_b_flops_per_element(nu=20, nf=40, nfaces=4):
@@ -359,7 +361,7 @@ def other_configs(args, torch, fr, W):
         out[f"tet24_{name}"].update({"volume_kernel_ms": b_ms, "volume_tflops": tfl,
                                      "flops_per_element": tet_phase_b_flops_per_element()})
         if prec == "fp64":
-            out[f"tet24_{name}"]["volume_fp64_pipe_frac"] = (tet_phase_b_fp64_pipe_flops_per_element() * nt / (b_ms * 1e-3) / 1e12
+            out[f"tet24_{name}"]["volume_fp64_pipe_frac"] = (dense_phase_b_fp64_pipe_flops_per_element() * nt / (b_ms * 1e-3) / 1e12
                                                              / FP64_PEAK_TFLOPS)
         del Uc, Rc
         if prec != "fp64":
@@ -414,7 +416,7 @@ def other_configs(args, torch, fr, W):
                                 "volume_tflops": fl_y * ny / (b_ms * 1e-3) / 1e12, "flops_per_element": fl_y}
         del Uc, Rc
         if prec == "fp64":
-            out["pyr20_fp64"]["volume_fp64_pipe_frac"] = (tet_phase_b_fp64_pipe_flops_per_element(30, 56) * ny / (b_ms * 1e-3)
+            out["pyr20_fp64"]["volume_fp64_pipe_frac"] = (dense_phase_b_fp64_pipe_flops_per_element(56) * ny / (b_ms * 1e-3)
                                                           / 1e12 / FP64_PEAK_TFLOPS)
             m64 = m
         else:

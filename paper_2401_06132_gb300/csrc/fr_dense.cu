@@ -182,7 +182,8 @@ k_dense_disu(HexArgs<float> a, const OPS *__restrict__ op, const FFOf<OPS> *__re
 }
 
 // The same in FP64, with the face values in block fixed point (fr_fx.cuh): on the FP64 pipe the 5 NU
-// multiply-adds per flux point bounded the kernel. A thread keeps its column of M0 in registers.
+// multiply-adds per flux point bounded the kernel (11^3 hexahedron/pyramid box, face phase 92 -> 38 us). A
+// thread keeps its column of M0 in registers.
 template <typename OPS, int EPB>
 __global__ void __launch_bounds__(OPS::NF * EPB) k_dense_disu_fx(HexArgs<double> a, const OPS *__restrict__ ops)
 {
@@ -944,7 +945,7 @@ __global__ void __launch_bounds__(128, OPS::NU <= 20 ? 5 : 4) k_dense_B32(HexArg
 // FP64 pipe. Blocks: each variable with its common solution; the three transformed flux components of
 // a variable, which the projection adds up. The quadrature-point fields never leave the registers: a
 // thread interpolates the 20 fields to its point, evaluates the flux there and keeps the 15 transformed
-// components until the CTA knows their largest magnitudes.
+// components until the CTA knows their largest magnitudes. Measured, 12^3 Kuhn box (10,368 tetrahedra): 2.53 -> 0.79 ms.
 template <typename OPS, int NTH>
 __global__ void __launch_bounds__(NTH, 4) k_dense_B_fx(HexArgs<double> a, const OPS *__restrict__ ops)
 {
@@ -1417,8 +1418,8 @@ int dense_phase(int phase, const HexArgs<T> &a, const OPS *ops, const FFOf<OPS> 
             fr_launch(k_dense_B_fx<OPS, NTH>, grid_elems(a.ne, 4), NTH, 0, s, a, ops);
         } else if (!tcdone && a.ne < 8 * fr_sms()) {
             // fewer elements than resident CTAs of one element: a small handle waits for one element's chain
-            // (B at 750 elements: tetrahedra 20.4 against 28.0 us with four per CTA, pyramids 29.2 against
-            // 37.4; at 1,296 tetrahedra 34.9 against 31.0)
+            // (B at 750 elements, below the line: tetrahedra 20.2 against 27.1 us with four per CTA, pyramids 26.4
+            // against 36.7; at 1,296, above it: 34.8 against 30.9 and 47.3 against 42.9)
             static SmemOptIn optin;
             optin(k_dense_B<NTH, OPS, 0>, base);
             fr_launch(k_dense_B<NTH, OPS, 0>, grid_elems(a.ne, 8), NTH, base, s, a, ops, opsff);

@@ -291,7 +291,7 @@ __device__ __forceinline__ void disu_blk_body(const HexArgs<T> &a, long long fir
 }
 
 // The same in FP64, with the traces in block fixed point (fr_fx.cuh): on the FP64 pipe the 20 multiply-adds
-// per flux point bounded the kernel.
+// per flux point bounded the kernel (48^3 p = 3: 0.378 -> 0.222 ms).
 template <int P, int EB, int NT>
 __device__ __forceinline__ void disu_fx_body(const HexArgs<double> &a, long long first, long long stride)
 {
@@ -666,7 +666,7 @@ __device__ __forceinline__ void project_5(const HexOps<T> &op, const T *src, T *
 // twelve decades inside an element.
 // What is left on the FP64 pipe: 80 operations per quadrature point and 70 per viscous flux point, 55% of
 // its cycles; the rest is latency (integer chains, barriers, instruction fetch) at 20 warps per SM.
-// Measured, 48^3 p = 3: 15.5 -> 5.48 ms per launch; 25^3 p = 4: 4.18 -> 1.60 ms. Collocation, per RHS:
+// Measured, 48^3 p = 3: 15.5 -> 5.44 ms per launch; 25^3 p = 4: 4.18 -> 1.61 ms. Collocation, per RHS:
 // 48^3 p = 3 7.72 -> 4.80 ms (this kernel 3.33), 25^3 p = 4 with every other kernel 2.42 -> 1.23 ms.
 // y = A x along one line, rows to fixed-point limbs.
 template <int R, int C, int LD>
@@ -1741,7 +1741,7 @@ __device__ __forceinline__ void fused_B_body(const HexArgs<T> &a, long long firs
 // (n^2 -> m^2 values), its z factor is formed by the quadrature point's own thread from 16-byte loads
 // that the points of a column share, and the projection is one thread's level (z, then x, then y,
 // streaming row by row). EPB elements per CTA fill the warps; the stages alternate between two buffers.
-// Measured: 5,800 warp instructions and 1,380 wavefronts per element; 48^3 p = 3 0.982 -> 0.781 ms,
+// Measured: 5,680 warp instructions and 1,510 wavefronts per element; 48^3 p = 3 0.982 -> 0.781 ms,
 // 32^3 p = 4 0.633 -> 0.541 ms per launch.
 // Layouts: a plane of the state and the gradient starts PS words after the last and a field FS words,
 // which spreads a warp's (field, plane) threads over distinct banks; interpolated planes and fluxes put
@@ -2098,8 +2098,9 @@ __device__ __forceinline__ void volume_body(const HexArgs<T> &a, long long first
 // The FP32 affine p = 3 volume kernel without a reference state is capped at 48 registers per thread: ten CTAs of 128 threads
 // per SM (more warps to hide its shared-memory latency; an eleventh, which its shared memory would
 // allow, needs 40 registers, spills and measured slower). The FP64 fixed-point kernel is capped at 96
-// registers, five CTAs of 128 threads per SM as its shared memory allows (measured on its first form: four CTAs
-// 6.99, three 7.50, five 6.66 ms at 48^3 p = 3). A minimum of 0 CTAs leaves the register count to the compiler (an
+// registers, five CTAs of 128 threads per SM as its shared memory allows at p = 3 (48^3: five CTAs 5.44, four and
+// three 5.55 ms; at p = 4, where shared memory holds three, the caps for four and three give 1.59 against
+// 1.61 ms at 25^3). A minimum of 0 CTAs leaves the register count to the compiler (an
 // explicit 1 lets it take up to 255).
 template <typename T, int P, int NT, int TCM, bool AA, bool SURF, bool CURV>
 constexpr int fused_B_min_ctas()
@@ -2127,7 +2128,7 @@ __global__ void __launch_bounds__(NT, 896 / NT) k_fused_B_surf32(HexArgs<float> 
 // ---------------------------------------------------------------------------------------------
 // FP64: R += lift of the common flux held in block fixed point (D: [variable][flux point], exponent fields
 // E), R *= -1/det J, and the RK4 stage update. On the FP64 pipe the six multiply-adds per value were half
-// of the lift kernel's operations.
+// of the lift kernel's operations (48^3 p = 3: 0.561 -> 0.404 ms).
 // p = 3 loads R and the stage sums of its three values per thread before the common flux arrives (the
 // kernel waits on memory: 0.404 to 0.375 ms at 48^3 elements); the five of p = 4 would cost too many
 // registers (0.103 to 0.145 ms at 25^3) and are loaded one by one.
@@ -3398,8 +3399,11 @@ static int fused_phase(int phase, const HexArgs<T> &a, cudaStream_t s, int varia
     if (a.ne == 0) return 0;
     if (phase == 0) {
         // fewer elements than one CTA of eight per SM: one element per CTA (the latency of eight elements'
-        // points in one CTA is what a small handle waits for: FP32 p = 3, 27 elements 12.4 to 8.6 us, 512
-        // elements 11.7 to 8.8; p = 4, 512 elements 15.1 to 11.3)
+        // points in one CTA is what a small handle waits for). Measured, us with one / eight per CTA, FP32 p = 3:
+        // 27 elements 8.6 / 12.4, 512 9.5 / 10.9, 1,000 9.0 / 11.4; above the line 1,331 9.4 / 11.5, 2,744
+        // 13.1 / 14.4, 4,096 14.7 / 14.8, 8,000 23.1 / 21.3, 21,952 54.5 / 44.8. The other forms cross later (FP64
+        // 8,000: 26.6 / 29.0, 21,952: 58.7 / 54.0; p = 4 FP32 8,000: 40.9 / 47.0), so the line lies on the safe side
+        // for many elements, where the face phase counts, at the price of 1 to 6 us between it and the crossing
         if (a.ne < 8 * fr_sms()) {
             fr_launch(k_disu_blk<T, P, 1, 128>, a.ne, 128, 0, s, a);
         } else {

